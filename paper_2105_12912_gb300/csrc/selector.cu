@@ -48,27 +48,50 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 
 // Forward and backward over rows gw, gw + nw, ... of every warp; per-CTA sums of the
 // unscaled gradient (d(e^2)/dy = 2e), of e^2 and of the row count go to part[cta].
+//
+// Bound by instruction issue (about 250 warp instructions a row).  Lane i owns row i of
+// W2 and dW2, whose packed layout puts the 32 lanes' words in 32 cache lines (and one
+// bank): the parameters are staged in shared memory with W2's rows padded to 33 words,
+// and dW2 is handed over transposed with the same padding, so that neither the loads
+// nor the reduction serialise (28,672 rows: 39 us a launch with the strided accesses,
+// 20 us so, both with the events around it).
+constexpr int kPitch = kMlpHid + 1;
+constexpr int kStage = kMlpHid * (kPitch - kMlpHid);  // words the padding adds
+// a parameter's word in the padded layout: W2's entries at pitch 33
+__device__ __forceinline__ int padded(int p) {
+  return p < kMlpW2 ? p : (p < kMlpB2 ? p + (p - kMlpW2) / kMlpHid : p + kStage);
+}
+// the same for the sums, which hold dW2 transposed
+__device__ __forceinline__ int padded_t(int p) {
+  if (p < kMlpW2 || p >= kMlpB2) return padded(p);
+  const int k = p - kMlpW2;
+  return kMlpW2 + (k % kMlpHid) * kPitch + k / kMlpHid;
+}
 __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __restrict__ w,
                                                                  const float* __restrict__ feat,
                                                                  const float* __restrict__ tgt,
                                                                  const uint8_t* __restrict__ valid,
                                                                  uint64_t n, float* __restrict__ part) {
-  __shared__ float s_red[kTrainWarps][kPart];
+  __shared__ float s_red[kTrainWarps][kPart + kStage];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float* sw = s_red[0];  // the staged parameters, until the sums need the words
+  for (int p = threadIdx.x; p < kMlpParams; p += kTrainThreads) sw[padded(p)] = w[p];
+  __syncthreads();
   float w1[kMlpIn], w2r[kMlpHid], w2c[kMlpHid], w3[kMlpOut], b3[kMlpOut];
-  const float b1 = w[kMlpB1 + lane], b2 = w[kMlpB2 + lane];
+  const float b1 = sw[kMlpB1 + lane], b2 = sw[kMlpB2 + kStage + lane];
 #pragma unroll
-  for (int j = 0; j < kMlpIn; j++) w1[j] = w[kMlpW1 + lane * kMlpIn + j];
+  for (int j = 0; j < kMlpIn; j++) w1[j] = sw[kMlpW1 + lane * kMlpIn + j];
 #pragma unroll
   for (int j = 0; j < kMlpHid; j++) {
-    w2r[j] = w[kMlpW2 + lane * kMlpHid + j];
-    w2c[j] = w[kMlpW2 + j * kMlpHid + lane];
+    w2r[j] = sw[kMlpW2 + lane * kPitch + j];
+    w2c[j] = sw[kMlpW2 + j * kPitch + lane];
   }
 #pragma unroll
   for (int c = 0; c < kMlpOut; c++) {
-    w3[c] = w[kMlpW3 + c * kMlpHid + lane];
-    b3[c] = w[kMlpB3 + c];
+    w3[c] = sw[kMlpW3 + kStage + c * kMlpHid + lane];
+    b3[c] = sw[kMlpB3 + kStage + c];
   }
+  __syncthreads();
   float g1[kMlpIn], g2[kMlpHid], g3[kMlpOut], gb3[kMlpOut];
   float gb1 = 0.0f, gb2 = 0.0f, loss = 0.0f, cnt = 0.0f;
 #pragma unroll
@@ -132,39 +155,69 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __
   for (int j = 0; j < kMlpIn; j++) my[kMlpW1 + lane * kMlpIn + j] = g1[j];
   my[kMlpB1 + lane] = gb1;
 #pragma unroll
-  for (int j = 0; j < kMlpHid; j++) my[kMlpW2 + lane * kMlpHid + j] = g2[j];
-  my[kMlpB2 + lane] = gb2;
+  for (int j = 0; j < kMlpHid; j++) my[kMlpW2 + j * kPitch + lane] = g2[j];
+  my[kMlpB2 + kStage + lane] = gb2;
 #pragma unroll
-  for (int c = 0; c < kMlpOut; c++) my[kMlpW3 + c * kMlpHid + lane] = g3[c];
+  for (int c = 0; c < kMlpOut; c++) my[kMlpW3 + kStage + c * kMlpHid + lane] = g3[c];
   if (lane == 0) {
 #pragma unroll
-    for (int c = 0; c < kMlpOut; c++) my[kMlpB3 + c] = gb3[c];
-    my[kMlpParams] = loss;
-    my[kMlpParams + 1] = cnt;
+    for (int c = 0; c < kMlpOut; c++) my[kMlpB3 + kStage + c] = gb3[c];
+    my[kStage + kMlpParams] = loss;
+    my[kStage + kMlpParams + 1] = cnt;
   }
   __syncthreads();
   for (int p = threadIdx.x; p < kPart; p += kTrainThreads) {
     float acc = 0.0f;
+    const int q = padded_t(p);
 #pragma unroll
-    for (int wv = 0; wv < kTrainWarps; wv++) acc += s_red[wv][p];
+    for (int wv = 0; wv < kTrainWarps; wv++) acc += s_red[wv][q];
     part[(uint64_t)blockIdx.x * kPart + p] = acc;
   }
 }
 
-// Sum of the CTA partials in CTA order (double), scaled to the mean over rows and
-// outputs; optionally one Adam step on the weights.  Thread p handles parameter p;
-// thread kMlpParams writes the loss.
-__global__ __launch_bounds__(256) void mlp_update_kernel(const float* __restrict__ part, int nparts,
-                                                         float* __restrict__ w, float* __restrict__ grad_out,
-                                                         double* __restrict__ loss_out, float* __restrict__ m,
-                                                         float* __restrict__ v, uint32_t step, float lr) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kMlpParams) return;
-  double cnt = 0.0, acc = 0.0;
-  for (int g = 0; g < nparts; g++) {
-    cnt += part[(uint64_t)g * kPart + kMlpParams + 1];
-    acc += part[(uint64_t)g * kPart + p];
+// Sum of the CTA partials (double), scaled to the mean over rows and outputs;
+// optionally one Adam step on the weights.  Parameter kMlpParams is the loss.
+//
+// Bound by latency: a thread that adds all 304 partials of its parameter waits for
+// them one after another (106 us a step).  So a CTA takes 32 parameters, its 32 warps
+// add every 32nd partial each (at most ten loads, all in flight, 128 bytes a row), and
+// warp w then adds parameter w's 32 sums across its lanes -- always in the same order,
+// so runs stay reproducible.  c1, c2: Adam's bias corrections of this step.
+constexpr int kUpdThreads = 1024, kUpdParams = 32;
+__global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* __restrict__ part, int nparts,
+                                                                 float* __restrict__ w,
+                                                                 float* __restrict__ grad_out,
+                                                                 double* __restrict__ loss_out,
+                                                                 float* __restrict__ m, float* __restrict__ v,
+                                                                 uint32_t step, float lr, float c1, float c2) {
+  __shared__ double s_sum[32][kUpdParams + 1];
+  __shared__ double s_c[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int p0 = blockIdx.x * kUpdParams;
+  {
+    double acc = 0.0;
+    const int p = min(p0 + lane, kMlpParams);
+#pragma unroll 10
+    for (int g = wid; g < nparts; g += 32) acc += part[(uint64_t)g * kPart + p];
+    s_sum[wid][lane] = acc;
   }
+  // row counts: whole numbers, at most 2^24 rows a CTA and 2^53 in all
+  double cnt = 0.0;
+  for (int g = threadIdx.x; g < nparts; g += kUpdThreads) cnt += part[(uint64_t)g * kPart + kMlpParams + 1];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
+  if (lane == 0) s_c[wid] = cnt;
+  __syncthreads();
+  const int p = p0 + wid;
+  if (p > kMlpParams) return;
+  double acc = s_sum[lane][wid];
+  cnt = s_c[lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    acc += __shfl_xor_sync(~0u, acc, o);
+    cnt += __shfl_xor_sync(~0u, cnt, o);
+  }
+  if (lane != 0) return;
   const double scale = cnt > 0.0 ? 1.0 / (3.0 * cnt) : 0.0;
   if (p == kMlpParams) {
     if (loss_out) *loss_out = acc * scale;
@@ -177,8 +230,6 @@ __global__ __launch_bounds__(256) void mlp_update_kernel(const float* __restrict
     const float vt = kAdamB2 * v[p] + (1.0f - kAdamB2) * gr * gr;
     m[p] = mt;
     v[p] = vt;
-    const float c1 = (float)(1.0 - pow((double)kAdamB1, (double)step));
-    const float c2 = (float)(1.0 - pow((double)kAdamB2, (double)step));
     w[p] -= lr * (mt / c1) / (sqrtf(vt / c2) + kAdamEps);
   }
 }
@@ -232,7 +283,10 @@ cudaError_t launch_mlp_grad(const float* w, const float* feat, const float* tgt,
 cudaError_t launch_mlp_update(const float* part, int nparts, float* w, float* grad, double* loss, float* m,
                               float* v, uint32_t step, float lr, cudaStream_t s) {
   trace_begin(K_MLP_UPDATE, s);
-  mlp_update_kernel<<<(kMlpParams + 1 + 255) / 256, 256, 0, s>>>(part, nparts, w, grad, loss, m, v, step, lr);
+  const float c1 = (float)(1.0 - std::pow((double)kAdamB1, (double)step));
+  const float c2 = (float)(1.0 - std::pow((double)kAdamB2, (double)step));
+  mlp_update_kernel<<<(kMlpParams + kUpdParams) / kUpdParams, kUpdThreads, 0, s>>>(part, nparts, w, grad, loss, m, v,
+                                                                                  step, lr, c1, c2);
   trace_end(K_MLP_UPDATE, s);
   return cudaGetLastError();
 }
