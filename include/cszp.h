@@ -230,7 +230,7 @@ typedef struct csz_batch csz_batch;
 #define CSZ_BATCH_STAGED 2     /* candidates: the staged launches */
 #define CSZ_BATCH_PERSISTENT 4 /* candidates: the single persistent launch */
 
-/* Workspace for a batch (0 if any field is invalid); it includes 124 KB per field of
+/* Workspace for a batch (0 if any field is invalid); it includes 92 KB per field of
    working memory for the persistent plan's run-length books. */
 size_t csz_batch_workspace_bytes(int nfields, const csz_field* fields);
 csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_options* opt,

@@ -396,7 +396,7 @@ __device__ const Log2Table kLog2Table = make_log2_table();
 __device__ __forceinline__ uint32_t log2_q16_small(uint32_t v) { return __ldg(&kLog2Table.v[v]); }
 
 // ---------------------------------------------------------------------------------
-// canonical Huffman codes from lengths (block-wide).  Codes are ordered by
+// canonical Huffman codes from lengths (block-wide, whole warps).  Codes are ordered by
 // (length, symbol); the first code of length l is (first(l-1) + count(l-1)) << 1.
 // Outputs per symbol its code and its rank in (length, symbol) order; per length
 // the first code, the count and the offset of its first symbol in that order.
@@ -417,6 +417,7 @@ __device__ inline void canonical_build(const uint8_t* len, int nsym, CanonSmem* 
   for (int l = tid; l <= kMaxLen; l += nt) cs->cnt[l] = 0;
   if (tid == 0) cs->bad = 0;
   const int nchunk = nsym / 32;
+  static_assert(kNsymLen / 32 <= 128 && kMaxLen == 64, "the prefixes below cover the chunks and the lengths");
   for (int i = tid; i < nchunk * (kMaxLen + 1); i += nt) wcnt[i] = 0;
   __syncthreads();
   // per-warp-chunk counts and ranks by length
@@ -431,25 +432,41 @@ __device__ inline void canonical_build(const uint8_t* len, int nsym, CanonSmem* 
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    unsigned long long c = 0;
-    uint32_t o = 0;
-    cs->first[0] = 0;
-    cs->off[0] = 0;
-    for (int l = 1; l <= kMaxLen; l++) {
-      c = (c + (l > 1 ? cs->cnt[l - 1] : 0u)) << 1;
-      cs->first[l] = c;
-      cs->off[l] = o;
-      o += cs->cnt[l];
+  // Warp 0: first codes and offsets by scans over the lengths (lane i: lengths 2i + 1 and
+  // 2i + 2).  With F(l) the 64-bit left-justified end of the codes shorter than l,
+  // first(l) = F(l) >> (64 - l): the recurrence above without its serial chain.  (F wraps
+  // to 0 only where a complete code ends: no longer code follows.)
+  if (tid < 32) {
+    const int l1 = 2 * tid + 1, l2 = l1 + 1;
+    const uint32_t n1 = cs->cnt[l1], n2 = cs->cnt[l2];
+    const unsigned long long e1 = (unsigned long long)n1 << (64 - l1), e2 = (unsigned long long)n2 << (64 - l2);
+    const unsigned long long F1 = warp_incl_scan(e1 + e2) - (e1 + e2);
+    const uint32_t o1 = warp_incl_scan(n1 + n2) - (n1 + n2);
+    cs->first[l1] = F1 >> (64 - l1);
+    cs->first[l2] = (F1 + e1) >> (64 - l2);
+    cs->off[l1] = o1;
+    cs->off[l2] = o1 + n1;
+    if (tid == 0) {
+      cs->first[0] = 0;
+      cs->off[0] = 0;
     }
   }
-  // prefix of per-chunk counts over chunks, per length (in place)
-  for (int l = 1 + tid; l <= kMaxLen; l += nt) {
-    uint32_t run = 0;
-    for (int ch = 0; ch < nchunk; ch++) {
-      uint16_t c = wcnt[ch * (kMaxLen + 1) + l];
-      wcnt[ch * (kMaxLen + 1) + l] = (uint16_t)run;
-      run += c;
+  // exclusive prefix of per-chunk counts over the chunks, a warp per length that occurs
+  // (in place; at most 128 chunks, four a lane)
+  for (int l = 1 + (tid >> 5); l <= kMaxLen; l += nt >> 5) {
+    if (cs->cnt[l] == 0) continue;
+    const int c0 = 4 * (tid & 31);
+    uint32_t c[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      c[k] = c0 + k < nchunk ? wcnt[(c0 + k) * (kMaxLen + 1) + l] : 0u;
+      sum += c[k];
+    }
+    uint32_t run = warp_incl_scan(sum) - sum;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (c0 + k < nchunk) wcnt[(c0 + k) * (kMaxLen + 1) + l] = (uint16_t)run;
+      run += c[k];
     }
   }
   __syncthreads();

@@ -260,13 +260,30 @@ __global__ __launch_bounds__(256) void range_batch_kernel(const RangeTask* __res
 
 constexpr int kBookThreads = 1024;
 
-// Ascending sort of L distinct keys by merging runs: an element's place in the merged
-// run is its index in its own run plus the number of smaller keys in the partner run
-// (binary search).  a holds the keys on entry and on exit; b is scratch of L keys.
+// Ascending sort of L distinct keys.  Warps first sort runs of 32 in registers (bitonic,
+// by shuffles; no barrier), then runs merge: an element's place in the merged run is its
+// index in its own run plus the number of smaller keys in the partner run (binary
+// search).  a holds the keys on entry and on exit; b is scratch.  Both have room for L
+// rounded up to 32.
 __device__ void rank_merge_sort_u64(uint64_t* a, uint64_t* b, int L) {
   uint64_t* src = a;
   uint64_t* dst = b;
-  for (int run = 1; run < L; run <<= 1) {
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < ((L + 31) & ~31); i += blockDim.x) {
+    uint64_t k = i < L ? a[i] : ~0ull;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+      for (int o = size >> 1; o; o >>= 1) {
+        const uint64_t z = __shfl_xor_sync(~0u, k, o);
+        const bool low = ((lane & o) == 0) == ((lane & size) == 0 || size == 32);
+        k = (z < k) == low ? z : k;
+      }
+    }
+    a[i] = k;
+  }
+  __syncthreads();
+  for (int run = 32; run < L; run <<= 1) {
     for (int i = threadIdx.x; i < L; i += blockDim.x) {
       const uint64_t k = src[i];
       const int r = i / run;
@@ -294,9 +311,9 @@ __device__ void rank_merge_sort_u64(uint64_t* a, uint64_t* b, int L) {
 }
 
 // One CTA per book: 0 quant codes [1024], 1 run values [1024], 2 run lengths [4096].
-// Shared memory (bytes): len 4K | sym 8K | weight by node 32K | parent by node 16K |
-// region A 32K (sort keys, live node list, canonical scratch) | region B 32K (sort
-// scratch, new nodes, depth pass).
+// Shared memory (bytes): len 4K | sym 8K | parent by node 16K | region A 32K (sort keys,
+// live node list, canonical scratch) | region B 32K (sort scratch, new nodes, depth
+// pass): 92 KB, two such CTAs an SM.
 // =================================================================================
 // record offsets: exclusive prefix of the blocks' record counts (one CTA)
 // =================================================================================
@@ -327,10 +344,65 @@ __device__ void record_offsets_body(const BookArgs& a) {
   }
 }
 
-// Working memory of one book over nsym symbols: len nsym B | sym 2 nsym | weight by
-// node 8 nsym | parent by node 4 nsym | region A 8 nsym (sort keys, live node list,
-// canonical scratch) | region B 8 nsym (sort scratch, new nodes, depth pass).
-__host__ __device__ constexpr uint32_t book_mem_bytes(int nsym) { return 31u * (uint32_t)nsym; }
+// Working memory of one book over nsym symbols: len nsym B | sym 2 nsym | parent by node
+// 4 nsym | region A 8 nsym (sort keys, live node list, canonical scratch) | region B
+// 8 nsym (sort scratch, new nodes, depth pass).
+__host__ __device__ constexpr uint32_t book_mem_bytes(int nsym) { return 23u * (uint32_t)nsym; }
+
+// Keys of live nodes: (weight, internal, node id), the order in which the sequential
+// two-queue method picks them (weight, leaves before internal nodes, creation order).
+constexpr uint64_t kNodeClass = 1ull << 13, kNodeId = kNodeClass - 1;
+
+// Merging rounds of one warp (no barrier) over the sorted live list A[0..n) and the
+// queue B[0..) of the nodes made here, which come in nondecreasing order: each round the
+// warp takes the 32 lightest live nodes in order (the elementwise minimum of one list
+// and the other reversed holds them as a bitonic sequence), and with t the sum of the
+// two lightest merges every consecutive pair whose second member weighs <= t: those
+// precede the node of weight t in the order above, so the sequential method would merge
+// them too before it comes up again.  Node ids next, next + 1, ...  Returns the number
+// of nodes made; *p_out, *q_out: the first live elements of A and B.  Stops when one
+// node is left, or after kDenseRounds full rounds in a row.
+//
+// Bound by latency: about 400 cycles a round for up to 16 merges, where the two-queue
+// method took one thread 190-220 cycles a merge (code histograms are sparse at their
+// rare end, so few pairs qualify at a time and rounds of the whole CTA, 2500 cycles
+// each, do not pay).  The launch with the 2-D 1800x3600 field's 1024-symbol book: 90 us
+// before, 33 us so (a run of 324 symbols: 39 and 19 us).
+constexpr int kDenseRounds = 12;
+__device__ __forceinline__ int merge_warp(const uint64_t* A, int n, uint64_t* B, uint16_t* par, uint32_t next,
+                                          int* p_out, int* q_out) {
+  const int lane = threadIdx.x & 31;
+  int p = 0, q = 0, e = 0, dense = 0;
+  while (n - p + e - q > 1 && dense < kDenseRounds) {
+    uint64_t x = p + lane < n ? A[p + lane] : ~0ull;
+    const int j = q + 31 - lane;
+    const uint64_t y = j < e ? B[j] : ~0ull;
+    x = y < x ? y : x;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const uint64_t z = __shfl_xor_sync(~0u, x, o);
+      x = (z < x) == ((lane & o) == 0) ? z : x;
+    }
+    const uint64_t mate = __shfl_xor_sync(~0u, x, 1);
+    const uint64_t sum = (x >> 14) + (mate >> 14);
+    const uint64_t t = __shfl_sync(~0u, sum, 0);
+    // (the pairs' heavier weights ascend: those within t are the first k)
+    const int k = __popc(__ballot_sync(~0u, !(lane & 1) && mate != ~0ull && (mate >> 14) <= t));
+    const bool in = lane < 2 * k;
+    const uint32_t id = next + (uint32_t)(e + (lane >> 1));
+    if (in) par[x & kNodeId] = (uint16_t)id;
+    if (in && !(lane & 1)) B[e + (lane >> 1)] = (sum << 14) | kNodeClass | id;
+    const int from_b = __popc(__ballot_sync(~0u, in && (uint32_t)(x & kNodeId) >= next));
+    q += from_b;
+    p += 2 * k - from_b;
+    e += k;
+    dense = k == 16 ? dense + 1 : 0;
+    __syncwarp();
+  }
+  *p_out = p;
+  *q_out = q;
+  return e;
+}
 
 // One canonical book (role 0 code, 1 run value, 2 run length) or, role 3, the
 // record offsets of a field, by a CTA of NT threads.  mem: book_mem_bytes(nsym) of
@@ -350,21 +422,26 @@ __device__ void codebook_core(const BookArgs& a, int role, unsigned char* mem) {
 
   uint8_t* s_len = mem;
   uint16_t* s_sym = reinterpret_cast<uint16_t*>(mem + nsym);
-  uint32_t* s_wt = reinterpret_cast<uint32_t*>(mem + 3 * nsym);
-  uint16_t* s_par = reinterpret_cast<uint16_t*>(mem + 11 * nsym);
-  uint64_t* A = reinterpret_cast<uint64_t*>(mem + 15 * nsym);
-  uint64_t* B = reinterpret_cast<uint64_t*>(mem + 23 * nsym);
+  uint16_t* s_par = reinterpret_cast<uint16_t*>(mem + 3 * nsym);
+  uint64_t* A = reinterpret_cast<uint64_t*>(mem + 7 * nsym);
+  uint64_t* B = reinterpret_cast<uint64_t*>(mem + 15 * nsym);
   __shared__ uint32_t s_L;
-  __shared__ int s_n, s_k, s_next;
+  __shared__ int s_n, s_k, s_next, s_p, s_q, s_e;
   __shared__ CanonSmem cs;
   const int tid = threadIdx.x;
 
   if (tid == 0) s_L = 0;
   for (int s = tid; s < nsym; s += blockDim.x) s_len[s] = 0;
   __syncthreads();
+  // the symbols that occur, in any order (one counter update a warp)
+#pragma unroll 4
   for (int s = tid; s < nsym; s += blockDim.x) {
     const uint32_t f = hist[s];
-    if (f) A[atomicAdd(&s_L, 1u)] = ((uint64_t)f << 12) | (uint64_t)s;
+    const uint32_t has = __ballot_sync(~0u, f != 0);
+    uint32_t at = 0;
+    if ((tid & 31) == 0 && has) at = atomicAdd(&s_L, (uint32_t)__popc(has));
+    at = __shfl_sync(~0u, at, 0) + __popc(has & ((1u << (tid & 31)) - 1u));
+    if (f) A[at] = ((uint64_t)f << 12) | (uint64_t)s;
   }
   __syncthreads();
   const int L = (int)s_L;
@@ -374,154 +451,115 @@ __device__ void codebook_core(const BookArgs& a, int role, unsigned char* mem) {
     // leaves in (frequency, symbol) order
     rank_merge_sort_u64(A, B, L);
     for (int i = tid; i < L; i += blockDim.x) {
-      s_wt[i] = (uint32_t)(A[i] >> 12);
-      s_sym[i] = (uint16_t)(A[i] & 0xfff);
+      const uint64_t key = A[i];
+      s_sym[i] = (uint16_t)(key & 0xfff);
+      A[i] = ((key >> 12) << 14) | (uint64_t)i;
     }
-    __syncthreads();
-    const int nn = 2 * L - 1;
-    // ---- pairing rounds ----------------------------------------------------------
-    // Keys order the live nodes as the sequential two-queue method picks them:
-    // (weight, leaves before internal nodes, creation order).  With t the sum of the
-    // two lightest, every consecutive pair whose second member weighs <= t precedes
-    // the new node of weight t in that order, so all such pairs merge in one round;
-    // the new nodes are rank-merged back.  When a round would merge few pairs the
-    // rest is finished by the sequential loop, from the same state.
-    constexpr uint64_t kClass = 1ull << 13, kIdx = kClass - 1;
-    for (int i = tid; i < L; i += blockDim.x) A[i] = ((uint64_t)s_wt[i] << 14) | (uint64_t)i;
     if (tid == 0) {
       s_n = L;
       s_next = L;
     }
     __syncthreads();
+    const int nn = 2 * L - 1;
+    // ---- merging rounds ----------------------------------------------------------
+    // A round of the whole CTA merges every qualifying pair of the live list (the rule of
+    // merge_warp) and rank-merges the new nodes back; it costs as much as six rounds of
+    // one warp, so warp 0 goes alone unless kBlockPairs pairs qualify, and the CTA
+    // rank-merges what it leaves in the same way.
+    constexpr int kBlockPairs = 96;
     while (true) {
       const int n = s_n;
       if (n <= 1) break;
-      if (tid == 0) {
+      const int next = s_next;
+      if (tid < 32) {
+        // qualifying pairs i, weight(A[2i+1]) <= t, up to kBlockPairs or, if that many, all
         const uint64_t t = (A[0] >> 14) + (A[1] >> 14);
-        int lo = 0, hi = n / 2;  // pairs i with weight(A[2i+1]) <= t
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if ((A[2 * mid + 1] >> 14) <= t) lo = mid + 1;
-          else hi = mid;
+        int k = 0;
+        if (n >= 2 * kBlockPairs && (A[2 * kBlockPairs - 1] >> 14) <= t) {
+          int lo = kBlockPairs, hi = n / 2;
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((A[2 * mid + 1] >> 14) <= t) lo = mid + 1;
+            else hi = mid;
+          }
+          k = lo;
+        } else {
+          int p, q;
+          const int e = merge_warp(A, n, B, s_par, (uint32_t)next, &p, &q);
+          if (tid == 0) {
+            s_p = p;
+            s_q = q;
+            s_e = e;
+          }
         }
-        s_k = lo;
+        if (tid == 0) s_k = k;
       }
       __syncthreads();
       const int k = s_k;
-      if (k < 16) break;
-      const int next = s_next;
-      for (int i = tid; i < k; i += blockDim.x) {
-        const uint64_t x = A[2 * i], y = A[2 * i + 1];
-        const uint64_t wn = (x >> 14) + (y >> 14);
-        const uint32_t id = (uint32_t)next + i;
-        s_par[x & kIdx] = (uint16_t)id;
-        s_par[y & kIdx] = (uint16_t)id;
-        s_wt[id] = (uint32_t)wn;
-        B[i] = (wn << 14) | kClass | id;
+      // left over after the round: A[p..n) and the new nodes B[q..e)
+      int p = 2 * k, q = 0, e = k;
+      if (k) {
+        for (int i = tid; i < k; i += blockDim.x) {
+          const uint64_t x = A[2 * i], y = A[2 * i + 1];
+          const uint64_t wn = (x >> 14) + (y >> 14);
+          const uint32_t id = (uint32_t)next + i;
+          s_par[x & kNodeId] = (uint16_t)id;
+          s_par[y & kNodeId] = (uint16_t)id;
+          B[i] = (wn << 14) | kNodeClass | id;
+        }
+        __syncthreads();
+      } else {
+        p = s_p;
+        q = s_q;
+        e = s_e;
       }
-      __syncthreads();
-      const int nr = n - 2 * k;
+      const int na = n - p, live = na + e - q;
+      if (live == 1) break;  // the root
       uint64_t mine[(kNsymLen + NT - 1) / NT];
       int dst[(kNsymLen + NT - 1) / NT], cnt = 0;
-      for (int i = tid; i < n - k; i += blockDim.x) {
-        const bool from_rest = i < nr;
-        const uint64_t x = from_rest ? A[2 * k + i] : B[i - nr];
-        const uint64_t* other = from_rest ? B : A + 2 * k;
-        int lo = 0, hi = from_rest ? k : nr;
+      for (int i = tid; i < live; i += blockDim.x) {
+        const bool from_a = i < na;
+        const uint64_t x = from_a ? A[p + i] : B[q + i - na];
+        const uint64_t* other = from_a ? B + q : A + p;
+        int lo = 0, hi = from_a ? e - q : na;
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
           if (other[mid] < x) lo = mid + 1;
           else hi = mid;
         }
         mine[cnt] = x;
-        dst[cnt] = (from_rest ? i : i - nr) + lo;
+        dst[cnt] = (from_a ? i : i - na) + lo;
         cnt++;
       }
       __syncthreads();
       for (int c = 0; c < cnt; c++) A[dst[c]] = mine[c];
       if (tid == 0) {
-        s_n = n - k;
-        s_next = next + k;
+        s_n = live;
+        s_next = next + e;
       }
       __syncthreads();
     }
-    if (tid == 0) {
-      // sequential finish; consumed leaves and internal nodes are prefixes of their
-      // queues, so the live list gives the queue fronts
-      const int n = s_n;
-      int live_leaves = 0;
-      for (int i = 0; i < n; i++) live_leaves += (A[i] & kClass) ? 0 : 1;
-      int qi = L - live_leaves, nxt = s_next, qj = nxt - (n - live_leaves);
-      constexpr uint32_t INF = 0xffffffffu;
-      uint32_t l0 = qi < L ? s_wt[qi] : INF, l1 = qi + 1 < L ? s_wt[qi + 1] : INF,
-               l2 = qi + 2 < L ? s_wt[qi + 2] : INF;
-      uint32_t i0 = qj < nxt ? s_wt[qj] : INF, i1 = qj + 1 < nxt ? s_wt[qj + 1] : INF;
-      while (nxt < nn) {
-        int pk[2];
-        uint32_t pw[2];
-#pragma unroll
-        for (int t = 0; t < 2; t++) {
-          if (l0 <= i0) {
-            pk[t] = qi;
-            pw[t] = l0;
-            qi++;
-            l0 = l1;
-            l1 = l2;
-            l2 = qi + 2 < L ? s_wt[qi + 2] : INF;
-          } else {
-            pk[t] = qj;
-            pw[t] = i0;
-            qj++;
-            i0 = i1;
-            i1 = qj + 1 < nxt ? s_wt[qj + 1] : INF;
-          }
-        }
-        const uint32_t sum = pw[0] + pw[1];
-        s_wt[nxt] = sum;
-        s_par[pk[0]] = (uint16_t)nxt;
-        s_par[pk[1]] = (uint16_t)nxt;
-        if (qj == nxt) {
-          i0 = sum;
-        } else if (qj + 1 == nxt) {
-          i1 = sum;
-        }
-        nxt++;
-      }
-      s_par[nn - 1] = (uint16_t)(nn - 1);
-    }
+    if (tid == 0) s_par[nn - 1] = (uint16_t)(nn - 1);
     __syncthreads();
-    // depths by pointer jumping (region B)
-    uint16_t* s_anc = reinterpret_cast<uint16_t*>(B);
-    uint16_t* s_dep = s_anc + 2 * nsym;
-    for (int i = tid; i < nn; i += blockDim.x) {
-      s_anc[i] = s_par[i];
-      s_dep[i] = (i == nn - 1) ? 0 : 1;
-    }
+    // depths by pointer jumping (region B): word i holds node i's ancestor and how far up
+    // it is.  The words are updated in place: one that has already moved on this round
+    // still names an ancestor and its distance.  Done once every ancestor is the root.
+    volatile uint32_t* s_up = reinterpret_cast<uint32_t*>(B);
+    for (int i = tid; i < nn; i += blockDim.x) s_up[i] = ((uint32_t)s_par[i] << 16) | (i == nn - 1 ? 0u : 1u);
     __syncthreads();
-    // (done once every node's ancestor is the root: the depths no longer change)
-    for (int step = 1; step < nn; step <<= 1) {
-      uint16_t na[(2 * kNsymLen + NT - 1) / NT], nd[(2 * kNsymLen + NT - 1) / NT];
-      int c = 0;
-      bool open = false;
+    bool open = true;
+    while (__syncthreads_or(open)) {
+      open = false;
       for (int i = tid; i < nn; i += blockDim.x) {
-        const uint16_t an = s_anc[i];
-        nd[c] = s_dep[i] + s_dep[an];
-        na[c] = s_anc[an];
-        open |= na[c] != (uint16_t)(nn - 1);
-        c++;
+        const uint32_t w = s_up[i], u = s_up[w >> 16];
+        const uint32_t v = (u & 0xffff0000u) | ((w & 0xffffu) + (u & 0xffffu));
+        s_up[i] = v;
+        open |= (v >> 16) != (uint32_t)(nn - 1);
       }
-      __syncthreads();
-      c = 0;
-      for (int i = tid; i < nn; i += blockDim.x) {
-        s_dep[i] = nd[c];
-        s_anc[i] = na[c];
-        c++;
-      }
-      if (!__syncthreads_or(open)) break;
     }
     for (int i = tid; i < L; i += blockDim.x) {
-      const uint16_t d = s_dep[i];
-      if (d > kMaxLen) atomicOr(&a.st->status, ERR_RANGE);
+      const uint32_t d = s_up[i] & 0xffffu;
+      if (d > (uint32_t)kMaxLen) atomicOr(&a.st->status, ERR_RANGE);
       s_len[s_sym[i]] = (uint8_t)d;
     }
   }
