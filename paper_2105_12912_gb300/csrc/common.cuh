@@ -38,6 +38,14 @@ __host__ __device__ constexpr uint32_t lut_entry(uint32_t sym, uint32_t len) { r
 __host__ __device__ constexpr int lut_len(uint32_t e) { return (int)(e & 15u); }
 __host__ __device__ constexpr int lut_sym(uint32_t e) { return (int)(e >> 4); }
 static_assert(kLutBits <= 15 && kNsymLen <= 4096, "symbol and length fit a 16-bit entry");
+// second level (books of 1024 symbols): 16-bit entries, (symbol << 4) | (length -
+// kLutBits), for codes of up to kLut2Max bits whose cell lies inside one code (0: not
+// resolved)
+constexpr int kLut2Size = 2048;
+constexpr int kLut2Max = kLutBits + 15;
+__host__ __device__ constexpr uint32_t lut2_entry(uint32_t sym, uint32_t len) { return (sym << 4) | (len - kLutBits); }
+__host__ __device__ constexpr int lut2_len(uint32_t e) { return (int)(e & 15u) + kLutBits; }
+__host__ __device__ constexpr int lut2_sym(uint32_t e) { return (int)(e >> 4); }
 constexpr uint32_t kSpinLimit = 1u << 20;
 
 enum : int { CODEC_HUFF = 0, CODEC_RLE = 1, CODEC_RLE_HUFF = 2 };

@@ -190,15 +190,22 @@ __device__ void dec_records_body(const DecodeArgs& a, uint32_t cta, uint32_t nct
   }
 }
 
-// One CTA per book: lengths from the archive, Kraft check, canonical tables and a
-// 14-bit lookup table (16-bit entries).
+// One CTA per book: lengths from the archive, Kraft check, canonical tables, the
+// kLutBits-bit lookup table (16-bit entries) and the second-level table of longer codes.
+// Bound by latency (one CTA per book, ahead of the whole decoding), so nothing here runs
+// serially over the 64 lengths or searches per table entry: lengths map to lanes, and a
+// thread fills eight lookup entries at a time, at one store where they share a code.
 __device__ void dec_tables_body(const DecodeArgs& a, int book) {
   if (a.dead) return;
   __shared__ uint8_t s_len[kNsymLen];
   __shared__ uint16_t s_wcnt[(kNsymLen / 32) * (kMaxLen + 1)];
+  __shared__ uint16_t s_sorted[kNsymLen];
   __shared__ CanonSmem cs;
   __shared__ uint32_t s_cnt[kMaxLen + 2];
-  __shared__ uint32_t s_bad;
+  // the limits' upper words, all ones once the code space is full (a limit of at most 31
+  // bits that is not full never reads all ones; longer ones are not looked up here)
+  __shared__ uint32_t s_lim[kMaxLen + 1];
+  __shared__ uint32_t s_bad, s_full[2];
   const int tid = threadIdx.x;
   const int nsym = book == 2 ? kNsymLen : kNsymCode;
   DecTab* t = &a.tabs[book];
@@ -220,16 +227,25 @@ __device__ void dec_tables_body(const DecodeArgs& a, int book) {
     else if (l) atomicAdd(&s_cnt[l], 1u);
   }
   __syncthreads();
-  if (tid == 0) {
-    long long avail = 1;
-    for (int l = 1; l <= kMaxLen; l++) {
-      avail = avail * 2 - (long long)s_cnt[l];
-      if (avail < 0) {
-        s_bad = 1;
-        break;
-      }
-      if (avail > (1ll << 40)) avail = 1ll << 40;
+  if (tid < 32) {
+    // Kraft sum in 2^-64 steps, exactly: whole parts, and the fractions' upper and lower
+    // words (no sum of 64 such words overflows 64 bits)
+    uint64_t whole = 0, fh = 0, fl = 0;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int l = 2 * tid + 1 + k;
+      const uint64_t c = s_cnt[l], f = c << (64 - l);
+      whole += l < 64 ? c >> l : 0ull;
+      fh += f >> 32;
+      fl += f & 0xffffffffull;
     }
+    whole = warp_sum(whole);
+    fh = warp_sum(fh);
+    fl = warp_sum(fl);
+    fh += fl >> 32;
+    whole += fh >> 32;
+    const bool frac = (fh & 0xffffffffull) != 0 || (fl & 0xffffffffull) != 0;
+    if (tid == 0 && (whole > 1 || (whole == 1 && frac))) s_bad = 1;
   }
   __syncthreads();
   if (s_bad) {
@@ -239,48 +255,83 @@ __device__ void dec_tables_body(const DecodeArgs& a, int book) {
     }
     return;
   }
-  canonical_build(s_len, nsym, &cs, s_wcnt, nullptr, t->sorted);
-  for (int l = tid; l <= kMaxLen; l += blockDim.x) {
+  canonical_build(s_len, nsym, &cs, s_wcnt, nullptr, s_sorted);
+  if (tid == 0) s_bad = s_full[0] = s_full[1] = 0;  // s_bad: now the largest length
+  __syncthreads();
+  if (tid <= kMaxLen) {
+    // canonical codes of length l, left-justified to 64 bits, end at
+    // (first_l + count_l) << (64-l); these ends never decrease, and wrap to 0 where the
+    // code space is exhausted
+    const int l = tid;
+    const unsigned long long end = cs.first[l] + cs.cnt[l];
+    const unsigned long long lim = l == 0 ? 0ull : end << (64 - l);
+    const bool full = l > 0 && lim == 0 && cs.off[l] + cs.cnt[l] > 0;
     t->first[l] = cs.first[l];
     t->count[l] = cs.cnt[l];
     t->off[l] = cs.off[l];
+    t->limit[l] = lim;
+    s_lim[l] = full ? ~0u : (uint32_t)(lim >> 32);
+    if (l > 0 && cs.cnt[l]) atomicMax(&s_bad, (uint32_t)l);
+    if (full && l < 64) atomicOr(&s_full[l >> 5], 1u << (l & 31));
   }
+  for (int s = tid; s < nsym; s += blockDim.x) t->sorted[s] = s_sorted[s];
+  __syncthreads();
+  const int maxlen = (int)s_bad;
+  // the second level: cells of 2^s2 in the code space above the codes of kLutBits bits
+  const uint32_t top = s_lim[kLutBits];
+  const uint32_t rest = 0u - top;  // 0 when the table holds every code (top all ones: 1)
+  int s2 = 0;
+  while (s2 < 32 && ((rest - 1u) >> s2) >= (uint32_t)kLut2Size) s2++;
   if (tid == 0) {
-    // canonical codes of length l, left-justified to 64 bits, occupy
-    // [first_l << (64-l), (first_l + count_l) << (64-l)); these ends never decrease
-    uint32_t mx = 0;
-    unsigned long long lim = 0, full = 0;
-    for (int l = 1; l <= kMaxLen; l++) {
-      if (cs.cnt[l]) {
-        mx = l;
-        const unsigned long long end = cs.first[l] + cs.cnt[l];
-        if (l == 64) {
-          lim = end;
-        } else if ((end >> l) != 0) {
-          full |= ~0ull << l;  // the code space is exhausted from this length on
-          lim = 0;
-        } else {
-          lim = end << (64 - l);
-        }
-      }
-      t->limit[l] = lim;
-    }
-    t->fullmask = full;
-    t->limit[0] = 0;
-    t->maxlen = mx;
+    t->fullmask = ((unsigned long long)s_full[1] << 32) | s_full[0];
+    t->maxlen = (uint32_t)maxlen;
     t->present = 1;
+    t->lut2_base = top;
+    t->lut2_shift = (uint32_t)s2;
   }
-  // lookup: for each kLutBits-bit prefix, the code of length <= kLutBits it starts with
-  for (int v = tid; v < (1 << kLutBits); v += blockDim.x) {
-    uint32_t e = 0;
-    for (int l = 1; l <= kLutBits; l++) {
-      const uint64_t c = (uint64_t)(v >> (kLutBits - l));
-      if (cs.cnt[l] && c >= cs.first[l] && c - cs.first[l] < cs.cnt[l]) {
-        e = lut_entry(t->sorted[cs.off[l] + (uint32_t)(c - cs.first[l])], (uint32_t)l);
-        break;
+  uint32_t lim[kLutBits + 1];
+#pragma unroll
+  for (int l = 1; l <= kLutBits; l++) lim[l] = s_lim[l];
+  // length of the code that prefix v starts with: the smallest whose codes end above it
+  auto entry = [&](uint32_t v) -> uint32_t {
+    const uint32_t x = v << (32 - kLutBits);
+    int l = 1;
+#pragma unroll
+    for (int k = 1; k <= kLutBits; k++) l += x >= lim[k] ? 1 : 0;
+    if (l > kLutBits) return 0u;
+    return lut_entry(s_sorted[cs.off[l] + (v >> (kLutBits - l)) - (uint32_t)cs.first[l]], (uint32_t)l);
+  };
+  for (uint32_t g = tid; g < (1u << kLutBits) / 8; g += blockDim.x) {
+    uint32_t e[8];
+    e[0] = entry(8 * g);
+    if (e[0] && lut_len(e[0]) <= kLutBits - 3) {
+#pragma unroll
+      for (int k = 1; k < 8; k++) e[k] = e[0];
+    } else {
+#pragma unroll 1
+      for (int k = 1; k < 8; k++) {
+        const uint32_t v = entry(8 * g + k);
+#pragma unroll
+        for (int j = 1; j < 8; j++) e[j] = j == k ? v : e[j];
       }
     }
-    t->lut[v] = (LutEntry)e;
+    reinterpret_cast<uint4*>(t->lut)[g] =
+        make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16);
+  }
+  for (uint32_t c = tid; book < 2 && c < (uint32_t)kLut2Size; c += blockDim.x) {
+    const uint64_t x = (uint64_t)top + ((uint64_t)c << s2);
+    uint32_t e = 0;
+    if (x < ~0u && rest > 1u) {
+      int l = kLutBits + 1;
+      while (l <= kLut2Max && l <= maxlen && (uint32_t)x >= s_lim[l]) l++;
+      // a cell inside one code (its 2^(32-l) values) resolves it
+      if (l <= kLut2Max && l <= maxlen && 32 - l >= s2) {
+        const uint64_t code = x >> (32 - l);
+        if (code - cs.first[l] < cs.cnt[l])
+          e = lut2_entry(s_sorted[cs.off[l] + (uint32_t)(code - cs.first[l])], (uint32_t)l);
+      }
+    }
+    t->lut2()[c] = (uint16_t)e;
   }
 }
 
@@ -307,16 +358,16 @@ struct BookView {
   const uint32_t* count;
   const uint32_t* off;
   const uint16_t* sorted;
+  const uint16_t* lut2;  // second-level table (codes just longer than kLutBits), lut2_n cells
+  uint32_t lut2_n, lut2_base, lut2_shift;
   int maxlen;
   unsigned long long fullmask;
 };
 
-// Matching the next codeword among the nb valid top bits of bb.  A table code of
-// length l <= nb found among the zero-padded top kLutBits bits is the next codeword (no
-// codeword is a prefix of another).  A table miss with more than kLutBits bits at hand is
-// a longer code: its length is the smallest one whose left-justified codes end above
-// bb (a binary search over the canonical limits), the true length whenever it is <= nb
-// (zero bits below nb cannot complete a shorter codeword), checked to be a codeword.
+// Matching the next codeword among the nb valid top bits of bb, for a code longer than
+// the lookup table's: its length is the smallest one whose left-justified codes end
+// above bb (a binary search over the canonical limits), the true length whenever it is
+// <= nb (zero bits below nb cannot complete a shorter codeword), checked to be a codeword.
 // Returns that length (0 if none fits in nb bits) and sets sym.
 __device__ __forceinline__ int ihs_match_long(uint64_t bb, int nb, const BookView& bk, int& sym) {
   int lo = kLutBits + 1, hi = bk.maxlen + 1;  // smallest k whose codes end above bb
@@ -332,109 +383,180 @@ __device__ __forceinline__ int ihs_match_long(uint64_t bb, int nb, const BookVie
   return lo;
 }
 
-// A warp's reader of one interleaved stream in[0..avail).  The warp reads the stream
-// strictly in order, so the next 96 units are kept in three 32-unit register windows
-// (lane i holds unit base+i of each); a top-up takes its unit from a window by
-// shuffle and a window is reloaded (one 64-byte load) two windows before it is
-// needed, so no load sits on the decode's critical path.
+// A warp's reader of one interleaved stream in[0..avail).
+//
+// Bound by instruction issue (it is the decoder's inner loop), so the step rests on two
+// facts of the unit order.  A lane takes units only until its next code is complete, so
+// it enters every step with at most 15 bits: its state is one 32-bit word.  And whether
+// nb bits hold a whole code needs no table: exactly when, zero-padded, they lie below the
+// end of the canonical codes of up to nb bits -- 16 words, one per lane, read by a
+// shuffle.  So a step is one compare, one ballot, one unit and one table lookup; a code
+// of up to 16 bits is complete after one unit, and the lookup misses only for codes
+// longer than the table (a second-level table, then a search).  The step this replaces
+// looked up twice and kept 64-bit windows: 159 warp instructions per 32 symbols with the
+// reconstruction, 693 us at 3-D 512^3 (rel 1e-4; 941 us when one block's run codec put
+// the other books' tables beside the code book's and halved the occupancy).  This one:
+// 415 us either way, 2-D 1800x3600 61 -> 33 us.
+//
+// The stream's next 128 units wait in a ring in shared memory; each half is refilled
+// from registers loaded one half ahead, so no load sits on the step's path.
 struct IhsReader {
   const uint16_t* __restrict__ in;
   uint32_t avail;
-  uint32_t w0, w1, w2;
-  uint32_t wbase;  // stream index of w0's lane 0
+  uint32_t ring;   // shared-memory address of the warp's 128 units, 256-byte aligned
+  uint32_t lim;    // lane 16 - k: the end of the codes of up to k bits, upper word
+  uint32_t p0, p1; // this lane's units of the half after the ring's
   uint32_t cur;    // units taken so far by the warp
-  uint64_t bb;     // this lane's bits, left-aligned
-  int nb;
+  uint32_t half;   // cur reaching this refills the half before it
+  uint32_t bb;     // this lane's bits, left-aligned
+  int sh;          // 16 - (number of bits): 1..16 between steps
   bool bad;        // this lane met a damaged stream
 
   __device__ __forceinline__ uint32_t fetch(uint32_t i) const { return i < avail ? (uint32_t)__ldg(&in[i]) : 0u; }
+  __device__ __forceinline__ uint32_t unit(uint32_t i) const {
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(((2u * i) & 254u) | ring) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ void put(uint32_t i, uint32_t v) const {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(((2u * i) & 254u) | ring), "h"((uint16_t)v) : "memory");
+  }
 
-  __device__ __forceinline__ void init(const uint16_t* p, uint32_t n) {
+  __device__ __forceinline__ void init(const uint16_t* p, uint32_t n, const BookView& bk, uint32_t ring_addr) {
     const uint32_t lane = threadIdx.x & 31;
     in = p;
     avail = n;
-    w0 = fetch(lane);
-    w1 = fetch(32 + lane);
-    w2 = fetch(64 + lane);
-    wbase = 0;
+    ring = ring_addr;
+    uint32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) v[k] = fetch(32 * k + lane);
+    p0 = fetch(128 + lane);
+    p1 = fetch(160 + lane);
+    const int k = 16 - (int)lane;  // (lanes 0 and 17 to 31 are never read)
+    lim = k >= 0 && k < 16 ? (((bk.fullmask >> k) & 1ull) ? ~0u : (uint32_t)(bk.limit[k] >> 32)) : 0u;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; i++) put(32 * i + lane, v[i]);
+    __syncwarp();
     cur = 0;
+    half = 64;
     bb = 0;
-    nb = 0;
+    sh = 16;
     bad = false;
   }
 
-  // One decoding step of the 32 lanes (every lane calls): each active lane tops up
-  // its bits in rounds until a codeword is complete, then consumes it.  Returns the
-  // symbol, meaningful where the lane was active and is not bad.  Control flow is
-  // warp-uniform: a round's unit goes in by selects, and the search for codes longer
-  // than the table runs only when some lane has one.
-  __device__ __forceinline__ int step(bool active, const BookView& bk) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
-    const bool live = active && !bad;
-    uint32_t e = bk.lut[(uint32_t)(bb >> (64 - kLutBits))];
-    int l = lut_len(e);
-    int sym = lut_sym(e);
-    int ml = (live && (uint32_t)(l - 1) < (uint32_t)nb) ? l : 0;  // a table code within the bits
-    bool lng = live && l == 0 && nb > kLutBits;
-    if (__any_sync(~0u, lng)) {
-      if (lng) ml = ihs_match_long(bb, nb, bk, sym);
+  __device__ __forceinline__ void advance(uint32_t taken) {
+    cur += taken;
+    if (cur >= half) {
+      const uint32_t lane = threadIdx.x & 31;
+      __syncwarp();
+      put(half + lane + 64, p0);
+      put(half + lane + 96, p1);
+      __syncwarp();
+      p0 = fetch(half + 128 + lane);
+      p1 = fetch(half + 160 + lane);
+      half += 64;
     }
-    bool need = live && ml == 0;
-    uint32_t ballot = __ballot_sync(~0u, need);
-    while (ballot != 0u) {
-      const uint32_t before = __popc(ballot & lt);
-      const uint32_t rel = cur - wbase + before;  // < 64 while cur - wbase < 32
-      const uint32_t u0 = __shfl_sync(~0u, w0, rel & 31);
-      const uint32_t u1 = __shfl_sync(~0u, w1, rel & 31);
-      const bool over = nb > 64 - 16 || cur + before >= avail;
-      bad = bad || (need && over);
-      const bool take = need && !over;
-      const uint64_t unit = (uint64_t)(rel < 32 ? u0 : u1) << ((48 - nb) & 63);
-      bb |= take ? unit : 0ull;
-      nb += take ? 16 : 0;
-      cur += __popc(ballot);
-      if (cur - wbase >= 32) {
-        w0 = w1;
-        w1 = w2;
-        wbase += 32;
-        w2 = fetch(wbase + 64 + lane);
-      }
-      // only lanes that took a unit look again
-      e = bk.lut[(uint32_t)(bb >> (64 - kLutBits))];
-      l = lut_len(e);
-      if (take && (uint32_t)(l - 1) < (uint32_t)nb) {
-        ml = l;
-        sym = lut_sym(e);
-      }
-      lng = take && l == 0 && nb > kLutBits;
-      if (__any_sync(~0u, lng)) {
-        if (lng) ml = ihs_match_long(bb, nb, bk, sym);
-      }
-      need = take && ml == 0;
-      ballot = __ballot_sync(~0u, need);
-    }
-    bb = ml >= 64 ? 0ull : bb << ml;  // ml = 0 where the lane consumes nothing
-    nb -= ml;
-    return live ? sym : 0;
   }
+
+  // Lanes with `open`: the code is longer than the tables resolve, or incomplete.  They
+  // search, and take further units in rounds until it is complete (at most 48 bits are
+  // held before a unit: more marks the stream damaged).  Returns the symbol and leaves
+  // the state past the code.
+  __device__ __forceinline__ int step_long(bool open, const BookView& bk) {
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+    uint64_t w = (uint64_t)bb << 32;
+    int nb = 16 - sh, ml = 0, sym = 0;
+    const bool mine = open;
+    while (true) {
+      if (open) ml = ihs_match_long(w, nb, bk, sym);
+      const bool need = open && ml == 0;
+      const uint32_t ballot = __ballot_sync(~0u, need);
+      if (ballot == 0u) break;
+      const bool over = nb > 48;
+      bad = bad || (need && over);
+      const uint64_t u = unit(cur + __popc(ballot & lt));
+      open = need && !over;
+      if (open) {
+        w |= u << (48 - nb);
+        nb += 16;
+      }
+      advance(__popc(ballot));
+    }
+    if (mine) {
+      w = ml > 0 && ml < 64 && !bad ? w << ml : 0ull;
+      bb = (uint32_t)(w >> 32);
+      sh = bad ? 16 : 16 - (nb - ml);
+    }
+    return sym;
+  }
+
+  // One decoding step of the 32 lanes (every lane calls): each active lane whose bits
+  // hold no whole code takes the next unit, then consumes its code.  Returns the
+  // symbol, meaningful where the lane was active and is not bad.
+  __device__ __forceinline__ int step(bool active, const BookView& bk) {
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+    const uint32_t end = __shfl_sync(~0u, lim, sh);  // (by every lane, active or not)
+    const bool need = active && bb >= end;
+    const uint32_t ballot = __ballot_sync(~0u, need);
+    const uint32_t u = unit(cur + __popc(ballot & lt));
+    if (need) {
+      bb |= u << sh;
+      sh -= 16;
+    }
+    advance(__popc(ballot));
+    const uint32_t e = bk.lut[bb >> (32 - kLutBits)];
+    int l = lut_len(e), sym = lut_sym(e);
+    const bool miss = active && e == 0u;
+    if (__builtin_expect(__any_sync(~0u, miss), 0)) {
+      bool open = miss;
+      if (miss) {
+        // (bb lies at or above the second level's base: the lookup missed.  A damaged
+        // stream can point past its cells.)
+        const uint32_t c = (bb - bk.lut2_base) >> bk.lut2_shift;
+        const uint32_t e2 = c < bk.lut2_n ? (uint32_t)__ldg(&bk.lut2[c]) : 0u;
+        const int l2 = lut2_len(e2);
+        if (e2 != 0u && l2 <= 16 - sh) {
+          l = l2;
+          sym = lut2_sym(e2);
+          open = false;
+        }
+      }
+      if (__any_sync(~0u, open)) {
+        const int s3 = step_long(open, bk);
+        if (open) {
+          sym = s3;
+          l = 0;
+        }
+      }
+    }
+    if (active) {
+      bb <<= l;
+      sh += l;
+    }
+    return sym;
+  }
+
+  // After the last step: the warp's verdict on the stream (uniform).
+  __device__ __forceinline__ bool sound() const { return !__any_sync(~0u, bad) && cur <= avail; }
 };
 
 // One warp decodes N symbols (+add) from in[0..avail) into out[].  Returns false
 // (warp-uniform) if the stream is damaged; *used gets the units read.
 __device__ bool ihs_decode_warp(const uint16_t* __restrict__ in, uint32_t avail, uint32_t N,
-                                const BookView& bk, uint16_t* out, int add, uint32_t* used) {
+                                const BookView& bk, uint16_t* out, int add, uint32_t* used, uint32_t ring) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t T = (N + 31) / 32;
   IhsReader rd;
-  rd.init(in, avail);
+  rd.init(in, avail, bk, ring);
+#pragma unroll 1
   for (uint32_t t = 0; t < T; t++) {
     const bool active = 32 * t + lane < N;
     const int sym = rd.step(active, bk);
     if (active && !rd.bad) out[32 * t + lane] = (uint16_t)(sym + add);
   }
   *used = rd.cur;
-  return !__any_sync(~0u, rd.bad);
+  return rd.sound();
 }
 
 __device__ __forceinline__ float scale(int32_t k, float ebx2) { return __fmul_rn(__int2float_rn(k), ebx2); }
@@ -549,11 +671,12 @@ struct RecordCursor {
 // writes its 2048 reconstructed elements.  The warp decodes 8 steps into a register
 // window, then runs their 8 prefix chains together (independent shuffles overlap)
 // and stores them.  Returns false (warp-uniform) if the stream is damaged or its records do not
-// match its outlier slots; *used gets the units read.  s_tab: this warp's 288 words
-// of shared memory (the record table, then the 3-D running sums).
+// match its outlier slots; *used gets the units read.  s_tab: this warp's 32 words of
+// shared memory (the record table), ring: its ring of units.
 template <int ND, typename E>
 __device__ bool fused_decode_reconstruct(const DecodeArgs& a, uint32_t b, uint32_t which, const uint16_t* u,
-                                         uint32_t avail, const BookView& bk, uint32_t* used, uint32_t* s_tab) {
+                                         uint32_t avail, const BookView& bk, uint32_t* used, uint32_t* s_tab,
+                                         uint32_t ring) {
   const uint32_t lane = threadIdx.x & 31;
   const int32_t r = (int32_t)a.radius;
   const Out<E> out(a);
@@ -564,36 +687,36 @@ __device__ bool fused_decode_reconstruct(const DecodeArgs& a, uint32_t b, uint32
   const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
   const uint32_t rs = a.rec_start[b], re = a.rec_start[b + 1];
   IhsReader rd;
-  rd.init(u, avail);
+  rd.init(u, avail, bk, ring);
   RecordCursor rc;
   rc.init(rec, rs, re, key0);
   bool bad = false;
-  // 3-D: the running z sum of each of the lane's 8 rows of a plane, in this warp's
-  // shared-memory strip (row s of lane l at zs[32 s + l]: no bank conflicts)
-  int32_t* zs = reinterpret_cast<int32_t*>(s_tab) + 32;
   int32_t carry = 0, ysum0 = 0, ysum1 = 0;
-  if (ND == 3) {
+  int32_t zs[8];  // 3-D: the running z sum of each of the lane's 8 rows of a plane
 #pragma unroll
-    for (int s = 0; s < 8; s++) zs[32 * s + lane] = 0;
-  }
+  for (int s = 0; s < 8; s++) zs[s] = 0;
 #pragma unroll 1
   for (uint32_t t0 = 0; t0 < 64; t0 += 8) {
-    // the decoding step runs two copies per iteration (four overflow the instruction
-    // cache); each pair of steps' q' shifts into an 8-register window
+    // four copies of the step per iteration (eight overflow the instruction cache: 507
+    // against 415 us at 3-D 512^3; two: 426)
     int32_t q[8];
 #pragma unroll 1
-    for (uint32_t s0 = 0; s0 < 8; s0 += 2) {
+    for (int s0 = 0; s0 < 8; s0 += 4) {
 #pragma unroll
-      for (uint32_t u = 0; u < 2; u++) {
-        const int sym = rd.step(true, bk);
-        int32_t v = sym - r;
-        rc.step(key0 + 64u * (t0 + s0 + u), sym, v, bad, s_tab);
-        q[6 + u] = v;
-      }
-      if (s0 + 2 < 8) {
+      for (int s = 0; s < 4; s++) q[s] = q[s + 4];
 #pragma unroll
-        for (int k = 0; k < 6; k++) q[k] = q[k + 2];
+      for (int s = 0; s < 4; s++) q[4 + s] = rd.step(true, bk) - r;
+    }
+    // the window's outlier records, if it reaches any (a code 0 without one is damage)
+    if (rc.next < key0 + 64u * (t0 + 8)) {
+#pragma unroll
+      for (int s = 0; s < 8; s++) {
+        const int sym = q[s] + r;
+        rc.step(key0 + 64u * (t0 + s), sym, q[s], bad, s_tab);
       }
+    } else {
+#pragma unroll
+      for (int s = 0; s < 8; s++) bad |= q[s] == -r;
     }
     if (ND == 1) {
       // 8 steps = one 256-element chunk: per-step warp scans, then the carries
@@ -652,15 +775,14 @@ __device__ bool fused_decode_reconstruct(const DecodeArgs& a, uint32_t b, uint32
       for (int s = 0; s < 8; s++) {
         const int32_t other = __shfl_xor_sync(~0u, q[s], 16);
         if (s == 4) pair = 0;  // rows 8-15: the second y chunk
-        const int32_t k = zs[32 * s + lane] + pair + q[s] + (p ? other : 0);
-        zs[32 * s + lane] = k;
+        zs[s] += pair + q[s] + (p ? other : 0);
         pair += q[s] + other;
-        out.put(base + (uint64_t)(2 * s) * nx, k);
+        out.put(base + (uint64_t)(2 * s) * nx, zs[s]);
       }
     }
   }
   *used = rd.cur;
-  const bool ok = !__any_sync(~0u, rd.bad || bad);
+  const bool ok = !__any_sync(~0u, bad) & rd.sound();
   // verbatim patches of this stream's slots overwrite their elements (after the
   // warp's own stores: __syncwarp orders them)
   __syncwarp();
@@ -679,7 +801,12 @@ __device__ bool fused_decode_reconstruct(const DecodeArgs& a, uint32_t b, uint32
 }
 
 constexpr int kStreamWarps = kStreamWarpsPerCta;
-constexpr int kRecTabWords = 288;  // per decoding warp of a fused stream: record table 32 + 3-D sums 256
+// per decoding warp: its ring of 128 units (64 words, 256-byte aligned) and, for fused
+// streams, its record table (32 words); 64 words of slack align the rings
+constexpr int kRingWords = 64, kRecTabWords = 32;
+static size_t stream_smem_bytes(int nluts, int warps) {
+  return (size_t)nluts * (1u << kLutBits) * sizeof(LutEntry) + 4u * (size_t)(kRingWords * (warps + 1) + kRecTabWords * warps);
+}
 
 // Entropy decoding, persistent: each CTA stages the lookup tables of the books the
 // archive uses in shared memory once, then its warps take (block, stream) slots from
@@ -710,10 +837,13 @@ __device__ void stream_decode_body(const DecodeArgs& a, uint32_t b_begin, uint32
   LutEntry* lut_code = s_luts;
   LutEntry* lut_val = s_luts + (huff ? (1 << kLutBits) : 0);
   LutEntry* lut_len = lut_val + (1 << kLutBits);
-  // fused streams: after the tables, per warp a record table (32 words) and the 3-D
-  // running sums (256 words); the launch sizes the dynamic shared memory for them
-  uint32_t* s_rectab =
+  // after the tables, the warps' rings and record tables (stream_smem_bytes)
+  uint32_t* s_tail =
       reinterpret_cast<uint32_t*>(s_luts + (huff ? (1 << kLutBits) : 0) + (rle ? 2 * (1 << kLutBits) : 0));
+  const uint32_t ring0 = (smem_u32(s_tail) + 255u) & ~255u;
+  const uint32_t wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const uint32_t ring = ring0 + 4u * kRingWords * wid;
+  uint32_t* s_rectab = s_tail + (ring0 - smem_u32(s_tail)) / 4 + kRingWords * nwarps + kRecTabWords * wid;
   // a chunk of blocks (batches) copies only the tables its own blocks use
   bool need_code = huff, need_runs = rle;
   if (b_end != 0) {
@@ -774,23 +904,17 @@ __device__ void stream_decode_body(const DecodeArgs& a, uint32_t b_begin, uint32
         continue;
       }
       const uint32_t h = huff_split(m);
-      const BookView bk{lut_code, s_first, s_limit, s_count, s_off, t->sorted, (int)t->maxlen, t->fullmask};
+      const BookView bk{lut_code, s_first, s_limit, s_count, s_off, t->sorted, t->sorted + kNsymCode,
+                        (uint32_t)kLut2Size, t->lut2_base, t->lut2_shift, (int)t->maxlen, t->fullmask};
+      const uint16_t* us = which == 0 ? u + 1 : u + 1 + na;
+      const uint32_t nus = which == 0 ? na : nu - 1 - na;
       if (ND != 0 && a.fuse && m == (uint32_t)kSlots) {
-        if (which == 0) {
-          ok = fused_decode_reconstruct<ND, E>(a, b, 0, u + 1, na, bk, &used, s_rectab + kRecTabWords * (threadIdx.x >> 5));
-          ok = ok && used == na;
-        } else {
-          ok = fused_decode_reconstruct<ND, E>(a, b, 1, u + 1 + na, nu - 1 - na, bk, &used,
-                                            s_rectab + kRecTabWords * (threadIdx.x >> 5));
-          ok = ok && ((2ull * (1ull + na + used) + 3) & ~3ull) == bytes;
-        }
-      } else if (which == 0) {
-        ok = ihs_decode_warp(u + 1, na, h, bk, a.codes + (uint64_t)b * kSlots, 0, &used);
-        ok = ok && used == na;
+        ok = fused_decode_reconstruct<ND, E>(a, b, which, us, nus, bk, &used, s_rectab, ring);
       } else {
-        ok = ihs_decode_warp(u + 1 + na, nu - 1 - na, m - h, bk, a.codes + (uint64_t)b * kSlots + h, 0, &used);
-        ok = ok && ((2ull * (1ull + na + used) + 3) & ~3ull) == bytes;
+        ok = ihs_decode_warp(us, nus, which == 0 ? h : m - h, bk, a.codes + (uint64_t)b * kSlots + (which == 0 ? 0u : h),
+                             0, &used, ring);
       }
+      ok = ok && (which == 0 ? used == na : ((2ull * (1ull + na + used) + 3) & ~3ull) == bytes);
     } else {
       const DecTab* tv = &a.tabs[1];
       const DecTab* tl = &a.tabs[2];
@@ -806,17 +930,13 @@ __device__ void stream_decode_body(const DecodeArgs& a, uint32_t b_begin, uint32
       }
       const uint32_t lavail = (uint32_t)((bytes - 8) / 2 - vu);
       const uint16_t* p16 = reinterpret_cast<const uint16_t*>(pay) + 4;
-      if (which == 0) {
-        const BookView bv{lut_val, tv->first, tv->limit, tv->count, tv->off, tv->sorted, (int)tv->maxlen,
-                          tv->fullmask};
-        ok = ihs_decode_warp(p16, vu, nr, bv, a.runv + (uint64_t)b * kSlots, 0, &used);
-        ok = ok && used == vu;
-      } else {
-        const BookView bl{lut_len, tl->first, tl->limit, tl->count, tl->off, tl->sorted, (int)tl->maxlen,
-                          tl->fullmask};
-        ok = ihs_decode_warp(p16 + vu, lavail, nr, bl, a.runl + (uint64_t)b * kSlots, 1, &used);
-        ok = ok && ((8ull + 2ull * (vu + used) + 3) & ~3ull) == bytes;
-      }
+      const DecTab* tb = which == 0 ? tv : tl;
+      const BookView bk{which == 0 ? lut_val : lut_len, tb->first, tb->limit, tb->count, tb->off, tb->sorted,
+                        tb->sorted + kNsymCode, which == 0 ? (uint32_t)kLut2Size : 0u, tb->lut2_base, tb->lut2_shift,
+                        (int)tb->maxlen, tb->fullmask};
+      ok = ihs_decode_warp(which == 0 ? p16 : p16 + vu, which == 0 ? vu : lavail, nr, bk,
+                           (which == 0 ? a.runv : a.runl) + (uint64_t)b * kSlots, (int)which, &used, ring);
+      ok = ok && (which == 0 ? used == vu : ((8ull + 2ull * (vu + used) + 3) & ~3ull) == bytes);
     }
     if (!ok && lane0) flag(a.st, ERR_CORRUPT);
   }
@@ -1575,7 +1695,7 @@ cudaError_t launch_decode_batch(const DecodeBatchLaunch& L, cudaStream_t s) {
   trace_end(K_DEC_SETUP, s);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int warps = L.warps ? L.warps : kStreamWarps;
-  const size_t smem = 3 * (1u << kLutBits) * sizeof(LutEntry) + (L.nd ? (size_t)warps * kRecTabWords * 4 : 0);
+  const size_t smem = stream_smem_bytes(3, warps);
   auto k = L.nd == 1 ? stream_decode_batch_kernel<1>
                      : (L.nd == 2 ? stream_decode_batch_kernel<2>
                                   : (L.nd == 3 ? stream_decode_batch_kernel<3> : stream_decode_batch_kernel<0>));
@@ -1632,27 +1752,32 @@ cudaError_t launch_decode_stages(const DecodeArgs& a, cudaStream_t s) {
   const int nd = a.g.ndim;
   const int nluts = ((a.flags & 1u) ? 1 : 0) + ((a.flags & 2u) ? 2 : 0);
   if (nluts) {
-    const size_t lut_bytes =
-        (size_t)nluts * (1u << kLutBits) * sizeof(LutEntry) + (size_t)kStreamWarps * kRecTabWords * 4;
-    static int sms = 0, occ[4][4] = {};
+    // warps per CTA: a stream is a chain of dependent steps, so a field with fewer streams
+    // than the chip's SMs take at full occupancy spreads them over more, smaller CTAs
+    // (each stages its own tables)
+    static int sms = 0, occ[4][4][3] = {};
     auto k = nd == 1 ? stream_decode_kernel<1, E> : (nd == 2 ? stream_decode_kernel<2, E> : stream_decode_kernel<3, E>);
     if (sms == 0) {
       int dev = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       for (auto kk : {stream_decode_kernel<1, E>, stream_decode_kernel<2, E>, stream_decode_kernel<3, E>})
-        cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(3 * (1u << kLutBits) * sizeof(LutEntry) + kStreamWarps * kRecTabWords * 4));
+        cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stream_smem_bytes(3, kStreamWarps));
     }
-    if (occ[nd][nluts] == 0) {
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[nd][nluts], k, 32 * kStreamWarps, lut_bytes);
-      if (occ[nd][nluts] <= 0) occ[nd][nluts] = 1;
+    const uint64_t streams = 2ull * a.g.nblk;
+    const int wi = streams >= 32ull * sms ? 2 : (streams >= 8ull * sms ? 1 : 0);
+    const int warps = 4 << wi;
+    static_assert(kStreamWarps == 16, "4, 8 or 16 warps");
+    const size_t smem = stream_smem_bytes(nluts, warps);
+    if (occ[nd][nluts][wi] == 0) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[nd][nluts][wi], k, 32 * warps, smem);
+      if (occ[nd][nluts][wi] <= 0) occ[nd][nluts][wi] = 1;
     }
-    const uint64_t want = (2ull * a.g.nblk + kStreamWarps - 1) / kStreamWarps;
-    const uint64_t cap = (uint64_t)sms * occ[nd][nluts];
+    const uint64_t want = (streams + warps - 1) / warps;
+    const uint64_t cap = (uint64_t)sms * occ[nd][nluts][wi];
     const unsigned grid = (unsigned)(want < cap ? want : cap);
     trace_begin(K_STREAM_DECODE, s);
-    k<<<grid, 32 * kStreamWarps, lut_bytes, s>>>(a);
+    k<<<grid, 32 * warps, smem, s>>>(a);
     trace_end(K_STREAM_DECODE, s);
   }
   if (a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF]) {  // run blocks present

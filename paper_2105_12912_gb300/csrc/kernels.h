@@ -124,7 +124,10 @@ struct DecTab {
   uint32_t off[kMaxLen + 1];
   uint32_t present;
   uint32_t maxlen;
-  uint16_t sorted[kNsymLen];
+  uint32_t lut2_base, lut2_shift;  // upper word of the codes' end at kLutBits bits; a cell's log2 size
+  uint16_t sorted[kNsymLen];  // (books of 1024 symbols: the second-level table sits behind them)
+  static_assert(kNsymCode + kLut2Size <= kNsymLen, "room for the second level");
+  __device__ uint16_t* lut2() { return sorted + kNsymCode; }
   alignas(16) LutEntry lut[1 << kLutBits];  // lut_entry(symbol, length), 0 = longer than kLutBits
 };
 
