@@ -91,8 +91,11 @@ __global__ __launch_bounds__(256) void range_d_kernel(const double* __restrict__
   const bool vec = (((uintptr_t)x) & 15) == 0;
   const uint64_t nvec = vec ? n / 2 : 0;
   const double2* x2 = reinterpret_cast<const double2*>(x);
+  // (integers only: one FP64 compare an element, at 2 a cycle and SM, took as long as the
+  // field's bytes; 3-D 256^3: 71 -> 39 us)
   auto take = [&](double a) {
-    if (!isfinite(a)) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+    if (((uint32_t)(u >> 32) & 0x7ff00000u) == 0x7ff00000u) {
       bad = 1;
     } else {
       const unsigned long long key = order_key_d(a);
@@ -100,7 +103,21 @@ __global__ __launch_bounds__(256) void range_d_kernel(const double* __restrict__
       hi = max(hi, key);
     }
   };
-  for (uint64_t i = tid; i < nvec; i += nth) {
+  // four independent 16-byte loads in flight per thread per iteration
+  uint64_t i = tid;
+  for (; i + 3 * nth < nvec; i += 4 * nth) {
+    const double2 v0 = __ldcs(&x2[i]), v1 = __ldcs(&x2[i + nth]), v2 = __ldcs(&x2[i + 2 * nth]),
+                  v3 = __ldcs(&x2[i + 3 * nth]);
+    take(v0.x);
+    take(v0.y);
+    take(v1.x);
+    take(v1.y);
+    take(v2.x);
+    take(v2.y);
+    take(v3.x);
+    take(v3.y);
+  }
+  for (; i < nvec; i += nth) {
     const double2 v = __ldcs(&x2[i]);
     take(v.x);
     take(v.y);

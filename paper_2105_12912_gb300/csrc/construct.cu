@@ -7,8 +7,9 @@ namespace cszp {
 
 using namespace cons;
 
+// (shared memory allows four CTAs an SM, two with double tiles)
 template <int ND, typename E, bool G = false>
-__global__ __launch_bounds__(kThreads, 4) void construct_kernel(const __grid_constant__ ConstructTask one,
+__global__ __launch_bounds__(kThreads, sizeof(E) == 8 ? 2 : 4) void construct_kernel(const __grid_constant__ ConstructTask one,
                                                              const ConstructTask* __restrict__ tasks,
                                                              const uint32_t* __restrict__ tile0, int nfields,
                                                              uint32_t ntiles, uint32_t* ticket,
@@ -84,7 +85,8 @@ void prepare_construct_task(ConstructTask& T) {
   if (rank == 1 && g.nelem >= (1ull << 32)) return;
   const CUresult r = fn(&T.tmap, f64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                         (cuuint32_t)rank, xp, dim, stride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        rank == 3 && !f64 && !T.a.global ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                        rank != 3 || T.a.global ? CU_TENSOR_MAP_SWIZZLE_NONE
+                                                : (f64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B),
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   T.use_tma = r == CUDA_SUCCESS ? 1 : 0;
 }

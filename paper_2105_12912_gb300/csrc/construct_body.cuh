@@ -70,16 +70,45 @@ struct Pq<float> {
     return prequant(x, eb_f, ebx2_f, ebx2_r, k, patch);
   }
 };
+// Doubles: the FP64 pipe gives 2 results a cycle and SM, and the plain fast path takes
+// seven of them an element (product, two conversions, product, difference, two compares),
+// which bounds the whole kernel (3-D 256^3: 298 us).  So the common case runs on
+// integers: |x / step| as the product of the two mantissas' upper 32 bits, shifted to a
+// 32-bit fraction (V).  Truncation loses less than 2^-29 of the product, so the true
+// value lies in [V, V + 8 K + 9] in units of 2^-32 with K its whole part; unless that
+// interval, widened by the rounding the FP64 product has (at most 2^-25), holds a half
+// point, the nearest integer is the one prequant_d finds: its distance to x is below
+// step / 2 = eb (1 - 2^-24), which the 2^-25 eb that fl64(k * step) may add keeps inside
+// the bound.  Everything else (a half point near, |k| close to the limit, non-finite x)
+// goes to prequant_d.  Now 58 us.
 template <>
 struct Pq<double> {
   double eb_d, step, rstep;
-  __device__ explicit Pq(const double* w) : eb_d(w[0]), step(w[1]), rstep(w[2]) {}
+  uint32_t mr;  // upper 32 bits of 1 / step's mantissa (the leading one among them)
+  int s0;       // product shift of an x with exponent field 0
+  __device__ explicit Pq(const double* w) : eb_d(w[0]), step(w[1]), rstep(w[2]) {
+    const uint32_t hi = (uint32_t)__double2hiint(rstep);
+    const int er = (int)(hi >> 20);  // (1 / step is positive)
+    mr = __funnelshift_l((uint32_t)__double2loint(rstep), hi, 11) | 0x80000000u;
+    // (with 1 / step in this range an x of exponent field 0 quantizes to 0 and a
+    // non-finite one fails the shift's test; outside it no x takes this path)
+    s0 = er >= 100 && er <= 1900 ? 2076 - er : -4096;
+  }
   __device__ static void load(const DevState* st, double* w) {
     w[0] = __ldcg(&st->eb_d);
     w[1] = __ldcg(&st->step_d);
     w[2] = __ldcg(&st->rstep_d);
   }
-  __device__ __forceinline__ bool fast(double x, int32_t& k) const { return prequant_fast_d(x, eb_d, step, rstep, k); }
+  __device__ __forceinline__ bool fast(double x, int32_t& k) const {
+    const int hi = __double2hiint(x);
+    const uint32_t mx = __funnelshift_l((uint32_t)__double2loint(x), (uint32_t)hi, 11) | 0x80000000u;
+    const int s = s0 - ((hi >> 20) & 0x7ff);
+    const uint64_t v = ((uint64_t)mx * mr) >> min((uint32_t)s, 63u);
+    const uint32_t K = (uint32_t)(v >> 32), f = (uint32_t)v;
+    k = (int32_t)(K + (f >> 31));
+    k = hi < 0 ? -k : k;
+    return (s >= 4) & (K < (1u << 27) - 8u) & (0x80000100u - f > 8u * K + 1024u);
+  }
   __device__ __forceinline__ uint32_t full(double x, int32_t& k, bool& patch) const {
     patch = false;
     return prequant_d(x, eb_d, step, rstep, k);
@@ -106,27 +135,46 @@ __device__ __forceinline__ void load16(const double* p, double (&f)[16]) {
   }
 }
 
-// ---- FP32 3-D tiles: 64-byte swizzled rows ------------------------------------------
-// A 16^3 FP32 box has 64-byte x rows.  Its TMA copy uses the 64-byte swizzle: the
-// 16-byte chunk c of row R lands at chunk c ^ ((R >> 1) & 3) of that row (the buffer
-// is 1024-byte aligned), so that eight threads reading one chunk of eight consecutive
-// rows touch all 32 banks.  Thread loads and every reader of such a box use the same
-// placement: element e of the box sits at swz64(e).
-__device__ __forceinline__ uint32_t swz64(uint32_t e) { return e ^ ((e >> 3) & 12u); }
+// ---- 3-D tiles: swizzled rows ---------------------------------------------------------
+// A 16^3 box has x rows of 64 bytes (FP32) or 128 (double).  Its TMA copy uses the
+// swizzle of that width: the 16-byte chunk c of row R lands at chunk c ^ row_key(R) of
+// that row (the buffer is 1024-byte aligned), so that eight threads reading one chunk of
+// eight consecutive rows touch all 32 banks.  Thread loads and every reader of such a box
+// use the same placement: element e of the box sits at swz(e).  k (int32) takes the first
+// four chunk places, by key, of each row.
 template <typename E>
-constexpr bool kRowSwizzled = false;
-template <>
-constexpr bool kRowSwizzled<float> = true;
+__device__ __forceinline__ uint32_t row_key(uint32_t row) {
+  return sizeof(E) == 4 ? (row >> 1) & 3u : row & 7u;
+}
+template <typename E>
+__device__ __forceinline__ uint32_t swz(uint32_t e) {
+  return sizeof(E) == 4 ? e ^ ((e >> 3) & 12u) : e ^ ((e >> 3) & 14u);
+}
+template <typename E>
+constexpr uint32_t kRowInts = 16 * sizeof(E) / 4;  // 32-bit words of a row
 
-__device__ __forceinline__ void ld_row(const float* row, uint32_t key, float (&f)[16]) {
+// prequantizes the 16 elements of a row; false if any of them needs the full decision
+__device__ __forceinline__ bool quant_row(const Pq<float>& pq, const float* row, uint32_t key, int32_t (&k)[16]) {
+  bool ok = true;
 #pragma unroll
   for (int c = 0; c < 4; c++) {
     const float4 v = reinterpret_cast<const float4*>(row)[c ^ key];
-    f[4 * c] = v.x;
-    f[4 * c + 1] = v.y;
-    f[4 * c + 2] = v.z;
-    f[4 * c + 3] = v.w;
+    ok = pq.fast(v.x, k[4 * c]) & ok;
+    ok = pq.fast(v.y, k[4 * c + 1]) & ok;
+    ok = pq.fast(v.z, k[4 * c + 2]) & ok;
+    ok = pq.fast(v.w, k[4 * c + 3]) & ok;
   }
+  return ok;
+}
+__device__ __forceinline__ bool quant_row(const Pq<double>& pq, const double* row, uint32_t key, int32_t (&k)[16]) {
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < 8; c++) {
+    const double2 v = reinterpret_cast<const double2*>(row)[c ^ key];
+    ok = pq.fast(v.x, k[2 * c]) & ok;
+    ok = pq.fast(v.y, k[2 * c + 1]) & ok;
+  }
+  return ok;
 }
 __device__ __forceinline__ void st_row(int32_t* row, uint32_t key, const int32_t (&k)[16]) {
 #pragma unroll
@@ -139,7 +187,7 @@ template <typename T, uint32_t NIN = kSlots>
 struct SmemT {
   T in[2][NIN];                 // TMA destinations (box layout); in 3-D the current
                                 // one then carries the partly differenced k
-  int32_t zrow[16];             // zeros: the neighbour row of a chunk's first row / plane
+  int32_t zrow[32];             // zeros: the neighbour row of a chunk's first row / plane
   uint16_t c[kSlots];           // codes of the current tile (dense order)
   uint32_t hc[kNsymCode];       // code histogram (per CTA, current field)
   uint32_t hv[kNsymCode];       // run-value histogram
@@ -206,8 +254,8 @@ __device__ __forceinline__ const float* field_ptr<float>(const ConstructArgs& A)
 template <>
 __device__ __forceinline__ const double* field_ptr<double>(const ConstructArgs& A) { return A.x64; }
 
-// Thread-loaded tile (fields TMA cannot describe): box layout (FP32 3-D boxes
-// swizzled like their TMA copies), zeros outside.
+// Thread-loaded tile (fields TMA cannot describe): box layout (3-D boxes swizzled like
+// their TMA copies), zeros outside.
 template <typename E>
 __device__ void load_tile_threads(const ConstructArgs& A, uint32_t b, E* buf) {
   const E* xs = field_ptr<E>(A);
@@ -232,7 +280,7 @@ __device__ void load_tile_threads(const ConstructArgs& A, uint32_t b, E* buf) {
     }
     E v = E(0);
     if (zz < w[0] && yy < w[1] && xx < w[2]) v = xs[((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + org[2] + xx];
-    buf[kRowSwizzled<E> && g.ndim == 3 ? swz64(p) : p] = v;
+    buf[g.ndim == 3 ? swz<E>(p) : p] = v;
   }
 }
 
@@ -278,7 +326,7 @@ __device__ __noinline__ uint32_t edge_codes(const ConstructArgs& A, uint32_t b, 
         xx = rr - yy * w[2];
       }
       uint32_t box = ND == 1 ? xx : (ND == 2 ? yy * 64 + xx : (zz * 16 + yy) * 16 + xx);
-      if (ND == 3 && kRowSwizzled<E>) box = swz64(box);
+      if (ND == 3) box = swz<E>(box);
       bool p;
       err |= pq.full(in[box], kv[i], p);
       pm |= (uint32_t)p << i;
@@ -557,26 +605,23 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
         const uint32_t j = (16 * ry + i) * 64 + xx;
         post(delta, j, anyp, (pm >> i) & 1u);
       }
-    } else if constexpr (kRowSwizzled<E>) {
-      // FP32: thread t holds the x row (z, y) = (t >> 4, t & 15), two 8-chunks along x,
-      // i.e. the 16 consecutive slots 16t .. 16t + 15.  The x difference runs in
-      // registers; the y and z differences read the rows t - 1, t - 16 and t - 17 (the
-      // zero row at a chunk's first row or plane), which by then hold their x differences.
-      const uint32_t zz = tid >> 4, yy = tid & 15, key = (tid >> 1) & 3;
-      float f[16];
-      ld_row(in + 16 * tid, key, f);
+    } else {
+      // thread t holds the x row (z, y) = (t >> 4, t & 15), two 8-chunks along x, i.e. the
+      // 16 consecutive slots 16t .. 16t + 15.  The x difference runs in registers; the y
+      // and z differences read the rows t - 1, t - 16 and t - 17 (the zero row at a
+      // chunk's first row or plane), which by then hold their x differences.
+      const uint32_t zz = tid >> 4, yy = tid & 15, key = row_key<E>(tid);
       int32_t k[16];
-      bool ok = true;
-#pragma unroll
-      for (int i = 0; i < 16; i++) ok = pq.fast(f[i], k[i]) & ok;
+      const bool ok = quant_row(pq, in + 16 * tid, key, k);
       uint32_t pm = 0;
       if (!__all_sync(~0u, ok)) {
 #pragma unroll
         for (int i = 0; i < 16; i++) {
+          const E v = in[swz<E>(16u * tid + i)];
           int32_t kk;
-          if (!pq.fast(f[i], kk)) {
+          if (!pq.fast(v, kk)) {
             bool p;
-            err |= pq.full(f[i], k[i], p);
+            err |= pq.full(v, k[i], p);
             pm |= (uint32_t)p << i;
           }
         }
@@ -588,15 +633,16 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
       // row, which only it has read, so no barrier comes first; the neighbour rows lie
       // in the same 8-plane chunk, and planes 0-7 (8-15) belong to threads 0-127
       // (128-255), so each half of the CTA waits only for itself (named barriers 1, 2)
-      st_row(s_k + 16 * tid, key, k);
+      constexpr uint32_t R = kRowInts<E>;
+      st_row(s_k + R * tid, key, k);
       asm volatile("bar.sync %0, %1;" ::"r"(1 + (tid >> 7)), "r"(128) : "memory");
       const bool hy = (yy & 7) != 0, hz = (zz & 7) != 0;
       const int ty = hy ? tid - 1 : 0, tz = hz ? tid - 16 : 0, tyz = hy && hz ? tid - 17 : 0;
-      const int4* ry = reinterpret_cast<const int4*>(hy ? s_k + 16 * ty : S.zrow);
-      const int4* rz = reinterpret_cast<const int4*>(hz ? s_k + 16 * tz : S.zrow);
-      const int4* ryz = reinterpret_cast<const int4*>(hy && hz ? s_k + 16 * tyz : S.zrow);
+      const int4* ry = reinterpret_cast<const int4*>(hy ? s_k + R * ty : S.zrow);
+      const int4* rz = reinterpret_cast<const int4*>(hz ? s_k + R * tz : S.zrow);
+      const int4* ryz = reinterpret_cast<const int4*>(hy && hz ? s_k + R * tyz : S.zrow);
       // rows t - 16 and t - 17 have the swizzle keys of rows t and t - 1
-      const uint32_t ky = ((uint32_t)(tid + 7) >> 1) & 3;  // = ((t - 1) >> 1) & 3 for t >= 1
+      const uint32_t ky = row_key<E>((uint32_t)(tid + 7));  // (t + 7 and t - 1 agree, for t >= 1)
       uint32_t u[16];
 #pragma unroll
       for (int c = 0; c < 4; c++) {
@@ -607,47 +653,6 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
         u[4 * c + 3] = (uint32_t)(k[4 * c + 3] - a.w - bz.w + d.w + r);
       }
       post16(S, u, pm, r, dglob);
-    } else {
-      // thread t: z column of (xx, yy) = (t & 15, t >> 4); z and x differences in
-      // registers and shuffles, the y difference through shared memory
-      const uint32_t xx = tid & 15, yy = tid >> 4;
-      int32_t k[16];
-      uint32_t pm = 0, slow = 0;
-#pragma unroll
-      for (int i = 0; i < 16; i++)
-        slow |= (uint32_t)!pq.fast(in[(i * 16 + yy) * 16 + xx], k[i]) << i;
-      if (__any_sync(~0u, slow != 0)) {
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-          if ((slow >> i) & 1u) {
-            bool p;
-            err |= pq.full(in[(i * 16 + yy) * 16 + xx], k[i], p);
-            pm |= (uint32_t)p << i;
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 15; i > 0; i--)
-        if (i & 7) k[i] -= k[i - 1];  // z difference within 8-chunks
-#pragma unroll
-      for (int i = 0; i < 16; i++) {
-        const int32_t left = __shfl_up_sync(~0u, k[i], 1);
-        if (xx & 7) k[i] -= left;  // x difference
-      }
-      const bool anyp = __any_sync(~0u, pm != 0);
-      // the box carries k from here: each thread overwrites only its own column, which
-      // only it has read, so no barrier comes first; the y difference reads the row
-      // below in the same 8-row chunk, and rows 0-7 (8-15) belong to warps 0-3 (4-7),
-      // so each group of four warps waits only for itself (named barriers 1 and 2)
-#pragma unroll
-      for (int i = 0; i < 16; i++) s_k[(i * 16 + yy) * 16 + xx] = k[i];
-      asm volatile("bar.sync %0, %1;" ::"r"(1 + (tid >> 7)), "r"(128) : "memory");
-#pragma unroll
-      for (int i = 0; i < 16; i++) {
-        const uint32_t j = (i * 16 + yy) * 16 + xx;
-        const int32_t below = (yy & 7) ? s_k[(i * 16 + yy - 1) * 16 + xx] : 0;
-        post(k[i] - below, j, anyp, (pm >> i) & 1u);
-      }
     }
     __syncthreads();
   } else {
@@ -875,7 +880,7 @@ __device__ __forceinline__ void construct_loop(const ConstructTask& one, const C
     pending = atomicAdd(ticket, 1u);
   }
   for (int i = tid; i < kNsymCode + kNsymCode + kHlShared; i += kThreads) S.hc[i] = 0;  // hc, hv, hl
-  if (tid < 16) S.zrow[tid] = 0;
+  if (tid < 32) S.zrow[tid] = 0;
   __syncthreads();
 
   int cur = 0, field = -1;

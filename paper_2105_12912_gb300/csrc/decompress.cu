@@ -582,7 +582,14 @@ struct Out<double> {
   double* __restrict__ p;
   double step;
   __device__ explicit Out(const DecodeArgs& a) : p(a.out64), step(a.step_d) {}
-  __device__ __forceinline__ void put(uint64_t i, int32_t k) const { __stcs(&p[i], __dmul_rn((double)k, step)); }
+  // (double)k built from bits: the conversion instruction would take the FP64 pipe, 2
+  // results a cycle and SM, once more beside the product (3-D 256^3: 107 -> 97 us)
+  __device__ __forceinline__ static double to_double(int32_t k) {
+    const uint32_t m = (uint32_t)abs(k), z = (uint32_t)__clz((int)m), t = m << (z & 31u);
+    const uint32_t hi = m ? ((1053u - z) << 20) + (t >> 11) : 0u;
+    return __hiloint2double((int)(hi | ((uint32_t)k & 0x80000000u)), (int)(t << 21));
+  }
+  __device__ __forceinline__ void put(uint64_t i, int32_t k) const { __stcs(&p[i], __dmul_rn(to_double(k), step)); }
   __device__ __forceinline__ void put_patch(uint64_t i, int32_t k, bool, uint32_t) const { put(i, k); }
   __device__ __forceinline__ void patch(uint64_t, uint32_t) const {}
 };
