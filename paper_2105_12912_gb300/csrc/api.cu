@@ -414,10 +414,16 @@ csz_status enqueue_decode(const uint8_t* d_ar, size_t bytes, const uint8_t* h, b
   da.fuse = global ? 0 : 1;
   da.f64 = f64 ? 1 : 0;
   if (global) {
-    // the x pass's look-back states, one per 4096 elements (at most one per codec block)
     da.global = 1;
-    da.scan_state = at<uint64_t>(d_ws, L.lb_e);
-    if (cudaMemsetAsync(da.scan_state, 0, 8ull * ((g.nelem + 4095) / 4096), s) != cudaSuccess) return CSZ_E_CUDA;
+    if (g.ndim == 1) {
+      da.scan_state = at<uint64_t>(d_ws, L.lb_e);
+      if (cudaMemsetAsync(da.scan_state, 0, 8ull * g.nblk, s) != cudaSuccess) return CSZ_E_CUDA;
+    } else {
+      // in the decoded run lengths' place (8 KB a block), read no more by then: 4 bytes a
+      // block row, at most 1 KB a block, each
+      da.gtotals = reinterpret_cast<int32_t*>(da.runl);
+      da.gstrips = da.gtotals + 256ull * g.nblk;
+    }
   }
   if (f64) {
     da.out64 = static_cast<double*>(d_out);

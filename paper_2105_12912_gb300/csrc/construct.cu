@@ -7,9 +7,9 @@ namespace cszp {
 
 using namespace cons;
 
-// (shared memory allows four CTAs an SM, two with double tiles)
+// (shared memory allows four CTAs an SM, two with double tiles, three with halo'd ones)
 template <int ND, typename E, bool G = false>
-__global__ __launch_bounds__(kThreads, sizeof(E) == 8 ? 2 : 4) void construct_kernel(const __grid_constant__ ConstructTask one,
+__global__ __launch_bounds__(kThreads, sizeof(E) == 8 ? 2 : (G ? 3 : 4)) void construct_kernel(const __grid_constant__ ConstructTask one,
                                                              const ConstructTask* __restrict__ tasks,
                                                              const uint32_t* __restrict__ tile0, int nfields,
                                                              uint32_t ntiles, uint32_t* ticket,
@@ -133,13 +133,9 @@ void launch_nd(const ConstructTask& one, uint32_t* ticket, cudaStream_t s) {
 cudaError_t launch_construct(const ConstructTask& one, uint32_t* ticket, cudaStream_t s) {
   const bool f64 = one.a.x64 != nullptr, global = one.a.global != 0;
   trace_begin(K_CONSTRUCT, s);
-  if (f64) {
-    if (global) launch_nd<double, true>(one, ticket, s);
-    else launch_nd<double, false>(one, ticket, s);
-  } else {
-    if (global) launch_nd<float, true>(one, ticket, s);
-    else launch_nd<float, false>(one, ticket, s);
-  }
+  if (f64) launch_nd<double, false>(one, ticket, s);  // (global prediction is FP32 only)
+  else if (global) launch_nd<float, true>(one, ticket, s);
+  else launch_nd<float, false>(one, ticket, s);
   trace_end(K_CONSTRUCT, s);
   return cudaGetLastError();
 }

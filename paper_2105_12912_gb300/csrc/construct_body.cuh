@@ -291,12 +291,13 @@ __device__ __forceinline__ void flush_hist(const uint32_t* h, int n, uint32_t* g
   }
 }
 
-// ---- edge blocks (not inlined: keeps the full-block paths compact in the
-// instruction cache): prequantize into registers in dense order, stage k, residuals
-// from the staged neighbours.  Returns error bits.
+// ---- edge blocks of 1-D and 2-D fields (not inlined: keeps the full-block paths compact
+// in the instruction cache): prequantize into registers in dense order, stage k,
+// residuals from the staged neighbours.  Returns error bits.
 template <int ND, typename E>
 __device__ __noinline__ uint32_t edge_codes(const ConstructArgs& A, uint32_t b, SmemT<E>& S, E* in,
                                             const uint32_t* w, uint32_t m, int32_t* dglob) {
+  static_assert(ND < 3, "3-D edge blocks go by rows (post_edge_rows)");
   const int tid = threadIdx.x, lane = tid & 31;
   const Pq<E> pq(S.pq);
   const int32_t r = (int32_t)A.radius;
@@ -309,26 +310,9 @@ __device__ __noinline__ uint32_t edge_codes(const ConstructArgs& A, uint32_t b, 
     const uint32_t j = tid + kThreads * i;
     kv[i] = 0;
     if (j < m) {
-      uint32_t zz, yy, xx;
-      if (ND == 1) {
-        zz = 0;
-        yy = 0;
-        xx = j;
-      } else if (ND == 2) {
-        zz = 0;
-        yy = j / w[2];
-        xx = j - yy * w[2];
-      } else {
-        const uint32_t p = w[1] * w[2];
-        zz = j / p;
-        const uint32_t rr = j - zz * p;
-        yy = rr / w[2];
-        xx = rr - yy * w[2];
-      }
-      uint32_t box = ND == 1 ? xx : (ND == 2 ? yy * 64 + xx : (zz * 16 + yy) * 16 + xx);
-      if (ND == 3) box = swz<E>(box);
+      const uint32_t yy = ND == 2 ? j / w[2] : 0u, xx = j - yy * w[2];
       bool p;
-      err |= pq.full(in[box], kv[i], p);
+      err |= pq.full(in[yy * 64 + xx], kv[i], p);
       pm |= (uint32_t)p << i;
     }
   }
@@ -341,37 +325,22 @@ __device__ __noinline__ uint32_t edge_codes(const ConstructArgs& A, uint32_t b, 
     if (lane == 0) S.patch[j >> 5] = pb;
   }
   __syncthreads();
-  const uint32_t sy = w[2], sz = w[1] * w[2];
+  const uint32_t sy = w[2];
 #pragma unroll
   for (int i = 0; i < kPer; i++) {
     const uint32_t j = tid + kThreads * i;
     int32_t delta = 0;
     uint16_t q = 0;
     const bool inb = j < m;
-    (void)delta;
     if (inb) {
-      uint32_t zz = 0, yy = 0, xx = j;
-      if (ND == 2) {
-        yy = j / w[2];
-        xx = j - yy * w[2];
-      } else if (ND == 3) {
-        zz = j / sz;
-        const uint32_t rr = j - zz * sz;
-        yy = rr / w[2];
-        xx = rr - yy * w[2];
-      }
+      const uint32_t yy = ND == 2 ? j / w[2] : 0u, xx = j - yy * w[2];
       const bool hx = (xx % Chunk<ND>::x) != 0;
       const bool hy = ND >= 2 && (yy % Chunk<ND>::y) != 0;
-      const bool hz = ND >= 3 && (zz % Chunk<ND>::z) != 0;
       int32_t p;
       if (ND == 1) {
         p = hx ? s_k[j - 1] : 0;
-      } else if (ND == 2) {
-        p = (hx ? s_k[j - 1] : 0) + (hy ? s_k[j - sy] : 0) - ((hx && hy) ? s_k[j - sy - 1] : 0);
       } else {
-        p = (hx ? s_k[j - 1] : 0) + (hy ? s_k[j - sy] : 0) + (hz ? s_k[j - sz] : 0) -
-            ((hx && hy) ? s_k[j - sy - 1] : 0) - ((hx && hz) ? s_k[j - sz - 1] : 0) -
-            ((hy && hz) ? s_k[j - sz - sy] : 0) + ((hx && hy && hz) ? s_k[j - sz - sy - 1] : 0);
+        p = (hx ? s_k[j - 1] : 0) + (hy ? s_k[j - sy] : 0) - ((hx && hy) ? s_k[j - sy - 1] : 0);
       }
       delta = s_k[j] - p;
       q = (delta > -r && delta < r) ? (uint16_t)(delta + r) : (uint16_t)0;
@@ -383,7 +352,7 @@ __device__ __noinline__ uint32_t edge_codes(const ConstructArgs& A, uint32_t b, 
     if (lane == 0) S.outl[j >> 5] = ob;
   }
   __syncthreads();
-    return err;
+  return err;
 }
 
 // ---- the tile's tail: run heads at word boundaries (full tiles), counts from the
@@ -502,6 +471,55 @@ __device__ __forceinline__ void post16(SM& S, const uint32_t (&u)[16], uint32_t 
   }
 }
 
+// Postquantization of a 3-D edge block (extent w, m elements) whose thread t holds u =
+// delta + r of the row (t >> 4, t & 15): its codes go to their dense slots, then the bit
+// words come from the codes.  S.patch has been cleared before the CTA's last barrier.  (A
+// thread per dense slot instead, with divisions to find its element and seven neighbour
+// reads, took four times the instructions; a fifth of a 100x500x500 field's blocks are
+// edge blocks: 100x500x500 construct 80 -> 71 us.)
+template <typename SM>
+__device__ __forceinline__ void post_edge_rows(SM& S, const uint32_t (&u)[16], uint32_t pm, const uint32_t* w,
+                                               uint32_t m, int32_t r, int32_t* dglob) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, zz = tid >> 4, yy = tid & 15;
+  if (zz < w[0] && yy < w[1]) {
+    const uint32_t j0 = (zz * w[1] + yy) * w[2], q0 = u[0] - 1u < (uint32_t)(2 * r - 1) ? u[0] : 0u;
+    bool same = true;
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++) {
+      const uint32_t q = u[i] - 1u < (uint32_t)(2 * r - 1) ? u[i] : 0u;  // |delta| < r
+      if (i < w[2]) {
+        S.c[j0 + i] = (uint16_t)q;
+        same &= q == q0;
+        if (q == 0) dglob[j0 + i] = (int32_t)(u[i] - (uint32_t)r);
+      }
+    }
+    if (same) {
+      atomicAdd(&S.hc[q0], w[2]);
+    } else {
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++)
+        if (i < w[2]) atomicAdd(&S.hc[u[i] - 1u < (uint32_t)(2 * r - 1) ? u[i] : 0u], 1u);
+    }
+    for (pm &= (1u << w[2]) - 1u; pm; pm &= pm - 1u) {
+      const uint32_t j = j0 + (uint32_t)(__ffs(pm) - 1);
+      atomicOr(&S.patch[j >> 5], 1u << (j & 31));
+    }
+  }
+  for (uint32_t j = m + tid; j < (uint32_t)kSlots; j += kThreads) S.c[j] = 0;
+  __syncthreads();
+#pragma unroll 4
+  for (int i = 0; i < kPer; i++) {
+    const uint32_t j = tid + kThreads * i;
+    const uint32_t q = S.c[j], left = j ? S.c[j - 1] : 0u;
+    const uint32_t ob = __ballot_sync(~0u, j < m && q == 0);
+    const uint32_t hb = __ballot_sync(~0u, j < m && (j == 0 || q != left));
+    if (lane == 0) {
+      S.outl[j >> 5] = ob;
+      S.head[j >> 5] = hb;
+    }
+  }
+}
+
 // ---- one tile ------------------------------------------------------------------------
 // Codes, records and histogram updates of codec block b (origin box[0..2], extent
 // box[3..5]) from the box in `in` (which this call overwrites with k and outlier
@@ -550,7 +568,7 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
   // ---- prequantization, Lorenzo residual (Sec. IV-B2), postquantization ----------
   // The residual is the mixed difference (1 - S_x)(1 - S_y)(1 - S_z) k, each shift
   // reading zero outside the chunk; that expansion is the paper's 1/2/3-D predictor.
-  if (full) {
+  if (ND == 3 || full) {
     if (ND == 1) {
       // thread t: 16 consecutive elements (a warp covers two whole 256-chunks)
       int32_t k[16];
@@ -609,8 +627,10 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
       // thread t holds the x row (z, y) = (t >> 4, t & 15), two 8-chunks along x, i.e. the
       // 16 consecutive slots 16t .. 16t + 15.  The x difference runs in registers; the y
       // and z differences read the rows t - 1, t - 16 and t - 17 (the zero row at a
-      // chunk's first row or plane), which by then hold their x differences.
+      // chunk's first row or plane), which by then hold their x differences.  Outside the
+      // field the box is zero, which quantizes to 0 and is nobody's neighbour.
       const uint32_t zz = tid >> 4, yy = tid & 15, key = row_key<E>(tid);
+      if (!full && tid < kSlots / 32) S.patch[tid] = 0;
       int32_t k[16];
       const bool ok = quant_row(pq, in + 16 * tid, key, k);
       uint32_t pm = 0;
@@ -635,7 +655,8 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
       // (128-255), so each half of the CTA waits only for itself (named barriers 1, 2)
       constexpr uint32_t R = kRowInts<E>;
       st_row(s_k + R * tid, key, k);
-      asm volatile("bar.sync %0, %1;" ::"r"(1 + (tid >> 7)), "r"(128) : "memory");
+      if (full) asm volatile("bar.sync %0, %1;" ::"r"(1 + (tid >> 7)), "r"(128) : "memory");
+      else __syncthreads();
       const bool hy = (yy & 7) != 0, hz = (zz & 7) != 0;
       const int ty = hy ? tid - 1 : 0, tz = hz ? tid - 16 : 0, tyz = hy && hz ? tid - 17 : 0;
       const int4* ry = reinterpret_cast<const int4*>(hy ? s_k + R * ty : S.zrow);
@@ -652,10 +673,11 @@ __device__ void process_tile(const ConstructArgs& A, uint32_t b, const uint32_t*
         u[4 * c + 2] = (uint32_t)(k[4 * c + 2] - a.z - bz.z + d.z + r);
         u[4 * c + 3] = (uint32_t)(k[4 * c + 3] - a.w - bz.w + d.w + r);
       }
-      post16(S, u, pm, r, dglob);
+      if (full) post16(S, u, pm, r, dglob);
+      else post_edge_rows(S, u, pm, w, m, r, dglob);
     }
     __syncthreads();
-  } else {
+  } else if constexpr (ND < 3) {
     err |= edge_codes<ND, E>(A, b, S, in, w, m, dglob);
     run_head_words(S.c, m, S.head);
     __syncthreads();
@@ -726,24 +748,133 @@ __device__ void load_halo_threads(const ConstructArgs& A, const uint32_t* org, E
   }
 }
 
-// Codes, records and histograms of codec block b under the global predictor: the
-// halo'd box is prequantized in place (each element's k as int32), then every slot's
-// residual is the mixed difference (1 - S_x)(1 - S_y)(1 - S_z) k over the box (the
-// paper's 1/2/3-D predictor, Sec. IV-B2, with no chunk restarts), then the tail.
+// k of the 16 elements p[0..15] of a halo box (16-byte aligned), differenced along x (p[-1]
+// is the element before them).  Returns their patch bits.
+template <typename E>
+__device__ __forceinline__ uint32_t quant_piece(const Pq<E>& pq, const E* p, int32_t (&k)[16], uint32_t& err) {
+  int32_t before;
+  bool ok = pq.fast(p[-1], before);
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const float4 v = reinterpret_cast<const float4*>(p)[c];
+    ok = pq.fast(v.x, k[4 * c]) & ok;
+    ok = pq.fast(v.y, k[4 * c + 1]) & ok;
+    ok = pq.fast(v.z, k[4 * c + 2]) & ok;
+    ok = pq.fast(v.w, k[4 * c + 3]) & ok;
+  }
+  uint32_t pm = 0;
+  if (!ok) {
+    bool patch;
+    err |= pq.full(p[-1], before, patch);
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      err |= pq.full(p[i], k[i], patch);
+      pm |= (uint32_t)patch << i;
+    }
+  }
+#pragma unroll
+  for (int i = 15; i > 0; i--) k[i] -= k[i - 1];
+  k[0] -= before;
+  return pm;
+}
+__device__ __forceinline__ void st_piece(void* p, const int32_t (&k)[16]) {
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    reinterpret_cast<int4*>(p)[c] = make_int4(k[4 * c], k[4 * c + 1], k[4 * c + 2], k[4 * c + 3]);
+}
+
+// Codes, records and histograms of codec block b under the global predictor: the mixed
+// difference (1 - S_x)(1 - S_y)(1 - S_z) k over the halo'd box (the paper's 1/2/3-D
+// predictor, Sec. IV-B2, with no chunk restarts), then the tail.
+//
+// As in process_tile, a thread takes 16 consecutive elements of a row: the x difference
+// runs in registers, and what it reads from its neighbours for y and z are four 16-byte
+// words each of rows that hold their x differences (the halo rows' among them: 33 more in
+// 3-D, 4 pieces in 2-D).  A thread per box element and then per slot, with a division or
+// two to place each and seven scalar neighbour reads, took 205 instructions per 32
+// elements and 280 us at 100x500x500; this: 77 us.  The box's row pitch (20 or 68
+// elements, an odd number of 16-byte words) spreads eight rows over all banks.
 template <int ND, typename E>
 __device__ void process_tile_global(const ConstructArgs& A, uint32_t b, const uint32_t* box,
                                     SmemT<E, kHaloMax>& S, E* in, uint32_t& n_rec_acc, uint32_t& n_patch_acc) {
   using H = Halo<ND>;
-  constexpr uint32_t NB = H::X * H::Y * H::Z;
-  constexpr uint32_t PER = (NB + kThreads - 1) / kThreads;
-  constexpr int hz = ND == 3 ? 1 : 0, hy = ND >= 2 ? 1 : 0;
+  static_assert(sizeof(E) == 4, "FP32 fields");
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t w[3] = {box[3], box[4], box[5]};
   const uint32_t m = w[0] * w[1] * w[2];
+  const Geom& g = A.g;
+  const bool full = w[0] == g.blk[0] && w[1] == g.blk[1] && w[2] == g.blk[2];
   const Pq<E> pq(S.pq);
   const int32_t r = (int32_t)A.radius;
   int32_t* dglob = A.deltas + (uint64_t)b * kSlots;
+  int32_t* K = reinterpret_cast<int32_t*>(in);
   uint32_t err = 0;
+  if (ND == 3 || full) {
+    int32_t k[16];
+    uint32_t u[16], pm;
+    if (ND == 1) {
+      pm = quant_piece(pq, in + kHaloPadX + 16 * tid, k, err);
+#pragma unroll
+      for (int i = 0; i < 16; i++) u[i] = (uint32_t)(k[i] + r);
+    } else if (ND == 2) {
+      // piece t & 3 of row t >> 2; threads 0 to 3 also take the row above the tile
+      const uint32_t at = ((tid >> 2) + 1) * H::X + kHaloPadX + 16 * (tid & 3);
+      const uint32_t above = kHaloPadX + 16 * (tid & 3);
+      if (tid < 32) {
+        if (tid < 4) quant_piece(pq, in + above, k, err);
+        __syncwarp();
+        if (tid < 4) st_piece(K + above, k);
+      }
+      pm = quant_piece(pq, in + at, k, err);
+      __syncthreads();  // every element read: the pieces now carry their x differences
+      st_piece(K + at, k);
+      __syncthreads();
+      const int4* ry = reinterpret_cast<const int4*>(K + at - H::X);
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const int4 a = ry[c];
+        u[4 * c] = (uint32_t)(k[4 * c] - a.x + r);
+        u[4 * c + 1] = (uint32_t)(k[4 * c + 1] - a.y + r);
+        u[4 * c + 2] = (uint32_t)(k[4 * c + 2] - a.z + r);
+        u[4 * c + 3] = (uint32_t)(k[4 * c + 3] - a.w + r);
+      }
+    } else {
+      // row (z, y) = (t >> 4, t & 15); threads 0 to 32 also take a halo row: the plane
+      // below the tile, then the row before each plane's first.  A row is read and
+      // overwritten by its own thread alone.
+      constexpr uint32_t PL = H::X * H::Y;
+      const uint32_t at = ((tid >> 4) + 1) * PL + ((tid & 15) + 1) * H::X + kHaloPadX;
+      if (!full && tid < kSlots / 32) S.patch[tid] = 0;
+      if (tid < 33) {
+        const uint32_t halo = (tid < 17 ? tid * H::X : (uint32_t)(tid - 16) * PL) + kHaloPadX;
+        quant_piece(pq, in + halo, k, err);
+        st_piece(K + halo, k);
+      }
+      pm = quant_piece(pq, in + at, k, err);
+      st_piece(K + at, k);
+      __syncthreads();
+      const int4* ry = reinterpret_cast<const int4*>(K + at - H::X);
+      const int4* rz = reinterpret_cast<const int4*>(K + at - PL);
+      const int4* ryz = reinterpret_cast<const int4*>(K + at - PL - H::X);
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const int4 a = ry[c], bz = rz[c], d = ryz[c];
+        u[4 * c] = (uint32_t)(k[4 * c] - a.x - bz.x + d.x + r);
+        u[4 * c + 1] = (uint32_t)(k[4 * c + 1] - a.y - bz.y + d.y + r);
+        u[4 * c + 2] = (uint32_t)(k[4 * c + 2] - a.z - bz.z + d.z + r);
+        u[4 * c + 3] = (uint32_t)(k[4 * c + 3] - a.w - bz.w + d.w + r);
+      }
+    }
+    if (full) post16(S, u, pm, r, dglob);
+    else post_edge_rows(S, u, pm, w, m, r, dglob);
+    __syncthreads();
+    tile_tail(A, b, S, m, full, err, n_rec_acc, n_patch_acc);
+    return;
+  }
+  // edge blocks of 1-D and 2-D fields: by box element, then by dense slot
+  constexpr uint32_t NB = H::X * H::Y * H::Z;
+  constexpr uint32_t PER = (NB + kThreads - 1) / kThreads;
+  constexpr int hy = ND >= 2 ? 1 : 0;
   if (tid < kSlots / 32) S.patch[tid] = 0;
   __syncthreads();
   // prequantize every box element the predictor reads (x >= -1) into registers
@@ -753,20 +884,18 @@ __device__ void process_tile_global(const ConstructArgs& A, uint32_t b, const ui
     const uint32_t p = tid + kThreads * i;
     kv[i] = 0;
     if (p < NB) {
-      const int x = (int)(p % H::X) - (int)kHaloPadX;
-      const int y = (int)((p / H::X) % H::Y) - hy, z = (int)(p / (H::X * H::Y)) - hz;
+      const int x = (int)(p % H::X) - (int)kHaloPadX, y = (int)(p / H::X) - hy;
       if (x >= -1) {
         bool patch = false;
         if (!pq.fast(in[p], kv[i])) err |= pq.full(in[p], kv[i], patch);
-        if (patch && x >= 0 && y >= 0 && z >= 0 && (uint32_t)x < w[2] && (uint32_t)y < w[1] && (uint32_t)z < w[0]) {
-          const uint32_t j = ((uint32_t)z * w[1] + (uint32_t)y) * w[2] + (uint32_t)x;
+        if (patch && x >= 0 && y >= 0 && (uint32_t)x < w[2] && (uint32_t)y < w[1]) {
+          const uint32_t j = (uint32_t)y * w[2] + (uint32_t)x;
           atomicOr(&S.patch[j >> 5], 1u << (j & 31));
         }
       }
     }
   }
-  __syncthreads();  // every element read: the box now carries k (int32, from its start)
-  int32_t* K = reinterpret_cast<int32_t*>(in);
+  __syncthreads();  // every element read: the box now carries k
 #pragma unroll
   for (uint32_t i = 0; i < PER; i++) {
     const uint32_t p = tid + kThreads * i;
@@ -779,25 +908,10 @@ __device__ void process_tile_global(const ConstructArgs& A, uint32_t b, const ui
     const bool inb = j < m;
     uint32_t q = 0;
     if (inb) {
-      uint32_t x = j, y = 0, z = 0;
-      if (ND == 2) {
-        y = j / w[2];
-        x = j - y * w[2];
-      } else if (ND == 3) {
-        const uint32_t pl = w[1] * w[2];
-        z = j / pl;
-        const uint32_t rr = j - z * pl;
-        y = rr / w[2];
-        x = rr - y * w[2];
-      }
-      const uint32_t p = ((z + hz) * H::Y + (y + hy)) * H::X + (x + kHaloPadX);
+      const uint32_t y = ND == 2 ? j / w[2] : 0u, x = j - y * w[2];
+      const uint32_t p = (y + hy) * H::X + (x + kHaloPadX);
       int32_t d = K[p] - K[p - 1];
       if (ND >= 2) d -= K[p - H::X] - K[p - H::X - 1];
-      if (ND == 3) {
-        constexpr uint32_t PL = H::X * H::Y;
-        d -= K[p - PL] - K[p - PL - 1];
-        d += K[p - PL - H::X] - K[p - PL - H::X - 1];
-      }
       const uint32_t u = (uint32_t)(d + r);
       q = u - 1u < (uint32_t)(2 * r - 1) ? u : 0u;  // |delta| < r
       atomicAdd(&S.hc[q], 1u);

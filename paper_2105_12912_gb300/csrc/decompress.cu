@@ -1308,41 +1308,249 @@ __global__ __launch_bounds__(kRecThreads) void reconstruct_kernel(DecodeArgs a) 
 
 // =================================================================================
 // global (unchunked) Lorenzo reconstruction: the N-D partial sum of q' over the whole
-// field (Sec. IV-B "Partial-Sum Lorenzo Reconstruction" holds without chunks), as
-// one pass per axis over an int32 copy of q' kept in the output buffer; the last pass
-// scales to FP32 in place, then the verbatim patches are written.
+// field (Sec. IV-B "Partial-Sum Lorenzo Reconstruction" holds without chunks).
+//
+// Bound by memory: the codes are read and the field written, and every full-size pass in
+// between costs as much again.  A pass per axis (q' written out, then a scan along x, y
+// and z, each reading and writing the field) took 296 us at 3-D 100x500x500, 143 of them
+// in the x scan's serial 4-byte loads.  Now only sums cross blocks: each block's row sums
+// (1/16 of the field) are scanned along x, each block forms the partial sums along x and
+// y of its own rows, with the row's sum before it, in shared memory and writes them once,
+// the strips' last rows (1/16 of the field) are scanned along y, and the last pass adds
+// those on its way along z: 95 us.  1-D fields take one pass with a look-back.
 // =================================================================================
-constexpr uint32_t kScanTile = 4096;  // elements per tile of the x pass (256 threads x 16)
 
-// q' of codec block b (q - r, or the outlier's delta) at its elements' field positions.
-__global__ __launch_bounds__(kRecThreads) void gfuse_kernel(DecodeArgs a) {
+// q' (q - r, or the outlier's delta) of the n <= 16 consecutive slots j0 .. j0 + n - 1 of
+// block b; zeros behind them.
+__device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, uint32_t j0, uint32_t n,
+                                             int32_t (&q)[16]) {
+  const uint16_t* codes = a.codes + (uint64_t)b * kSlots + j0;
+  const int32_t r = (int32_t)a.radius;
+  if (n == 16 && (j0 & 7) == 0) {
+    const uint4 v[2] = {reinterpret_cast<const uint4*>(codes)[0], reinterpret_cast<const uint4*>(codes)[1]};
+    const uint32_t u[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      q[2 * i] = (int32_t)(u[i] & 0xffffu) - r;
+      q[2 * i + 1] = (int32_t)(u[i] >> 16) - r;
+    }
+  } else {
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++) q[i] = i < n ? (int32_t)codes[i] - r : 0;
+  }
+  uint32_t lo = a.rec_start[b];
+  const uint32_t re = a.rec_start[b + 1];
+  if (lo == re || n == 0) return;
+  // the row's records (sorted by key): the first one by a search, then in order
+  const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
+  const uint32_t k0 = (b * (uint32_t)kSlots + j0) * 2u, k1 = k0 + 2u * n;
+  uint32_t hi = re;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (rec[mid].x < k0) lo = mid + 1;
+    else hi = mid;
+  }
+  for (; lo < re; lo++) {
+    const uint2 kv = rec[lo];
+    if (kv.x >= k1) break;
+    const uint32_t at = (kv.x - k0) >> 1;
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++)
+      if (i == at && !(kv.x & 1u)) q[i] = (int32_t)kv.y;
+  }
+}
+
+// The row piece of thread t of a block: 3-D row (z, y) = (t / 16, t % 16), up to 16
+// elements; 2-D piece t % 4 (16 elements) of row t / 4.  row: its row index in the field.
+struct RowPiece {
+  uint32_t j0, n;  // first slot and number of slots
+  uint32_t z, y;   // in the block
+  bool valid;
+};
+template <int ND>
+__device__ __forceinline__ RowPiece row_piece(const uint32_t* w) {
+  const uint32_t t = threadIdx.x;
+  RowPiece p;
+  const uint32_t x0 = ND == 3 ? 0u : 16u * (t & 3u);
+  p.z = ND == 3 ? t >> 4 : 0u;
+  p.y = ND == 3 ? t & 15u : t >> 2;
+  p.valid = p.z < w[0] && p.y < w[1] && x0 < w[2];
+  p.n = p.valid ? min(16u, w[2] - x0) : 0u;
+  p.j0 = p.valid ? (p.z * w[1] + p.y) * w[2] + x0 : 0u;
+  return p;
+}
+
+// Sums of the block's rows: totals[bx][row], row over the field's rows.
+template <int ND>
+__global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) {
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint32_t b = blockIdx.x;
   uint32_t org[3], w[3];
   block_box(a.g, b, org, w);
-  const uint32_t m = w[0] * w[1] * w[2];
-  const int32_t r = (int32_t)a.radius;
-  int32_t* q = reinterpret_cast<int32_t*>(a.out);
-  const uint16_t* codes = a.codes + (uint64_t)b * kSlots;
-  const uint64_t ny = a.g.n[1], nx = a.g.n[2];
-  auto elem = [&](uint32_t j) -> uint64_t {
-    const uint32_t pl = w[1] * w[2], zz = j / pl, rr = j - zz * pl, yy = rr / w[2], xx = rr - yy * w[2];
-    return ((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + org[2] + xx;
-  };
-  for (uint32_t j = threadIdx.x; j < m; j += kRecThreads) q[elem(j)] = (int32_t)codes[j] - r;
-  __syncthreads();  // orders the outliers' writes after the codes' writes
-  const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
-  for (uint32_t i = a.rec_start[b] + threadIdx.x; i < a.rec_start[b + 1]; i += kRecThreads) {
-    const uint2 kv = rec[i];
-    if ((kv.x & 1u) == 0) q[elem((kv.x >> 1) % kSlots)] = (int32_t)kv.y;
+  const RowPiece p = row_piece<ND>(w);
+  int32_t q[16], sum = 0;
+  load_fused16(a, b, p.j0, p.n, q);
+#pragma unroll
+  for (int i = 0; i < 16; i++) sum += q[i];
+  if (ND == 2) {
+    sum += __shfl_xor_sync(~0u, sum, 1);
+    sum += __shfl_xor_sync(~0u, sum, 2);
+  }
+  const uint64_t nrows = (uint64_t)a.g.n[0] * a.g.n[1];
+  if (p.valid && (ND == 3 || (threadIdx.x & 3) == 0))
+    a.gtotals[(b % a.g.g[2]) * nrows + (uint64_t)(org[0] + p.z) * a.g.n[1] + org[1] + p.y] = sum;
+}
+
+// Row sums to the sums before each block, in place (a thread per row).
+__global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint64_t nrows = (uint64_t)a.g.n[0] * a.g.n[1];
+  const uint64_t row = blockIdx.x * 256ull + threadIdx.x;
+  if (row >= nrows) return;
+  const uint32_t nb = a.g.g[2];
+  int32_t* t = a.gtotals + row;
+  int32_t acc = 0;
+  for (uint32_t i = 0; i < nb; i += 8) {
+    int32_t v[8];
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = i + k < nb ? t[(i + k) * nrows] : 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) {
+      if (i + k < nb) t[(i + k) * nrows] = acc;
+      acc += v[k];
+    }
   }
 }
 
-// Exclusive prefix, for a segmented scan, of the tiles before `tile`: the aggregates
-// back to the nearest tile that published an inclusive value (a tile holding a segment
-// start), summed modulo 2^62 and read back as a signed value.  One full warp calls;
-// the wait is bounded (ERR_TIMEOUT and 0 on expiry).
-__device__ int64_t seg_lookback_warp(const uint64_t* state, uint32_t tile, uint32_t* status, uint32_t spin_limit) {
+// Partial sums along x, over the whole row, and along y, within the block, of one block.
+// Rows cross from threads to columns in shared memory; 16-byte chunk c of the 16-element
+// piece R sits at c ^ ((R >> 1) & 3), so that eight threads writing their pieces touch
+// all banks.
+template <int ND>
+__global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
+  __shared__ __align__(16) int32_t s_k[kSlots];
+  __shared__ int32_t s_band[4][64];
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint32_t b = blockIdx.x, tid = threadIdx.x;
+  uint32_t org[3], w[3];
+  block_box(a.g, b, org, w);
+  const uint64_t ny = a.g.n[1], nx = a.g.n[2], nrows = (uint64_t)a.g.n[0] * ny;
+  const RowPiece p = row_piece<ND>(w);
+  int32_t k[16];
+  load_fused16(a, b, p.j0, p.n, k);
+  int32_t carry = p.valid ? a.gtotals[(b % a.g.g[2]) * nrows + (uint64_t)(org[0] + p.z) * ny + org[1] + p.y] : 0;
+#pragma unroll
+  for (int i = 1; i < 16; i++) k[i] += k[i - 1];
+  if (ND == 2) {
+    // the row's earlier pieces
+    const int32_t u1 = __shfl_up_sync(~0u, k[15], 1, 4), u2 = __shfl_up_sync(~0u, k[15], 2, 4),
+                  u3 = __shfl_up_sync(~0u, k[15], 3, 4);
+    const uint32_t at = tid & 3;
+    carry += (at >= 1 ? u1 : 0) + (at >= 2 ? u2 : 0) + (at >= 3 ? u3 : 0);
+  }
+  const uint32_t key = (tid >> 1) & 3;
+#pragma unroll
+  for (uint32_t c = 0; c < 4; c++)
+    reinterpret_cast<int4*>(s_k + 16 * tid)[c ^ key] =
+        make_int4(k[4 * c] + carry, k[4 * c + 1] + carry, k[4 * c + 2] + carry, k[4 * c + 3] + carry);
+  __syncthreads();
+  auto at = [&](uint32_t e) -> int32_t { return s_k[e ^ ((e >> 3) & 12u)]; };
+  int32_t* q = reinterpret_cast<int32_t*>(a.out);
+  if (ND == 3) {
+    const uint32_t x = tid & 15, z = tid >> 4;
+    if (x < w[2] && z < w[0]) {
+      int32_t* o = q + ((uint64_t)(org[0] + z) * ny + org[1]) * nx + org[2] + x;
+      int32_t acc = 0;
+#pragma unroll
+      for (uint32_t y = 0; y < 16; y++) {
+        acc += at((z * 16 + y) * 16 + x);
+        if (y < w[1]) o[y * nx] = acc;
+      }
+    }
+  } else {
+    // column x, rows 16 band .. 16 band + 15; bands chain through their sums
+    const uint32_t x = tid & 63, band = tid >> 6;
+    int32_t v[16], sum = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++) {
+      const uint32_t y = 16 * band + i;
+      sum += y < w[1] ? at(y * 64 + x) : 0;
+      v[i] = sum;
+    }
+    s_band[band][x] = sum;
+    __syncthreads();
+    int32_t before = 0;
+    for (uint32_t i = 0; i < band; i++) before += s_band[i][x];
+    if (x < w[2]) {
+      int32_t* o = q + (uint64_t)(org[1] + 16 * band) * nx + org[2] + x;
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++)
+        if (16 * band + i < w[1]) o[i * nx] = v[i] + before;
+    }
+  }
+}
+
+// Strips of block height along y: the sums before each strip, from the last row of the
+// strips before it (a thread per plane and column): gstrips[(z gy + by) nx + x].
+__global__ __launch_bounds__(256) void gy_carry_kernel(DecodeArgs a) {
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
+  const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
+  if (c >= nz * nx) return;
+  const uint64_t z = c / nx, x = c - z * nx;
+  const uint32_t gy = a.g.g[1], h = a.g.blk[1];
+  const int32_t* q = reinterpret_cast<const int32_t*>(a.out) + (z * ny + h - 1) * nx + x;
+  int32_t* o = a.gstrips + z * gy * nx + x;
+  int32_t acc = 0;
+  o[0] = 0;
+  for (uint32_t i = 0; i + 1 < gy; i += 8) {
+    int32_t v[8];
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = i + k + 1 < gy ? q[(uint64_t)(i + k) * h * nx] : 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) {
+      acc += v[k];
+      if (i + k + 1 < gy) o[(uint64_t)(i + k + 1) * nx] = acc;
+    }
+  }
+}
+
+// The last pass, in place: the strips' sums added, partial sums along z (a thread per
+// column; 2-D fields have one plane), scaled.
+__global__ __launch_bounds__(256) void gfinal_kernel(DecodeArgs a) {
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
+  const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
+  if (c >= ny * nx) return;
+  const uint64_t y = c / nx, x = c - y * nx;
+  const uint32_t gy = a.g.g[1];
+  float* out = a.out + c;
+  const int32_t* q = reinterpret_cast<const int32_t*>(out);
+  const int32_t* st = a.gstrips + (y / a.g.blk[1]) * nx + x;
+  const uint64_t plane = ny * nx, splane = (uint64_t)gy * nx;
+  const float ebx2 = a.ebx2_f;
+  int32_t acc = 0;
+  uint64_t z = 0;
+  for (; z + 8 <= nz; z += 8) {
+    int32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = q[(z + i) * plane] + st[(z + i) * splane];
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      acc += v[i];
+      __stcs(&out[(z + i) * plane], scale(acc, ebx2));
+    }
+  }
+  for (; z < nz; z++) {
+    acc += q[z * plane] + st[z * splane];
+    __stcs(&out[z * plane], scale(acc, ebx2));
+  }
+}
+
+// Exclusive prefix of the tiles before `tile`: the aggregates back to the nearest tile
+// that published an inclusive value, summed modulo 2^62 and read back as a signed value.
+// One full warp calls; the wait is bounded (ERR_TIMEOUT and 0 on expiry).
+__device__ int64_t signed_lookback_warp(const uint64_t* state, uint32_t tile, uint32_t* status, uint32_t spin_limit) {
   const int lane = threadIdx.x & 31;
   if (tile == 0) return 0;
   uint64_t excl = 0;
@@ -1371,17 +1579,11 @@ __device__ int64_t seg_lookback_warp(const uint64_t* state, uint32_t tile, uint3
   return (int64_t)(excl << 2) >> 2;
 }
 
-__device__ __forceinline__ void seg_publish(uint64_t* state, uint32_t tile, bool inclusive, int64_t v) {
-  st_relaxed(&state[tile], (inclusive ? LB_INC : LB_AGG) | ((uint64_t)v & LB_VAL));
-}
-
-// Pass along x: an inclusive scan of the flattened field restarted at every row start
-// (a segment of n[2] elements), one tile of 4096 elements per CTA in ticket order;
-// tiles chain their carries by decoupled look-back.  `last`: scale to FP32 in place.
-__global__ __launch_bounds__(256) void gscan_x_kernel(DecodeArgs a, uint64_t* state, int last) {
+// 1-D fields: the inclusive scan of the whole field in one pass, one codec block (4096
+// consecutive elements) per CTA in ticket order; blocks chain by decoupled look-back.
+__global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state) {
   __shared__ uint32_t s_tile;
   __shared__ int s_go;
-  __shared__ int s_wf[8];
   __shared__ int32_t s_ws[8];
   __shared__ int32_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1392,125 +1594,39 @@ __global__ __launch_bounds__(256) void gscan_x_kernel(DecodeArgs a, uint64_t* st
   __syncthreads();
   if (!s_go) return;  // every CTA leaves: no tile waits on another
   const uint32_t tile = s_tile;
-  const uint64_t n = a.g.nelem, seg = a.g.n[2];
-  int32_t* q = reinterpret_cast<int32_t*>(a.out);
-  const uint64_t base = (uint64_t)tile * kScanTile + 16u * tid;
-  int32_t v[16];
-  uint32_t heads = 0;
-  uint64_t rpos = base % seg;
+  const uint64_t first = (uint64_t)tile * kSlots + 16u * tid;
+  const uint32_t n = first < a.g.nelem ? (uint32_t)min((unsigned long long)16, (unsigned long long)(a.g.nelem - first)) : 0u;
+  int32_t k[16];
+  load_fused16(a, tile, 16u * tid, n, k);
 #pragma unroll
-  for (int i = 0; i < 16; i++) {
-    const uint64_t idx = base + i;
-    v[i] = idx < n ? q[idx] : 0;
-    if (idx < n && rpos == 0) heads |= 1u << i;
-    rpos = rpos + 1 == seg ? 0 : rpos + 1;
-  }
-  // the thread's own segmented inclusive scan, and its pair (head seen, sum since it)
-  bool f = false;
-  int32_t run = 0;
-#pragma unroll
-  for (int i = 0; i < 16; i++) {
-    if ((heads >> i) & 1u) {
-      run = v[i];
-      f = true;
-    } else {
-      run += v[i];
-    }
-    v[i] = run;
-  }
-  // warp scan of the pairs (combine a then b: (fa | fb, fb ? sb : sa + sb))
-  bool F = f;
-  int32_t S = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const bool fu = __shfl_up_sync(~0u, (int)F, o) != 0;
-    const int32_t su = __shfl_up_sync(~0u, S, o);
-    if (lane >= o) {
-      if (!F) S += su;
-      F = F || fu;
-    }
-  }
-  bool Fe = __shfl_up_sync(~0u, (int)F, 1) != 0;
-  int32_t Se = __shfl_up_sync(~0u, S, 1);
-  if (lane == 0) {
-    Fe = false;
-    Se = 0;
-  }
-  if (lane == 31) {
-    s_wf[wid] = F;
-    s_ws[wid] = S;
-  }
+  for (int i = 1; i < 16; i++) k[i] += k[i - 1];
+  const int32_t incl = warp_incl_scan(k[15]);
+  if (lane == 31) s_ws[wid] = incl;
   __syncthreads();
-  bool Fw = false;
-  int32_t Sw = 0;
-  for (int ww = 0; ww < wid; ww++) {
-    Sw = s_wf[ww] ? s_ws[ww] : Sw + s_ws[ww];
-    Fw = Fw || s_wf[ww];
-  }
-  const bool Ft = Fw || Fe;               // a segment starts before this thread, in the tile
-  const int32_t St = Fe ? Se : Sw + Se;   // and the sum since the latest such start
+  int32_t pre = incl - k[15];
+  for (int v = 0; v < wid; v++) pre += s_ws[v];
   if (wid == 0) {
-    bool TF = false;
-    int32_t TS = 0;
-    for (int ww = 0; ww < 8; ww++) {
-      TS = s_wf[ww] ? s_ws[ww] : TS + s_ws[ww];
-      TF = TF || s_wf[ww];
-    }
-    if (lane == 0) seg_publish(state, tile, TF, TS);  // a tile with a segment start needs no carry
-    int64_t c = 0;
-    if ((uint64_t)tile * kScanTile % seg != 0) c = seg_lookback_warp(state, tile, &a.st->status, kSpinLimit);
+    const int64_t total = (int64_t)warp_sum(lane < 8 ? s_ws[lane] : 0);
+    if (lane == 0) st_relaxed(&state[tile], (tile == 0 ? LB_INC : LB_AGG) | ((uint64_t)total & LB_VAL));
+    const int64_t c = signed_lookback_warp(state, tile, &a.st->status, kSpinLimit);
     if (lane == 0) {
-      if (!TF) seg_publish(state, tile, true, c + TS);
+      if (tile) st_relaxed(&state[tile], LB_INC | ((uint64_t)(c + total) & LB_VAL));
       s_carry = (int32_t)c;
     }
   }
   __syncthreads();
-  const int32_t pre = Ft ? St : s_carry + St;  // what precedes the thread's first element
-  const float ebx2 = a.ebx2_f;
-  float* out = a.out;
+  pre += s_carry;
+  float* out = a.out + first;
+  if (n == 16 && ((uintptr_t)out & 15) == 0) {
 #pragma unroll
-  for (int i = 0; i < 16; i++) {
-    const uint64_t idx = base + i;
-    // elements before the thread's first head add what precedes the thread
-    const bool own = (heads & ((2u << i) - 1u)) != 0;
-    const int32_t k = own ? v[i] : pre + v[i];
-    if (idx < n) {
-      if (last) out[idx] = scale(k, ebx2);
-      else q[idx] = k;
-    }
-  }
-}
-
-// Pass along y (or z): thread (outer, x) runs down its column; `last`: scale in place.
-__global__ __launch_bounds__(256) void gscan_col_kernel(DecodeArgs a, int axis, int last) {
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
-  const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
-  // axis 1 (y): columns (z, x), stride nx, length ny; axis 0 (z): columns (y, x), stride ny nx, length nz
-  const uint64_t ncol = axis == 1 ? nz * nx : ny * nx;
-  const uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (c >= ncol) return;
-  const uint64_t stride = axis == 1 ? nx : ny * nx, len = axis == 1 ? ny : nz;
-  const uint64_t start = axis == 1 ? (c / nx) * ny * nx + c % nx : c;
-  int32_t* q = reinterpret_cast<int32_t*>(a.out);
-  float* out = a.out;
-  const float ebx2 = a.ebx2_f;
-  int32_t acc = 0;
-  uint64_t i = 0;
-  for (; i + 4 <= len; i += 4) {
-    int32_t t[4];
+    for (int i = 0; i < 4; i++)
+      __stcs(reinterpret_cast<float4*>(out) + i,
+             make_float4(scale(k[4 * i] + pre, a.ebx2_f), scale(k[4 * i + 1] + pre, a.ebx2_f),
+                         scale(k[4 * i + 2] + pre, a.ebx2_f), scale(k[4 * i + 3] + pre, a.ebx2_f)));
+  } else {
 #pragma unroll
-    for (int u = 0; u < 4; u++) t[u] = q[start + (i + u) * stride];
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-      acc += t[u];
-      if (last) out[start + (i + u) * stride] = scale(acc, ebx2);
-      else q[start + (i + u) * stride] = acc;
-    }
-  }
-  for (; i < len; i++) {
-    acc += q[start + i * stride];
-    if (last) out[start + i * stride] = scale(acc, ebx2);
-    else q[start + i * stride] = acc;
+    for (uint32_t i = 0; i < 16; i++)
+      if (i < n) out[i] = scale(k[i] + pre, a.ebx2_f);
   }
 }
 
@@ -1533,17 +1649,19 @@ __global__ void gpatch_kernel(DecodeArgs a) {
 // The global reconstruction's launches (after set-up, decoding and run expansion).
 cudaError_t launch_global_reconstruct(const DecodeArgs& a, cudaStream_t s) {
   trace_begin(K_RECONSTRUCT, s);
-  gfuse_kernel<<<a.g.nblk, kRecThreads, 0, s>>>(a);
   const int nd = a.g.ndim;
-  const uint64_t ntiles = (a.g.nelem + kScanTile - 1) / kScanTile;
-  gscan_x_kernel<<<(unsigned)ntiles, 256, 0, s>>>(a, a.scan_state, nd == 1 ? 1 : 0);
-  if (nd >= 2) {
-    const uint64_t cy = (uint64_t)a.g.n[0] * a.g.n[2];
-    gscan_col_kernel<<<(unsigned)((cy + 255) / 256), 256, 0, s>>>(a, 1, nd == 2 ? 1 : 0);
-  }
-  if (nd == 3) {
-    const uint64_t cz = (uint64_t)a.g.n[1] * a.g.n[2];
-    gscan_col_kernel<<<(unsigned)((cz + 255) / 256), 256, 0, s>>>(a, 0, 1);
+  const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
+  auto ctas = [](uint64_t threads) { return (unsigned)((threads + 255) / 256); };
+  if (nd == 1) {
+    g1d_kernel<<<a.g.nblk, 256, 0, s>>>(a, a.scan_state);
+  } else {
+    if (nd == 2) grow_totals_kernel<2><<<a.g.nblk, kRecThreads, 0, s>>>(a);
+    else grow_totals_kernel<3><<<a.g.nblk, kRecThreads, 0, s>>>(a);
+    gx_carry_kernel<<<ctas(nz * ny), 256, 0, s>>>(a);
+    if (nd == 2) gblock_kernel<2><<<a.g.nblk, kRecThreads, 0, s>>>(a);
+    else gblock_kernel<3><<<a.g.nblk, kRecThreads, 0, s>>>(a);
+    gy_carry_kernel<<<ctas(nz * nx), 256, 0, s>>>(a);
+    gfinal_kernel<<<ctas(ny * nx), 256, 0, s>>>(a);
   }
   if (a.n_rec) gpatch_kernel<<<(unsigned)((a.n_rec + 255) / 256 < 1024 ? (a.n_rec + 255) / 256 : 1024), 256, 0, s>>>(a);
   trace_end(K_RECONSTRUCT, s);

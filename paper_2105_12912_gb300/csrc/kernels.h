@@ -156,8 +156,10 @@ struct DecodeArgs {
   double step_d;
   int f64;
   uint64_t* prep_lb;   // set-up chunks' look-back states (2 per 1024 blocks), zeroed per call
-  int global;          // global (unchunked) Lorenzo archive: reconstruction by per-axis passes
-  uint64_t* scan_state;  // their look-back states (one per 4096 elements), zeroed per call
+  int global;          // global (unchunked) Lorenzo archive: partial sums over the whole field
+  uint64_t* scan_state;  // 1-D: their look-back states (one per block), zeroed per call
+  int32_t* gtotals;      // 2-D, 3-D: row sums by block along x, then the sums before each
+  int32_t* gstrips;      // and the sums before each strip of blocks along y
   int dead;            // batches: the header failed validation, do nothing
   int check_hdr;       // the arguments come from a host copy of the header (hdr): the
   uint32_t hdr[32];    // set-up compares the device archive's header with it
