@@ -5,10 +5,10 @@
 //                          validation and each block's first record
 //   stream_decode_kernel   one warp per interleaved 32-lane stream (Huffman code
 //                          streams, RLE+Huffman value and length streams)
-//   rle_expand_kernel      one CTA per listed RLE / RLE+Huffman block: runs to codes
-//   reconstruct_kernel<ND> fuse outliers (q' = q - r, or delta), N-D partial sums
-//                          per chunk (Alg. 1, Sec. IV-B2), scale by 2eb, verbatim
-//                          patches
+//   reconstruct_kernel<ND> one CTA per listed block (runs, or cut by the field's edge):
+//                          runs to codes, fuse outliers (q' = q - r, or delta), N-D
+//                          partial sums per chunk (Alg. 1, Sec. IV-B2), scale by 2eb,
+//                          verbatim patches
 //   dec_status_kernel      the status word of an asynchronous decompression
 // and their batch forms (per-field tables in device memory, headers read and checked
 // on the device by dec_header_batch_kernel).
@@ -572,8 +572,11 @@ struct Out<float> {
   __device__ explicit Out(const DecodeArgs& a) : p(a.out), ebx2(a.ebx2_f) {}
   __device__ __forceinline__ float value(int32_t k) const { return scale(k, ebx2); }
   __device__ __forceinline__ void put(uint64_t i, int32_t k) const { __stcs(&p[i], scale(k, ebx2)); }
-  __device__ __forceinline__ void put_patch(uint64_t i, int32_t k, bool patch, uint32_t bits) const {
-    __stcs(&p[i], patch ? __uint_as_float(bits) : scale(k, ebx2));
+  // four consecutive elements, i a multiple of four elements from x0: vec4(x0) must hold
+  __device__ __forceinline__ bool vec4(uint64_t x0) const { return ((uintptr_t)(p + x0) & 15) == 0; }
+  __device__ __forceinline__ void put4(uint64_t i, int4 k) const {
+    __stcs(reinterpret_cast<float4*>(&p[i]),
+           make_float4(scale(k.x, ebx2), scale(k.y, ebx2), scale(k.z, ebx2), scale(k.w, ebx2)));
   }
   __device__ __forceinline__ void patch(uint64_t i, uint32_t bits) const { p[i] = __uint_as_float(bits); }
 };
@@ -590,7 +593,12 @@ struct Out<double> {
     return __hiloint2double((int)(hi | ((uint32_t)k & 0x80000000u)), (int)(t << 21));
   }
   __device__ __forceinline__ void put(uint64_t i, int32_t k) const { __stcs(&p[i], __dmul_rn(to_double(k), step)); }
-  __device__ __forceinline__ void put_patch(uint64_t i, int32_t k, bool, uint32_t) const { put(i, k); }
+  __device__ __forceinline__ bool vec4(uint64_t x0) const { return ((uintptr_t)(p + x0) & 15) == 0; }
+  __device__ __forceinline__ void put4(uint64_t i, int4 k) const {
+    __stcs(reinterpret_cast<double2*>(&p[i]), make_double2(__dmul_rn(to_double(k.x), step), __dmul_rn(to_double(k.y), step)));
+    __stcs(reinterpret_cast<double2*>(&p[i + 2]),
+           make_double2(__dmul_rn(to_double(k.z), step), __dmul_rn(to_double(k.w), step)));
+  }
   __device__ __forceinline__ void patch(uint64_t, uint32_t) const {}
 };
 
@@ -954,25 +962,35 @@ __global__ __launch_bounds__(32 * kStreamWarps, 2) void stream_decode_kernel(Dec
   stream_decode_body<ND, E>(a, 0, 0);
 }
 
-constexpr int kRleThreads = 256;
+// =================================================================================
+// blocks that no decoding warp reconstructs: run blocks, blocks cut by the field's edge,
+// and all blocks of a batch of mixed dimensionality
+//
+// Bound by latency and barriers, not by bytes: one CTA a block, and what it needs arrives
+// step after step.  So a thread keeps 16 consecutive slots (one row, or a piece of one) in
+// registers from the codes, or straight from the runs, to the sums along x; shared memory
+// only turns rows into columns for the other axes.  Runs become codes by a bit per run
+// start and population counts.  (A word per slot for the starts and a scan of maxima over
+// them took a dozen barriers, and the codes went through memory once more, in a launch of
+// their own for single fields: 40 mixed fields, 51 M elements: 175 -> 82 us;
+// 2-D 1800x3600: 12 us in two launches -> 6 us in one.)
+// =================================================================================
+constexpr int kRecThreads = 256;
 
-// RLE and RLE+Huffman blocks: run starts by a block scan, then every code position
-// finds its run by binary search.
-// Runs of run block b to its 4096 codes at `out` (global or shared memory, 16-byte
-// aligned), with shared scratch s_v, s_l (kSlots each) and s_start (kSlots + 1).
-// Returns false (the same in every thread) when the block is not expanded: not a run
-// block, corrupt (flagged), or its field already flagged corrupt.
-__device__ bool rle_expand_into(const DecodeArgs& a, uint32_t b, uint16_t* out, uint16_t* s_v, uint16_t* s_l,
-                                uint32_t* s_start) {
-  __shared__ uint32_t s_scan[33];
-  __shared__ uint32_t s_bad;
-  const int tid = threadIdx.x;
-  if (a.dead) return false;
-  const int codec = a.ar[a.off_codec + b];
-  if (codec != CODEC_RLE && codec != CODEC_RLE_HUFF) return false;
-  uint32_t org[3], w[3];
-  block_box(a.g, b, org, w);
-  const uint32_t m = w[0] * w[1] * w[2];
+struct RebuildSmem {
+  int32_t k[kSlots];          // sums along x, swizzled; before that, codes of a cut run block
+  uint16_t v[kSlots];         // run values
+  uint32_t bits[kSlots / 32]; // run starts
+  uint32_t tot[2][kRecThreads / 32];
+  int go;
+};
+
+// The runs of run block b (m elements) as codes: thread t gets slots 16t .. 16t + 15, two a
+// word (slots beyond m hold no code).  Returns false, the same in every thread, when the
+// block is corrupt (flagged).  Contains barriers.
+__device__ __forceinline__ bool expand_runs(const DecodeArgs& a, uint32_t b, int codec, uint32_t m, RebuildSmem& S,
+                                            uint32_t (&c)[8]) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint64_t bytes = a.blk_off[b + 1] - a.blk_off[b];
   const uint8_t* pay = a.ar + a.off_pay + a.blk_off[b];
   const uint32_t lim = 2 * a.radius;
@@ -991,341 +1009,95 @@ __device__ bool rle_expand_into(const DecodeArgs& a, uint32_t b, uint16_t* out, 
     if (tid == 0) flag(a.st, ERR_CORRUPT);
     return false;
   }
-  // the status is read once, by thread 0, and acted on after the barrier, so that a
-  // corruption flagged by another CTA meanwhile cannot split this CTA's threads
-  if (tid == 0) s_bad = (a.st->status & ERR_CORRUPT) ? 2u : 0u;
-  __syncthreads();
-  if (s_bad == 2u) return false;
-  for (uint32_t i = tid; i < nr; i += blockDim.x) {
-    s_v[i] = v[i];
-    s_l[i] = l[i];
+  if (tid < kSlots / 32) S.bits[tid] = 0;
+  bool bad = false;
+  uint32_t total = 0;
+  for (uint32_t i0 = 0, k = 0; i0 < nr; i0 += kRecThreads, k ^= 1) {
+    const uint32_t i = i0 + tid;
+    uint32_t len = 0;
+    if (i < nr) {
+      const uint16_t val = v[i];
+      len = l[i];
+      S.v[i] = val;
+      bad |= val >= lim || len == 0;
+    }
+    const uint32_t incl = warp_incl_scan(len);
+    if (lane == 31) S.tot[k][wid] = incl;
+    __syncthreads();  // (the other half of tot is free: every thread has read it before this barrier)
+    uint32_t start = total + incl - len;
+#pragma unroll
+    for (uint32_t w = 0; w < kRecThreads / 32; w++) {
+      const uint32_t t = S.tot[k][w];
+      if (w < wid) start += t;
+      total += t;
+    }
+    if (len && start < (uint32_t)kSlots) atomicOr(&S.bits[start >> 5], 1u << (start & 31));
   }
-  __syncthreads();
-  const uint32_t per = (nr + blockDim.x - 1) / blockDim.x;
-  const uint32_t lo = min(nr, tid * per), hi = min(nr, lo + per);
-  uint32_t sum = 0;
-  for (uint32_t i = lo; i < hi; i++) {
-    if (s_v[i] >= lim || s_l[i] == 0) s_bad = 1;
-    sum += s_l[i];
-  }
-  uint32_t tot;
-  uint32_t off = block_excl_scan<uint32_t>(sum, s_scan, &tot);
-  for (uint32_t i = lo; i < hi; i++) {
-    s_start[i] = off;
-    off += s_l[i];
-  }
-  if (tid == 0) s_start[nr] = tot;
-  __syncthreads();
-  if (s_bad || tot != m) {
+  if (__syncthreads_or(bad) || total != m) {
     if (tid == 0) flag(a.st, ERR_CORRUPT);
     return false;
   }
-  // run index of every position: mark run starts, then a running maximum
-  uint32_t* s_idx = s_start;  // starts are no longer needed once marked below
-  uint32_t my_starts[16];
-  const uint32_t cnt = hi - lo;
-  for (uint32_t i = 0; i < cnt && i < 16; i++) my_starts[i] = s_start[lo + i];
-  __syncthreads();
-  for (int i = tid; i < kSlots; i += blockDim.x) s_idx[i] = 0;
-  __syncthreads();
-  if (cnt <= 16) {
-    for (uint32_t i = 0; i < cnt; i++)
-      if (my_starts[i] < m) s_idx[my_starts[i]] = lo + i;
-  }
-  __syncthreads();
-  // contiguous 16 positions per thread: local running max, then a block scan of maxima
-  uint32_t run = 0;
-  const uint32_t p0 = 16 * tid;
-#pragma unroll
-  for (int i = 0; i < 16; i++) run = max(run, s_idx[p0 + i]);
-  // exclusive running max over threads (warp scan + per-warp carries)
-  uint32_t incl = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t u = __shfl_up_sync(~0u, incl, o);
-    if ((tid & 31) >= o) incl = max(incl, u);
-  }
-  if ((tid & 31) == 31) s_scan[tid >> 5] = incl;
-  __syncthreads();
-  uint32_t carry = 0;
-  for (int wv = 0; wv < (tid >> 5); wv++) carry = max(carry, s_scan[wv]);
-  uint32_t excl = __shfl_up_sync(~0u, incl, 1);
-  if ((tid & 31) == 0) excl = 0;
-  uint32_t cur = max(carry, excl);
-  uint32_t vals[8];
+  // runs that start before slot 16t: the words of earlier warps, then the warp's own
+  const uint32_t hb = (S.bits[tid >> 1] >> (16 * (tid & 1))) & 0xffffu;
+  const uint4 w4 = reinterpret_cast<const uint4*>(S.bits)[lane];
+  const uint32_t n4 = __popc(w4.x) + __popc(w4.y) + __popc(w4.z) + __popc(w4.w), n = __popc(hb);
+  uint32_t run = __reduce_add_sync(~0u, lane < 4 * wid ? n4 : 0u) + warp_incl_scan(n) - n;
+  uint32_t cur = run ? S.v[run - 1] : 0u;
 #pragma unroll
   for (int i = 0; i < 16; i++) {
-    cur = max(cur, s_idx[p0 + i]);
-    const uint16_t v = s_v[cur];
-    if (i & 1) vals[i >> 1] |= (uint32_t)v << 16;
-    else vals[i >> 1] = v;
+    if ((hb >> i) & 1u) cur = S.v[run++];
+    c[i >> 1] = i & 1 ? c[i >> 1] | cur << 16 : cur;
   }
-  // positions >= m get whatever run they fall in; they are never read
-  uint4* o4 = reinterpret_cast<uint4*>(out + p0);
-  o4[0] = make_uint4(vals[0], vals[1], vals[2], vals[3]);
-  o4[1] = make_uint4(vals[4], vals[5], vals[6], vals[7]);
   return true;
 }
 
-// Run block b expanded in place in the code stream (global), with its own scratch.
-__device__ void rle_expand_body(const DecodeArgs& a, uint32_t b) {
-  __shared__ __align__(16) uint16_t s_v[kSlots];
-  __shared__ __align__(16) uint16_t s_l[kSlots];
-  __shared__ __align__(16) uint32_t s_start[kSlots + 1];
-  rle_expand_into(a, b, a.codes + (uint64_t)b * kSlots, s_v, s_l, s_start);
-}
-
-// One CTA per listed run block (the list the set-up wrote; it holds exactly the
-// header's count unless the archive is corrupt, which the set-up has flagged and
-// the body checks).
-__global__ __launch_bounds__(kRleThreads) void rle_expand_kernel(DecodeArgs a) {
+// Global prediction: the codes of a listed run block into the code stream (the list the
+// set-up wrote holds exactly the header's count unless the archive is corrupt, which the
+// set-up has flagged).
+__global__ __launch_bounds__(kRecThreads) void rle_expand_kernel(DecodeArgs a) {
+  __shared__ __align__(16) RebuildSmem S;
   if (a.dead) return;
   const uint32_t b = a.runblk[blockIdx.x];
   if (b >= a.g.nblk) return;
-  rle_expand_body(a, b);
-}
-
-// =================================================================================
-// reconstruction: N-D partial sums per chunk (Sec. IV-B2), scaled by 2eb
-// =================================================================================
-constexpr int kRecThreads = 256;
-
-// codes: the block's 4096 code slots (global memory, or a shared-memory copy)
-template <int ND, typename E>
-__device__ void reconstruct_body(const DecodeArgs& a, uint32_t b, int32_t* s_q, const uint16_t* codes) {
-  // (the caller has checked the field's status, the same way in every thread)
-  const int tid = threadIdx.x;
-  uint32_t org[3], w[3];
+  const int codec = a.ar[a.off_codec + b];
+  if (codec != CODEC_RLE && codec != CODEC_RLE_HUFF) return;
+  // the status is read once, by thread 0, and acted on after the barrier, so that a
+  // corruption flagged by another CTA meanwhile cannot split this CTA's threads
+  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT);
+  __syncthreads();
+  if (!S.go) return;
+  uint32_t org[3], w[3], c[8];
   block_box(a.g, b, org, w);
-  const uint32_t m = w[0] * w[1] * w[2];
-  const int32_t r = (int32_t)a.radius;
-  const Out<E> out(a);
-  const uint32_t rs = a.rec_start[b], re = a.rec_start[b + 1];
-  const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
-  // a full 3-D block without records reads its codes directly; otherwise
-  // codes -> q' = q - r in s_q, then the outliers' deltas
-  const bool direct = ND == 3 && m == (uint32_t)kSlots && rs == re;
-  if (!direct) {
-    const uint4* src = reinterpret_cast<const uint4*>(codes);
-    for (uint32_t i = tid; i < (m + 7) / 8; i += kRecThreads) {
-      const uint4 v = src[i];
-      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        s_q[8 * i + 2 * k] = (int32_t)(u[k] & 0xffffu) - r;
-        s_q[8 * i + 2 * k + 1] = (int32_t)(u[k] >> 16) - r;
-      }
-    }
-    __syncthreads();
-    for (uint32_t i = rs + tid; i < re; i += kRecThreads) {
-      const uint2 kv = rec[i];
-      if ((kv.x & 1u) == 0) s_q[(kv.x >> 1) % kSlots] = (int32_t)kv.y;
-    }
-    __syncthreads();
-  }
-  const uint64_t ny = a.g.n[1], nx = a.g.n[2];
-  if (ND == 1) {
-    // each warp scans whole 256-chunks, 32 elements per step
-    const int lane = tid & 31, wid = tid >> 5;
-    for (uint32_t c = wid; c * 256 < m; c += kRecThreads / 32) {
-      int32_t carry = 0;
-#pragma unroll
-      for (int i = 0; i < 8; i++) {
-        const uint32_t j = c * 256 + i * 32 + lane;
-        const int32_t v = j < m ? s_q[j] : 0;
-        const int32_t inc = warp_incl_scan(v) + carry;
-        carry = __shfl_sync(~0u, inc, 31);
-        if (j < m) out.put((uint64_t)org[2] + j, inc);
-      }
-    }
-  } else if (ND == 2) {
-    // thread = (column x, 16-row chunk band): y sums in registers, x sums by shuffles
-    const uint32_t x = tid & 63, ry = tid >> 6;
-    const bool xin = x < w[2];
-    int32_t v[16];
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-      const uint32_t y = ry * 16 + i;
-      v[i] = (xin && y < w[1]) ? s_q[y * w[2] + x] : 0;
-    }
-#pragma unroll
-    for (int i = 1; i < 16; i++) v[i] += v[i - 1];
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) {
-        const int32_t u = __shfl_up_sync(~0u, v[i], o);
-        if ((x & 15) >= (uint32_t)o) v[i] += u;
-      }
-    }
-    if (xin) {
-      const uint64_t base = (uint64_t)org[1] * nx + org[2] + x;
-#pragma unroll
-      for (int i = 0; i < 16; i++) {
-        const uint32_t y = ry * 16 + i;
-        if (y < w[1]) out.put(base + (uint64_t)y * nx, v[i]);
-      }
-    }
-  } else if (m == (uint32_t)kSlots) {
-    // full 16^3 block: thread (x, y) takes the z column -- z sums in registers, x
-    // sums by shuffles -- then, after one exchange through shared memory, thread
-    // (x, z) takes the y column, adds along y in registers and stores its row
-    // segment (16 consecutive floats per half-warp)
-    const uint32_t x = tid & 15, y = tid >> 4;
-    int32_t v[16];
-#pragma unroll
-    for (int i = 0; i < 16; i++)
-      v[i] = direct ? (int32_t)codes[(i * 16 + y) * 16 + x] - r : s_q[(i * 16 + y) * 16 + x];
-#pragma unroll
-    for (int i = 1; i < 16; i++)
-      if (i & 7) v[i] += v[i - 1];
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-        const int32_t u = __shfl_up_sync(~0u, v[i], o);
-        if ((x & 7) >= (uint32_t)o) v[i] += u;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 16; i++) s_q[(i * 16 + y) * 16 + x] = v[i];
-    __syncthreads();
-    const uint32_t z = tid >> 4;
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = s_q[(z * 16 + i) * 16 + x];
-#pragma unroll
-    for (int i = 1; i < 16; i++)
-      if (i & 7) v[i] += v[i - 1];
-    const uint64_t base = ((uint64_t)(org[0] + z) * ny + org[1]) * nx + org[2] + x;
-#pragma unroll
-    for (int i = 0; i < 16; i++) out.put(base + (uint64_t)i * nx, v[i]);
-  } else {
-    // edge block: z sums in registers, x sums by shuffles, y sums through shared
-    // memory
-    const uint32_t x = tid & 15, y = tid >> 4;
-    const bool in_xy = x < w[2] && y < w[1];
-    int32_t v[16];
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = (in_xy && (uint32_t)i < w[0]) ? s_q[(i * w[1] + y) * w[2] + x] : 0;
-#pragma unroll
-    for (int i = 1; i < 16; i++)
-      if (i & 7) v[i] += v[i - 1];
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-        const int32_t u = __shfl_up_sync(~0u, v[i], o);
-        if ((x & 7) >= (uint32_t)o) v[i] += u;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 16; i++)
-      if (in_xy && (uint32_t)i < w[0]) s_q[(i * w[1] + y) * w[2] + x] = v[i];
-    __syncthreads();
-    {
-      const uint32_t xx = tid & 15, zz = tid >> 4;
-      if (xx < w[2] && zz < w[0]) {
-        int32_t acc = 0;
-        for (uint32_t yy = 0; yy < w[1]; yy++) {
-          const uint32_t j = (zz * w[1] + yy) * w[2] + xx;
-          acc = (yy & 7) ? acc + s_q[j] : s_q[j];
-          s_q[j] = acc;
-        }
-      }
-    }
-    __syncthreads();
-    for (uint32_t j = tid; j < m; j += kRecThreads) {
-      const uint32_t p = w[1] * w[2];
-      const uint32_t zz = j / p, rem = j - zz * p, yy = rem / w[2], xx = rem - yy * w[2];
-      out.put(((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + org[2] + xx, s_q[j]);
-    }
-  }
-  __syncthreads();
-  // verbatim patches overwrite their elements (ordered after the block's stores)
-  for (uint32_t i = rs + tid; i < re; i += kRecThreads) {
-    const uint2 kv = rec[i];
-    if (kv.x & 1u) {
-      const uint32_t j = (kv.x >> 1) % kSlots;
-      const uint32_t p = w[1] * w[2];
-      const uint32_t zz = j / p, rem = j - zz * p, yy = rem / w[2], xx = rem - yy * w[2];
-      out.patch(((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + org[2] + xx, kv.y);
-    }
-  }
+  if (!expand_runs(a, b, codec, w[0] * w[1] * w[2], S, c)) return;
+  uint4* o = reinterpret_cast<uint4*>(a.codes + (uint64_t)b * kSlots + 16 * threadIdx.x);
+  o[0] = make_uint4(c[0], c[1], c[2], c[3]);
+  o[1] = make_uint4(c[4], c[5], c[6], c[7]);
 }
 
-// Persistent: CTA c takes work items c, c + grid, ...; while it reconstructs one
-// block, a bulk copy is already bringing the next block's 8 KB of codes into shared
-// memory.  The work items are all blocks, or, when the entropy decoder reconstructs
-// full Huffman blocks itself (a.fuse), the listed other blocks.
-template <int ND, typename E>
-__global__ __launch_bounds__(kRecThreads) void reconstruct_kernel(DecodeArgs a) {
-  __shared__ __align__(128) uint16_t s_codes[2][kSlots];
-  __shared__ __align__(16) int32_t s_q[kSlots];
-  __shared__ unsigned long long s_bar[2];
-  __shared__ uint32_t s_fail;
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
-  const int tid = threadIdx.x;
-  const uint32_t grid = gridDim.x;
-  const uint32_t nwork = a.fuse ? a.st->n_slow : a.g.nblk;
-  auto block_of = [&](uint32_t i) -> uint32_t { return a.fuse ? a.slowblk[i] : i; };
-  auto issue = [&](uint32_t b, int buf) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&s_bar[buf], kSlots * 2);
-    bulk_load(s_codes[buf], a.codes + (uint64_t)b * kSlots, kSlots * 2, &s_bar[buf]);
-  };
-  if (tid == 0) {
-    mbar_init(&s_bar[0]);
-    mbar_init(&s_bar[1]);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_fail = 0;
-    if (blockIdx.x < nwork) issue(block_of(blockIdx.x), 0);
-  }
-  __syncthreads();
-  uint32_t it = 0, i = blockIdx.x;
-  bool next_issued = false;
-  for (; i < nwork; i += grid, it++) {
-    const int cur = it & 1;
-    const uint32_t b = block_of(i);
-    next_issued = i + grid < nwork;
-    if (tid == 0 && next_issued) issue(block_of(i + grid), cur ^ 1);
-    if (!mbar_wait(&s_bar[cur], (it >> 1) & 1u, kSpinLimit)) {
-      atomicOr(&a.st->status, ERR_TIMEOUT);
-      s_fail = 1;
-    }
-    __syncthreads();
-    if (s_fail) break;
-    reconstruct_body<ND, E>(a, b, s_q, s_codes[cur]);
-    __syncthreads();
-  }
-  if (s_fail && tid == 0) {
-    // wait once more (bounded) for this block's copy and the next one in flight
-    mbar_wait(&s_bar[it & 1], (it >> 1) & 1u, kSpinLimit);
-    if (next_issued) mbar_wait(&s_bar[(it + 1) & 1], ((it + 1) >> 1) & 1u, kSpinLimit);
-  }
+// The row piece of thread t of a block: 3-D row (z, y) = (t / 16, t % 16), up to 16
+// elements; 2-D piece t % 4 (16 elements) of row t / 4; 1-D elements 16t on.
+struct RowPiece {
+  uint32_t j0, n;  // first slot and number of slots
+  uint32_t z, y;   // in the block
+  bool valid;
+};
+template <int ND>
+__device__ __forceinline__ RowPiece row_piece(const uint32_t* w) {
+  const uint32_t t = threadIdx.x;
+  RowPiece p;
+  const uint32_t x0 = ND == 3 ? 0u : (ND == 2 ? 16u * (t & 3u) : 16u * t);
+  p.z = ND == 3 ? t >> 4 : 0u;
+  p.y = ND == 3 ? t & 15u : (ND == 2 ? t >> 2 : 0u);
+  p.valid = p.z < w[0] && p.y < w[1] && x0 < w[2];
+  p.n = p.valid ? min(16u, w[2] - x0) : 0u;
+  p.j0 = p.valid ? (p.z * w[1] + p.y) * w[2] + x0 : 0u;
+  return p;
 }
 
-// =================================================================================
-// global (unchunked) Lorenzo reconstruction: the N-D partial sum of q' over the whole
-// field (Sec. IV-B "Partial-Sum Lorenzo Reconstruction" holds without chunks).
-//
-// Bound by memory: the codes are read and the field written, and every full-size pass in
-// between costs as much again.  A pass per axis (q' written out, then a scan along x, y
-// and z, each reading and writing the field) took 296 us at 3-D 100x500x500, 143 of them
-// in the x scan's serial 4-byte loads.  Now only sums cross blocks: each block's row sums
-// (1/16 of the field) are scanned along x, each block forms the partial sums along x and
-// y of its own rows, with the row's sum before it, in shared memory and writes them once,
-// the strips' last rows (1/16 of the field) are scanned along y, and the last pass adds
-// those on its way along z: 95 us.  1-D fields take one pass with a look-back.
-// =================================================================================
-
-// q' (q - r, or the outlier's delta) of the n <= 16 consecutive slots j0 .. j0 + n - 1 of
-// block b; zeros behind them.
-__device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, uint32_t j0, uint32_t n,
+// q = code - r of n <= 16 slots (zeros behind them)
+__device__ __forceinline__ void load_codes16(const uint16_t* codes, uint32_t j0, uint32_t n, int32_t r,
                                              int32_t (&q)[16]) {
-  const uint16_t* codes = a.codes + (uint64_t)b * kSlots + j0;
-  const int32_t r = (int32_t)a.radius;
+  codes += j0;
   if (n == 16 && (j0 & 7) == 0) {
     const uint4 v[2] = {reinterpret_cast<const uint4*>(codes)[0], reinterpret_cast<const uint4*>(codes)[1]};
     const uint32_t u[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
@@ -1338,10 +1110,15 @@ __device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, ui
 #pragma unroll
     for (uint32_t i = 0; i < 16; i++) q[i] = i < n ? (int32_t)codes[i] - r : 0;
   }
+}
+
+// The outliers' deltas among block b's slots j0 .. j0 + n - 1: the records (sorted by key)
+// from the first one there, found by a search.
+__device__ __forceinline__ void overlay_outliers(const DecodeArgs& a, uint32_t b, uint32_t j0, uint32_t n,
+                                                 int32_t (&q)[16]) {
   uint32_t lo = a.rec_start[b];
   const uint32_t re = a.rec_start[b + 1];
   if (lo == re || n == 0) return;
-  // the row's records (sorted by key): the first one by a search, then in order
   const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
   const uint32_t k0 = (b * (uint32_t)kSlots + j0) * 2u, k1 = k0 + 2u * n;
   uint32_t hi = re;
@@ -1360,24 +1137,169 @@ __device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, ui
   }
 }
 
-// The row piece of thread t of a block: 3-D row (z, y) = (t / 16, t % 16), up to 16
-// elements; 2-D piece t % 4 (16 elements) of row t / 4.  row: its row index in the field.
-struct RowPiece {
-  uint32_t j0, n;  // first slot and number of slots
-  uint32_t z, y;   // in the block
-  bool valid;
-};
-template <int ND>
-__device__ __forceinline__ RowPiece row_piece(const uint32_t* w) {
-  const uint32_t t = threadIdx.x;
-  RowPiece p;
-  const uint32_t x0 = ND == 3 ? 0u : 16u * (t & 3u);
-  p.z = ND == 3 ? t >> 4 : 0u;
-  p.y = ND == 3 ? t & 15u : t >> 2;
-  p.valid = p.z < w[0] && p.y < w[1] && x0 < w[2];
-  p.n = p.valid ? min(16u, w[2] - x0) : 0u;
-  p.j0 = p.valid ? (p.z * w[1] + p.y) * w[2] + x0 : 0u;
-  return p;
+// The 16 k of thread t's row piece to the block's rows in shared memory: 16-byte chunk c of
+// piece R sits at c ^ ((R >> 1) & 3), so that eight threads writing their pieces touch all
+// banks; element e of the block (16 R + its place in the piece) is at swz_k(e).
+__device__ __forceinline__ uint32_t swz_k(uint32_t e) { return e ^ ((e >> 3) & 12u); }
+__device__ __forceinline__ void st_piece(int32_t* s_k, const int32_t (&k)[16], int32_t add) {
+  const uint32_t tid = threadIdx.x, key = (tid >> 1) & 3;
+#pragma unroll
+  for (uint32_t c = 0; c < 4; c++)
+    reinterpret_cast<int4*>(s_k + 16 * tid)[c ^ key] =
+        make_int4(k[4 * c] + add, k[4 * c + 1] + add, k[4 * c + 2] + add, k[4 * c + 3] + add);
+}
+
+// Block b from its codes (or runs) to the output: outliers, partial sums within the Lorenzo
+// chunks (Sec. IV-B2), scaled; then the verbatim patches.  (The caller has checked the
+// field's status, the same way in every thread.)
+template <int ND, typename E>
+__device__ void reconstruct_body(const DecodeArgs& a, uint32_t b, RebuildSmem& S) {
+  const uint32_t tid = threadIdx.x;
+  uint32_t org[3], w[3];
+  block_box(a.g, b, org, w);
+  const uint32_t m = w[0] * w[1] * w[2];
+  const int32_t r = (int32_t)a.radius;
+  const Out<E> out(a);
+  const RowPiece p = row_piece<ND>(w);
+  const int codec = a.ar[a.off_codec + b];
+  int32_t q[16];
+  if (codec == CODEC_RLE || codec == CODEC_RLE_HUFF) {
+    uint32_t c[8];
+    if (!expand_runs(a, b, codec, m, S, c)) return;
+    if (ND == 1 || m == (uint32_t)kSlots) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        q[2 * i] = (int32_t)(c[i] & 0xffffu) - r;
+        q[2 * i + 1] = (int32_t)(c[i] >> 16) - r;
+      }
+    } else {  // slots to row pieces
+      uint16_t* s_c = reinterpret_cast<uint16_t*>(S.k);
+      reinterpret_cast<uint4*>(s_c)[2 * tid] = make_uint4(c[0], c[1], c[2], c[3]);
+      reinterpret_cast<uint4*>(s_c)[2 * tid + 1] = make_uint4(c[4], c[5], c[6], c[7]);
+      __syncthreads();
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++) q[i] = i < p.n ? (int32_t)s_c[p.j0 + i] - r : 0;
+      __syncthreads();
+    }
+  } else {
+    load_codes16(a.codes + (uint64_t)b * kSlots, p.j0, p.n, r, q);
+  }
+  overlay_outliers(a, b, p.j0, p.n, q);
+  // sums along x: chunks of 256 (16 threads), 16 or 8
+#pragma unroll
+  for (int i = 1; i < 16; i++)
+    if (ND != 3 || (i & 7)) q[i] += q[i - 1];
+  int32_t before = 0;
+  if (ND == 1) {
+    int32_t t = q[15];
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const int32_t u = __shfl_up_sync(~0u, t, o, 16);
+      if ((tid & 15) >= (uint32_t)o) t += u;
+    }
+    before = t - q[15];
+  }
+  st_piece(S.k, q, before);
+  __syncthreads();
+  const uint64_t ny = a.g.n[1], nx = a.g.n[2];
+  if (ND == 1) {
+    if (m == (uint32_t)kSlots && out.vec4(org[2])) {
+#pragma unroll
+      for (uint32_t i = 0; i < 4; i++) {
+        const uint32_t e = 4 * (tid + kRecThreads * i);
+        out.put4((uint64_t)org[2] + e, *reinterpret_cast<const int4*>(S.k + swz_k(e)));
+      }
+    } else {
+#pragma unroll 4
+      for (uint32_t i = 0; i < 16; i++) {
+        const uint32_t e = tid + kRecThreads * i;
+        if (e < m) out.put((uint64_t)org[2] + e, S.k[swz_k(e)]);
+      }
+    }
+  } else if (ND == 2) {
+    // column x of the 16-row chunk band
+    const uint32_t x = tid & 63, y0 = 16 * (tid >> 6);
+    if (x < w[2]) {
+      const uint64_t base = (uint64_t)(org[1] + y0) * nx + org[2] + x;
+      int32_t acc = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++) {
+        acc += S.k[swz_k((y0 + i) * 64 + x)];
+        if (y0 + i < w[1]) out.put(base + i * nx, acc);
+      }
+    }
+  } else {
+    // columns along z in place, then along y
+    const uint32_t x = tid & 15, h = tid >> 4;
+    {
+      int32_t acc = 0;
+#pragma unroll
+      for (uint32_t z = 0; z < 16; z++) {
+        int32_t& k = S.k[swz_k((z * 16 + h) * 16 + x)];
+        acc = (z & 7) ? acc + k : k;
+        k = acc;
+      }
+    }
+    __syncthreads();
+    if (x < w[2] && h < w[0]) {
+      const uint64_t base = ((uint64_t)(org[0] + h) * ny + org[1]) * nx + org[2] + x;
+      int32_t acc = 0;
+#pragma unroll
+      for (uint32_t y = 0; y < 16; y++) {
+        const int32_t k = S.k[swz_k((h * 16 + y) * 16 + x)];
+        acc = (y & 7) ? acc + k : k;
+        if (y < w[1]) out.put(base + y * nx, acc);
+      }
+    }
+  }
+  // verbatim patches overwrite their elements (ordered after the block's stores)
+  const uint32_t rs = a.rec_start[b], re = a.rec_start[b + 1];
+  if (rs == re) return;
+  __syncthreads();
+  const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
+  for (uint32_t i = rs + tid; i < re; i += kRecThreads) {
+    const uint2 kv = rec[i];
+    if (kv.x & 1u) {
+      const uint32_t j = (kv.x >> 1) % kSlots;
+      const uint32_t pl = w[1] * w[2];
+      const uint32_t zz = j / pl, rem = j - zz * pl, yy = rem / w[2], xx = rem - yy * w[2];
+      out.patch(((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + org[2] + xx, kv.y);
+    }
+  }
+}
+
+// One CTA per listed block (the set-up's list: run blocks and cut blocks).
+template <int ND, typename E>
+__global__ __launch_bounds__(kRecThreads, 6) void reconstruct_kernel(DecodeArgs a) {
+  __shared__ __align__(16) RebuildSmem S;
+  if (a.dead) return;
+  // the status is read once, by thread 0 (run expansions in other CTAs may flag
+  // corruption meanwhile), so every thread takes the same path
+  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT) && blockIdx.x < a.st->n_slow;
+  __syncthreads();
+  if (!S.go) return;
+  reconstruct_body<ND, E>(a, a.slowblk[blockIdx.x], S);
+}
+
+// =================================================================================
+// global (unchunked) Lorenzo reconstruction: the N-D partial sum of q' over the whole
+// field (Sec. IV-B "Partial-Sum Lorenzo Reconstruction" holds without chunks).
+//
+// Bound by memory: the codes are read and the field written, and every full-size pass in
+// between costs as much again.  A pass per axis (q' written out, then a scan along x, y
+// and z, each reading and writing the field) took 296 us at 3-D 100x500x500, 143 of them
+// in the x scan's serial 4-byte loads.  Now only sums cross blocks: each block's row sums
+// (1/16 of the field) are scanned along x, each block forms the partial sums along x and
+// y of its own rows, with the row's sum before it, in shared memory and writes them once,
+// the strips' last rows (1/16 of the field) are scanned along y, and the last pass adds
+// those on its way along z: 95 us.  1-D fields take one pass with a look-back.
+// =================================================================================
+
+// q' (q - r, or the outlier's delta) of a row piece of block b.
+__device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, uint32_t j0, uint32_t n,
+                                             int32_t (&q)[16]) {
+  load_codes16(a.codes + (uint64_t)b * kSlots, j0, n, (int32_t)a.radius, q);
+  overlay_outliers(a, b, j0, n, q);
 }
 
 // Sums of the block's rows: totals[bx][row], row over the field's rows.
@@ -1423,9 +1345,6 @@ __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
 }
 
 // Partial sums along x, over the whole row, and along y, within the block, of one block.
-// Rows cross from threads to columns in shared memory; 16-byte chunk c of the 16-element
-// piece R sits at c ^ ((R >> 1) & 3), so that eight threads writing their pieces touch
-// all banks.
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
   __shared__ __align__(16) int32_t s_k[kSlots];
@@ -1448,13 +1367,9 @@ __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
     const uint32_t at = tid & 3;
     carry += (at >= 1 ? u1 : 0) + (at >= 2 ? u2 : 0) + (at >= 3 ? u3 : 0);
   }
-  const uint32_t key = (tid >> 1) & 3;
-#pragma unroll
-  for (uint32_t c = 0; c < 4; c++)
-    reinterpret_cast<int4*>(s_k + 16 * tid)[c ^ key] =
-        make_int4(k[4 * c] + carry, k[4 * c + 1] + carry, k[4 * c + 2] + carry, k[4 * c + 3] + carry);
+  st_piece(s_k, k, carry);
   __syncthreads();
-  auto at = [&](uint32_t e) -> int32_t { return s_k[e ^ ((e >> 3) & 12u)]; };
+  auto at = [&](uint32_t e) -> int32_t { return s_k[swz_k(e)]; };
   int32_t* q = reinterpret_cast<int32_t*>(a.out);
   if (ND == 3) {
     const uint32_t x = tid & 15, z = tid >> 4;
@@ -1774,17 +1689,10 @@ __global__ __launch_bounds__(1024) void stream_decode_batch_kernel(const DecodeA
   stream_decode_body<ND, float>(a, b0, b1);
 }
 
-// Reconstruction of a batch, one CTA per codec block of every field.  A run block's
-// runs are expanded here, into shared memory, instead of by a separate launch: the
-// expansion's scratch then serves as the reconstruction's (s_q overlays the run
-// values and lengths, read no more once the codes are out).
-__global__ __launch_bounds__(kRecThreads) void reconstruct_batch_kernel(const DecodeArgs* __restrict__ tasks,
+// Reconstruction of a batch, one CTA per codec block of every field.
+__global__ __launch_bounds__(kRecThreads, 6) void reconstruct_batch_kernel(const DecodeArgs* __restrict__ tasks,
                                                                         const uint32_t* __restrict__ tile0, int nfields) {
-  static_assert(kRecThreads == kRleThreads, "run expansion assumes its CTA size");
-  __shared__ __align__(16) uint32_t s_scr[kSlots + (kSlots + 1) + 3];  // run values and lengths, then starts
-  __shared__ __align__(16) uint16_t s_codes[kSlots];
-  __shared__ int s_go;
-  int32_t* s_q = reinterpret_cast<int32_t*>(s_scr);
+  __shared__ __align__(16) RebuildSmem S;
   const int f = field_of(tile0, nfields, blockIdx.x);
   const DecodeArgs& a = tasks[f];
   const uint32_t b = blockIdx.x - tile0[f];
@@ -1793,20 +1701,12 @@ __global__ __launch_bounds__(kRecThreads) void reconstruct_batch_kernel(const De
   if (a.fuse && a.ar[a.off_codec + b] == CODEC_HUFF && block_is_full(a.g, b)) return;
   // the status is read once, by thread 0 (run expansions in other CTAs may flag
   // corruption meanwhile), so every thread takes the same path
-  if (threadIdx.x == 0) s_go = !(a.st->status & ERR_CORRUPT);
+  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT);
   __syncthreads();
-  if (!s_go) return;
-  const int codec = a.ar[a.off_codec + b];
-  const uint16_t* codes = a.codes + (uint64_t)b * kSlots;
-  if (codec == CODEC_RLE || codec == CODEC_RLE_HUFF) {
-    uint16_t* sv = reinterpret_cast<uint16_t*>(s_scr);
-    if (!rle_expand_into(a, b, s_codes, sv, sv + kSlots, s_scr + kSlots)) return;
-    __syncthreads();
-    codes = s_codes;
-  }
-  if (a.g.ndim == 1) reconstruct_body<1, float>(a, b, s_q, codes);
-  else if (a.g.ndim == 2) reconstruct_body<2, float>(a, b, s_q, codes);
-  else reconstruct_body<3, float>(a, b, s_q, codes);
+  if (!S.go) return;
+  if (a.g.ndim == 1) reconstruct_body<1, float>(a, b, S);
+  else if (a.g.ndim == 2) reconstruct_body<2, float>(a, b, S);
+  else reconstruct_body<3, float>(a, b, S);
 }
 
 cudaError_t launch_decode_batch(const DecodeBatchLaunch& L, cudaStream_t s) {
@@ -1905,39 +1805,25 @@ cudaError_t launch_decode_stages(const DecodeArgs& a, cudaStream_t s) {
     k<<<grid, 32 * warps, smem, s>>>(a);
     trace_end(K_STREAM_DECODE, s);
   }
-  if (a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF]) {  // run blocks present
-    trace_begin(K_RLE_EXPAND, s);
-    rle_expand_kernel<<<a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF], kRleThreads, 0, s>>>(a);
-    trace_end(K_RLE_EXPAND, s);
+  const uint32_t nrun = a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF];
+  if (a.global) {
+    if (nrun) {
+      trace_begin(K_RLE_EXPAND, s);
+      rle_expand_kernel<<<nrun, kRecThreads, 0, s>>>(a);
+      trace_end(K_RLE_EXPAND, s);
+    }
+    return launch_global_reconstruct(a, s);
   }
-  if (a.global) return launch_global_reconstruct(a, s);
-  // blocks left to the reconstruction kernel: with fusion at most the edge blocks and
-  // the run blocks (the header's counts, which the set-up checks); none, and the launch
-  // is skipped
-  uint64_t work = a.g.nblk;
-  if (a.fuse) {
-    uint64_t full = 1;
-    for (int d = 0; d < 3; d++) full *= a.g.n[d] / a.g.blk[d];
-    work = (a.g.nblk - full) + a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF];
-    if (work > a.g.nblk) work = a.g.nblk;
-  }
+  // blocks left to the reconstruction kernel: at most the cut blocks and the run blocks
+  // (the header's counts, which the set-up checks); none, and the launch is skipped
+  uint64_t full = 1;
+  for (int d = 0; d < 3; d++) full *= a.g.n[d] / a.g.blk[d];
+  uint64_t work = (a.g.nblk - full) + nrun;
+  if (work > a.g.nblk) work = a.g.nblk;
   if (work) {
-    static int sms = 0, occ[4] = {0, 0, 0, 0};
     auto k = nd == 1 ? reconstruct_kernel<1, E> : (nd == 2 ? reconstruct_kernel<2, E> : reconstruct_kernel<3, E>);
-    if (sms == 0) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    if (occ[nd] == 0) {
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[nd], k, kRecThreads, 0);
-      if (occ[nd] <= 0) occ[nd] = 1;
-    }
-    // persistent only when every CTA gets several blocks to prefetch
-    const uint64_t cap = (uint64_t)sms * occ[nd];
-    const unsigned grid = (unsigned)(work <= 3 * cap ? work : cap);
     trace_begin(K_RECONSTRUCT, s);
-    k<<<grid, kRecThreads, 0, s>>>(a);
+    k<<<(unsigned)work, kRecThreads, 0, s>>>(a);
     trace_end(K_RECONSTRUCT, s);
   }
   return cudaGetLastError();
