@@ -332,8 +332,7 @@ csz_status run_pipeline(const void* d_field, int ndim, const uint64_t* dims, int
   ea.off_codec = kHdr;
   ea.off_bb = off_bb;
   ea.off_rec = off_rec;
-  ea.lb = at<uint64_t>(d_ws, L.lb_e);
-  ea.spin_limit = g_spin_limit;
+  ea.groups = at<uint64_t>(d_ws, L.lb_e);
   ea.place_records = an ? 0 : 1;
   ea.rec = ra;
   FinalizeArgs& fa = ea.fin;

@@ -24,7 +24,7 @@ struct csz_batch {
   // device tables and regions (inside the caller's workspace)
   unsigned char* zero_base = nullptr;
   uint64_t zero_bytes = 0;
-  uint32_t* tickets = nullptr;  // [0] construction, [1] encoding
+  uint32_t* tickets = nullptr;  // see PersistArgs
   DevState* states = nullptr;   // nfields, kStateStride apart
   ConstructTask* ctasks = nullptr;
   uint32_t* tile0 = nullptr;  // nfields + 1
@@ -72,7 +72,7 @@ FieldLayout field_layout(const Geom& g) {
   L.lens = o;
   o += a256(2 * kNsymCode + kNsymLen);
   L.bcodes = o;
-  o += a256(8ull * (2 * kNsymCode + kNsymLen));
+  o += a256(kBookCodeBytes);
   L.codes = o;
   o += a256(2ull * kSlots * g.nblk);
   L.counts = o;
@@ -89,12 +89,12 @@ FieldLayout field_layout(const Geom& g) {
   return L;
 }
 
-// Whole-batch layout: zeroed part (tickets, states, histograms, look-back states),
+// Whole-batch layout: zeroed part (tickets, states, histograms, group totals),
 // tables, then the fields' own regions.
 struct BatchLayout {
-  uint64_t tickets, states, hists, lb, zero_end;
+  uint64_t tickets, states, hists, zero_end;
   uint64_t ctasks, tile0, rtasks, cta0, btasks, etasks, len_books, fields_begin;
-  std::vector<uint64_t> lb_at, field_at;
+  std::vector<uint64_t> group_at, field_at;
   uint64_t total;
 };
 
@@ -108,11 +108,10 @@ BatchLayout batch_layout(const std::vector<Geom>& gs) {
   o += kStateStride * F;
   B.hists = o;
   o += a256(kHistBytes) * F;
-  B.lb = o;
-  B.lb_at.resize(F);
+  B.group_at.resize(F);
   for (uint64_t f = 0; f < F; f++) {
-    B.lb_at[f] = o;
-    o += a256(8ull * gs[f].nblk);
+    B.group_at[f] = o;
+    o += a256(8ull * ((gs[f].nblk + 255) / 256));
   }
   B.zero_end = o;
   B.ctasks = o;
@@ -168,7 +167,7 @@ cudaError_t enqueue(const csz_batch* b, int construct_grid, cudaStream_t s) {
                                   construct_grid, b->common_nd, s)) != cudaSuccess)
     return e;
   if ((e = launch_codebook_batch(b->btasks, b->nfields, s)) != cudaSuccess) return e;
-  return launch_encode_batch(b->etasks, b->tile0, b->nfields, b->ntiles, &b->tickets[1], s);
+  return launch_encode_batch(b->etasks, b->tile0, b->nfields, b->ntiles, s);
 }
 
 // The same batch as one launch of the persistent kernel.
@@ -317,8 +316,7 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
     ea.off_codec = kHdr;
     ea.off_bb = off_bb;
     ea.off_rec = off_rec;
-    ea.lb = at<uint64_t>(ws, B.lb_at[f]);
-    ea.spin_limit = kSpinLimit;
+    ea.groups = at<uint64_t>(ws, B.group_at[f]);
     ea.place_records = 1;
     ea.rec = ra;
     FinalizeArgs& fa = ea.fin;

@@ -102,6 +102,13 @@ __host__ __device__ inline void block_box(const Geom& g, uint32_t b, uint32_t or
   }
 }
 
+// number of in-field elements of codec block b
+__host__ __device__ inline uint32_t block_elems(const Geom& g, uint32_t b) {
+  uint32_t org[3], w[3];
+  block_box(g, b, org, w);
+  return w[0] * w[1] * w[2];
+}
+
 // codec block b has the full block extent on every axis (not cut by the field's edge)
 __host__ __device__ inline bool block_is_full(const Geom& g, uint32_t b) {
   uint32_t org[3], w[3];
@@ -137,6 +144,10 @@ struct DevState {
   uint32_t tiles_flushed;  // tiles whose histograms, counts and codes are in place
   uint32_t books_done;     // book-phase items finished (three books and the record offsets)
 };
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
 
 // ---------------------------------------------------------------------------------
 // memory-model helpers for the decoupled look-back
@@ -406,12 +417,19 @@ __device__ __forceinline__ uint32_t log2_q16_small(uint32_t v) { return __ldg(&k
 // ---------------------------------------------------------------------------------
 // canonical Huffman codes from lengths (block-wide, whole warps).  Codes are ordered by
 // (length, symbol); the first code of length l is (first(l-1) + count(l-1)) << 1.
-// Outputs per symbol its code and its rank in (length, symbol) order; per length
+// Outputs per symbol its code (code_out with packed_out, or neither) and its rank in (length, symbol) order; per length
 // the first code, the count and the offset of its first symbol in that order.
 // smem: cnt[kMaxLen+1] u32, first[kMaxLen+1] u64, off[kMaxLen+1] u32,
 //       wcnt[(nsym/32)*(kMaxLen+1)] u16
 // Contains __syncthreads; all threads call.
 // ---------------------------------------------------------------------------------
+// A code of up to kPackedMax bits with its length in one word, as the encoder reads it:
+// the code left-aligned, the length in the low five bits (kPackedLong: a longer code; 0: no
+// code).
+constexpr uint32_t kPackedMax = 27, kPackedLong = 31;
+__device__ __forceinline__ uint32_t packed_code(uint64_t code, int len) {
+  return len > (int)kPackedMax ? kPackedLong : ((uint32_t)code << (32 - len)) | (uint32_t)len;
+}
 struct CanonSmem {
   uint32_t cnt[kMaxLen + 1];
   uint32_t off[kMaxLen + 1];
@@ -420,7 +438,7 @@ struct CanonSmem {
 };
 
 __device__ inline void canonical_build(const uint8_t* len, int nsym, CanonSmem* cs, uint16_t* wcnt,
-                                       uint64_t* code_out, uint16_t* sorted_out) {
+                                       uint64_t* code_out, uint32_t* packed_out, uint16_t* sorted_out) {
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int l = tid; l <= kMaxLen; l += nt) cs->cnt[l] = 0;
   if (tid == 0) cs->bad = 0;
@@ -484,10 +502,15 @@ __device__ inline void canonical_build(const uint8_t* len, int nsym, CanonSmem* 
     const uint32_t peers = __match_any_sync(~0u, l);
     if (l && l <= kMaxLen) {
       uint32_t rank = wcnt[(s >> 5) * (kMaxLen + 1) + l] + __popc(peers & ((1u << (tid & 31)) - 1u));
-      if (code_out) code_out[s] = cs->first[l] + rank;
+      if (code_out) {
+        const uint64_t code = cs->first[l] + rank;
+        code_out[s] = code;
+        packed_out[s] = packed_code(code, l);
+      }
       if (sorted_out) sorted_out[cs->off[l] + rank] = (uint16_t)s;
     } else if (code_out) {
       code_out[s] = 0;
+      packed_out[s] = 0;
     }
   }
   __syncthreads();
@@ -586,45 +609,6 @@ __device__ __forceinline__ uint32_t next_head(const uint32_t* head, const uint32
 // consume their code.
 // ---------------------------------------------------------------------------------
 
-// One warp encodes sym[0..N) (+add) with a book into out[]; returns the unit count.
-__device__ inline uint32_t ihs_encode_warp(const uint16_t* sym, uint32_t N, int add,
-                                           const uint8_t* __restrict__ lens,
-                                           const uint64_t* __restrict__ codes, uint16_t* out) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t mine = N > lane ? (N - lane + 31) / 32 : 0;
-  uint64_t acc = 0;   // produced, not yet emitted bits (MSB-aligned)
-  int nacc = 0;
-  uint32_t enext = 0;  // next own symbol to produce
-  int nb = 0;          // bits the simulated decoder lane holds
-  uint32_t base = 0;
-  const uint32_t T = (N + 31) / 32;
-  for (uint32_t t = 0; t < T; t++) {
-    const bool active = t < mine;
-    const int len = active ? (int)__ldg(&lens[sym[32 * t + lane] + add]) : 0;
-    while (true) {
-      const bool need = active && len > nb;
-      const uint32_t ballot = __ballot_sync(~0u, need);
-      if (!ballot) break;
-      if (need) {
-        while (nacc < 16 && enext < mine) {
-          const int s = sym[32 * enext + lane] + add;
-          const int l = __ldg(&lens[s]);
-          acc |= (__ldg(&codes[s]) << (64 - l)) >> nacc;
-          nacc += l;
-          enext++;
-        }
-        out[base + __popc(ballot & ((1u << lane) - 1u))] = (uint16_t)(acc >> 48);
-        acc <<= 16;
-        nacc = nacc > 16 ? nacc - 16 : 0;
-        nb += 16;
-      }
-      base += __popc(ballot);
-    }
-    nb -= len;
-  }
-  return base;
-}
-
 // Block-wide encoder of the same stream (blockDim.x == 256): thread (lane l, warp w)
 // owns lane l's steps 16w..16w+15.  A lane holding cum(t) bits of codes after step t
 // has taken U(t) = ceil(cum(t)/16) units, so at step t it takes U(t) - U(t-1) units,
@@ -715,203 +699,123 @@ __host__ __device__ __forceinline__ uint32_t huff_split(uint32_t m) {
   return h < m ? h : m;
 }
 
-// Block-wide encoder of one Huffman block's two streams (256 threads).  Pass 1
-// (ihs_plan2): thread (lane l, warp w) reads the lengths of lane l's steps
-// 16(w&3)..16(w&3)+15 of stream w>>2 once into registers; per-lane totals give both
-// streams' sizes.  Pass 2 (ihs_emit2): each thread appends its codes to its lane's
-// bit string in shared memory (64 strings of 64 words, word index XOR-swizzled by
-// the lane so a warp's 32 lanes hit 32 banks), then every unit is cut straight out
-// of its lane's string and stored at its decoder-order position (rounds within
-// steps, lanes in order within a round).  Lanes above 2016 bits take the gather
-// encoder instead.
-struct IhsPlan {
-  uint32_t len4[4];    // the thread's 16 code lengths, 8 bits each
-  uint32_t pre;        // bits of the lane before the thread's first step
-  uint32_t cum;        // bits of the thread's 16 steps
-};
-
-constexpr uint32_t kLaneWords = 64;                       // words per lane string
-constexpr uint32_t kLaneBitsMax = 32 * (kLaneWords - 1);  // 2016 bits: a string and the word after it fit
-
-__device__ __forceinline__ uint32_t plan_len(const IhsPlan& P, int i) {
-  // selects rather than an indexed load, so the plan stays in registers
-  const uint32_t wsel = i < 8 ? (i < 4 ? P.len4[0] : P.len4[1]) : (i < 12 ? P.len4[2] : P.len4[3]);
-  return (wsel >> (8 * (i & 3))) & 0xffu;
-}
-
-struct IhsPlan2Out {
+// Block-wide encoder of a pair of interleaved streams (256 threads): a Huffman block's
+// streams A and B, or the value and the length stream of an RLE+Huffman block.  Warp w
+// takes quarter w & 3 of stream w >> 2, thread (lane l) lane l's symbols of the quarter's
+// up to 16 steps, whose packed codes it keeps in registers from the sizes to the payload.
+//
+// Bound by instruction issue and barriers (3-D 512^3, rel 1e-4: 109 instructions per 32
+// symbols and 533 us in the encoder this replaced, which looked lengths and codes up apart
+// in global memory, gathered each lane's bits in shared memory and cut the units out of
+// them again).  What makes it short is the order of the units: a lane takes its next unit
+// with the first code that does not fit the bits taken so far, so by then the unit before
+// is complete.  Each thread holds the one unit it has a place for but not all bits of;
+// a code that overflows it completes and stores it and takes the next place, one ballot a
+// step.  A thread's first bits complete a unit placed by an earlier quarter: they go to
+// shared memory and are added after the barrier.  Now 390 us with
+// the sizes in a pass of their own (plan_body).
+struct PairPlan {
+  uint32_t e[16];             // packed codes of the thread's steps (0 behind the last)
+  uint32_t pre;               // bits of the lane before them
+  uint32_t base;              // units of the stream before them
   uint32_t units_a, units_b;  // units of each stream
-  uint32_t max_lane_bits;     // over both streams
+  bool packed;                // every code packed and every step held: pair_emit applies
 };
 
-// Fills P; returns the units of both streams and the largest lane total.  scratch:
-// >= 256 + 4 u32.  Contains __syncthreads.
-__device__ inline IhsPlan2Out ihs_plan2(const uint16_t* sym, uint32_t m, const uint8_t* __restrict__ lens,
-                                       uint32_t* scratch, IhsPlan& P) {
-  const uint32_t tid = threadIdx.x, l = tid & 31, w = tid >> 5, sidx = w >> 2, wl = w & 3;
-  const uint32_t h = huff_split(m);
-  const uint32_t N = sidx ? m - h : h;
-  const uint16_t* ss = sym + (sidx ? h : 0);
-  const uint32_t t0 = 16 * wl;
-  uint32_t cum = 0;
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    uint32_t pk = 0;
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const uint32_t j = 32 * (t0 + 4 * q + k) + l;
-      const uint32_t L = j < N ? (uint32_t)__ldg(&lens[ss[j]]) : 0u;
-      pk |= L << (8 * k);
-      cum += L;
-    }
-    P.len4[q] = pk;
-  }
-  P.cum = cum;
+// The steps of a quarter of a stream of n symbols.
+__device__ __forceinline__ uint32_t quarter_steps(uint32_t n) { return (n + 127u) / 128u; }
+
+// Completes P from the thread's bit total (bit 31: not packed).  scratch: 256 words that no
+// thread reads or writes otherwise before the next barrier.  Contains one barrier.
+__device__ __forceinline__ void pair_plan(PairPlan& P, uint32_t cum, uint32_t* scratch) {
+  const uint32_t l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  scratch[threadIdx.x] = cum;
   __syncthreads();
-  scratch[32 * w + l] = cum;
-  __syncthreads();
-  uint32_t pre = 0, tot = 0;
+  uint32_t all = 0, pre = 0, tot[2] = {0u, 0u};
 #pragma unroll
-  for (uint32_t v = 0; v < 4; v++) {
-    const uint32_t c = scratch[32 * (4 * sidx + v) + l];
-    if (v < wl) pre += c;
-    tot += c;
+  for (uint32_t v = 0; v < 8; v++) {
+    const uint32_t c = scratch[32 * v + l];
+    all |= c;
+    tot[v >> 2] += c & 0x7fffffffu;
+    if (v >> 2 == w >> 2 && v < w) pre += c & 0x7fffffffu;
   }
   P.pre = pre;
-  if (wl == 0) {  // warps 0 and 4 total their stream
-    const uint32_t units = warp_sum((tot + 15) >> 4);
-    uint32_t mx = tot;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(~0u, mx, o));
-    if (l == 0) {
-      scratch[256 + sidx] = units;
-      scratch[258 + sidx] = mx;
-    }
-  }
-  __syncthreads();
-  IhsPlan2Out r;
-  r.units_a = scratch[256];
-  r.units_b = scratch[257];
-  r.max_lane_bits = max(scratch[258], scratch[259]);
-  __syncthreads();
-  return r;
+  P.base = __reduce_add_sync(~0u, (pre + 15) >> 4);
+  P.units_a = __reduce_add_sync(~0u, (tot[0] + 15) >> 4);
+  P.units_b = __reduce_add_sync(~0u, (tot[1] + 15) >> 4);
+  P.packed = !(__any_sync(~0u, all >> 31));
 }
 
-// Pass 2; requires every lane total <= kLaneBitsMax.  out16[0] receives units_a,
-// stream A starts at out16[1], stream B at out16[1 + units_a].  lanebuf: 64 *
-// kLaneWords u32, all zero if `clean` (cleared before a block barrier the caller
-// passed), else cleared here.  scratch: >= 8 u32.  Contains __syncthreads.
-__device__ inline void ihs_emit2(const uint16_t* sym, uint32_t m, const uint64_t* __restrict__ codes,
-                                 const IhsPlan& P, uint32_t units_a, uint32_t* lanebuf, uint16_t* out16,
-                                 uint32_t* scratch, bool clean) {
-  const uint32_t tid = threadIdx.x, l = tid & 31, w = tid >> 5, sidx = w >> 2, wl = w & 3;
-  const uint32_t h = huff_split(m);
-  const uint16_t* ss = sym + (sidx ? h : 0);
-  const uint32_t t0 = 16 * wl;
-  uint32_t* mine = lanebuf + kLaneWords * (32 * sidx + l);
-  // each thread clears the words its bits land in (and the one after them); together
-  // the threads of a lane clear every word that is read
-  if (!clean) {
-    const uint32_t w0 = P.pre >> 5, w1 = min((P.pre + P.cum + 31) >> 5, kLaneWords - 1);
-    for (uint32_t wi = w0; wi <= w1; wi++) mine[wi ^ l] = 0;
-    __syncthreads();
-  }
-  // codes gather in a 64-bit window (left-aligned, `fill` bits used, < 32 between
-  // codes); each completed word is stored.  Only the thread's first and last words
-  // can be shared with the neighbouring steps of the lane: those two are OR-ed in.
-  {
-    uint32_t wi = P.pre >> 5;
-    int fill = (int)(P.pre & 31);
-    uint64_t win = 0;
-    bool first = true;
-    auto flush = [&]() {
-      const uint32_t word = (uint32_t)(win >> 32);
-      if (first) atomicOr(&mine[wi ^ l], word);
-      else mine[wi ^ l] = word;
-      first = false;
-      win <<= 32;
-      fill -= 32;
-      wi++;
-    };
-#pragma unroll 4
-    for (int i = 0; i < 16; i++) {
-      const int L = (int)plan_len(P, i);
-      if (L == 0) continue;
-      const uint64_t C = __ldg(&codes[ss[32 * (t0 + i) + l]]);
-      if (L <= 32) {
-        win |= C << (64 - fill - L);
-        fill += L;
-        if (fill >= 32) flush();
-      } else {  // a code longer than 32 bits: its top L - 32 bits, then the low 32
-        const int hl = L - 32;
-        win |= (C >> 32) << (64 - fill - hl);
-        fill += hl;
-        if (fill >= 32) flush();
-        win |= (C & 0xffffffffull) << (32 - fill);
-        fill += 32;
-        flush();
-      }
-    }
-    if (fill > 0) atomicOr(&mine[wi ^ l], (uint32_t)(win >> 32));
-  }
-  // units each warp's steps take, for the warp's first output position in its stream
-  const uint32_t u_begin = (P.pre + 15) >> 4, u_end = (P.pre + P.cum + 15) >> 4;
-  const uint32_t wtot = warp_sum(u_end - u_begin);
-  if (l == 0) scratch[w] = wtot;
-  __syncthreads();
-  uint32_t base = 1 + (sidx ? units_a : 0);
-  for (uint32_t v = 0; v < wl; v++) base += scratch[4 * sidx + v];
-  if (tid == 0) out16[0] = (uint16_t)units_a;
+// Writes both streams to out (shared memory), stream A from unit a0 on, stream B behind
+// it.  heads: 256 words.  Contains one barrier; the units are complete after another.
+__device__ __forceinline__ void pair_emit(const PairPlan& P, uint16_t* out, uint32_t a0, uint32_t* heads) {
+  const uint32_t tid = threadIdx.x, l = tid & 31, w = tid >> 5;
   const uint32_t lt = (1u << l) - 1u;
-  // unit k of this lane's string: units are 16-bit aligned, so unit k is the upper
-  // (k even) or lower (k odd) half of word k / 2
-  auto unit_at = [&](uint32_t k) -> uint16_t { return (uint16_t)(mine[(k >> 1) ^ l] >> ((~k & 1u) << 4)); };
-  uint32_t c = P.pre, uprev = u_begin;
-  // four steps at a time; a lane takes two or more units in one step only for a code
-  // longer than 16 bits, so usually one ballot per step gives every position
+  // places are shared-memory addresses; the first is the thread's word of heads
+  const uint32_t head = smem_u32(heads + tid);
+  uint32_t next = smem_u32(out) + 2u * (a0 + (w >> 2 ? P.units_a : 0u) + P.base);
+  uint32_t fill = ((P.pre + 15u) & 15u) + 1u;  // bits of the lane's last unit so far, 1 to 16
+  uint32_t win = 0;                            // this thread's bits of it and behind it, placed after `fill` bits
+  uint32_t pos = head;                         // its place
+  uint32_t any_len = 0;
 #pragma unroll
-  for (int i0 = 0; i0 < 16; i0 += 4) {
-    uint32_t D[4], up[4];
-    bool multi = false;
+  for (int i = 0; i < 16; i++) any_len |= P.e[i];
+  const bool wide = __any_sync(~0u, (any_len & 16u) != 0);  // (a code of 17 bits or more may take two units)
+  auto store = [](uint32_t at, uint32_t unit) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)unit) : "memory");
+  };
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const uint32_t cn = c + plan_len(P, i0 + k);
-      const uint32_t u = (cn + 15) >> 4;
-      D[k] = u - uprev;
-      up[k] = uprev;
-      multi |= D[k] >= 2;
-      c = cn;
-      uprev = u;
-    }
-    if (!__any_sync(~0u, multi)) {
-      uint32_t b1[4];
-#pragma unroll
-      for (int k = 0; k < 4; k++) b1[k] = __ballot_sync(~0u, D[k] != 0);
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        if (D[k]) out16[base + __popc(b1[k] & lt)] = unit_at(up[k]);
-        base += __popc(b1[k]);
+  for (int i = 0; i < 16; i++) {
+    const uint32_t L = P.e[i] & 31u, c = P.e[i] & ~31u;
+    const uint32_t n = fill + L;
+    const bool need = n > 16;
+    const uint32_t b1 = __ballot_sync(~0u, need);
+    const uint32_t p1 = next + 2u * __popc(b1 & lt);
+    next += 2u * __popc(b1);
+    if (wide && __any_sync(~0u, n > 32)) {
+      const uint32_t b2 = __ballot_sync(~0u, n > 32);
+      const uint64_t both = ((uint64_t)win << 32) | (((uint64_t)c << 32) >> fill);
+      win = (uint32_t)(both >> 32);
+      fill = n;
+      if (need) {
+        store(pos, win >> 16);
+        pos = p1;
+        win <<= 16;
+        fill -= 16;
       }
+      if (n > 32) {
+        store(p1, win >> 16);
+        pos = next + 2u * __popc(b2 & lt);
+        win = (uint32_t)both;
+        fill -= 16;
+      }
+      next += 2u * __popc(b2);
     } else {
-      // rounds, as the decoder takes them
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-#pragma unroll 1
-        for (uint32_t r = 1; r <= 4; r++) {
-          const uint32_t br = __ballot_sync(~0u, D[k] >= r);
-          if (!br) break;
-          if (D[k] >= r) out16[base + __popc(br & lt)] = unit_at(up[k] + r - 1);
-          base += __popc(br);
-        }
+      win |= c >> fill;
+      fill = n;
+      if (need) {
+        store(pos, win >> 16);
+        pos = p1;
+        win <<= 16;
+        fill -= 16;
       }
     }
   }
+  // (the upper half of the word: whether the thread has taken a unit)
+  if (pos == head) store(head, win >> 16);
+  store(head + 2, pos != head);
   __syncthreads();
+  if (pos != head) {
+    // the later quarters' first bits, up to the first of them that took a unit of its own
+    uint32_t unit = win >> 16;
+    for (uint32_t v = tid + 32; (v & ~127u) == (tid & ~127u); v += 32) {
+      const uint32_t h = heads[v];
+      unit |= h & 0xffffu;
+      if (h >> 16) break;
+    }
+    store(pos, unit);
+  }
 }
-
-// Units lane `lane` of a stream needs: ceil(bits/16), given its bit total.
-__device__ __forceinline__ uint32_t ihs_lane_units(uint32_t bits) { return (bits + 15) / 16; }
-
 
 // One forward pass of the selector MLP by a full warp: lane i owns hidden unit i, and
 // every dot product is a chain of fused multiply-adds from the bias over the inputs
@@ -940,9 +844,6 @@ __device__ __forceinline__ void mlp_forward_warp(const float* __restrict__ w, co
 // ---------------------------------------------------------------------------------
 // mbarrier helpers for bulk asynchronous copies (TMA)
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 
 __device__ __forceinline__ void mbar_init(unsigned long long* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");

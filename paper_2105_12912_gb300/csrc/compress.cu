@@ -6,10 +6,10 @@
 //     device code construct_body.cuh) record counts, bit words, residuals, histograms
 //   codebook_kernel                   three canonical Huffman books; a fourth CTA
 //                                     scans the blocks' record counts
-//   encode_kernel                     per block: its records, exact sizes or heuristic /
-//                                     MLP pick, payload placement by decoupled
-//                                     look-back, payload
-//   (the block counted last)          header, padding, books
+//   plan_kernel                       per block: its records, exact sizes or heuristic /
+//                                     MLP pick
+//   payload_kernel                    per block: its place among the payloads, payload;
+//                                     block 0: header, padding, books
 // Batches run the same bodies either as one launch per stage (the *_batch kernels)
 // or as the phases of one persistent kernel (batch_persistent_kernel).
 #include "common.cuh"
@@ -436,6 +436,7 @@ __device__ void codebook_core(const BookArgs& a, int role, unsigned char* mem) {
   const uint32_t* hist = book == 0 ? a.hist_code : (book == 1 ? a.hist_val : a.hist_len);
   uint8_t* len_out = a.lens + (book == 0 ? 0 : (book == 1 ? kNsymCode : 2 * kNsymCode));
   uint64_t* code_out = a.codes + (book == 0 ? 0 : (book == 1 ? kNsymCode : 2 * kNsymCode));
+  uint32_t* packed_out = packed_books(a.codes) + (code_out - a.codes);
 
   uint8_t* s_len = mem;
   uint16_t* s_sym = reinterpret_cast<uint16_t*>(mem + nsym);
@@ -582,7 +583,7 @@ __device__ void codebook_core(const BookArgs& a, int role, unsigned char* mem) {
   }
   __syncthreads();
   for (int s = tid; s < nsym; s += blockDim.x) len_out[s] = s_len[s];
-  canonical_build(s_len, nsym, &cs, reinterpret_cast<uint16_t*>(A), code_out, nullptr);
+  canonical_build(s_len, nsym, &cs, reinterpret_cast<uint16_t*>(A), code_out, packed_out, nullptr);
 }
 
 __global__ __launch_bounds__(kBookThreads) void codebook_kernel(BookArgs a) {
@@ -744,9 +745,9 @@ __device__ __forceinline__ void mlp_forward_staged(const float* sw, const float 
 }
 
 // smallest exact size; ties prefer HUFF, then RLE_HUFF, then RLE
-__device__ __forceinline__ int exhaustive_pick(uint64_t sh, uint64_t sr, uint64_t srh) {
+__device__ __forceinline__ int exhaustive_pick(uint32_t sh, uint32_t sr, uint32_t srh) {
   int c = CODEC_HUFF;
-  uint64_t best = sh;
+  uint32_t best = sh;
   if (srh < best) {
     c = CODEC_RLE_HUFF;
     best = srh;
@@ -755,188 +756,243 @@ __device__ __forceinline__ int exhaustive_pick(uint64_t sh, uint64_t sr, uint64_
   return c;
 }
 
-// interleaved-stream units from per-thread bit partials: thread t's symbols all belong
-// to lane t % 32 (strided mapping over 256 threads); called by warp 0
-__device__ __forceinline__ uint32_t units_from_partials(const uint32_t* part) {
-  const int lane = threadIdx.x & 31;
-  uint32_t bits = 0;
-#pragma unroll
-  for (int wv = 0; wv < kEncThreads / 32; wv++) bits += part[32 * wv + lane];
-  return warp_sum(ihs_lane_units(bits));
-}
-
 static_assert(kEncThreads % kMadoN == 0, "madogram distances by thread");
 
-// Selection and encoding of codec block b of one field (all threads of the CTA).
-// smem: encode_smem_bytes() of dynamic shared memory.
-__device__ void encode_body(const EncodeArgs& a, uint32_t b, unsigned char* smem) {
-  uint16_t* s_c = reinterpret_cast<uint16_t*>(smem);             // 4096 codes
-  uint16_t* s_rv = s_c + kSlots;                                 // run values
-  uint16_t* s_rl = s_rv + kSlots;                                // run lengths
-  uint32_t* s_buf = reinterpret_cast<uint32_t*>(s_rl + kSlots);  // 16 KB
-  uint32_t* s_head = s_buf + kBufBytes / 4;                      // 128
-  uint32_t* s_woff = s_head + kSlots / 32;                       // 129 (+3)
-  uint32_t* s_next = s_woff + kSlots / 32 + 4;                   // 128
-  uint32_t* s_part = s_next + kSlots / 32;                       // 2 x 256
-  uint32_t* s_scan = s_part + 2 * kEncThreads;                   // 34
-  uint64_t* s_scan64 = reinterpret_cast<uint64_t*>(s_scan + 34); // 33
-  __shared__ uint32_t s_codec, s_units[3];
-  __shared__ uint64_t s_prefix;
-  __shared__ float s_feat[8];
-
-  const int tid = threadIdx.x, wid = tid >> 5;
-  uint32_t org[3], w[3];
-  block_box(a.g, b, org, w);
-  const uint32_t m = w[0] * w[1] * w[2];
-  const int sel = a.select;
-  const uint32_t r = a.radius;
-  const uint8_t* clen = a.lens;
-  const uint8_t* vlen = a.lens + kNsymCode;
-  const uint8_t* llen = a.lens + 2 * kNsymCode;
-  const uint64_t* ccode = a.bcodes;
-  const uint64_t* vcode = a.bcodes + kNsymCode;
-  const uint64_t* lcode = a.bcodes + 2 * kNsymCode;
-
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(a.codes + (uint64_t)b * kSlots);
-    uint4* dst = reinterpret_cast<uint4*>(s_c);
-    for (int i = tid; i < kSlots / 8; i += kEncThreads) dst[i] = __ldcs(&src[i]);
-    // the Huffman emitter's lane strings (s_rv and s_rl, 16 KB) start cleared; run
-    // extraction overwrites them, and the emitter then clears what it uses itself
-    uint4* lanes = reinterpret_cast<uint4*>(s_rv);
-    for (int i = tid; i < 2 * kSlots * 2 / 16; i += kEncThreads) lanes[i] = make_uint4(0u, 0u, 0u, 0u);
-  }
-  // the block statistics' code histogram (the first 1024 words of s_buf, which holds
-  // no payload until assembly) starts at zero, and the learned selector's parameters
-  // sit after it; both are ready at the barrier after the records
-  const bool analyze = a.analyze != 0;
-  static_assert(kNsymCode == 4 * kEncThreads && 4 * (kNsymCode + kSwWords) <= kBufBytes, "s_buf layout");
-  if (analyze || sel == SEL_HEURISTIC || sel == SEL_LEARNED)
-    reinterpret_cast<uint4*>(s_buf)[tid] = make_uint4(0u, 0u, 0u, 0u);
-  if (sel == SEL_LEARNED && !analyze) stage_mlp(a.mlp_w, reinterpret_cast<float*>(s_buf) + kNsymCode);
-
-  // this block's outlier and patch records, in slot order, at its record offset
-  if (a.place_records && a.rec.counts[b] != 0) {
-    const RecordArgs& R = a.rec;
-    const uint32_t lo = tid * 16;
-    const uint32_t* mw = R.masks + (uint64_t)b * 256;
-    const uint32_t pb = (mw[lo >> 5] >> (lo & 31)) & 0xffffu;
-    const uint32_t ob = (mw[128 + (lo >> 5)] >> (lo & 31)) & 0xffffu;
-    uint64_t pos = R.rec_off[b] + block_excl_scan<uint64_t>((uint64_t)(__popc(ob) + __popc(pb)), s_scan64, nullptr);
-    if (ob | pb) {
-      const int32_t* dl = R.deltas + (uint64_t)b * kSlots;
-      const uint64_t ny = a.g.n[1], nx = a.g.n[2];
-      uint32_t err = 0;
-      for (int i = 0; i < 16; i++) {
-        const uint32_t j = lo + i;
-        const uint32_t slot2 = (b * (uint32_t)kSlots + j) * 2u;
-        if ((ob >> i) & 1u) {
-          if (pos < R.rec_cap) reinterpret_cast<uint2*>(R.rec)[pos] = make_uint2(slot2, (uint32_t)dl[j]);
-          else err |= ERR_CAPACITY;
-          pos++;
-        }
-        if ((pb >> i) & 1u) {
-          uint32_t zz = 0, yy = 0, xx = j;
-          if (a.g.ndim == 2) {
-            yy = j / w[2];
-            xx = j - yy * w[2];
-          } else if (a.g.ndim == 3) {
-            const uint32_t pl = w[1] * w[2];
-            zz = j / pl;
-            const uint32_t rr = j - zz * pl;
-            yy = rr / w[2];
-            xx = rr - yy * w[2];
-          }
-          const uint64_t e = ((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + (org[2] + xx);
-          if (pos < R.rec_cap) reinterpret_cast<uint2*>(R.rec)[pos] = make_uint2(slot2 + 1u, __float_as_uint(R.x[e]));
-          else err |= ERR_CAPACITY;
-          pos++;
-        }
+// Block b's outlier and patch records, in slot order, at its record offset (all threads;
+// not inlined: few blocks have any, and the registers are the payload's).
+__device__ __noinline__ void place_records(const EncodeArgs& a, uint32_t b, const uint32_t* org, const uint32_t* w,
+                                           uint64_t* s_scan64) {
+  const uint32_t tid = threadIdx.x;
+  const RecordArgs& R = a.rec;
+  const uint32_t lo = tid * 16;
+  const uint32_t* mw = R.masks + (uint64_t)b * 256;
+  const uint32_t pb = (mw[lo >> 5] >> (lo & 31)) & 0xffffu;
+  const uint32_t ob = (mw[128 + (lo >> 5)] >> (lo & 31)) & 0xffffu;
+  uint64_t pos = R.rec_off[b] + block_excl_scan<uint64_t>((uint64_t)(__popc(ob) + __popc(pb)), s_scan64, nullptr);
+  if (ob | pb) {
+    const int32_t* dl = R.deltas + (uint64_t)b * kSlots;
+    const uint64_t ny = a.g.n[1], nx = a.g.n[2];
+    uint32_t err = 0;
+    for (int i = 0; i < 16; i++) {
+      const uint32_t j = lo + i;
+      const uint32_t slot2 = (b * (uint32_t)kSlots + j) * 2u;
+      if ((ob >> i) & 1u) {
+        if (pos < R.rec_cap) reinterpret_cast<uint2*>(R.rec)[pos] = make_uint2(slot2, (uint32_t)dl[j]);
+        else err |= ERR_CAPACITY;
+        pos++;
       }
-      if (err) atomicOr(&a.st->status, err);
+      if ((pb >> i) & 1u) {
+        uint32_t zz = 0, yy = 0, xx = j;
+        if (a.g.ndim == 2) {
+          yy = j / w[2];
+          xx = j - yy * w[2];
+        } else if (a.g.ndim == 3) {
+          const uint32_t pl = w[1] * w[2];
+          zz = j / pl;
+          const uint32_t rr = j - zz * pl;
+          yy = rr / w[2];
+          xx = rr - yy * w[2];
+        }
+        const uint64_t e = ((uint64_t)(org[0] + zz) * ny + (org[1] + yy)) * nx + (org[2] + xx);
+        if (pos < R.rec_cap) reinterpret_cast<uint2*>(R.rec)[pos] = make_uint2(slot2 + 1u, __float_as_uint(R.x[e]));
+        else err |= ERR_CAPACITY;
+        pos++;
+      }
+    }
+    if (err) atomicOr(&a.st->status, err);
+  }
+}
+
+// The runs of a block's codes (s_c: 4096 codes, staged here from the code stream): their
+// values and lengths, in order.  All threads; ends with a barrier.
+__device__ __noinline__ void extract_runs(const uint16_t* codes, uint32_t m, uint16_t* s_c, uint32_t* s_head,
+                                          uint32_t* s_woff, uint32_t* s_next, uint16_t* s_rv, uint16_t* s_rl) {
+  const uint32_t tid = threadIdx.x;
+  const uint4* src = reinterpret_cast<const uint4*>(codes);
+  uint4* dst = reinterpret_cast<uint4*>(s_c);
+  for (int i = tid; i < kSlots / 8; i += kEncThreads) dst[i] = __ldcg(&src[i]);
+  __syncthreads();
+  block_run_heads(s_c, m, s_head, s_woff, s_next);
+#pragma unroll 4
+  for (int i = 0; i < kSlots / kEncThreads; i++) {
+    const uint32_t j = tid + kEncThreads * i;
+    if (j < m) {
+      const uint32_t hb = s_head[j >> 5], bit = j & 31;
+      if ((hb >> bit) & 1u) {
+        const uint32_t ri = s_woff[j >> 5] + __popc(hb & ((1u << bit) - 1u));
+        s_rv[ri] = s_c[j];
+        s_rl[ri] = (uint16_t)(next_head(s_head, s_next, j, m) - j);
+      }
     }
   }
   __syncthreads();
+}
 
-  // Analysis (selector training data): every size and every feature of every block,
-  // no payload.  Otherwise runs are counted in every mode except forced Huffman and
-  // extracted (values, lengths) only when a run codec or the statistics need them.
-  uint32_t nr = 0;
-  bool have_runs = false;
-  // the run count comes from construction; the run index is built only when runs
-  // are extracted
-  if (sel != SEL_HUFF || analyze) nr = a.block_runs[b];
+// Encoding takes two launches (or phases): the plan of every block -- records, runs,
+// statistics, exact sizes, the pick -- then, when every size is known, the payloads.  One
+// launch with a decoupled look-back for the payload offsets held a CTA's place on its SM
+// until the slowest of the hundreds of blocks before it had its size, half of the time it
+// was resident (100x500x500 learned: 176 us with the look-back, 96 us with made-up
+// offsets).  Now the plan adds each block's size to its group's total and a payload CTA
+// sums what precedes it, with nothing to wait for; the codes are read twice for it.
+// 3-D 512^3: 525 -> 390 us for both.
+//
+// Groups of kGroup blocks: one 64-bit total each, payload bytes below bit 40, the numbers
+// of RLE and of RLE+Huffman blocks from bits 40 and 52.
+constexpr uint32_t kGroup = 256;
+static_assert(kGroup == kEncThreads, "a thread per block of the group");
+constexpr uint64_t kGroupBytes = (1ull << 40) - 1;
+
+// The Huffman streams' symbols of this thread (pair_plan); kNsymCode behind the last.
+struct HuffPart {
+  const uint16_t* src;
+  uint32_t n, steps, j0;
+  bool full;
+  __device__ __forceinline__ HuffPart(const uint16_t* codes, uint32_t m) {
+    const uint32_t w = threadIdx.x >> 5, h = huff_split(m);
+    n = w >> 2 ? m - h : h;
+    steps = quarter_steps(n);
+    j0 = 32 * (w & 3) * steps + (threadIdx.x & 31);
+    src = codes + (w >> 2 ? h : 0u) + j0;
+    full = m == (uint32_t)kSlots;
+  }
+  __device__ __forceinline__ void load(uint32_t (&sym)[16]) const {
+    if (full) {
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++) sym[i] = __ldcg(&src[32 * i]);
+    } else {
+#pragma unroll
+      for (uint32_t i = 0; i < 16; i++)
+        sym[i] = i < steps && j0 + 32 * i < n ? (uint32_t)__ldcg(&src[32 * i]) : (uint32_t)kNsymCode;
+    }
+  }
+};
+
+// The code book's packed codes in shared memory, and an empty one for "no symbol" (a
+// barrier follows at the caller)
+__device__ __forceinline__ void stage_book(const EncodeArgs& a, uint32_t* s_tab) {
+  reinterpret_cast<uint4*>(s_tab)[threadIdx.x] = __ldcg(&reinterpret_cast<const uint4*>(packed_books(a.bcodes))[threadIdx.x]);
+  if (threadIdx.x == 0) s_tab[kNsymCode] = 0;
+}
+
+// P of the Huffman block whose symbols the thread holds.  Contains one barrier.
+__device__ __forceinline__ void plan_huff(PairPlan& P, const EncodeArgs& a, const HuffPart& part, uint32_t (&sym)[16],
+                                          const uint32_t* s_tab, uint32_t* s_part) {
+  uint32_t cum = 0, odd = 0, longest = 0;
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    P.e[i] = s_tab[sym[i]];
+    cum += P.e[i] & 31u;
+    longest = max(longest, P.e[i] & 31u);
+  }
+  if (longest == kPackedLong) {
+    part.load(sym);  // (again: not held for this rare case)
+    odd = 1u << 31;
+#pragma unroll
+    for (int i = 0; i < 16; i++)
+      if ((P.e[i] & 31u) == kPackedLong) cum += __ldg(&a.lens[sym[i]]) - kPackedLong;
+  }
+  pair_plan(P, cum | odd, s_part);
+}
+
+// P of an RLE+Huffman block's nr runs.  Contains one barrier.
+__device__ __forceinline__ void plan_runs(PairPlan& P, const EncodeArgs& a, const uint16_t* rv, const uint16_t* rl,
+                                          uint32_t nr, uint32_t* s_part) {
+  const uint32_t lane = threadIdx.x & 31, which = threadIdx.x >> 7, quarter = (threadIdx.x >> 5) & 3;
+  const uint32_t steps = quarter_steps(nr), j0 = 32 * quarter * steps + lane;
+  const uint16_t* sy = which ? rl : rv;
+  const uint32_t at = which ? 2 * kNsymCode : kNsymCode;
+  const uint32_t* book = packed_books(a.bcodes) + at;
+  const uint8_t* lens = a.lens + at;
+  uint32_t cum = 0, odd = steps > 16 ? 1u << 31 : 0u;
+  auto take = [&](uint32_t i) -> uint32_t {
+    const uint32_t j = j0 + 32 * i;
+    if (i >= steps || j >= nr) return 0u;
+    const uint32_t sym = (uint32_t)sy[j] - which;  // (run lengths are coded less one)
+    const uint32_t e = book[sym];
+    uint32_t L = e & 31u;
+    if (L == kPackedLong) {
+      odd = 1u << 31;
+      L = __ldg(&lens[sym]);
+    }
+    cum += L;
+    return e;
+  };
+#pragma unroll
+  for (uint32_t i = 0; i < 16; i++) P.e[i] = take(i);
+  for (uint32_t i = 16; i < steps; i++) take(i);
+  pair_plan(P, cum | odd, s_part);
+}
+
+// Payload bytes of a Huffman block (u16 unit count, both streams) and of an RLE+Huffman
+// block (two words, both streams), from its plan
+__device__ __forceinline__ uint32_t huff_bytes(const PairPlan& P) { return (2 * (1 + P.units_a + P.units_b) + 3) & ~3u; }
+__device__ __forceinline__ uint32_t rlehuff_bytes(const PairPlan& P) { return (8 + 2 * (P.units_a + P.units_b) + 3) & ~3u; }
+
+// Where the plan leaves the runs of a block that is coded by them: values, then lengths, in
+// the block's outlier residuals, which its records no longer need.
+__device__ __forceinline__ uint16_t* block_run_store(const EncodeArgs& a, uint32_t b) {
+  return reinterpret_cast<uint16_t*>(const_cast<int32_t*>(a.rec.deltas) + (uint64_t)b * kSlots);
+}
+
+// The plan of codec block b of one field (all threads of the CTA).  box: its origin and
+// extent (block_box).  smem: plan_smem_bytes() of dynamic shared memory.
+__device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, unsigned char* smem) {
+  uint16_t* s_c = reinterpret_cast<uint16_t*>(smem);              // 4096 codes
+  uint16_t* s_rv = s_c + kSlots;                                  // run values
+  uint16_t* s_rl = s_rv + kSlots;                                 // run lengths
+  uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_rl + kSlots);  // 1024: the statistics' code histogram
+  uint32_t* s_sw = s_hist + kNsymCode;                            // the learned selector's parameters
+  uint32_t* s_tab = s_sw + (kSwWords + 3) / 4 * 4;                // the code book, packed (+4)
+  uint32_t* s_head = s_tab + kNsymCode + 4;                       // 128
+  uint32_t* s_woff = s_head + kSlots / 32;                        // 129 (+3)
+  uint32_t* s_next = s_woff + kSlots / 32 + 4;                    // 128
+  uint32_t* s_part = s_next + kSlots / 32;                        // 2 x 256
+  uint64_t* s_scan64 = reinterpret_cast<uint64_t*>(s_part + 2 * kEncThreads);  // 33
+  __shared__ int s_codec;
+  __shared__ float s_feat[8];
+
+  const int tid = threadIdx.x, wid = tid >> 5;
+  const uint32_t m = box[3] * box[4] * box[5];
+  const int sel = a.select;
+  const uint32_t r = a.radius;
+  // the symbols are on their way while the block's run count and records are looked at; read
+  // again where that takes more (L2 has them), rather than held
+  const uint16_t* codes = a.codes + (uint64_t)b * kSlots;
+  const HuffPart part(codes, m);
+  uint32_t sym[16];
+  part.load(sym);
+  bool fresh = true;  // sym holds the symbols
+  // the run count comes from construction; forced Huffman does without
+  const bool analyze = a.analyze != 0;
+  const uint32_t nr = sel != SEL_HUFF || analyze ? a.block_runs[b] : 0u;
   const bool eligible = a.all_runs || 4 * nr <= m;
-  auto extract_runs = [&]() {
-    if (have_runs) return;
-    block_run_heads(s_c, m, s_head, s_woff, s_next);
-#pragma unroll 4
-    for (int i = 0; i < kSlots / kEncThreads; i++) {
-      const uint32_t j = tid + kEncThreads * i;
-      if (j < m) {
-        const uint32_t hb = s_head[j >> 5], bit = j & 31;
-        if ((hb >> bit) & 1u) {
-          const uint32_t ri = s_woff[j >> 5] + __popc(hb & ((1u << bit) - 1u));
-          s_rv[ri] = s_c[j];
-          s_rl[ri] = (uint16_t)(next_head(s_head, s_next, j, m) - j);
-        }
-      }
-    }
-    __syncthreads();
-    have_runs = true;
-  };
-  if (analyze || (sel != SEL_HUFF && eligible && sel != SEL_RLE)) extract_runs();
-
-  // exact sizes: Huffman units from per-lane bit totals; the plan (code lengths in
-  // registers, lane offsets) is kept for the payload
-  IhsPlan plan;
-  IhsPlan2Out plan_out{0u, 0u, ~0u};
-  auto huff_units = [&]() {  // u16 count + both streams
-    plan_out = ihs_plan2(s_c, m, clen, s_part, plan);
-    return 1u + plan_out.units_a + plan_out.units_b;
-  };
-  auto rlehuff_units = [&]() {
-    uint32_t vb = 0, lb = 0;
-    for (uint32_t i = tid; i < nr; i += kEncThreads) {
-      vb += __ldg(&vlen[s_rv[i]]);
-      lb += __ldg(&llen[s_rl[i] - 1]);
-    }
-    s_part[tid] = vb;
-    s_part[kEncThreads + tid] = lb;
-    __syncthreads();
-    if (tid < 32) {
-      const uint32_t vu = units_from_partials(s_part);
-      const uint32_t lu = units_from_partials(s_part + kEncThreads);
-      if (tid == 0) {
-        s_units[1] = vu;
-        s_units[2] = lu;
-      }
-    }
-    __syncthreads();
-  };
-  uint64_t size_h = ~0ull, size_r = ~0ull, size_rh = ~0ull;
-  // for_pick: the sizes only decide an exhaustive pick, so the Huffman size is left
-  // unknown (~0) when a run codec is already smaller than any Huffman payload can be:
-  // every code takes at least one bit, so a Huffman block of m codes holds at least
-  // m / 16 units plus its unit count, 2 + m / 8 bytes.  The pick is the same.
-  auto exact_sizes = [&](bool h, bool rl, bool rh, bool for_pick) {
-    if (rl) size_r = 4ull * nr;
-    if (rh && eligible && size_rh == ~0ull) {
-      rlehuff_units();
-      size_rh = (8ull + 2ull * (s_units[1] + s_units[2]) + 3) & ~3ull;
-    }
-    const bool beaten = for_pick && min(size_r, size_rh) < 2ull + m / 8;
-    if (h && size_h == ~0ull && !beaten) size_h = (2ull * huff_units() + 3) & ~3ull;
-  };
-  exact_sizes(analyze || sel == SEL_HUFF || sel == SEL_EXHAUSTIVE, analyze || sel == SEL_RLE || sel == SEL_EXHAUSTIVE,
-              analyze || sel == SEL_RLE_HUFF || sel == SEL_EXHAUSTIVE, sel == SEL_EXHAUSTIVE && !analyze);
-
-  // selection
+  // Runs are extracted (values, lengths) when a run codec or the statistics may need them.
+  bool runs = analyze || (sel != SEL_HUFF && eligible);
   const bool statistics = analyze || ((sel == SEL_HEURISTIC || sel == SEL_LEARNED) && eligible);
-  if ((sel == SEL_HEURISTIC || sel == SEL_LEARNED) && !eligible && !analyze) {
-    if (tid == 0) s_codec = CODEC_HUFF;  // both pick between Huffman and RLE+Huffman
-  } else if (statistics) {
-    uint32_t* s_hist = s_buf;  // 1024 words (zeroed above), before the payload is assembled
+  // the histogram starts at zero; it and the parameters are ready at the barriers of the
+  // run extraction
+  static_assert(kNsymCode == 4 * kEncThreads, "a 16-byte store a thread");
+  if (statistics) {
+    reinterpret_cast<uint4*>(s_hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    if (sel == SEL_LEARNED) stage_mlp(a.mlp_w, reinterpret_cast<float*>(s_sw));
+  }
+  if (a.place_records && a.rec.counts[b] != 0) {
+    place_records(a, b, box, box + 3, s_scan64);
+    fresh = false;
+  }
+  if (runs) {
+    extract_runs(codes, m, s_c, s_head, s_woff, s_next, s_rv, s_rl);
+    fresh = false;
+  }
+
+  // selection by the block's statistics; -1: by exact sizes
+  int codec = sel == SEL_HUFF || (!eligible && (sel == SEL_HEURISTIC || sel == SEL_LEARNED)) ? CODEC_HUFF
+              : sel == SEL_RLE || sel == SEL_RLE_HUFF                                       ? sel
+                                                                                            : -1;
+  if (analyze) codec = -1;
+  if (statistics) {
+    const bool heuristic = sel == SEL_HEURISTIC && !analyze;
     for (uint32_t i = tid; i < nr; i += kEncThreads) atomicAdd(&s_hist[s_rv[i]], (uint32_t)s_rl[i]);
     __syncthreads();
     // block statistics in one pass and one reduction: entropy sum, |delta| sum, top
@@ -956,7 +1012,7 @@ __device__ void encode_body(const EncodeArgs& a, uint32_t b, unsigned char* smem
         }
       }
     }
-    const bool want_mado = !(sel == SEL_HEURISTIC && !analyze);
+    const bool want_mado = !heuristic;
     if (want_mado) {
       // kEncThreads is a multiple of kMadoN, so a thread's distance is fixed
       const uint32_t d = kMadoD0 + kMadoStep * (tid % kMadoN);
@@ -978,8 +1034,7 @@ __device__ void encode_body(const EncodeArgs& a, uint32_t b, unsigned char* smem
     }
     __syncthreads();
     const int64_t Lm = log2_q16_small(m);
-    __shared__ bool s_fallback;
-    if (sel == SEL_HEURISTIC && !analyze) {
+    if (heuristic) {
       if (tid == 0) {
         S_ = 0;
         f1 = 0;
@@ -1052,176 +1107,208 @@ __device__ void encode_body(const EncodeArgs& a, uint32_t b, unsigned char* smem
           float f[kMlpIn], y[kMlpOut];
 #pragma unroll
           for (int j = 0; j < kMlpIn; j++) f[j] = __shfl_sync(~0u, fk, j);
-          mlp_forward_staged(reinterpret_cast<const float*>(s_buf) + kNsymCode, f, y);
+          mlp_forward_staged(reinterpret_cast<const float*>(s_sw), f, y);
           bool fb;
           const int c = learned_pick(y, fb);
-          if (lane == 0) {
-            s_codec = (uint32_t)c;
-            s_fallback = fb;
-          }
+          if (lane == 0) s_codec = fb ? -1 : c;
         }
-      }
-      __syncthreads();
-      if (analyze) {
-        // one training row: features, log2 bits per element of each codec (Q16-exact),
-        // exact sizes, and whether the learned selector decides this block
-        if (tid < kMlpIn) a.feat_out[(uint64_t)b * kMlpIn + tid] = s_feat[tid];
-        if (tid < kMlpOut) {
-          const uint64_t sz = tid == CODEC_HUFF ? size_h : (tid == CODEC_RLE ? size_r : size_rh);
-          const bool have = sz != ~0ull;
-          a.size_out[(uint64_t)b * kMlpOut + tid] = have ? (uint32_t)sz : 0xffffffffu;
-          a.tgt_out[(uint64_t)b * kMlpOut + tid] =
-              have ? (float)((int64_t)log2_q16(8 * sz) - (int64_t)log2_q16(m)) * (1.0f / 65536.0f) : 0.0f;
-          if (tid == 0) a.valid_out[b] = eligible ? 1 : 0;
-        }
-        return;
-      }
-      if (s_fallback) {
-        // the network is unsure: exact sizes decide
-        exact_sizes(true, true, true, true);
-        if (tid == 0) s_codec = (uint32_t)exhaustive_pick(size_h, size_r, size_rh);
       }
     }
     __syncthreads();
-  } else if (tid == 0) {
-    s_codec = sel <= SEL_RLE_HUFF ? (uint32_t)sel : (uint32_t)exhaustive_pick(size_h, size_r, size_rh);
-  }
-  __syncthreads();
-  const int codec = (int)s_codec;
-  if (codec == CODEC_RLE || codec == CODEC_RLE_HUFF) extract_runs();
-  exact_sizes(codec == CODEC_HUFF, codec == CODEC_RLE, codec == CODEC_RLE_HUFF, false);
-  const uint64_t size = codec == CODEC_HUFF ? size_h : (codec == CODEC_RLE ? 4ull * nr : size_rh);
-  // The block's codec and size are counted, then the block counts itself done with
-  // release semantics: the block that takes the last count (acquire) writes the
-  // header from complete totals once its own payload is out.  No other block's
-  // payload bytes are needed for that, so the count need not wait for them.
-  __shared__ bool s_last;
-  uint32_t done = 0;
-  if (tid == 0) {
-    lookback_publish(a.lb, b, size);
-    atomicAdd(&a.st->ncodec[codec], 1u);
-    atomicAdd(&a.st->payload, (unsigned long long)size);
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(done) : "l"(&a.st->encode_done) : "memory");
+    if (!analyze) codec = s_codec;  // (-1 where the network is unsure)
   }
 
-  // payload assembly in shared memory while predecessors publish (every chosen size
-  // fits 16 KB unless a forced Huffman mode meets very long codes; those go direct)
-  auto assemble = [&](uint16_t* out16) {
-    if (codec == CODEC_HUFF) {
-      const uint32_t u = 1u + plan_out.units_a + plan_out.units_b;
-      if (plan_out.max_lane_bits <= kLaneBitsMax) {
-        ihs_emit2(s_c, m, ccode, plan, plan_out.units_a, reinterpret_cast<uint32_t*>(s_rv), out16, s_part,
-                  !have_runs);
-      } else {
-        const uint32_t h = huff_split(m);
-        if (tid == 0) out16[0] = (uint16_t)plan_out.units_a;
-        ihs_encode_block(s_c, h, 0, clen, ccode, out16 + 1, s_part);
-        ihs_encode_block(s_c + h, m - h, 0, clen, ccode, out16 + 1 + plan_out.units_a, s_part);
-      }
-      if ((u & 1u) && tid == 0) out16[u] = 0;
-    } else if (codec == CODEC_RLE_HUFF) {
-      const uint32_t vu = s_units[1], lu = s_units[2];
-      if (tid == 0) {
-        uint32_t* out32 = reinterpret_cast<uint32_t*>(out16);
-        out32[0] = nr;
-        out32[1] = vu;
-        if ((vu + lu) & 1u) out16[4 + vu + lu] = 0;
-      }
-      ihs_encode_block(s_rv, nr, 0, vlen, vcode, out16 + 4, s_part);
-      ihs_encode_block(s_rl, nr, -1, llen, lcode, out16 + 4 + vu, s_part);
+  // A pick by sizes takes the runs' first, then the Huffman size, unless a run codec is
+  // already smaller than any Huffman payload can be: every code takes at least one bit, so
+  // a block of m codes holds at least m / 16 units plus its unit count, 2 + m / 8 bytes.
+  PairPlan plan;
+  uint32_t size_h = ~0u, size_rh = ~0u;
+  const uint32_t size_r = 4 * nr;
+  if (codec == CODEC_RLE_HUFF || (codec < 0 && eligible)) {
+    plan_runs(plan, a, s_rv, s_rl, nr, s_part);
+    size_rh = rlehuff_bytes(plan);
+  }
+  if (codec == CODEC_HUFF || (codec < 0 && (analyze || min(size_r, size_rh) >= 2 + m / 8))) {
+    stage_book(a, s_tab);
+    if (!fresh) part.load(sym);
+    __syncthreads();
+    plan_huff(plan, a, part, sym, s_tab, s_part + kEncThreads);
+    size_h = huff_bytes(plan);
+  }
+  if (analyze) {
+    // one training row: features, log2 bits per element of each codec (Q16-exact),
+    // exact sizes, and whether the learned selector decides this block
+    if (tid < kMlpIn) a.feat_out[(uint64_t)b * kMlpIn + tid] = s_feat[tid];
+    if (tid < kMlpOut) {
+      const uint32_t sz = tid == CODEC_HUFF ? size_h : (tid == CODEC_RLE ? size_r : size_rh);
+      const bool have = sz != ~0u;
+      a.size_out[(uint64_t)b * kMlpOut + tid] = have ? sz : 0xffffffffu;
+      a.tgt_out[(uint64_t)b * kMlpOut + tid] =
+          have ? (float)((int64_t)log2_q16(8ull * sz) - (int64_t)log2_q16(m)) * (1.0f / 65536.0f) : 0.0f;
+      if (tid == 0) a.valid_out[b] = eligible ? 1 : 0;
     }
-  };
-  const bool in_smem = size <= (uint64_t)kBufBytes;
-  if (in_smem) assemble(reinterpret_cast<uint16_t*>(s_buf));
-  if (tid == 0) s_last = done == a.g.nblk - 1;
-  __syncthreads();
-
-  // placement
-  if (tid < 32) {
-    const uint64_t pre = lookback_warp(a.lb, b, size, &a.st->status, a.spin_limit);
-    if (tid == 0) s_prefix = pre;
-  }
-  __syncthreads();
-  const uint64_t off_pay = a.off_rec + 8ull * a.st->n_rec;
-  const uint64_t dst_off = off_pay + s_prefix;
-  if (tid == 0) {
-    a.ar[a.off_codec + b] = (uint8_t)codec;
-    reinterpret_cast<uint32_t*>(a.ar + a.off_bb)[b] = (uint32_t)size;
-  }
-  if (dst_off + size > a.cap) {
-    if (tid == 0) atomicOr(&a.st->status, ERR_CAPACITY);
     return;
   }
-  uint32_t* dst = reinterpret_cast<uint32_t*>(a.ar + dst_off);
-  const uint32_t nwords = (uint32_t)(size / 4);
-  if (codec == CODEC_RLE) {
-    uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
+  if (codec < 0) codec = exhaustive_pick(size_h, size_r, size_rh);  // (the same in every thread)
+  const uint32_t size = codec == CODEC_HUFF ? size_h : (codec == CODEC_RLE ? size_r : size_rh);
+  if (codec != CODEC_HUFF) {
+    if (!runs) extract_runs(codes, m, s_c, s_head, s_woff, s_next, s_rv, s_rl);
+    uint16_t* rv = block_run_store(a, b);
     for (uint32_t i = tid; i < nr; i += kEncThreads) {
-      d16[i] = s_rv[i];
-      d16[nr + i] = s_rl[i];
+      rv[i] = s_rv[i];
+      rv[kSlots + i] = s_rl[i];
     }
-  } else if (in_smem) {
-    for (uint32_t i = tid; i < nwords; i += kEncThreads) dst[i] = s_buf[i];
+  }
+  if (tid == 0) {
+    a.ar[a.off_codec + b] = (uint8_t)codec;
+    reinterpret_cast<uint32_t*>(a.ar + a.off_bb)[b] = size;
+    atomicAdd(reinterpret_cast<unsigned long long*>(a.groups) + b / kGroup,
+              (unsigned long long)size | (codec == CODEC_RLE ? 1ull << 40 : (codec == CODEC_RLE_HUFF ? 1ull << 52 : 0ull)));
+  }
+}
+
+// The field's totals from its groups', then the header, section padding and books (one
+// CTA; not inlined, as the two below, for the registers of the common path).
+__device__ __noinline__ void finish_field(const EncodeArgs& a) {
+  __shared__ uint64_t s_sum[kEncThreads / 32], s_all[kEncThreads / 32];
+  const uint32_t tid = threadIdx.x, wid = tid >> 5;
+  const uint32_t ngroups = (a.g.nblk + kGroup - 1) / kGroup;
+  uint64_t bytes = 0, counts = 0;  // (RLE blocks, RLE+Huffman blocks from bit 32)
+  for (uint32_t k = tid; k < ngroups; k += kEncThreads) {
+    const uint64_t v = __ldcg(&a.groups[k]);
+    bytes += v & kGroupBytes;
+    counts += ((v >> 40) & 0xfffu) | (v >> 52) << 32;
+  }
+  bytes = warp_sum(bytes);
+  counts = warp_sum(counts);
+  if ((tid & 31) == 0) {
+    s_sum[wid] = bytes;
+    s_all[wid] = counts;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < kEncThreads / 32; w++) {
+      bytes += s_sum[w];
+      counts += s_all[w];
+    }
+    a.st->payload = bytes;
+    a.st->ncodec[CODEC_RLE] = (uint32_t)counts;
+    a.st->ncodec[CODEC_RLE_HUFF] = (uint32_t)(counts >> 32);
+    a.st->ncodec[CODEC_HUFF] = a.g.nblk - (uint32_t)counts - (uint32_t)(counts >> 32);
+  }
+  finalize_body(a.fin);
+}
+
+// A block with codes longer than a packed one's, or one whose payload does not fit the
+// buffer: both streams by the gathering encoder.  first: units before stream A.
+__device__ __noinline__ void encode_long(const EncodeArgs& a, int codec, const uint16_t* codes, uint32_t m,
+                                         const uint16_t* rv, uint32_t nr, uint32_t ua, uint16_t* out16,
+                                         uint32_t* s_part) {
+  if (codec == CODEC_HUFF) {
+    const uint32_t h = huff_split(m);
+    ihs_encode_block(codes, h, 0, a.lens, a.bcodes, out16 + 1, s_part);
+    ihs_encode_block(codes + h, m - h, 0, a.lens, a.bcodes, out16 + 1 + ua, s_part);
   } else {
-    assemble(reinterpret_cast<uint16_t*>(dst));
+    const uint8_t* vlen = a.lens + kNsymCode;
+    const uint64_t* vcode = a.bcodes + kNsymCode;
+    ihs_encode_block(rv, nr, 0, vlen, vcode, out16 + 4, s_part);
+    ihs_encode_block(rv + kSlots, nr, -1, vlen + kNsymCode, vcode + kNsymCode, out16 + 4 + ua, s_part);
   }
-  // the block that counted last writes the header, section padding and books
-  if (s_last) finalize_body(a.fin);
 }
 
-// Blocks are taken in ticket order, so the payload look-back only ever waits on
-// blocks that CTAs already hold.
-__global__ __launch_bounds__(kEncThreads, 5) void encode_kernel(EncodeArgs a) {
-  __shared__ uint32_t s_tile;
-  extern __shared__ __align__(16) unsigned char smem[];
-  if (threadIdx.x == 0) s_tile = atomicAdd(&a.st->ticket_encode, 1u);
-  __syncthreads();
-  encode_body(a, s_tile, smem);
-}
-
-// Batch: one CTA per codec block of every field; the ticket runs over the blocks of
-// all fields in order (tile0[f] = first block of field f).
-__global__ __launch_bounds__(kEncThreads, 5) void encode_batch_kernel(const EncodeArgs* __restrict__ tasks,
-                                                                   const uint32_t* __restrict__ tile0, int nfields,
-                                                                   uint32_t* ticket) {
-  __shared__ uint32_t s_tile;
-  __shared__ int s_field;
-  if (threadIdx.x == 0) {
-    const uint32_t t = atomicAdd(ticket, 1u);
-    int lo = 0, hi = nfields - 1;  // last field with tile0[f] <= t
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (tile0[mid] <= t) lo = mid;
-      else hi = mid - 1;
+// The payload of codec block b (all threads of the CTA), after the plans of all the field's
+// blocks; block 0 also writes the header, section padding and books.  m: the block's
+// elements.  smem: payload_smem_bytes() of dynamic shared memory.
+__device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsigned char* smem) {
+  uint32_t* s_buf = reinterpret_cast<uint32_t*>(smem);  // 16 KB: the payload; before it, the code book
+  uint32_t* s_part = s_buf + kBufBytes / 4;             // 256 (+ 8)
+  uint32_t* s_heads = s_part + kEncThreads + 8;         // 256
+  __shared__ uint64_t s_sum[kEncThreads / 32];
+  const uint32_t tid = threadIdx.x, wid = tid >> 5;
+  const uint16_t* codes = a.codes + (uint64_t)b * kSlots;
+  const HuffPart part(codes, m);
+  uint32_t sym[16];
+  part.load(sym);
+  const int codec = __ldcg(&a.ar[a.off_codec + b]);
+  const uint32_t* bb = reinterpret_cast<const uint32_t*>(a.ar + a.off_bb);
+  const uint32_t size = __ldcg(&bb[b]);
+  const uint64_t n_rec = __ldcg(&a.st->n_rec);
+  // what precedes the block: the groups before its own, the blocks before it in its own
+  const uint32_t group = b / kGroup, in_group = b % kGroup;
+  uint64_t before = tid < in_group ? (uint64_t)__ldcg(&bb[group * kGroup + tid]) : 0ull;
+  for (uint32_t k = tid; k < group; k += kEncThreads) before += __ldcg(&a.groups[k]) & kGroupBytes;
+  const uint32_t nr = a.block_runs[b];
+  const uint16_t* rv = block_run_store(a, b);
+  before = warp_sum(before);
+  if ((tid & 31) == 0) s_sum[wid] = before;
+  PairPlan plan;
+  const bool in_smem = size <= (uint32_t)kBufBytes;
+  if (codec == CODEC_HUFF) {
+    stage_book(a, s_buf);
+    __syncthreads();
+    plan_huff(plan, a, part, sym, s_buf, s_part);
+  } else if (codec == CODEC_RLE_HUFF) {
+    plan_runs(plan, a, rv, rv + kSlots, nr, s_part);
+  } else {
+    __syncthreads();
+  }
+  uint64_t dst_off = a.off_rec + 8ull * n_rec;
+#pragma unroll
+  for (int w = 0; w < kEncThreads / 32; w++) dst_off += s_sum[w];
+  if (dst_off + size > a.cap) {
+    if (tid == 0) atomicOr(&a.st->status, ERR_CAPACITY);
+  } else {
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.ar + dst_off);
+    if (codec == CODEC_RLE) {
+      uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
+      for (uint32_t i = tid; i < nr; i += kEncThreads) {
+        d16[i] = rv[i];
+        d16[nr + i] = rv[kSlots + i];
+      }
+    } else {
+      // assembled in shared memory (every chosen size fits 16 KB unless a forced mode meets
+      // very long codes; those go direct)
+      uint16_t* out16 = in_smem ? reinterpret_cast<uint16_t*>(s_buf) : reinterpret_cast<uint16_t*>(dst);
+      const uint32_t ua = plan.units_a, ub = plan.units_b;
+      const uint32_t first = codec == CODEC_HUFF ? 1u : 4u, units = first + ua + ub;  // before stream A; in all
+      if (plan.packed && in_smem) {
+        pair_emit(plan, reinterpret_cast<uint16_t*>(s_buf), first, s_heads);
+      } else {
+        encode_long(a, codec, codes, m, rv, nr, ua, out16, s_part);
+      }
+      if (tid == 0) {
+        if (codec == CODEC_HUFF) {
+          out16[0] = (uint16_t)ua;
+        } else {
+          reinterpret_cast<uint32_t*>(out16)[0] = nr;
+          reinterpret_cast<uint32_t*>(out16)[1] = ua;
+        }
+        if (units & 1u) out16[units] = 0;
+      }
+      if (in_smem) {
+        __syncthreads();
+        for (uint32_t i = tid; i < size / 4; i += kEncThreads) dst[i] = s_buf[i];
+      }
     }
-    s_field = lo;
-    s_tile = t - tile0[lo];
   }
-  __syncthreads();
+  if (b == 0) finish_field(a);
+}
+
+__global__ __launch_bounds__(kEncThreads, 5) void plan_kernel(EncodeArgs a) {
+  __shared__ uint32_t s_box[6];
   extern __shared__ __align__(16) unsigned char smem[];
-  encode_body(tasks[s_field], s_tile, smem);
+  if (threadIdx.x == 0) block_box(a.g, blockIdx.x, s_box, s_box + 3);
+  __syncthreads();
+  plan_body(a, blockIdx.x, s_box, smem);
 }
 
-static size_t encode_smem_bytes() {
-  return kSlots * 2 * 3 + kBufBytes + (kSlots / 32) * 4 * 3 + 16 + 2 * kEncThreads * 4 + 34 * 4 + 33 * 8 + 16;
+__global__ __launch_bounds__(kEncThreads, 5) void payload_kernel(EncodeArgs a) {
+  __shared__ uint32_t s_m;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (threadIdx.x == 0) s_m = block_elems(a.g, blockIdx.x);
+  __syncthreads();
+  payload_body(a, blockIdx.x, s_m, smem);
 }
-
-// =================================================================================
-// batched compression in one persistent launch
-// =================================================================================
-// Every CTA runs the four phases of the staged batch in order, so the work items of
-// each phase are taken (by ticket) only after those of the phases before it were all
-// taken: a waiting CTA waits on items that running CTAs hold (only a running CTA takes
-// an item), and those wait only on earlier phases, so the launch cannot deadlock even
-// when not all of its CTAs are resident at once.  The
-// hand-overs are per field (DevState ready_range, tiles_flushed, books_done: a
-// release by the producer, an acquire by thread 0 of the consumer, then a CTA
-// barrier), so one field's books and encoding start while other fields are still
-// being constructed.  Every wait is bounded (ERR_TIMEOUT in the field's status).
-// The output is the staged path's, byte for byte: the same bodies run on the same
-// items.
-constexpr int kPersistThreads = 256;
-static_assert(kPersistThreads == kEncThreads, "one CTA shape for every phase");
 
 __device__ __forceinline__ int field_of_prefix(const uint32_t* prefix, int nfields, uint32_t c) {
   int lo = 0, hi = nfields - 1;  // last field with prefix[f] <= c
@@ -1232,6 +1319,58 @@ __device__ __forceinline__ int field_of_prefix(const uint32_t* prefix, int nfiel
   }
   return lo;
 }
+
+// Batch: one CTA per codec block of every field (tile0[f] = first block of field f).
+__global__ __launch_bounds__(kEncThreads, 5) void plan_batch_kernel(const EncodeArgs* __restrict__ tasks,
+                                                                 const uint32_t* __restrict__ tile0, int nfields) {
+  __shared__ uint32_t s_box[6];
+  __shared__ int s_field;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (threadIdx.x == 0) {
+    const int f = field_of_prefix(tile0, nfields, blockIdx.x);
+    s_field = f;
+    block_box(tasks[f].g, blockIdx.x - tile0[f], s_box, s_box + 3);
+  }
+  __syncthreads();
+  plan_body(tasks[s_field], blockIdx.x - tile0[s_field], s_box, smem);
+}
+
+__global__ __launch_bounds__(kEncThreads, 5) void payload_batch_kernel(const EncodeArgs* __restrict__ tasks,
+                                                                    const uint32_t* __restrict__ tile0, int nfields) {
+  __shared__ uint32_t s_m;
+  __shared__ int s_field;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (threadIdx.x == 0) {
+    const int f = field_of_prefix(tile0, nfields, blockIdx.x);
+    s_field = f;
+    s_m = block_elems(tasks[f].g, blockIdx.x - tile0[f]);
+  }
+  __syncthreads();
+  payload_body(tasks[s_field], blockIdx.x - tile0[s_field], s_m, smem);
+}
+
+static size_t plan_smem_bytes() {
+  return kSlots * 2 * 3 + 4 * (kNsymCode + (kSwWords + 3) / 4 * 4 + kNsymCode + 4 + (kSlots / 32) * 3 + 4 + 2 * kEncThreads) +
+         33 * 8 + 16;
+}
+static size_t payload_smem_bytes() { return kBufBytes + 4 * (2 * kEncThreads + 8); }
+
+// =================================================================================
+// batched compression in one persistent launch
+// =================================================================================
+// Every CTA runs the phases of the staged batch in order, so the work items of
+// each phase are taken (by ticket) only after those of the phases before it were all
+// taken: a waiting CTA waits on items that running CTAs hold (only a running CTA takes
+// an item), and those wait only on earlier phases, so the launch cannot deadlock even
+// when not all of its CTAs are resident at once.  The
+// hand-overs are per field (DevState ready_range, tiles_flushed, books_done, encode_done: a
+// release by the producer, an acquire by thread 0 of the consumer, then a CTA
+// barrier), so one field's books and encoding start while other fields are still
+// being constructed.  Every wait is bounded (ERR_TIMEOUT in the field's status).
+// The output is the staged path's, byte for byte: the same bodies run on the same
+// items.
+constexpr int kPersistThreads = 256;
+static_assert(kPersistThreads == kEncThreads, "one CTA shape for every phase");
 
 // thread 0 draws the next item of a phase; every thread gets it (two barriers, so the
 // word is free for the next draw)
@@ -1256,7 +1395,7 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
   // which would pad the static shared memory of every kernel in this file
   extern __shared__ __align__(16) unsigned char smem_dyn[];
   unsigned char* smem_raw = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
-  __shared__ uint32_t s_word;
+  __shared__ uint32_t s_word, s_box[6];
   const int tid = threadIdx.x;
   // ---- phase 1: value ranges and bounds ---------------------------------------------
   while (true) {
@@ -1292,7 +1431,7 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
       atomicAdd(&ba.st->books_done, 1u);
     }
   }
-  // ---- phase 4: encoding (waits for each field's books) -------------------------------
+  // ---- phase 4: block plans (wait for each field's books) ------------------------------
   int ready_field = -1;
   while (true) {
     const uint32_t t = draw_item(&p.tickets[1], &s_word);
@@ -1303,14 +1442,37 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
       await_field(&ea.st->books_done, 4u, ea.st, p.spin_limit);
       ready_field = f;
     }
-    encode_body(ea, t - p.tile0[f], smem_raw);
+    if (tid == 0) block_box(ea.g, t - p.tile0[f], s_box, s_box + 3);
+    __syncthreads();
+    plan_body(ea, t - p.tile0[f], s_box, smem_raw);
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(&ea.st->encode_done, 1u);
+    }
+  }
+  // ---- phase 5: payloads (wait for each field's plans) ---------------------------------
+  ready_field = -1;
+  while (true) {
+    const uint32_t t = draw_item(&p.tickets[4], &s_word);
+    if (t >= p.ntiles) break;
+    const int f = field_of_prefix(p.tile0, p.nfields, t);
+    const EncodeArgs& ea = p.etasks[f];
+    if (f != ready_field) {
+      await_field(&ea.st->encode_done, ea.g.nblk, ea.st, p.spin_limit);
+      ready_field = f;
+    }
+    if (tid == 0) s_box[0] = block_elems(ea.g, t - p.tile0[f]);
+    __syncthreads();
+    payload_body(ea, t - p.tile0[f], s_box[0], smem_raw);
     __syncthreads();
   }
 }
 
 static size_t persist_smem_bytes() {
   size_t b = construct_smem_bytes();
-  if (encode_smem_bytes() > b) b = encode_smem_bytes();
+  if (plan_smem_bytes() > b) b = plan_smem_bytes();
+  if (payload_smem_bytes() > b) b = payload_smem_bytes();
   if (book_mem_bytes(kNsymCode) > b) b = book_mem_bytes(kNsymCode);
   return b + 1024;  // alignment slack
 }
@@ -1390,7 +1552,8 @@ cudaError_t launch_codebook(const BookArgs& a, cudaStream_t s) {
 
 cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s) {
   trace_begin(K_ENCODE, s);
-  encode_kernel<<<a.g.nblk, kEncThreads, encode_smem_bytes(), s>>>(a);
+  plan_kernel<<<a.g.nblk, kEncThreads, plan_smem_bytes(), s>>>(a);
+  if (!a.analyze) payload_kernel<<<a.g.nblk, kEncThreads, payload_smem_bytes(), s>>>(a);
   trace_end(K_ENCODE, s);
   return cudaGetLastError();
 }
@@ -1428,9 +1591,10 @@ cudaError_t launch_codebook_batch(const BookArgs* d_tasks, int nfields, cudaStre
 }
 
 cudaError_t launch_encode_batch(const EncodeArgs* d_tasks, const uint32_t* d_tile0, int nfields, uint32_t ntiles,
-                                uint32_t* ticket, cudaStream_t s) {
+                                cudaStream_t s) {
   trace_begin(K_ENCODE, s);
-  encode_batch_kernel<<<ntiles, kEncThreads, encode_smem_bytes(), s>>>(d_tasks, d_tile0, nfields, ticket);
+  plan_batch_kernel<<<ntiles, kEncThreads, plan_smem_bytes(), s>>>(d_tasks, d_tile0, nfields);
+  payload_batch_kernel<<<ntiles, kEncThreads, payload_smem_bytes(), s>>>(d_tasks, d_tile0, nfields);
   trace_end(K_ENCODE, s);
   return cudaGetLastError();
 }

@@ -255,7 +255,7 @@ __device__ void dec_tables_body(const DecodeArgs& a, int book) {
     }
     return;
   }
-  canonical_build(s_len, nsym, &cs, s_wcnt, nullptr, s_sorted);
+  canonical_build(s_len, nsym, &cs, s_wcnt, nullptr, nullptr, s_sorted);
   if (tid == 0) s_bad = s_full[0] = s_full[1] = 0;  // s_bad: now the largest length
   __syncthreads();
   if (tid <= kMaxLen) {

@@ -39,8 +39,8 @@ inline bool make_geom(int ndim, const uint64_t* dims, Geom& g) {
   return true;
 }
 
-// Workspace: [DevState | set-up look-back states | histograms | look-back states]
-// (zeroed per compression; decompression zeroes the first two),
+// Workspace: [DevState | set-up look-back states | histograms | group totals] (zeroed per
+// compression; decompression zeroes the first two),
 // books, decode tables and offsets, block-major code stream, decoded run lengths,
 // the lists of run blocks and of blocks reconstructed apart from their decoding
 // (the part decompression needs ends at dec_total), then compression-only scratch:
@@ -65,14 +65,16 @@ inline Layout layout(const Geom& g) {
   o += kNsymCode * 4;
   L.hist_len = o;
   o += kNsymLen * 4;
+  // compression: the totals of groups of 256 blocks (zeroed per call); decompression of
+  // 1-D global archives: a look-back state per block (zeroed there)
   L.lb_e = o;
+  L.zero_end = o + 8ull * ((g.nblk + 255) / 256);
   o += 8ull * g.nblk;
-  L.zero_end = o;
   o = a256(o);
   L.lens = o;
   o += a256(2 * kNsymCode + kNsymLen);
   L.bcodes = o;
-  o += 8ull * (2 * kNsymCode + kNsymLen);
+  o += a256(kBookCodeBytes);
   L.blk_off = o;
   o += a256(8ull * (g.nblk + 1));
   L.rec_start = o;

@@ -60,12 +60,21 @@ struct ConstructTask {
   int use_tma;
 };
 
+// The three books (quant codes, run values, run lengths) one after the other: 64-bit codes,
+// then the same codes packed with their lengths (packed_code).
+constexpr int kBookSyms = 2 * kNsymCode + kNsymLen;
+constexpr uint64_t kBookCodeBytes = 12ull * kBookSyms;
+__host__ __device__ inline uint32_t* packed_books(uint64_t* codes) { return reinterpret_cast<uint32_t*>(codes + kBookSyms); }
+__host__ __device__ inline const uint32_t* packed_books(const uint64_t* codes) {
+  return reinterpret_cast<const uint32_t*>(codes + kBookSyms);
+}
+
 struct BookArgs {
   const uint32_t* hist_code;
   const uint32_t* hist_val;
   const uint32_t* hist_len;
   uint8_t* lens;    // 1024 + 1024 + 4096
-  uint64_t* codes;  // 1024 + 1024 + 4096
+  uint64_t* codes;  // 1024 + 1024 + 4096, then the packed codes (packed_books)
   DevState* st;
   int place_records;  // a fourth CTA scans the record counts into rec.rec_off
   uint32_t nblk;
@@ -108,11 +117,10 @@ struct EncodeArgs {
   uint8_t* ar;
   uint64_t cap;
   uint64_t off_codec, off_bb, off_rec;
-  uint64_t* lb;
-  uint32_t spin_limit;
+  uint64_t* groups;  // [nblk / 256, rounded up] totals of groups of 256 blocks (zeroed per call; compress.cu)
   int place_records;  // write each block's records (compression, not analysis)
   RecordArgs rec;
-  FinalizeArgs fin;  // used by the last block to finish
+  FinalizeArgs fin;  // used by block 0
 };
 
 // decode tables of one canonical book
@@ -213,7 +221,7 @@ cudaError_t launch_range_batch(const RangeTask* d_tasks, const uint32_t* d_cta0,
                                cudaStream_t s);
 cudaError_t launch_codebook_batch(const BookArgs* d_tasks, int nfields, cudaStream_t s);
 cudaError_t launch_encode_batch(const EncodeArgs* d_tasks, const uint32_t* d_tile0, int nfields, uint32_t ntiles,
-                                uint32_t* ticket, cudaStream_t s);
+                                cudaStream_t s);
 
 // Batched compression as one persistent kernel: every CTA goes through the same
 // four phases in order, taking work items from one ticket per phase -- value-range
@@ -231,7 +239,7 @@ struct PersistArgs {
   unsigned char* len_books;  // nfields x persist_len_book_bytes(): working memory of the run-length books
   const EncodeArgs* etasks;
   int nfields;
-  uint32_t* tickets;  // [0] construction, [1] encoding, [2] value range, [3] books
+  uint32_t* tickets;  // [0] construction, [1] block plans, [2] value range, [3] books, [4] payloads
   uint32_t spin_limit;
 };
 size_t persist_len_book_bytes();
