@@ -4,9 +4,9 @@
 // encoded sizes of every block).  The loss is the mean over rows and outputs of the
 // squared error; the optimiser is Adam.
 //
-// Kernel layout: one warp per row at a time, lane i owning hidden unit i of both
-// layers, so the forward pass is a shuffle-broadcast of the activations and the
-// backward pass accumulates each lane's rows of dW1 and dW2 in registers.  Partial
+// Kernel layout: one warp per pair of rows at a time, lane i owning hidden unit i of both
+// layers, so the activations go to every lane through shared memory and the backward
+// pass accumulates each lane's rows of dW1 and dW2 in registers.  Partial
 // sums per CTA go to the workspace and are added in a fixed order by the update
 // kernel, so a training run is reproducible bit for bit on one GPU model.
 #include <cmath>
@@ -18,7 +18,7 @@
 namespace cszp {
 namespace {
 
-constexpr int kTrainThreads = 256;
+constexpr int kTrainThreads = 384;
 constexpr int kTrainWarps = kTrainThreads / 32;
 constexpr int kPart = kMlpParams + 2;  // gradient sums, loss sum, row count
 constexpr float kAdamB1 = 0.9f, kAdamB2 = 0.999f, kAdamEps = 1e-8f;
@@ -49,12 +49,18 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // Forward and backward over rows gw, gw + nw, ... of every warp; per-CTA sums of the
 // unscaled gradient (d(e^2)/dy = 2e), of e^2 and of the row count go to part[cta].
 //
-// Bound by instruction issue (about 250 warp instructions a row).  Lane i owns row i of
-// W2 and dW2, whose packed layout puts the 32 lanes' words in 32 cache lines (and one
-// bank): the parameters are staged in shared memory with W2's rows padded to 33 words,
-// and dW2 is handed over transposed with the same padding, so that neither the loads
-// nor the reduction serialise (28,672 rows: 39 us a launch with the strided accesses,
-// 20 us so, both with the events around it).
+// Bound by instruction issue (about 200 warp instructions a row) and, with few warps an SM
+// for the registers the weights take, by the chains in between.  A row's activations reach
+// the 32 lanes as 16-byte shared-memory words (a shuffle each, 64 a row, kept the one
+// shuffle result a cycle and SM busy for half the time) and are read again for dW2 instead
+// of held, which leaves registers for 12 warps an SM where 198 a thread left 8; and a warp
+// works on two rows at once.  Rows that take no part are skipped by a ballot over 32 of
+// them.  A training step on 28,672 rows, with the update below: 35 -> 21 us.
+//
+// Lane i owns row i of W2 and dW2, whose packed layout puts the 32 lanes' words in 32 cache
+// lines (and one bank): the parameters are staged in shared memory with W2's rows padded to
+// 33 words, and dW2 is handed over transposed with the same padding, so that neither the
+// loads nor the reduction serialise.
 constexpr int kPitch = kMlpHid + 1;
 constexpr int kStage = kMlpHid * (kPitch - kMlpHid);  // words the padding adds
 // a parameter's word in the padded layout: W2's entries at pitch 33
@@ -67,12 +73,28 @@ __device__ __forceinline__ int padded_t(int p) {
   const int k = p - kMlpW2;
   return kMlpW2 + (k % kMlpHid) * kPitch + k / kMlpHid;
 }
+// One row's sums over the lanes' hidden units, four independent chains
+__device__ __forceinline__ float dot32(const float (&w)[kMlpHid], const float* s, float first) {
+  float acc[4] = {first, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int j = 0; j < kMlpHid; j += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(s + j);
+    acc[0] = fmaf(w[j], v.x, acc[0]);
+    acc[1] = fmaf(w[j + 1], v.y, acc[1]);
+    acc[2] = fmaf(w[j + 2], v.z, acc[2]);
+    acc[3] = fmaf(w[j + 3], v.w, acc[3]);
+  }
+  return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+constexpr int kRedWarps = kTrainWarps / 2;  // the warps' sums meet in two turns
 __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __restrict__ w,
                                                                  const float* __restrict__ feat,
                                                                  const float* __restrict__ tgt,
                                                                  const uint8_t* __restrict__ valid,
                                                                  uint64_t n, float* __restrict__ part) {
-  __shared__ float s_red[kTrainWarps][kPart + kStage];
+  __shared__ float s_red[kRedWarps][kPart + kStage];
+  __shared__ __align__(16) float s_act[kTrainWarps][4][kMlpHid];  // per warp: h1 and da2 of two rows
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float* sw = s_red[0];  // the staged parameters, until the sums need the words
   for (int p = threadIdx.x; p < kMlpParams; p += kTrainThreads) sw[padded(p)] = w[p];
@@ -101,129 +123,192 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __
 #pragma unroll
   for (int c = 0; c < kMlpOut; c++) g3[c] = gb3[c] = 0.0f;
 
+  float(*act)[kMlpHid] = s_act[wid];
   const uint64_t nw = (uint64_t)gridDim.x * kTrainWarps;
-  for (uint64_t r = (uint64_t)blockIdx.x * kTrainWarps + wid; r < n; r += nw) {
-    if (valid && !valid[r]) continue;  // warp-uniform
-    float x[kMlpIn];
+  for (uint64_t r0 = (uint64_t)blockIdx.x * kTrainWarps + wid; r0 < n; r0 += 32 * nw) {
+    const uint64_t mine = r0 + lane * nw;
+    uint32_t todo = __ballot_sync(~0u, mine < n && (!valid || valid[mine]));
+    while (todo) {
+      // two of the rows, or one (then the second repeats it and adds nothing)
+      uint64_t row[2];
+      row[0] = r0 + (__ffs(todo) - 1) * nw;
+      todo &= todo - 1;
+      const bool both = todo != 0;
+      row[1] = both ? r0 + (__ffs(todo) - 1) * nw : row[0];
+      todo &= todo - 1;
+      float x[2][kMlpIn], a1[2], a2[2], h2[2], dy[2][kMlpOut], da2[2], da1[2];
+      // forward
 #pragma unroll
-    for (int j = 0; j < kMlpIn; j++) x[j] = __ldg(&feat[r * kMlpIn + j]);
-    // forward
-    float a1 = b1;
+      for (int k = 0; k < 2; k++) {
+        a1[k] = b1;
 #pragma unroll
-    for (int j = 0; j < kMlpIn; j++) a1 = fmaf(w1[j], x[j], a1);
-    const float h1 = a1 > 0.0f ? a1 : 0.0f;
-    float h1all[kMlpHid];
-    float a2 = b2;
+        for (int j = 0; j < kMlpIn; j++) x[k][j] = __ldg(&feat[row[k] * kMlpIn + j]);
 #pragma unroll
-    for (int j = 0; j < kMlpHid; j++) {
-      h1all[j] = __shfl_sync(~0u, h1, j);
-      a2 = fmaf(w2r[j], h1all[j], a2);
+        for (int j = 0; j < kMlpIn; j++) a1[k] = fmaf(w1[j], x[k][j], a1[k]);
+        act[k][lane] = a1[k] > 0.0f ? a1[k] : 0.0f;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        a2[k] = dot32(w2r, act[k], b2);
+        h2[k] = a2[k] > 0.0f ? a2[k] : 0.0f;
+      }
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+#pragma unroll
+        for (int c = 0; c < kMlpOut; c++) {
+          const float y = b3[c] + warp_sum_f(w3[c] * h2[k]);
+          const float e = k == 0 || both ? y - __ldg(&tgt[row[k] * kMlpOut + c]) : 0.0f;
+          loss = fmaf(e, e, loss);
+          dy[k][c] = 2.0f * e;
+        }
+      }
+      cnt += both ? 2.0f : 1.0f;
+      // backward
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        float dh2 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < kMlpOut; c++) {
+          g3[c] = fmaf(dy[k][c], h2[k], g3[c]);
+          gb3[c] += dy[k][c];
+          dh2 = fmaf(dy[k][c], w3[c], dh2);
+        }
+        da2[k] = a2[k] > 0.0f ? dh2 : 0.0f;
+        act[2 + k][lane] = da2[k];
+        gb2 += da2[k];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+#pragma unroll
+        for (int j = 0; j < kMlpHid; j += 4) {
+          const float4 h = *reinterpret_cast<const float4*>(&act[k][j]);
+          g2[j] = fmaf(da2[k], h.x, g2[j]);
+          g2[j + 1] = fmaf(da2[k], h.y, g2[j + 1]);
+          g2[j + 2] = fmaf(da2[k], h.z, g2[j + 2]);
+          g2[j + 3] = fmaf(da2[k], h.w, g2[j + 3]);
+        }
+        const float dh1 = dot32(w2c, act[2 + k], 0.0f);
+        da1[k] = a1[k] > 0.0f ? dh1 : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kMlpIn; j++) g1[j] = fmaf(da1[k], x[k][j], g1[j]);
+        gb1 += da1[k];
+      }
+      __syncwarp();  // act is free again
     }
-    const float h2 = a2 > 0.0f ? a2 : 0.0f;
-    float dy[kMlpOut];
-#pragma unroll
-    for (int c = 0; c < kMlpOut; c++) {
-      const float y = b3[c] + warp_sum_f(w3[c] * h2);
-      const float e = y - __ldg(&tgt[r * kMlpOut + c]);
-      loss = fmaf(e, e, loss);
-      dy[c] = 2.0f * e;
-    }
-    cnt += 1.0f;
-    // backward
-    float dh2 = 0.0f;
-#pragma unroll
-    for (int c = 0; c < kMlpOut; c++) {
-      g3[c] = fmaf(dy[c], h2, g3[c]);
-      gb3[c] += dy[c];
-      dh2 = fmaf(dy[c], w3[c], dh2);
-    }
-    const float da2 = a2 > 0.0f ? dh2 : 0.0f;
-#pragma unroll
-    for (int j = 0; j < kMlpHid; j++) g2[j] = fmaf(da2, h1all[j], g2[j]);
-    gb2 += da2;
-    float dh1 = 0.0f;
-#pragma unroll
-    for (int i = 0; i < kMlpHid; i++) dh1 = fmaf(w2c[i], __shfl_sync(~0u, da2, i), dh1);
-    const float da1 = a1 > 0.0f ? dh1 : 0.0f;
-#pragma unroll
-    for (int j = 0; j < kMlpIn; j++) g1[j] = fmaf(da1, x[j], g1[j]);
-    gb1 += da1;
   }
 
-  float* my = s_red[wid];
+  // the sums of warps kRedWarps and up, then those of the others added to them
+  for (int turn = 1; turn >= 0; turn--) {
+    if (wid / kRedWarps == turn) {
+      float* my = s_red[wid % kRedWarps];
+      auto put = [&](int at, float v) { my[at] = turn ? v : my[at] + v; };
 #pragma unroll
-  for (int j = 0; j < kMlpIn; j++) my[kMlpW1 + lane * kMlpIn + j] = g1[j];
-  my[kMlpB1 + lane] = gb1;
+      for (int j = 0; j < kMlpIn; j++) put(kMlpW1 + lane * kMlpIn + j, g1[j]);
+      put(kMlpB1 + lane, gb1);
 #pragma unroll
-  for (int j = 0; j < kMlpHid; j++) my[kMlpW2 + j * kPitch + lane] = g2[j];
-  my[kMlpB2 + kStage + lane] = gb2;
+      for (int j = 0; j < kMlpHid; j++) put(kMlpW2 + j * kPitch + lane, g2[j]);
+      put(kMlpB2 + kStage + lane, gb2);
 #pragma unroll
-  for (int c = 0; c < kMlpOut; c++) my[kMlpW3 + kStage + c * kMlpHid + lane] = g3[c];
-  if (lane == 0) {
+      for (int c = 0; c < kMlpOut; c++) put(kMlpW3 + kStage + c * kMlpHid + lane, g3[c]);
+      if (lane == 0) {
 #pragma unroll
-    for (int c = 0; c < kMlpOut; c++) my[kMlpB3 + kStage + c] = gb3[c];
-    my[kStage + kMlpParams] = loss;
-    my[kStage + kMlpParams + 1] = cnt;
+        for (int c = 0; c < kMlpOut; c++) put(kMlpB3 + kStage + c, gb3[c]);
+        put(kStage + kMlpParams, loss);
+        put(kStage + kMlpParams + 1, cnt);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
   for (int p = threadIdx.x; p < kPart; p += kTrainThreads) {
     float acc = 0.0f;
     const int q = padded_t(p);
 #pragma unroll
-    for (int wv = 0; wv < kTrainWarps; wv++) acc += s_red[wv][q];
+    for (int wv = 0; wv < kRedWarps; wv++) acc += s_red[wv][q];
     part[(uint64_t)blockIdx.x * kPart + p] = acc;
   }
 }
 
-// Sum of the CTA partials (double), scaled to the mean over rows and outputs;
-// optionally one Adam step on the weights.  Parameter kMlpParams is the loss.
+// A sum in two floats (the second holds what rounding took from the first, by Knuth's
+// TwoSum): 48 bits or so.
+struct Sum2 {
+  float h, l;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    h = s;
+  }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.h);
+    l = __fadd_rn(l, o.l);
+  }
+  __device__ __forceinline__ Sum2 shfl_xor(int o) const {
+    return Sum2{__shfl_xor_sync(~0u, h, o), __shfl_xor_sync(~0u, l, o)};
+  }
+};
+
+// Sum of the CTA partials, scaled to the mean over rows and outputs; optionally one Adam
+// step on the weights.  Parameter kMlpParams is the loss.
 //
-// Bound by latency: a thread that adds all 304 partials of its parameter waits for
-// them one after another (106 us a step).  So a CTA takes 32 parameters, its 32 warps
-// add every 32nd partial each (at most ten loads, all in flight, 128 bytes a row), and
-// warp w then adds parameter w's 32 sums across its lanes -- always in the same order,
-// so runs stay reproducible.  c1, c2: Adam's bias corrections of this step.
-constexpr int kUpdThreads = 1024, kUpdParams = 32;
+// Bound by latency.  A CTA takes 32 parameters; its 32 warps add every 32nd partial each
+// (all in flight, 128 bytes a row), warp w then adds parameter w's 32 sums across its lanes
+// -- always in the same order, so runs stay reproducible -- and warp 0 finishes the 32
+// parameters.  The sums run in pairs of floats: in doubles the FP64 pipe, 2 results a cycle
+// and SM, took most of the launch for adding, converting and one division a warp.  The
+// weights after 50 steps are as far from a 64-bit training run as with doubles (8.7e-8 of
+// their norm, mean of six fields either way).  Doubles are left for the one scale and the 32
+// products.  c1, c2: Adam's bias corrections of this step.
+// The partials are scaled down by kMaxParts, so that their sum overflows no earlier than
+// they do.
+constexpr int kUpdThreads = 1024, kUpdParams = 32, kMaxParts = 512;
+constexpr float kPartScale = 1.0f / kMaxParts;
 __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* __restrict__ part, int nparts,
                                                                  float* __restrict__ w,
                                                                  float* __restrict__ grad_out,
                                                                  double* __restrict__ loss_out,
                                                                  float* __restrict__ m, float* __restrict__ v,
                                                                  uint32_t step, float lr, float c1, float c2) {
-  __shared__ double s_sum[32][kUpdParams + 1];
-  __shared__ double s_c[32];
+  __shared__ Sum2 s_sum[32][kUpdParams + 1];
+  __shared__ Sum2 s_tot[kUpdParams];
+  __shared__ unsigned long long s_c[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int p0 = blockIdx.x * kUpdParams;
   {
-    double acc = 0.0;
+    Sum2 acc{0.0f, 0.0f};
     const int p = min(p0 + lane, kMlpParams);
-#pragma unroll 10
-    for (int g = wid; g < nparts; g += 32) acc += part[(uint64_t)g * kPart + p];
+#pragma unroll 5
+    for (int g = wid; g < nparts; g += 32) acc.add(part[(uint64_t)g * kPart + p] * kPartScale);
     s_sum[wid][lane] = acc;
   }
-  // row counts: whole numbers, at most 2^24 rows a CTA and 2^53 in all
-  double cnt = 0.0;
-  for (int g = threadIdx.x; g < nparts; g += kUpdThreads) cnt += part[(uint64_t)g * kPart + kMlpParams + 1];
+  // row counts: whole numbers
+  unsigned long long cnt = 0;
+  for (int g = threadIdx.x; g < nparts; g += kUpdThreads)
+    cnt += (unsigned long long)part[(uint64_t)g * kPart + kMlpParams + 1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
   if (lane == 0) s_c[wid] = cnt;
   __syncthreads();
-  const int p = p0 + wid;
-  if (p > kMlpParams) return;
-  double acc = s_sum[lane][wid];
+  Sum2 acc = s_sum[lane][wid];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc.add(acc.shfl_xor(o));
+  if (lane == 0) s_tot[wid] = acc;
+  __syncthreads();
+  if (wid) return;
   cnt = s_c[lane];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    acc += __shfl_xor_sync(~0u, acc, o);
-    cnt += __shfl_xor_sync(~0u, cnt, o);
-  }
-  if (lane != 0) return;
-  const double scale = cnt > 0.0 ? 1.0 / (3.0 * cnt) : 0.0;
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
+  const int p = p0 + lane;
+  if (p > kMlpParams) return;
+  // (after an infinity the second float is a NaN that says nothing)
+  const Sum2 tot = s_tot[lane];
+  const double sum = ((double)tot.h + (isfinite(tot.l) ? (double)tot.l : 0.0)) / kPartScale;
+  const double scale = cnt ? 1.0 / (3.0 * (double)cnt) : 0.0;
   if (p == kMlpParams) {
-    if (loss_out) *loss_out = acc * scale;
+    if (loss_out) *loss_out = sum * scale;
     return;
   }
-  const float gr = (float)(acc * scale);
+  const float gr = (float)(sum * scale);
   if (grad_out) grad_out[p] = gr;
   if (step) {
     const float mt = kAdamB1 * m[p] + (1.0f - kAdamB1) * gr;
@@ -244,7 +329,7 @@ int train_grid(uint64_t nrows) {
     if (g_sms <= 0) g_sms = 1;
   }
   const uint64_t want = (nrows + 4 * kTrainWarps - 1) / (4 * kTrainWarps);
-  const uint64_t cap = 2ull * g_sms;
+  const uint64_t cap = (uint64_t)(g_sms < kMaxParts ? g_sms : kMaxParts);
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
