@@ -149,6 +149,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The first statement of a kernel in a chain of launches (launch_chained): waits until the
+// launch before it has completed and its writes are visible -- which that launch did in its
+// turn, so everything before it is too -- then lets the next launch's CTAs take places that
+// become free.  Does nothing in an ordinary launch.
+__device__ __forceinline__ void chained_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------------
 // memory-model helpers for the decoupled look-back
 // ---------------------------------------------------------------------------------

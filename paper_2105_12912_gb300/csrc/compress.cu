@@ -48,6 +48,7 @@ __device__ void derive_eb(DevState* st, int mode, double eb, float vmin, float v
 }
 
 __global__ void abs_params_kernel(DevState* st, double eb) {
+  chained_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) derive_eb(st, 0, eb, 0.0f, 0.0f);
 }
 
@@ -67,6 +68,7 @@ __device__ void derive_eb_d(DevState* st, int mode, double eb, double vmin, doub
 }
 
 __global__ void abs_params_d_kernel(DevState* st, double eb) {
+  chained_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) derive_eb_d(st, 0, eb, 0.0, 0.0);
 }
 
@@ -82,6 +84,7 @@ __device__ __forceinline__ double key_to_double(unsigned long long k) {
 // bound and the step.
 __global__ __launch_bounds__(256) void range_d_kernel(const double* __restrict__ x, uint64_t n, DevState* st,
                                                       int mode, double eb) {
+  chained_begin();
   __shared__ unsigned long long s_red[2][33];
   __shared__ bool s_last;
   unsigned long long lo_inv = 0, hi = 0;
@@ -248,6 +251,7 @@ __device__ __forceinline__ void range_body(const float* __restrict__ x, uint64_t
 
 __global__ __launch_bounds__(256) void range_kernel(const float* __restrict__ x, uint64_t n, DevState* st, int mode,
                                                     double eb) {
+  chained_begin();
   range_body(x, n, st, mode, eb, blockIdx.x, gridDim.x);
 }
 
@@ -587,6 +591,7 @@ __device__ void codebook_core(const BookArgs& a, int role, unsigned char* mem) {
 }
 
 __global__ __launch_bounds__(kBookThreads) void codebook_kernel(BookArgs a) {
+  chained_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   codebook_core<kBookThreads>(a, blockIdx.x, smem);
 }
@@ -1295,6 +1300,7 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsign
 }
 
 __global__ __launch_bounds__(kEncThreads, 5) void plan_kernel(EncodeArgs a) {
+  chained_begin();
   __shared__ uint32_t s_box[6];
   extern __shared__ __align__(16) unsigned char smem[];
   if (threadIdx.x == 0) block_box(a.g, blockIdx.x, s_box, s_box + 3);
@@ -1303,6 +1309,7 @@ __global__ __launch_bounds__(kEncThreads, 5) void plan_kernel(EncodeArgs a) {
 }
 
 __global__ __launch_bounds__(kEncThreads, 5) void payload_kernel(EncodeArgs a) {
+  chained_begin();
   __shared__ uint32_t s_m;
   extern __shared__ __align__(16) unsigned char smem[];
   if (threadIdx.x == 0) s_m = block_elems(a.g, blockIdx.x);
@@ -1545,15 +1552,15 @@ cudaError_t launch_codebook(const BookArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int grid = a.place_records ? 4 : 3;
   trace_begin(K_CODEBOOK, s);
-  codebook_kernel<<<grid, kBookThreads, sm, s>>>(a);
+  launch_chained(codebook_kernel, grid, kBookThreads, sm, s, a);
   trace_end(K_CODEBOOK, s);
   return cudaGetLastError();
 }
 
 cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s) {
   trace_begin(K_ENCODE, s);
-  plan_kernel<<<a.g.nblk, kEncThreads, plan_smem_bytes(), s>>>(a);
-  if (!a.analyze) payload_kernel<<<a.g.nblk, kEncThreads, payload_smem_bytes(), s>>>(a);
+  launch_chained(plan_kernel, a.g.nblk, kEncThreads, plan_smem_bytes(), s, a);
+  if (!a.analyze) launch_chained(payload_kernel, a.g.nblk, kEncThreads, payload_smem_bytes(), s, a);
   trace_end(K_ENCODE, s);
   return cudaGetLastError();
 }

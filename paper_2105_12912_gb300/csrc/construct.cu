@@ -14,6 +14,7 @@ __global__ __launch_bounds__(kThreads, sizeof(E) == 8 ? 2 : (G ? 3 : 4)) void co
                                                              const uint32_t* __restrict__ tile0, int nfields,
                                                              uint32_t ntiles, uint32_t* ticket,
                                                              uint32_t spin_limit) {
+  chained_begin();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   construct_loop<ND, E, G, false>(one, tasks, tile0, nfields, ntiles, ticket, spin_limit, smem_raw);
 }
@@ -118,7 +119,7 @@ template <int ND, typename E, bool G>
 void launch_one(const ConstructTask& one, uint32_t* ticket, cudaStream_t s) {
   using SM = SmemT<E, G ? kHaloMax : kSlots>;
   const int grid = grid_of<ND, E, G>(one.a.g.nblk);
-  construct_kernel<ND, E, G><<<grid, kThreads, sizeof(SM), s>>>(one, nullptr, nullptr, 1, one.a.g.nblk, ticket,
+  launch_chained(construct_kernel<ND, E, G>, grid, kThreads, sizeof(SM), s, one, nullptr, nullptr, 1, one.a.g.nblk, ticket,
                                                                 one.a.spin_limit);
 }
 

@@ -339,6 +339,7 @@ __device__ void dec_tables_body(const DecodeArgs& a, int book) {
 // block sizes (one chunk of 1024 blocks each), the next three build the decode tables
 // of the three books, the rest validate records and find each block's first record.
 __global__ __launch_bounds__(1024) void dec_setup_kernel(DecodeArgs a, uint32_t nchunks) {
+  chained_begin();
   if (blockIdx.x < nchunks) {
     dec_prep_chunk_body(a, nchunks);
   } else if (blockIdx.x < nchunks + 3) {
@@ -959,6 +960,7 @@ __device__ void stream_decode_body(const DecodeArgs& a, uint32_t b_begin, uint32
 
 template <int ND, typename E>
 __global__ __launch_bounds__(32 * kStreamWarps, 2) void stream_decode_kernel(DecodeArgs a) {
+  chained_begin();
   stream_decode_body<ND, E>(a, 0, 0);
 }
 
@@ -1055,6 +1057,7 @@ __device__ __forceinline__ bool expand_runs(const DecodeArgs& a, uint32_t b, int
 // set-up wrote holds exactly the header's count unless the archive is corrupt, which the
 // set-up has flagged).
 __global__ __launch_bounds__(kRecThreads) void rle_expand_kernel(DecodeArgs a) {
+  chained_begin();
   __shared__ __align__(16) RebuildSmem S;
   if (a.dead) return;
   const uint32_t b = a.runblk[blockIdx.x];
@@ -1271,6 +1274,7 @@ __device__ void reconstruct_body(const DecodeArgs& a, uint32_t b, RebuildSmem& S
 // One CTA per listed block (the set-up's list: run blocks and cut blocks).
 template <int ND, typename E>
 __global__ __launch_bounds__(kRecThreads, 6) void reconstruct_kernel(DecodeArgs a) {
+  chained_begin();
   __shared__ __align__(16) RebuildSmem S;
   if (a.dead) return;
   // the status is read once, by thread 0 (run expansions in other CTAs may flag
@@ -1305,6 +1309,7 @@ __device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, ui
 // Sums of the block's rows: totals[bx][row], row over the field's rows.
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) {
+  chained_begin();
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint32_t b = blockIdx.x;
   uint32_t org[3], w[3];
@@ -1325,6 +1330,7 @@ __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) 
 
 // Row sums to the sums before each block, in place (a thread per row).
 __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
+  chained_begin();
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint64_t nrows = (uint64_t)a.g.n[0] * a.g.n[1];
   const uint64_t row = blockIdx.x * 256ull + threadIdx.x;
@@ -1347,6 +1353,7 @@ __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
 // Partial sums along x, over the whole row, and along y, within the block, of one block.
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
+  chained_begin();
   __shared__ __align__(16) int32_t s_k[kSlots];
   __shared__ int32_t s_band[4][64];
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
@@ -1408,6 +1415,7 @@ __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
 // Strips of block height along y: the sums before each strip, from the last row of the
 // strips before it (a thread per plane and column): gstrips[(z gy + by) nx + x].
 __global__ __launch_bounds__(256) void gy_carry_kernel(DecodeArgs a) {
+  chained_begin();
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
   const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
@@ -1433,6 +1441,7 @@ __global__ __launch_bounds__(256) void gy_carry_kernel(DecodeArgs a) {
 // The last pass, in place: the strips' sums added, partial sums along z (a thread per
 // column; 2-D fields have one plane), scaled.
 __global__ __launch_bounds__(256) void gfinal_kernel(DecodeArgs a) {
+  chained_begin();
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
   const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
@@ -1497,6 +1506,7 @@ __device__ int64_t signed_lookback_warp(const uint64_t* state, uint32_t tile, ui
 // 1-D fields: the inclusive scan of the whole field in one pass, one codec block (4096
 // consecutive elements) per CTA in ticket order; blocks chain by decoupled look-back.
 __global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state) {
+  chained_begin();
   __shared__ uint32_t s_tile;
   __shared__ int s_go;
   __shared__ int32_t s_ws[8];
@@ -1547,6 +1557,7 @@ __global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state)
 
 // Verbatim patches (after the last pass).
 __global__ void gpatch_kernel(DecodeArgs a) {
+  chained_begin();
   if (a.dead || (a.st->status & ERR_CORRUPT)) return;
   const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
   const uint64_t ny = a.g.n[1], nx = a.g.n[2];
@@ -1568,17 +1579,17 @@ cudaError_t launch_global_reconstruct(const DecodeArgs& a, cudaStream_t s) {
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
   auto ctas = [](uint64_t threads) { return (unsigned)((threads + 255) / 256); };
   if (nd == 1) {
-    g1d_kernel<<<a.g.nblk, 256, 0, s>>>(a, a.scan_state);
+    launch_chained(g1d_kernel, a.g.nblk, 256, 0, s, a, a.scan_state);
   } else {
-    if (nd == 2) grow_totals_kernel<2><<<a.g.nblk, kRecThreads, 0, s>>>(a);
-    else grow_totals_kernel<3><<<a.g.nblk, kRecThreads, 0, s>>>(a);
-    gx_carry_kernel<<<ctas(nz * ny), 256, 0, s>>>(a);
-    if (nd == 2) gblock_kernel<2><<<a.g.nblk, kRecThreads, 0, s>>>(a);
-    else gblock_kernel<3><<<a.g.nblk, kRecThreads, 0, s>>>(a);
-    gy_carry_kernel<<<ctas(nz * nx), 256, 0, s>>>(a);
-    gfinal_kernel<<<ctas(ny * nx), 256, 0, s>>>(a);
+    if (nd == 2) launch_chained(grow_totals_kernel<2>, a.g.nblk, kRecThreads, 0, s, a);
+    else launch_chained(grow_totals_kernel<3>, a.g.nblk, kRecThreads, 0, s, a);
+    launch_chained(gx_carry_kernel, ctas(nz * ny), 256, 0, s, a);
+    if (nd == 2) launch_chained(gblock_kernel<2>, a.g.nblk, kRecThreads, 0, s, a);
+    else launch_chained(gblock_kernel<3>, a.g.nblk, kRecThreads, 0, s, a);
+    launch_chained(gy_carry_kernel, ctas(nz * nx), 256, 0, s, a);
+    launch_chained(gfinal_kernel, ctas(ny * nx), 256, 0, s, a);
   }
-  if (a.n_rec) gpatch_kernel<<<(unsigned)((a.n_rec + 255) / 256 < 1024 ? (a.n_rec + 255) / 256 : 1024), 256, 0, s>>>(a);
+  if (a.n_rec) launch_chained(gpatch_kernel, (unsigned)((a.n_rec + 255) / 256 < 1024 ? (a.n_rec + 255) / 256 : 1024), 256, 0, s, a);
   trace_end(K_RECONSTRUCT, s);
   return cudaGetLastError();
 }
@@ -1761,12 +1772,13 @@ cudaError_t launch_wait_selftest(int which, uint32_t spin_limit, uint64_t* lb, D
 }
 
 __global__ void dec_status_kernel(const DevState* st, uint32_t* d_status) {
+  chained_begin();
   *d_status = (uint32_t)fold(st->status);
 }
 
 cudaError_t launch_dec_status(const DevState* st, uint32_t* d_status, cudaStream_t s) {
   trace_begin(K_DEC_STATUS, s);
-  dec_status_kernel<<<1, 1, 0, s>>>(st, d_status);
+  launch_chained(dec_status_kernel, 1, 1, 0, s, st, d_status);
   trace_end(K_DEC_STATUS, s);
   return cudaGetLastError();
 }
@@ -1802,14 +1814,14 @@ cudaError_t launch_decode_stages(const DecodeArgs& a, cudaStream_t s) {
     const uint64_t cap = (uint64_t)sms * occ[nd][nluts][wi];
     const unsigned grid = (unsigned)(want < cap ? want : cap);
     trace_begin(K_STREAM_DECODE, s);
-    k<<<grid, 32 * warps, smem, s>>>(a);
+    launch_chained(k, grid, 32 * warps, smem, s, a);
     trace_end(K_STREAM_DECODE, s);
   }
   const uint32_t nrun = a.n_codec[CODEC_RLE] + a.n_codec[CODEC_RLE_HUFF];
   if (a.global) {
     if (nrun) {
       trace_begin(K_RLE_EXPAND, s);
-      rle_expand_kernel<<<nrun, kRecThreads, 0, s>>>(a);
+      launch_chained(rle_expand_kernel, nrun, kRecThreads, 0, s, a);
       trace_end(K_RLE_EXPAND, s);
     }
     return launch_global_reconstruct(a, s);
@@ -1823,7 +1835,7 @@ cudaError_t launch_decode_stages(const DecodeArgs& a, cudaStream_t s) {
   if (work) {
     auto k = nd == 1 ? reconstruct_kernel<1, E> : (nd == 2 ? reconstruct_kernel<2, E> : reconstruct_kernel<3, E>);
     trace_begin(K_RECONSTRUCT, s);
-    k<<<(unsigned)work, kRecThreads, 0, s>>>(a);
+    launch_chained(k, (unsigned)work, kRecThreads, 0, s, a);
     trace_end(K_RECONSTRUCT, s);
   }
   return cudaGetLastError();

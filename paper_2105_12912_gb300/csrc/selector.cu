@@ -93,6 +93,7 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __
                                                                  const float* __restrict__ tgt,
                                                                  const uint8_t* __restrict__ valid,
                                                                  uint64_t n, float* __restrict__ part) {
+  chained_begin();
   __shared__ float s_red[kRedWarps][kPart + kStage];
   __shared__ __align__(16) float s_act[kTrainWarps][4][kMlpHid];  // per warp: h1 and da2 of two rows
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -269,6 +270,7 @@ __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* __
                                                                  double* __restrict__ loss_out,
                                                                  float* __restrict__ m, float* __restrict__ v,
                                                                  uint32_t step, float lr, float c1, float c2) {
+  chained_begin();
   __shared__ Sum2 s_sum[32][kUpdParams + 1];
   __shared__ Sum2 s_tot[kUpdParams];
   __shared__ unsigned long long s_c[32];
@@ -360,7 +362,7 @@ T* at(void* base, uint64_t off) {
 cudaError_t launch_mlp_grad(const float* w, const float* feat, const float* tgt, const uint8_t* valid,
                             uint64_t n, float* part, int grid, cudaStream_t s) {
   trace_begin(K_MLP_GRAD, s);
-  mlp_grad_kernel<<<grid, kTrainThreads, 0, s>>>(w, feat, tgt, valid, n, part);
+  launch_chained(mlp_grad_kernel, grid, kTrainThreads, 0, s, w, feat, tgt, valid, n, part);
   trace_end(K_MLP_GRAD, s);
   return cudaGetLastError();
 }
@@ -370,7 +372,7 @@ cudaError_t launch_mlp_update(const float* part, int nparts, float* w, float* gr
   trace_begin(K_MLP_UPDATE, s);
   const float c1 = (float)(1.0 - std::pow((double)kAdamB1, (double)step));
   const float c2 = (float)(1.0 - std::pow((double)kAdamB2, (double)step));
-  mlp_update_kernel<<<(kMlpParams + kUpdParams) / kUpdParams, kUpdThreads, 0, s>>>(part, nparts, w, grad, loss, m, v,
+  launch_chained(mlp_update_kernel, (kMlpParams + kUpdParams) / kUpdParams, kUpdThreads, 0, s, part, nparts, w, grad, loss, m, v,
                                                                                   step, lr, c1, c2);
   trace_end(K_MLP_UPDATE, s);
   return cudaGetLastError();
