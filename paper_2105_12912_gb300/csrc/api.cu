@@ -316,6 +316,7 @@ csz_status run_pipeline(const void* d_field, int ndim, const uint64_t* dims, int
   ea.select = select;
   ea.codes = ca.codes;
   ea.block_runs = ca.block_runs;
+  ea.masks = ca.masks;
   ea.lens = ba.lens;
   ea.bcodes = ba.codes;
   ea.mlp_w = opt ? opt->selector_weights : nullptr;

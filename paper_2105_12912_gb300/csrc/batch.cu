@@ -78,7 +78,7 @@ FieldLayout field_layout(const Geom& g) {
   L.counts = o;
   o += a256(4ull * g.nblk);
   L.masks = o;
-  o += a256(1024ull * g.nblk);
+  o += a256(4ull * kMaskWords * g.nblk);
   L.deltas = o;
   o += a256(4ull * kSlots * g.nblk);
   L.rec_off = o;
@@ -307,6 +307,7 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
     ea.select = select;
     ea.codes = ca.codes;
     ea.block_runs = ca.block_runs;
+    ea.masks = ca.masks;
     ea.lens = ba.lens;
     ea.bcodes = ba.codes;
     ea.mlp_w = opt ? opt->selector_weights : nullptr;

@@ -26,6 +26,7 @@ constexpr int kSlots = 4096;
 constexpr int kNsymCode = 1024;
 constexpr int kNsymLen = 4096;
 constexpr int kHdr = 128;
+constexpr int kMaskWords = 3 * kSlots / 32;  // bit words of a block: patches, outliers, run starts
 constexpr uint32_t kMagic = 0x2B5A5343u;  // "CSZ+"
 constexpr uint32_t kVersion = 2;
 constexpr int kLanes = 32;  // interleave width of Huffman streams (header field)
@@ -588,16 +589,6 @@ __device__ inline void run_head_index(const uint32_t* head, uint32_t m, uint32_t
     nexthead[4 * lane + k] = cur == 0xffffffffu ? m : cur;
   }
   if (lane == 31) woff[kSlots / 32] = incl;
-}
-
-// Both of the above for a whole CTA of 256 threads; returns the number of runs.
-__device__ inline uint32_t block_run_heads(const uint16_t* c, uint32_t m, uint32_t* head, uint32_t* woff,
-                                           uint32_t* nexthead) {
-  run_head_words(c, m, head);
-  __syncthreads();
-  if (threadIdx.x < 32) run_head_index(head, m, woff, nexthead);
-  __syncthreads();
-  return woff[kSlots / 32];
 }
 
 // position of the run start after position j (a run start), using the head words

@@ -770,7 +770,7 @@ __device__ __noinline__ void place_records(const EncodeArgs& a, uint32_t b, cons
   const uint32_t tid = threadIdx.x;
   const RecordArgs& R = a.rec;
   const uint32_t lo = tid * 16;
-  const uint32_t* mw = R.masks + (uint64_t)b * 256;
+  const uint32_t* mw = R.masks + (uint64_t)b * kMaskWords;
   const uint32_t pb = (mw[lo >> 5] >> (lo & 31)) & 0xffffu;
   const uint32_t ob = (mw[128 + (lo >> 5)] >> (lo & 31)) & 0xffffu;
   uint64_t pos = R.rec_off[b] + block_excl_scan<uint64_t>((uint64_t)(__popc(ob) + __popc(pb)), s_scan64, nullptr);
@@ -808,28 +808,32 @@ __device__ __noinline__ void place_records(const EncodeArgs& a, uint32_t b, cons
   }
 }
 
-// The runs of a block's codes (s_c: 4096 codes, staged here from the code stream): their
-// values and lengths, in order.  All threads; ends with a barrier.
-__device__ __noinline__ void extract_runs(const uint16_t* codes, uint32_t m, uint16_t* s_c, uint32_t* s_head,
-                                          uint32_t* s_woff, uint32_t* s_next, uint16_t* s_rv, uint16_t* s_rl) {
-  const uint32_t tid = threadIdx.x;
-  const uint4* src = reinterpret_cast<const uint4*>(codes);
-  uint4* dst = reinterpret_cast<uint4*>(s_c);
-  for (int i = tid; i < kSlots / 8; i += kEncThreads) dst[i] = __ldcg(&src[i]);
-  __syncthreads();
-  block_run_heads(s_c, m, s_head, s_woff, s_next);
-#pragma unroll 4
-  for (int i = 0; i < kSlots / kEncThreads; i++) {
-    const uint32_t j = tid + kEncThreads * i;
-    if (j < m) {
-      const uint32_t hb = s_head[j >> 5], bit = j & 31;
-      if ((hb >> bit) & 1u) {
-        const uint32_t ri = s_woff[j >> 5] + __popc(hb & ((1u << bit) - 1u));
-        s_rv[ri] = s_c[j];
-        s_rl[ri] = (uint16_t)(next_head(s_head, s_next, j, m) - j);
-      }
+// The nr runs of a block: their values and lengths, in order, from its codes and the run
+// starts that construction left as bits.  A thread takes 16 consecutive codes; runs before
+// them are counted in the bit words, which every warp reads for itself, so one barrier
+// comes before the lengths and one after them.  s_at: scratch, the run starts.  (Finding the
+// starts again from codes in shared memory took three more barriers, with one warp's index of
+// the words between them: 40 mixed fields, most of their blocks in runs, compression 553 ->
+// 511 us.)  All threads.
+__device__ __noinline__ void extract_runs(const uint16_t* codes, const uint32_t* heads, uint32_t m, uint32_t nr,
+                                          uint16_t* s_at, uint16_t* s_rv, uint16_t* s_rl) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint4* src = reinterpret_cast<const uint4*>(codes + 16 * tid);
+  const uint4 c0 = __ldcg(&src[0]), c1 = __ldcg(&src[1]), w4 = __ldcg(&reinterpret_cast<const uint4*>(heads)[lane]);
+  const uint32_t hb = (__ldcg(&heads[tid >> 1]) >> (16 * (tid & 1))) & 0xffffu;
+  const uint32_t c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+  const uint32_t n4 = __popc(w4.x) + __popc(w4.y) + __popc(w4.z) + __popc(w4.w), n = __popc(hb);
+  uint32_t run = __reduce_add_sync(~0u, lane < 4 * wid ? n4 : 0u) + warp_incl_scan(n) - n;
+#pragma unroll
+  for (uint32_t i = 0; i < 16; i++) {
+    if ((hb >> i) & 1u) {
+      s_rv[run] = (uint16_t)(c[i >> 1] >> (16 * (i & 1)));
+      s_at[run] = (uint16_t)(16 * tid + i);
+      run++;
     }
   }
+  __syncthreads();
+  for (uint32_t i = tid; i < nr; i += kEncThreads) s_rl[i] = (uint16_t)((i + 1 < nr ? s_at[i + 1] : m) - s_at[i]);
   __syncthreads();
 }
 
@@ -943,16 +947,13 @@ __device__ __forceinline__ uint16_t* block_run_store(const EncodeArgs& a, uint32
 // The plan of codec block b of one field (all threads of the CTA).  box: its origin and
 // extent (block_box).  smem: plan_smem_bytes() of dynamic shared memory.
 __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, unsigned char* smem) {
-  uint16_t* s_c = reinterpret_cast<uint16_t*>(smem);              // 4096 codes
+  uint16_t* s_c = reinterpret_cast<uint16_t*>(smem);              // 4096 codes; before them the run starts
   uint16_t* s_rv = s_c + kSlots;                                  // run values
   uint16_t* s_rl = s_rv + kSlots;                                 // run lengths
   uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_rl + kSlots);  // 1024: the statistics' code histogram
   uint32_t* s_sw = s_hist + kNsymCode;                            // the learned selector's parameters
   uint32_t* s_tab = s_sw + (kSwWords + 3) / 4 * 4;                // the code book, packed (+4)
-  uint32_t* s_head = s_tab + kNsymCode + 4;                       // 128
-  uint32_t* s_woff = s_head + kSlots / 32;                        // 129 (+3)
-  uint32_t* s_next = s_woff + kSlots / 32 + 4;                    // 128
-  uint32_t* s_part = s_next + kSlots / 32;                        // 2 x 256
+  uint32_t* s_part = s_tab + kNsymCode + 4;                       // 2 x 256
   uint64_t* s_scan64 = reinterpret_cast<uint64_t*>(s_part + 2 * kEncThreads);  // 33
   __shared__ int s_codec;
   __shared__ float s_feat[8];
@@ -964,6 +965,7 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
   // the symbols are on their way while the block's run count and records are looked at; read
   // again where that takes more (L2 has them), rather than held
   const uint16_t* codes = a.codes + (uint64_t)b * kSlots;
+  const uint32_t* heads = a.masks + (uint64_t)b * kMaskWords + 2 * (kSlots / 32);
   const HuffPart part(codes, m);
   uint32_t sym[16];
   part.load(sym);
@@ -987,7 +989,7 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
     fresh = false;
   }
   if (runs) {
-    extract_runs(codes, m, s_c, s_head, s_woff, s_next, s_rv, s_rl);
+    extract_runs(codes, heads, m, nr, s_c, s_rv, s_rl);
     fresh = false;
   }
 
@@ -999,6 +1001,11 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
   if (statistics) {
     const bool heuristic = sel == SEL_HEURISTIC && !analyze;
     for (uint32_t i = tid; i < nr; i += kEncThreads) atomicAdd(&s_hist[s_rv[i]], (uint32_t)s_rl[i]);
+    const bool want_mado = !heuristic;
+    if (want_mado) {  // the codes, in the place of the run starts
+      const uint4* src = reinterpret_cast<const uint4*>(codes);
+      for (int i = tid; i < kSlots / 8; i += kEncThreads) reinterpret_cast<uint4*>(s_c)[i] = __ldcg(&src[i]);
+    }
     __syncthreads();
     // block statistics in one pass and one reduction: entropy sum, |delta| sum, top
     // count and largest in-range |delta|, and (selector) the madogram's code changes
@@ -1017,7 +1024,6 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
         }
       }
     }
-    const bool want_mado = !heuristic;
     if (want_mado) {
       // kEncThreads is a multiple of kMadoN, so a thread's distance is fixed
       const uint32_t d = kMadoD0 + kMadoStep * (tid % kMadoN);
@@ -1157,7 +1163,7 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
   if (codec < 0) codec = exhaustive_pick(size_h, size_r, size_rh);  // (the same in every thread)
   const uint32_t size = codec == CODEC_HUFF ? size_h : (codec == CODEC_RLE ? size_r : size_rh);
   if (codec != CODEC_HUFF) {
-    if (!runs) extract_runs(codes, m, s_c, s_head, s_woff, s_next, s_rv, s_rl);
+    if (!runs) extract_runs(codes, heads, m, nr, s_c, s_rv, s_rl);
     uint16_t* rv = block_run_store(a, b);
     for (uint32_t i = tid; i < nr; i += kEncThreads) {
       rv[i] = s_rv[i];
@@ -1357,7 +1363,7 @@ __global__ __launch_bounds__(kEncThreads, 5) void payload_batch_kernel(const Enc
 }
 
 static size_t plan_smem_bytes() {
-  return kSlots * 2 * 3 + 4 * (kNsymCode + (kSwWords + 3) / 4 * 4 + kNsymCode + 4 + (kSlots / 32) * 3 + 4 + 2 * kEncThreads) +
+  return kSlots * 2 * 3 + 4 * (kNsymCode + (kSwWords + 3) / 4 * 4 + kNsymCode + 4 + 2 * kEncThreads) +
          33 * 8 + 16;
 }
 static size_t payload_smem_bytes() { return kBufBytes + 4 * (2 * kEncThreads + 8); }

@@ -192,7 +192,7 @@ struct SmemT {
   uint32_t hc[kNsymCode];       // code histogram (per CTA, current field)
   uint32_t hv[kNsymCode];       // run-value histogram
   uint32_t hl[kHlShared];       // run-length histogram (length - 1), short runs
-  uint32_t patch[kSlots / 32];  // verbatim-patch positions
+  uint32_t patch[kSlots / 32];  // verbatim-patch positions (these three are copied out together)
   uint32_t outl[kSlots / 32];   // outlier positions
   uint32_t head[kSlots / 32];   // run heads
   uint32_t woff[kSlots / 32 + 4];
@@ -393,15 +393,15 @@ __device__ void tile_tail(const ConstructArgs& A, uint32_t b, SmemT<E, NIN>& S, 
     A.block_runs[b] = (uint16_t)nruns;
     n_rec_acc += n_out + n_patch;
     n_patch_acc += n_patch;
-    // codes to the block-major stream (whole 4096-slot block, zero tail) and the
-    // patch / outlier bit words: bulk copies from shared memory, waited for before
+    // codes to the block-major stream (whole 4096-slot block, zero tail) and the patch,
+    // outlier and run-start bit words: bulk copies from shared memory, waited for before
     // those buffers are written again
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(A.codes + (uint64_t)b * kSlots),
                  "r"(smem_u32(S.c)), "r"((uint32_t)(kSlots * 2))
                  : "memory");
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(A.masks + (uint64_t)b * 256),
-                 "r"(smem_u32(S.patch)), "r"((uint32_t)(2 * (kSlots / 32) * 4))
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(A.masks + (uint64_t)b * kMaskWords),
+                 "r"(smem_u32(S.patch)), "r"((uint32_t)(kMaskWords * 4))
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }

@@ -93,7 +93,7 @@ inline Layout layout(const Geom& g) {
   L.counts = o;
   o += a256(4ull * g.nblk);
   L.masks = o;
-  o += a256(1024ull * g.nblk);
+  o += a256(4ull * kMaskWords * g.nblk);
   L.deltas = o;
   o += a256(4ull * kSlots * g.nblk);
   L.rec_off = o;

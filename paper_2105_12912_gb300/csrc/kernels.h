@@ -42,7 +42,7 @@ struct ConstructArgs {
   uint32_t* hist_val;  // [1024]
   uint32_t* hist_len;  // [4096]
   uint32_t* counts;    // [nblk] (outliers << 16) | patches of each block
-  uint32_t* masks;     // [nblk][256] patch bit words [128], then outlier bit words [128]
+  uint32_t* masks;     // [nblk][kMaskWords] patch, outlier and run-start bit words, 128 each
   int32_t* deltas;     // [nblk * 4096] outlier residuals by slot (written at outliers only)
   uint16_t* block_runs;  // [nblk] runs of equal codes in each block
   uint32_t spin_limit;
@@ -65,7 +65,7 @@ struct RangeTask {
 struct RecordArgs {
   const float* x;
   const uint32_t* counts;  // [nblk] (outliers << 16) | patches
-  const uint32_t* masks;   // [nblk][256] patch words, then outlier words
+  const uint32_t* masks;   // [nblk][kMaskWords] patch, outlier and run-start words
   const int32_t* deltas;   // [nblk * 4096] outlier residuals by slot
   uint64_t* rec_off;       // [nblk] exclusive prefix of record counts
   uint32_t* rec;           // archive record section (u32 key, u32 val pairs)
@@ -124,6 +124,7 @@ struct EncodeArgs {
   int select;
   const uint16_t* codes;
   const uint16_t* block_runs;  // [nblk] runs per block (from construction)
+  const uint32_t* masks;       // [nblk][kMaskWords] bit words (from construction): the run starts
   const uint8_t* lens;
   const uint64_t* bcodes;
   const float* mlp_w;
