@@ -229,6 +229,13 @@ __device__ __forceinline__ void tma_load(int rank, void* dst, const CUtensorMap*
   }
 }
 
+template <typename E>
+__device__ __forceinline__ const E* field_ptr(const ConstructArgs& A);
+template <>
+__device__ __forceinline__ const float* field_ptr<float>(const ConstructArgs& A) { return A.x; }
+template <>
+__device__ __forceinline__ const double* field_ptr<double>(const ConstructArgs& A) { return A.x64; }
+
 // Start fetching tile b of task T into buffer `buf` (thread 0 only).  The buffer was
 // last touched by ordinary loads and stores, hence the proxy fence.
 template <typename E>
@@ -236,8 +243,12 @@ __device__ void issue_tile(const ConstructTask* T, const uint32_t* org, E* buf, 
   const Geom& g = T->a.g;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   mbar_expect_tx(bar, (uint32_t)(kSlots * sizeof(E)));
-  if (g.ndim == 1) {
-    // a 1-D box holds at most 256 elements: 16 copies
+  if (g.ndim == 1 && org[2] + (uint64_t)kSlots <= g.nelem) {
+    // a whole 1-D tile is one stretch of memory: one copy (a tensor copy's box holds at most
+    // 256 elements, and issuing 16 of them was most of thread 0's work on a tile: 40 mixed fields, compression 511 -> 500 us)
+    bulk_load(buf, field_ptr<E>(T->a) + org[2], (uint32_t)(kSlots * sizeof(E)), bar);
+  } else if (g.ndim == 1) {
+    // the last tile, zero-filled behind the field: 16 boxes
     for (int i = 0; i < kSlots / 256; i++)
       tma_load(1, buf + 256 * i, &T->tmap, (int32_t)(org[2] + 256 * i), 0, 0, bar);
   } else if (g.ndim == 2) {
@@ -246,13 +257,6 @@ __device__ void issue_tile(const ConstructTask* T, const uint32_t* org, E* buf, 
     tma_load(3, buf, &T->tmap, (int32_t)org[2], (int32_t)org[1], (int32_t)org[0], bar);
   }
 }
-
-template <typename E>
-__device__ __forceinline__ const E* field_ptr(const ConstructArgs& A);
-template <>
-__device__ __forceinline__ const float* field_ptr<float>(const ConstructArgs& A) { return A.x; }
-template <>
-__device__ __forceinline__ const double* field_ptr<double>(const ConstructArgs& A) { return A.x64; }
 
 // Thread-loaded tile (fields TMA cannot describe): box layout (3-D boxes swizzled like
 // their TMA copies), zeros outside.
@@ -726,7 +730,12 @@ __device__ void issue_tile_global(const ConstructTask* T, const uint32_t* org, E
   const Geom& g = T->a.g;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   const int32_t x0 = (int32_t)org[2] - (int32_t)kHaloPadX;
-  if (g.ndim == 1) {
+  if (g.ndim == 1 && org[2] && org[2] + (uint64_t)kSlots <= g.nelem) {
+    // a whole tile and the elements before it: one stretch of memory, as in issue_tile
+    constexpr uint32_t bytes = (kSlots + kHaloPadX) * (uint32_t)sizeof(E);
+    mbar_expect_tx(bar, bytes);
+    bulk_load(buf, field_ptr<E>(T->a) + (org[2] - kHaloPadX), bytes, bar);
+  } else if (g.ndim == 1) {
     mbar_expect_tx(bar, (uint32_t)(Halo<1>::X * sizeof(E)));
     for (int i = 0; i < 17; i++) tma_load(1, buf + 256 * i, &T->tmap, x0 + 256 * i, 0, 0, bar);
   } else if (g.ndim == 2) {
