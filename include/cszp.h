@@ -129,6 +129,22 @@ csz_status csz_decompress(const uint8_t* d_archive, size_t bytes, float* d_out,
                           void* stream);
 
 /*
+ * For callers that allocate the output themselves: csz_archive_head copies the archive's
+ * 128-byte header to h_header (host memory; synchronises `stream`) and gives its shape and
+ * bytes per element (4: FP32, 8: double); csz_decompress_with_header then decompresses
+ * with that copy, so the header crosses to the host once, where csz_archive_info followed
+ * by csz_decompress reads it twice.  The device compares the archive's own header with the
+ * copy (a mismatch is CSZ_E_CORRUPT).  f64: d_out holds doubles; an archive of the other
+ * type is CSZ_E_ARG.  Otherwise arguments, workspace, ownership, errors and the one
+ * synchronisation are csz_decompress's.
+ */
+csz_status csz_archive_head(const uint8_t* d_archive, size_t bytes, uint8_t* h_header, int* ndim,
+                            uint64_t* dims, int* elem_bytes, void* stream);
+csz_status csz_decompress_with_header(const uint8_t* d_archive, size_t bytes, const uint8_t* h_header,
+                                      int f64, void* d_out, uint64_t out_cap_elems, void* d_workspace,
+                                      size_t workspace_bytes, void* stream);
+
+/*
  * csz_decompress without any host synchronisation.  The caller passes the archive's
  * 128-byte header as a host copy (h_header: e.g. from csz_compress_with_header, or
  * read once and kept), so nothing is read back before the launches; the device

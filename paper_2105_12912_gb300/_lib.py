@@ -57,6 +57,10 @@ SIGNATURES = {
                                    C.POINTER(C.c_size_t), C.c_void_p]),
     "csz_decompress_f64": (C.c_int, [C.c_void_p, C.c_size_t, C.c_void_p, C.c_uint64, C.c_void_p, C.c_size_t,
                                      C.c_void_p]),
+    "csz_archive_head": (C.c_int, [C.c_void_p, C.c_size_t, C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_uint64),
+                                   C.POINTER(C.c_int), C.c_void_p]),
+    "csz_decompress_with_header": (C.c_int, [C.c_void_p, C.c_size_t, C.c_void_p, C.c_int, C.c_void_p, C.c_uint64,
+                                             C.c_void_p, C.c_size_t, C.c_void_p]),
     "csz_archive_elem_bytes": (C.c_int, [C.c_void_p, C.c_size_t]),
     "csz_wait_selftest": (C.c_int, [C.c_int, C.c_uint32, C.c_void_p, C.c_size_t, C.c_void_p]),
     "csz_decompress_static": (C.c_int, [C.c_void_p, C.c_size_t, C.c_void_p, C.c_uint64, C.c_void_p]),

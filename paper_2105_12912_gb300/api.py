@@ -145,19 +145,33 @@ def decompress(archive: torch.Tensor, nbytes: int | None = None, out: torch.Tens
         raise ValueError("archive must be a uint8 CUDA tensor")
     if nbytes is None:
         nbytes = archive.numel()
+    head = None
     if dims is None or out is None:
-        head = bytes(archive[:128].cpu().numpy().tobytes())
+        # the header crosses to the host once: its copy gives the shape here and drives the
+        # decompression (which compares it with the archive's own on the device)
+        head = (C.c_uint8 * 128)()
+        nd, esz = C.c_int(), C.c_int()
+        shape = (C.c_uint64 * 3)()
+        st = L.lib().csz_archive_head(C.c_void_p(archive.data_ptr()), archive.numel(), head, C.byref(nd), shape,
+                                      C.byref(esz), _stream_ptr(None))
         if dims is None:
-            dims, _, _ = archive_info(head)
+            _check(st, "csz_archive_info")
+            dims = tuple(shape[:nd.value])
+        if st != L.OK:
+            head = None  # (csz_decompress says what is wrong with it)
         if out is None:
-            esz = elem_bytes(head)
-            out = torch.empty(tuple(dims), dtype=torch.float64 if esz == 8 else torch.float32,
+            out = torch.empty(tuple(dims), dtype=torch.float64 if esz.value == 8 else torch.float32,
                               device=archive.device)
     ws = _ws(archive.device, workspace).get(workspace_bytes(dims) or 256)
     f64 = out.dtype == torch.float64
-    fn = L.lib().csz_decompress_f64 if f64 else L.lib().csz_decompress
-    st = fn(C.c_void_p(archive.data_ptr()), int(nbytes), C.c_void_p(out.data_ptr()), out.numel(),
-            C.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream))
+    if head is not None:
+        st = L.lib().csz_decompress_with_header(C.c_void_p(archive.data_ptr()), int(nbytes), head, int(f64),
+                                                C.c_void_p(out.data_ptr()), out.numel(), C.c_void_p(ws.data_ptr()),
+                                                ws.numel(), _stream_ptr(stream))
+    else:
+        fn = L.lib().csz_decompress_f64 if f64 else L.lib().csz_decompress
+        st = fn(C.c_void_p(archive.data_ptr()), int(nbytes), C.c_void_p(out.data_ptr()), out.numel(),
+                C.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream))
     if raise_on_error:
         _check(st, "csz_decompress_f64" if f64 else "csz_decompress")
     return out, st

@@ -1,6 +1,7 @@
 // Host side of the cszp C ABI: argument and archive-header validation, workspace
 // layout, kernel sequencing on the caller's stream, one synchronisation per call.
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 
 #include "cszp.h"
@@ -352,16 +353,24 @@ csz_status run_pipeline(const void* d_field, int ndim, const uint64_t* dims, int
   fa.off_bb = off_bb;
   fa.off_rec = off_rec;
   fa.lens = ba.lens;
+  fa.hdr_copy = h_header ? at<uint32_t>(d_ws, L.hdr) : nullptr;
   if (launch_encode(ea, s) != cudaSuccess) return CSZ_E_CUDA;
 
-  DevState hs;
-  if (cudaMemcpyAsync(&hs, st, sizeof(hs), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
-  if (h_header && cudaMemcpyAsync(h_header, d_ar, kHdr, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  // the state and, where it is asked for, the header behind it: one copy
+  struct {
+    alignas(256) DevState st;
+    alignas(256) uint8_t hdr[kHdr];
+  } back;
+  static_assert(offsetof(decltype(back), hdr) == (sizeof(DevState) + 255) / 256 * 256, "as in the workspace");
+  const DevState& hs = back.st;
+  if (cudaMemcpyAsync(&back, st, h_header ? offsetof(decltype(back), hdr) + kHdr : sizeof(hs), cudaMemcpyDeviceToHost,
+                      s) != cudaSuccess)
     return CSZ_E_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
   trace_collect();
   const csz_status r = fold(hs.status);
   if (r != CSZ_OK) return r;
+  if (h_header) memcpy(h_header, back.hdr, kHdr);
   if (h_bytes) *h_bytes = an ? 0 : (size_t)hs.total;
   return CSZ_OK;
 }
@@ -438,6 +447,35 @@ csz_status enqueue_decode(const uint8_t* d_ar, size_t bytes, const uint8_t* h, b
   return CSZ_OK;
 }
 
+// A decompression with its one last synchronisation; h as in enqueue_decode.
+csz_status decode_and_wait(const uint8_t* d_ar, size_t bytes, const uint8_t* h, bool check_hdr, void* d_out,
+                           uint64_t out_cap, void* d_ws, size_t ws_bytes, cudaStream_t s, bool f64) {
+  DevState* st = nullptr;
+  const csz_status r = enqueue_decode(d_ar, bytes, h, check_hdr, d_out, out_cap, d_ws, ws_bytes, s, &st, f64);
+  if (r != CSZ_OK) return r;
+  DevState hs;
+  if (cudaMemcpyAsync(&hs, st, sizeof(hs), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
+  trace_collect();
+  return fold(hs.status);
+}
+
+csz_status read_header(const uint8_t* d_ar, uint8_t* h, cudaStream_t s) {
+  if (cudaMemcpyAsync(h, d_ar, kHdr, cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
+  return cudaStreamSynchronize(s) == cudaSuccess ? CSZ_OK : CSZ_E_CUDA;
+}
+
+csz_status decompress_any(const uint8_t* d_ar, size_t bytes, void* d_out, uint64_t out_cap, void* d_ws,
+                          size_t ws_bytes, void* stream, bool f64) {
+  if (!d_ar || !d_out || !d_ws) return CSZ_E_ARG;
+  if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  uint8_t h[kHdr];
+  const csz_status r = read_header(d_ar, h, s);
+  if (r != CSZ_OK) return r;
+  return decode_and_wait(d_ar, bytes, h, false, d_out, out_cap, d_ws, ws_bytes, s, f64);
+}
+
 }  // namespace
 
 extern "C" {
@@ -477,20 +515,26 @@ csz_status csz_archive_info(const uint8_t* h, size_t bytes, int* ndim, uint64_t*
 
 csz_status csz_decompress(const uint8_t* d_ar, size_t bytes, float* d_out, uint64_t out_cap, void* d_ws,
                           size_t ws_bytes, void* stream) {
-  if (!d_ar || !d_out || !d_ws) return CSZ_E_ARG;
+  return decompress_any(d_ar, bytes, d_out, out_cap, d_ws, ws_bytes, stream, false);
+}
+
+csz_status csz_archive_head(const uint8_t* d_ar, size_t bytes, uint8_t* h_header, int* ndim, uint64_t* dims,
+                            int* elem_bytes, void* stream) {
+  if (!d_ar || !h_header) return CSZ_E_ARG;
   if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  uint8_t h[kHdr];
-  if (cudaMemcpyAsync(h, d_ar, kHdr, cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
-  DevState* st = nullptr;
-  const csz_status r = enqueue_decode(d_ar, bytes, h, false, d_out, out_cap, d_ws, ws_bytes, s, &st);
+  csz_status r = read_header(d_ar, h_header, static_cast<cudaStream_t>(stream));
   if (r != CSZ_OK) return r;
-  DevState hs;
-  if (cudaMemcpyAsync(&hs, st, sizeof(hs), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
-  trace_collect();
-  return fold(hs.status);
+  r = csz_archive_info(h_header, kHdr, ndim, dims, nullptr, nullptr);
+  if (r == CSZ_OK && elem_bytes) *elem_bytes = csz_archive_elem_bytes(h_header, kHdr);
+  return r;
+}
+
+csz_status csz_decompress_with_header(const uint8_t* d_ar, size_t bytes, const uint8_t* h_header, int f64, void* d_out,
+                                      uint64_t out_cap, void* d_ws, size_t ws_bytes, void* stream) {
+  if (!d_ar || !h_header || !d_out || !d_ws) return CSZ_E_ARG;
+  if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;
+  return decode_and_wait(d_ar, bytes, h_header, true, d_out, out_cap, d_ws, ws_bytes,
+                         static_cast<cudaStream_t>(stream), f64 != 0);
 }
 
 csz_status csz_compress_f64(const double* d_field, int ndim, const uint64_t* dims, int eb_mode, double eb,
@@ -502,20 +546,7 @@ csz_status csz_compress_f64(const double* d_field, int ndim, const uint64_t* dim
 
 csz_status csz_decompress_f64(const uint8_t* d_ar, size_t bytes, double* d_out, uint64_t out_cap, void* d_ws,
                               size_t ws_bytes, void* stream) {
-  if (!d_ar || !d_out || !d_ws) return CSZ_E_ARG;
-  if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  uint8_t h[kHdr];
-  if (cudaMemcpyAsync(h, d_ar, kHdr, cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
-  DevState* st = nullptr;
-  const csz_status r = enqueue_decode(d_ar, bytes, h, false, d_out, out_cap, d_ws, ws_bytes, s, &st, true);
-  if (r != CSZ_OK) return r;
-  DevState hs;
-  if (cudaMemcpyAsync(&hs, st, sizeof(hs), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CSZ_E_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CSZ_E_CUDA;
-  trace_collect();
-  return fold(hs.status);
+  return decompress_any(d_ar, bytes, d_out, out_cap, d_ws, ws_bytes, stream, true);
 }
 
 int csz_archive_elem_bytes(const uint8_t* h, size_t bytes) {

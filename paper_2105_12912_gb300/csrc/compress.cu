@@ -660,7 +660,10 @@ __device__ void finalize_body(const FinalizeArgs& a) {
   __syncthreads();
   if (s_total > a.cap) return;
   uint8_t* ar = a.ar;
-  for (int i = tid; i < kHdr / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(ar)[i] = s_hdr[i];
+  for (int i = tid; i < kHdr / 4; i += blockDim.x) {
+    reinterpret_cast<uint32_t*>(ar)[i] = s_hdr[i];
+    if (a.hdr_copy) a.hdr_copy[i] = s_hdr[i];
+  }
   // zero padding: codec section, blk_bytes section, payload tail
   for (uint64_t i = kHdr + a.nblk + tid; i < a.off_bb; i += blockDim.x) ar[i] = 0;
   for (uint64_t i = a.off_bb + 4ull * a.nblk + tid; i < a.off_rec; i += blockDim.x) ar[i] = 0;

@@ -39,15 +39,15 @@ inline bool make_geom(int ndim, const uint64_t* dims, Geom& g) {
   return true;
 }
 
-// Workspace: [DevState | set-up look-back states | histograms | group totals] (zeroed per
-// compression; decompression zeroes the first two),
+// Workspace: [DevState | header | set-up look-back states | histograms | group totals] (zeroed per
+// compression; decompression zeroes what precedes the histograms),
 // books, decode tables and offsets, block-major code stream, decoded run lengths,
 // the lists of run blocks and of blocks reconstructed apart from their decoding
 // (the part decompression needs ends at dec_total), then compression-only scratch:
 // per-block record counts, patch / outlier bit masks, outlier residuals and record
 // offsets.
 struct Layout {
-  uint64_t st, prep_lb, hist_code, hist_val, hist_len, lb_e, zero_end;
+  uint64_t st, hdr, prep_lb, hist_code, hist_val, hist_len, lb_e, zero_end;
   uint64_t lens, bcodes, blk_off, rec_start, tabs, codes, runl, runblk, slowblk, dec_total;
   uint64_t counts, masks, deltas, rec_off, runs, total;
 };
@@ -57,6 +57,8 @@ inline Layout layout(const Geom& g) {
   uint64_t o = 0;
   L.st = o;
   o += a256(sizeof(DevState));
+  L.hdr = o;  // compression: the archive's header, to be read back with the state
+  o += 256;
   L.prep_lb = o;  // decompression set-up: two look-back states per 1024 blocks
   o += a256(16ull * ((g.nblk + 1023) / 1024));
   L.hist_code = o;

@@ -115,6 +115,7 @@ struct FinalizeArgs {
   int select;
   uint64_t nblk, off_bb, off_rec;
   const uint8_t* lens;
+  uint32_t* hdr_copy;  // a second copy of the header (or null)
 };
 
 struct EncodeArgs {
