@@ -250,7 +250,7 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
     tile0[f] = tiles;
     tiles += g.nblk;
     cta0[f] = ctas;
-    ctas += d.eb_mode == CSZ_EB_REL ? range_ctas(g.nelem) : 1u;
+    ctas += d.eb_mode == CSZ_EB_REL ? range_ctas_batch(g.nelem) : 1u;
 
     RangeTask& R = rt[f];
     R.x = d.d_field;

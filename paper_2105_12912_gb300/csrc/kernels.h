@@ -239,7 +239,8 @@ cudaError_t launch_construct_batch(const ConstructTask* d_tasks, const uint32_t*
 cudaError_t launch_codebook(const BookArgs& a, cudaStream_t s);
 cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s);
 // batches: per-field tables in device memory
-uint32_t range_ctas(uint64_t n);  // CTAs the range pass gives a REL field of n elements
+uint32_t range_ctas(uint64_t n);        // CTAs the range pass gives a REL field of n elements
+uint32_t range_ctas_batch(uint64_t n);  // and in a batch
 cudaError_t launch_range_batch(const RangeTask* d_tasks, const uint32_t* d_cta0, int nfields, uint32_t nctas,
                                cudaStream_t s);
 cudaError_t launch_codebook_batch(const BookArgs* d_tasks, int nfields, cudaStream_t s);
