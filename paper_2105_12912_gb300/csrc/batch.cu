@@ -529,7 +529,7 @@ csz_status csz_batch_plan(const csz_batch* b, int* persistent, int* grid, double
 }  // extern "C"
 
 // Stream-decode CTA shapes the batch's tuner chooses among (warps per CTA; a CTA
-// decodes kDecChunkRounds * warps / 2 codec blocks).  None changes the output.
+// decodes up to kDecChunkRounds * warps / 2 codec blocks).  None changes the output.
 constexpr int kDecShapes[3] = {8, 16, 32};
 
 struct csz_batch_dec {
@@ -668,6 +668,14 @@ csz_status csz_batch_dec_create(int nfields, const csz_dfield* fields, void* d_w
   uint32_t nsetup = 0, ntiles = 0, nchunks_v[3] = {0, 0, 0};
   // fields that share their dimensionality decode with the fused reconstruction
   int common_nd = gs[0].ndim;
+  uint64_t blocks = 0;
+  for (const Geom& g : gs) blocks += g.nblk;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  uint32_t rounds = kDecChunkRounds;
+  while (rounds > 1 && blocks / (rounds * (uint32_t)kDecShapes[1] / 2) < (uint64_t)kDecChunkWaves * (uint32_t)(sms > 0 ? sms : 1))
+    rounds /= 2;
   for (int f = 1; f < nfields; f++)
     if (gs[f].ndim != common_nd) common_nd = 0;
   for (int f = 0; f < nfields; f++) {
@@ -696,7 +704,7 @@ csz_status csz_batch_dec_create(int nfields, const csz_dfield* fields, void* d_w
     if (rec_ctas > 256) rec_ctas = 256;
     nsetup += prep_chunks(g) + 3 + (uint32_t)rec_ctas;
     for (int v = 0; v < 3; v++) {
-      const uint32_t per = kDecChunkRounds * ((uint32_t)kDecShapes[v] / 2);
+      const uint32_t per = rounds * ((uint32_t)kDecShapes[v] / 2);
       chunk0s[v][f] = nchunks_v[v];
       nchunks_v[v] += (g.nblk + per - 1) / per;
     }
@@ -720,7 +728,7 @@ csz_status csz_batch_dec_create(int nfields, const csz_dfield* fields, void* d_w
     return CSZ_E_CUDA;
   }
   b->launch = DecodeBatchLaunch{b->d_tasks, nfields, at<uint32_t>(ws, B.setup0), nsetup, b->chunk0[1],
-                                b->nchunks[1], at<uint32_t>(ws, B.tile0), ntiles, common_nd, kDecShapes[1]};
+                                b->nchunks[1], at<uint32_t>(ws, B.tile0), ntiles, common_nd, kDecShapes[1], rounds};
   if (dec_capture(b) != cudaSuccess) {
     delete b;
     return CSZ_E_CUDA;

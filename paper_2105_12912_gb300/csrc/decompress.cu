@@ -1691,10 +1691,11 @@ __global__ __launch_bounds__(1024) void dec_setup_batch_kernel(const DecodeArgs*
 // warps, as for single fields
 template <int ND>
 __global__ __launch_bounds__(1024) void stream_decode_batch_kernel(const DecodeArgs* __restrict__ tasks,
-                                                                   const uint32_t* __restrict__ chunk0, int nfields) {
+                                                                   const uint32_t* __restrict__ chunk0, int nfields,
+                                                                   uint32_t rounds) {
   const int f = field_of(chunk0, nfields, blockIdx.x);
   const DecodeArgs& a = tasks[f];
-  const uint32_t per = kDecChunkRounds * (blockDim.x / 64);  // blocks per CTA: two streams each
+  const uint32_t per = rounds * (blockDim.x / 64);  // blocks per CTA: two streams each
   const uint32_t b0 = (blockIdx.x - chunk0[f]) * per;
   const uint32_t b1 = min(a.g.nblk, b0 + per);
   stream_decode_body<ND, float>(a, b0, b1);
@@ -1738,7 +1739,7 @@ cudaError_t launch_decode_batch(const DecodeBatchLaunch& L, cudaStream_t s) {
   e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   trace_begin(K_STREAM_DECODE, s);
-  k<<<L.nchunks, 32 * warps, smem, s>>>(L.tasks, L.chunk0, L.nfields);
+  k<<<L.nchunks, 32 * warps, smem, s>>>(L.tasks, L.chunk0, L.nfields, L.rounds);
   trace_end(K_STREAM_DECODE, s);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // (run blocks are expanded inside the reconstruction)

@@ -290,12 +290,15 @@ struct DecodeBatchLaunch {
   uint32_t ntiles;
   int nd;                  // the fields' common dimensionality (fused decoding), 0 if mixed
   int warps;               // stream-decode warps per CTA (8, 16 or 32; 0 = 16)
+  uint32_t rounds;         // blocks per stream-decode CTA: rounds * warps / 2
 };
 constexpr int kStreamWarpsPerCta = 16;
-// batched decoding: a decoding CTA of w warps takes kDecChunkRounds * w / 2 codec
-// blocks (its decode tables staged once for them), its warps drawing the blocks'
-// streams one at a time
-constexpr uint32_t kDecChunkRounds = 4;
+// batched decoding: a decoding CTA of w warps takes rounds * w / 2 codec blocks, so that it
+// copies the lookup tables once for several streams a warp.  A Huffman stream takes ten times
+// as long as one of a run block's, so with few CTAs in all the last Huffman chunk sets the
+// time: rounds halve until the batch has kDecChunkWaves CTAs an SM (40 mixed fields, 12,664
+// blocks: 396 CTAs of 16 warps -> 1,594, a call 240 -> 206 us).
+constexpr uint32_t kDecChunkRounds = 4, kDecChunkWaves = 8;
 cudaError_t launch_decode_batch(const DecodeBatchLaunch& L, cudaStream_t s);
 
 }  // namespace cszp
