@@ -1306,7 +1306,9 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsign
   if (b == 0) finish_field(a);
 }
 
-__global__ __launch_bounds__(kEncThreads, 5) void plan_kernel(EncodeArgs a) {
+// (four CTAs an SM: with the registers of five the plan spills, 3-D 512^3 compression 818
+// against 805 us, 40 mixed fields 486 against 474; the payload's place is better at five)
+__global__ __launch_bounds__(kEncThreads, 4) void plan_kernel(EncodeArgs a) {
   chained_begin();
   __shared__ uint32_t s_box[6];
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1335,7 +1337,7 @@ __device__ __forceinline__ int field_of_prefix(const uint32_t* prefix, int nfiel
 }
 
 // Batch: one CTA per codec block of every field (tile0[f] = first block of field f).
-__global__ __launch_bounds__(kEncThreads, 5) void plan_batch_kernel(const EncodeArgs* __restrict__ tasks,
+__global__ __launch_bounds__(kEncThreads, 4) void plan_batch_kernel(const EncodeArgs* __restrict__ tasks,
                                                                  const uint32_t* __restrict__ tile0, int nfields) {
   __shared__ uint32_t s_box[6];
   __shared__ int s_field;
