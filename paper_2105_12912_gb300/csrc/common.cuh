@@ -180,7 +180,8 @@ __device__ __forceinline__ void lookback_publish(uint64_t* state, uint32_t tile,
   st_relaxed(&state[tile], (tile == 0 ? LB_INC : LB_AGG) | agg);
 }
 
-// Decoupled look-back (single-pass prefix scan over tiles taken in ticket order):
+// Decoupled look-back (single-pass prefix scan over tiles taken in ticket order, as by the
+// chunks of the decode set-up):
 // called by one full warp after lookback_publish; returns the exclusive prefix and
 // publishes the inclusive one.  The wait is bounded; on expiry the status gets
 // ERR_TIMEOUT and the tile publishes what it has so successors finish too.

@@ -15,7 +15,7 @@
 // tiles of one field and added to the field's global histograms when the CTA moves
 // to another field or finishes.  Records are not placed here: each tile leaves its
 // outlier / patch counts, bit words and outlier residuals; the codebook launch scans
-// the counts and the encode CTAs write the records in slot order.
+// the counts and the plan CTAs write the records in slot order.
 //
 // This header holds the device code: construct.cu instantiates it as the
 // construction kernels, compress.cu as one phase of the batched persistent kernel.

@@ -1750,7 +1750,7 @@ cudaError_t launch_decode_batch(const DecodeBatchLaunch& L, cudaStream_t s) {
 }
 
 // One bounded wait that nothing satisfies (a test aid for the failure path): which 0,
-// the payload look-back of tile 1 behind a tile 0 that never publishes; which 1, an
+// the look-back of tile 1 behind a tile 0 that never publishes; which 1, an
 // mbarrier phase no copy or arrival completes.  Either gives up after `spin_limit`
 // tries and leaves ERR_TIMEOUT in the status, and the kernel returns normally.
 __global__ void wait_selftest_kernel(int which, uint32_t spin_limit, uint64_t* lb, DevState* st) {

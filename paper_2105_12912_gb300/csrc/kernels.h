@@ -60,7 +60,7 @@ struct RangeTask {
 };
 
 // Record placement: the exclusive prefix of the blocks' record counts (one CTA of
-// the codebook launch), then each encode CTA writes its block's outlier and patch
+// the codebook launch), then each plan CTA writes its block's outlier and patch
 // records in slot order at that offset.
 struct RecordArgs {
   const float* x;
