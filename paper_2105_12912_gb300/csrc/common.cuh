@@ -703,7 +703,8 @@ __host__ __device__ __forceinline__ uint32_t huff_split(uint32_t m) {
 // Block-wide encoder of a pair of interleaved streams (256 threads): a Huffman block's
 // streams A and B, or the value and the length stream of an RLE+Huffman block.  Warp w
 // takes quarter w & 3 of stream w >> 2, thread (lane l) lane l's symbols of the quarter's
-// up to 16 steps, whose packed codes it keeps in registers from the sizes to the payload.
+// steps, whose packed codes it keeps in registers from the sizes to the payload (16 steps: a
+// whole Huffman block, or 2048 runs; more runs, in forced modes, are read a second time).
 //
 // Bound by instruction issue and barriers (3-D 512^3, rel 1e-4: 109 instructions per 32
 // symbols and 533 us in the encoder this replaced, which looked lengths and codes up apart
@@ -716,11 +717,11 @@ __host__ __device__ __forceinline__ uint32_t huff_split(uint32_t m) {
 // shared memory and are added after the barrier.  Now 390 us with
 // the sizes in a pass of their own (plan_body).
 struct PairPlan {
-  uint32_t e[16];             // packed codes of the thread's steps (0 behind the last)
+  uint32_t e[16];             // packed codes of 16 of the thread's steps (0 behind the last)
   uint32_t pre;               // bits of the lane before them
   uint32_t base;              // units of the stream before them
   uint32_t units_a, units_b;  // units of each stream
-  bool packed;                // every code packed and every step held: pair_emit applies
+  bool packed;                // every code is packed: PairEmitter applies
 };
 
 // The steps of a quarter of a stream of n symbols.
@@ -747,76 +748,91 @@ __device__ __forceinline__ void pair_plan(PairPlan& P, uint32_t cum, uint32_t* s
   P.packed = !(__any_sync(~0u, all >> 31));
 }
 
-// Writes both streams to out (shared memory), stream A from unit a0 on, stream B behind
-// it.  heads: 256 words.  Contains one barrier; the units are complete after another.
-__device__ __forceinline__ void pair_emit(const PairPlan& P, uint16_t* out, uint32_t a0, uint32_t* heads) {
-  const uint32_t tid = threadIdx.x, l = tid & 31, w = tid >> 5;
-  const uint32_t lt = (1u << l) - 1u;
-  // places are shared-memory addresses; the first is the thread's word of heads
-  const uint32_t head = smem_u32(heads + tid);
-  uint32_t next = smem_u32(out) + 2u * (a0 + (w >> 2 ? P.units_a : 0u) + P.base);
-  uint32_t fill = ((P.pre + 15u) & 15u) + 1u;  // bits of the lane's last unit so far, 1 to 16
-  uint32_t win = 0;                            // this thread's bits of it and behind it, placed after `fill` bits
-  uint32_t pos = head;                         // its place
-  uint32_t any_len = 0;
-#pragma unroll
-  for (int i = 0; i < 16; i++) any_len |= P.e[i];
-  const bool wide = __any_sync(~0u, (any_len & 16u) != 0);  // (a code of 17 bits or more may take two units)
-  auto store = [](uint32_t at, uint32_t unit) {
+// Writes both streams to shared memory: init, then steps for every 16 steps, then finish.
+struct PairEmitter {
+  uint32_t head;  // places are shared-memory addresses; the first is the thread's word of heads
+  uint32_t next;  // the warp's next place
+  uint32_t fill;  // bits of the lane's last unit so far, 1 to 16
+  uint32_t win;   // this thread's bits of it and behind it, placed after `fill` bits
+  uint32_t pos;   // its place
+
+  static __device__ __forceinline__ void store(uint32_t at, uint32_t unit) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)unit) : "memory");
-  };
+  }
+
+  // Stream A from unit a0 of out on, stream B behind it.  heads: 256 words.
+  __device__ __forceinline__ void init(const PairPlan& P, uint16_t* out, uint32_t a0, uint32_t* heads) {
+    head = smem_u32(heads + threadIdx.x);
+    next = smem_u32(out) + 2u * (a0 + (threadIdx.x >> 7 ? P.units_a : 0u) + P.base);
+    fill = ((P.pre + 15u) & 15u) + 1u;
+    win = 0;
+    pos = head;
+  }
+
+  __device__ __forceinline__ void steps(const uint32_t (&e)[16]) {
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+    uint32_t any_len = 0;
 #pragma unroll
-  for (int i = 0; i < 16; i++) {
-    const uint32_t L = P.e[i] & 31u, c = P.e[i] & ~31u;
-    const uint32_t n = fill + L;
-    const bool need = n > 16;
-    const uint32_t b1 = __ballot_sync(~0u, need);
-    const uint32_t p1 = next + 2u * __popc(b1 & lt);
-    next += 2u * __popc(b1);
-    if (wide && __any_sync(~0u, n > 32)) {
-      const uint32_t b2 = __ballot_sync(~0u, n > 32);
-      const uint64_t both = ((uint64_t)win << 32) | (((uint64_t)c << 32) >> fill);
-      win = (uint32_t)(both >> 32);
-      fill = n;
-      if (need) {
-        store(pos, win >> 16);
-        pos = p1;
-        win <<= 16;
-        fill -= 16;
-      }
-      if (n > 32) {
-        store(p1, win >> 16);
-        pos = next + 2u * __popc(b2 & lt);
-        win = (uint32_t)both;
-        fill -= 16;
-      }
-      next += 2u * __popc(b2);
-    } else {
-      win |= c >> fill;
-      fill = n;
-      if (need) {
-        store(pos, win >> 16);
-        pos = p1;
-        win <<= 16;
-        fill -= 16;
+    for (int i = 0; i < 16; i++) any_len |= e[i];
+    const bool wide = __any_sync(~0u, (any_len & 16u) != 0);  // (a code of 17 bits or more may take two units)
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const uint32_t L = e[i] & 31u, c = e[i] & ~31u;
+      const uint32_t n = fill + L;
+      const bool need = n > 16;
+      const uint32_t b1 = __ballot_sync(~0u, need);
+      const uint32_t p1 = next + 2u * __popc(b1 & lt);
+      next += 2u * __popc(b1);
+      if (wide && __any_sync(~0u, n > 32)) {
+        const uint32_t b2 = __ballot_sync(~0u, n > 32);
+        const uint64_t both = ((uint64_t)win << 32) | (((uint64_t)c << 32) >> fill);
+        win = (uint32_t)(both >> 32);
+        fill = n;
+        if (need) {
+          store(pos, win >> 16);
+          pos = p1;
+          win <<= 16;
+          fill -= 16;
+        }
+        if (n > 32) {
+          store(p1, win >> 16);
+          pos = next + 2u * __popc(b2 & lt);
+          win = (uint32_t)both;
+          fill -= 16;
+        }
+        next += 2u * __popc(b2);
+      } else {
+        win |= c >> fill;
+        fill = n;
+        if (need) {
+          store(pos, win >> 16);
+          pos = p1;
+          win <<= 16;
+          fill -= 16;
+        }
       }
     }
   }
-  // (the upper half of the word: whether the thread has taken a unit)
-  if (pos == head) store(head, win >> 16);
-  store(head + 2, pos != head);
-  __syncthreads();
-  if (pos != head) {
-    // the later quarters' first bits, up to the first of them that took a unit of its own
-    uint32_t unit = win >> 16;
-    for (uint32_t v = tid + 32; (v & ~127u) == (tid & ~127u); v += 32) {
-      const uint32_t h = heads[v];
-      unit |= h & 0xffffu;
-      if (h >> 16) break;
+
+  // Contains one barrier; the units are complete after another.
+  __device__ __forceinline__ void finish(const uint32_t* heads) {
+    const uint32_t tid = threadIdx.x;
+    // (the upper half of the word: whether the thread has taken a unit)
+    if (pos == head) store(head, win >> 16);
+    store(head + 2, pos != head);
+    __syncthreads();
+    if (pos != head) {
+      // the later quarters' first bits, up to the first of them that took a unit of its own
+      uint32_t unit = win >> 16;
+      for (uint32_t v = tid + 32; (v & ~127u) == (tid & ~127u); v += 32) {
+        const uint32_t h = heads[v];
+        unit |= h & 0xffffu;
+        if (h >> 16) break;
+      }
+      store(pos, unit);
     }
-    store(pos, unit);
   }
-}
+};
 
 // One forward pass of the selector MLP by a full warp: lane i owns hidden unit i, and
 // every dot product is a chain of fused multiply-adds from the bias over the inputs

@@ -905,32 +905,54 @@ __device__ __forceinline__ void plan_huff(PairPlan& P, const EncodeArgs& a, cons
   pair_plan(P, cum | odd, s_part);
 }
 
-// P of an RLE+Huffman block's nr runs.  Contains one barrier.
-__device__ __forceinline__ void plan_runs(PairPlan& P, const EncodeArgs& a, const uint16_t* rv, const uint16_t* rl,
-                                          uint32_t nr, uint32_t* s_part) {
-  const uint32_t lane = threadIdx.x & 31, which = threadIdx.x >> 7, quarter = (threadIdx.x >> 5) & 3;
-  const uint32_t steps = quarter_steps(nr), j0 = 32 * quarter * steps + lane;
-  const uint16_t* sy = which ? rl : rv;
-  const uint32_t at = which ? 2 * kNsymCode : kNsymCode;
-  const uint32_t* book = packed_books(a.bcodes) + at;
-  const uint8_t* lens = a.lens + at;
-  uint32_t cum = 0, odd = steps > 16 ? 1u << 31 : 0u;
-  auto take = [&](uint32_t i) -> uint32_t {
-    const uint32_t j = j0 + 32 * i;
-    if (i >= steps || j >= nr) return 0u;
-    const uint32_t sym = (uint32_t)sy[j] - which;  // (run lengths are coded less one)
-    const uint32_t e = book[sym];
-    uint32_t L = e & 31u;
-    if (L == kPackedLong) {
-      odd = 1u << 31;
-      L = __ldg(&lens[sym]);
-    }
-    cum += L;
-    return e;
-  };
+// The runs of this thread (values or lengths) in an RLE+Huffman block of nr runs.
+struct RunPart {
+  const uint16_t* sy;
+  const uint32_t* book;
+  const uint8_t* lens;
+  uint32_t which, steps, j0, nr;
+  __device__ __forceinline__ RunPart(const EncodeArgs& a, const uint16_t* rv, const uint16_t* rl, uint32_t n) {
+    which = threadIdx.x >> 7;
+    nr = n;
+    steps = quarter_steps(n);
+    j0 = 32 * ((threadIdx.x >> 5) & 3) * steps + (threadIdx.x & 31);
+    sy = which ? rl : rv;
+    const uint32_t at = which ? 2 * kNsymCode : kNsymCode;
+    book = packed_books(a.bcodes) + at;
+    lens = a.lens + at;
+  }
+  // Packed codes of the steps from `first` on; returns their bits (odd: bit 31 set where a
+  // code is not packed).
+  __device__ __forceinline__ uint32_t load(uint32_t first, uint32_t (&e)[16], uint32_t& odd) const {
+    uint32_t cum = 0;
 #pragma unroll
-  for (uint32_t i = 0; i < 16; i++) P.e[i] = take(i);
-  for (uint32_t i = 16; i < steps; i++) take(i);
+    for (uint32_t i = 0; i < 16; i++) {
+      const uint32_t j = j0 + 32 * (first + i);
+      e[i] = 0;
+      if (first + i < steps && j < nr) {
+        const uint32_t sym = (uint32_t)sy[j] - which;  // (run lengths are coded less one)
+        e[i] = book[sym];
+        uint32_t L = e[i] & 31u;
+        if (L == kPackedLong) {
+          odd = 1u << 31;
+          L = __ldg(&lens[sym]);
+        }
+        cum += L;
+      }
+    }
+    return cum;
+  }
+};
+
+// P of an RLE+Huffman block's runs, with the codes of their first 16 steps.  Contains one
+// barrier.
+__device__ __forceinline__ void plan_runs(PairPlan& P, const RunPart& part, uint32_t* s_part) {
+  uint32_t cum = 0, odd = 0;
+#pragma unroll 1
+  for (uint32_t first = part.steps > 16 ? 16u : 0u;; first -= 16) {  // (the later steps first)
+    cum += part.load(first, P.e, odd);
+    if (first == 0) break;
+  }
   pair_plan(P, cum | odd, s_part);
 }
 
@@ -1137,7 +1159,7 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
   uint32_t size_h = ~0u, size_rh = ~0u;
   const uint32_t size_r = 4 * nr;
   if (codec == CODEC_RLE_HUFF || (codec < 0 && eligible)) {
-    plan_runs(plan, a, s_rv, s_rl, nr, s_part);
+    plan_runs(plan, RunPart(a, s_rv, s_rl, nr), s_part);
     size_rh = rlehuff_bytes(plan);
   }
   if (codec == CODEC_HUFF || (codec < 0 && (analyze || min(size_r, size_rh) >= 2 + m / 8))) {
@@ -1228,6 +1250,28 @@ __device__ __noinline__ void encode_long(const EncodeArgs& a, int codec, const u
   }
 }
 
+// The streams of an RLE+Huffman block of more than 2048 runs (forced modes): two turns of
+// 16 steps, the codes read again.  (Not inlined: a loop in the payload's common path costs it
+// its registers, 3-D 512^3 compression 803 -> 842 us.  The gathering encoder, which such
+// blocks took before: 1426 us for 60 M elements of a walk; now 897.)
+__device__ __noinline__ void emit_many_runs(const EncodeArgs& a, uint32_t pre, uint32_t base, uint32_t units_a,
+                                            const uint16_t* rv, uint32_t nr, uint32_t* s_buf, uint32_t* s_heads) {
+  PairPlan P;
+  P.pre = pre;
+  P.base = base;
+  P.units_a = units_a;
+  const RunPart part(a, rv, rv + kSlots, nr);
+  PairEmitter em;
+  em.init(P, reinterpret_cast<uint16_t*>(s_buf), 4u, s_heads);
+  uint32_t odd = 0;
+#pragma unroll 1
+  for (uint32_t f = 0; f < part.steps; f += 16) {
+    part.load(f, P.e, odd);
+    em.steps(P.e);
+  }
+  em.finish(s_heads);
+}
+
 // The payload of codec block b (all threads of the CTA), after the plans of all the field's
 // blocks; block 0 also writes the header, section padding and books.  m: the block's
 // elements.  smem: payload_smem_bytes() of dynamic shared memory.
@@ -1260,7 +1304,7 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsign
     __syncthreads();
     plan_huff(plan, a, part, sym, s_buf, s_part);
   } else if (codec == CODEC_RLE_HUFF) {
-    plan_runs(plan, a, rv, rv + kSlots, nr, s_part);
+    plan_runs(plan, RunPart(a, rv, rv + kSlots, nr), s_part);
   } else {
     __syncthreads();
   }
@@ -1284,7 +1328,14 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsign
       const uint32_t ua = plan.units_a, ub = plan.units_b;
       const uint32_t first = codec == CODEC_HUFF ? 1u : 4u, units = first + ua + ub;  // before stream A; in all
       if (plan.packed && in_smem) {
-        pair_emit(plan, reinterpret_cast<uint16_t*>(s_buf), first, s_heads);
+        if (codec == CODEC_RLE_HUFF && quarter_steps(nr) > 16) {
+          emit_many_runs(a, plan.pre, plan.base, plan.units_a, rv, nr, s_buf, s_heads);
+        } else {
+          PairEmitter em;
+          em.init(plan, reinterpret_cast<uint16_t*>(s_buf), first, s_heads);
+          em.steps(plan.e);
+          em.finish(s_heads);
+        }
       } else {
         encode_long(a, codec, codes, m, rv, nr, ua, out16, s_part);
       }
