@@ -260,31 +260,6 @@ __device__ T block_excl_scan(T v, T* scratch, T* total) {
   return r;
 }
 
-template <typename T>
-__device__ T block_sum(T v, T* scratch) {
-  T t;
-  block_excl_scan(v, scratch, &t);
-  return t;
-}
-
-__device__ inline uint32_t block_max_u32(uint32_t v, uint32_t* scratch) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(~0u, v, o));
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    uint32_t s = lane < nw ? scratch[lane] : 0u;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s = max(s, __shfl_xor_sync(~0u, s, o));
-    if (lane == 0) scratch[32] = s;
-  }
-  __syncthreads();
-  uint32_t r = scratch[32];
-  __syncthreads();
-  return r;
-}
-
 // ---------------------------------------------------------------------------------
 // prequantization arithmetic (Sec. IV-A1), bit-identical to a plain C reading
 // ---------------------------------------------------------------------------------
@@ -378,13 +353,6 @@ __device__ __forceinline__ uint32_t prequant_d(double x, double eb_d, double ste
     return 0;
   }
   return ERR_RANGE;  // unreachable by the step's margin
-}
-
-__device__ __forceinline__ bool prequant_fast_d(double x, double eb_d, double step, double rstep, int32_t& k) {
-  const double v = __dmul_rn(x, rstep);
-  k = __double2int_rn(v);
-  const double s = __dsub_rn(x, __dmul_rn((double)k, step));
-  return (fabs(v) < kMaxK64) & (fabs(s) < eb_d);
 }
 
 // Binary logarithm in Q16 by bit-by-bit squaring of the mantissa (integer only).

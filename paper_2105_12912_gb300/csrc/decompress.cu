@@ -23,59 +23,6 @@ __device__ __forceinline__ void flag(DevState* st, uint32_t bits) { atomicOr(&st
 // =================================================================================
 // archive validation and offsets
 // =================================================================================
-__device__ void dec_prep_body(const DecodeArgs& a) {
-  if (a.dead) return;
-  __shared__ uint64_t s_scan[33];
-  __shared__ uint32_t s_nc[3];
-  const int tid = threadIdx.x;
-  if (a.check_hdr && tid < 32) {
-    // the launch was set up from a host copy of the header: it must be this archive's
-    const uint8_t* h = a.ar + 4 * tid;
-    const uint32_t v = (uint32_t)h[0] | ((uint32_t)h[1] << 8) | ((uint32_t)h[2] << 16) | ((uint32_t)h[3] << 24);
-    if (__any_sync(~0u, v != a.hdr[tid]) && tid == 0) flag(a.st, ERR_CORRUPT);
-  }
-  if (tid < 3) s_nc[tid] = 0;
-  __syncthreads();
-  // payload offsets and, packed above them in the same scan (bits 40-51 and 52-63; a
-  // scan step covers at most 1024 blocks), the lists of run blocks and of the blocks
-  // the reconstruction kernel takes (those not reconstructed by their decoder warps)
-  constexpr uint64_t kLow = (1ull << 40) - 1, kMid = (1ull << 12) - 1;
-  uint64_t carry = 0, rcarry = 0, scarry = 0;
-  bool bad = false;
-  for (uint32_t base = 0; base < a.g.nblk; base += blockDim.x) {
-    const uint32_t b = base + tid;
-    uint64_t bb = 0;
-    bool run = false, slow = false;
-    if (b < a.g.nblk) {
-      const uint32_t c = a.ar[a.off_codec + b];
-      bb = reinterpret_cast<const uint32_t*>(a.ar + a.off_bb)[b];
-      if (c > 2 || (bb & 3) || bb >= (1ull << 30)) bad = true;  // a valid block is below 2^17 bytes
-      else atomicAdd(&s_nc[c], 1u);
-      run = c == CODEC_RLE || c == CODEC_RLE_HUFF;
-      slow = !(a.fuse && c == CODEC_HUFF && block_is_full(a.g, b));
-    }
-    if (bb >= (1ull << 30)) bb = 0;
-    uint64_t tot;
-    const uint64_t ex =
-        block_excl_scan<uint64_t>(bb | ((uint64_t)slow << 40) | ((uint64_t)run << 52), s_scan, &tot);
-    if (b < a.g.nblk) a.blk_off[b] = carry + (ex & kLow);
-    if (run && a.runblk) a.runblk[rcarry + (ex >> 52)] = b;
-    if (slow && a.slowblk) a.slowblk[scarry + ((ex >> 40) & kMid)] = b;
-    carry += tot & kLow;
-    rcarry += tot >> 52;
-    scarry += (tot >> 40) & kMid;
-  }
-  if (tid == 0) {
-    a.st->n_slow = (uint32_t)scarry;
-    a.blk_off[a.g.nblk] = carry;
-    if (carry != a.payload) bad = true;
-    if ((s_nc[CODEC_HUFF] && !(a.flags & 1u)) || (s_nc[CODEC_RLE_HUFF] && !(a.flags & 2u))) bad = true;
-    for (int c = 0; c < 3; c++)
-      if (s_nc[c] != a.n_codec[c]) bad = true;  // the header's counts decide which kernels run
-  }
-  if (bad) flag(a.st, ERR_CORRUPT);
-}
-
 // Single-field set-up, one CTA per 1024 codec blocks (chunks taken by ticket and
 // chained by decoupled look-back, so no CTA scans the whole block list): codec and
 // block-size validation, payload offsets, the lists of run blocks and of the blocks
