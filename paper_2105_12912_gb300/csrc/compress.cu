@@ -967,9 +967,17 @@ __device__ __forceinline__ uint16_t* block_run_store(const EncodeArgs& a, uint32
   return reinterpret_cast<uint16_t*>(const_cast<int32_t*>(a.rec.deltas) + (uint64_t)b * kSlots);
 }
 
+// The field's status as far as encoding goes by it.  An expired wait (ERR_TIMEOUT) may have
+// left blocks that construction never wrote: their codes, run counts, sizes and picks are
+// whatever the memory held, good for no index, so such a field's blocks are passed over (the
+// call reports the status).  Every other error leaves valid codes.  Read through L2, by every
+// thread beside loads it waits for anyway; the launches before have set all there is to set.
+__device__ __forceinline__ uint32_t encode_status(const EncodeArgs& a) { return __ldcg(&a.st->status); }
+
 // The plan of codec block b of one field (all threads of the CTA).  box: its origin and
-// extent (block_box).  smem: plan_smem_bytes() of dynamic shared memory.
-__device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, unsigned char* smem) {
+// extent (block_box).  status: the field's, the same in every thread.  smem:
+// plan_smem_bytes() of dynamic shared memory.
+__device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, uint32_t status, unsigned char* smem) {
   uint16_t* s_c = reinterpret_cast<uint16_t*>(smem);              // 4096 codes; before them the run starts
   uint16_t* s_rv = s_c + kSlots;                                  // run values
   uint16_t* s_rl = s_rv + kSlots;                                 // run lengths
@@ -996,6 +1004,8 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
   // the run count comes from construction; forced Huffman does without
   const bool analyze = a.analyze != 0;
   const uint32_t nr = sel != SEL_HUFF || analyze ? a.block_runs[b] : 0u;
+  const uint32_t records = a.place_records ? a.rec.counts[b] : 0u;
+  if (status & ERR_TIMEOUT) return;  // (every load above is on its way by now)
   const bool eligible = a.all_runs || 4 * nr <= m;
   // Runs are extracted (values, lengths) when a run codec or the statistics may need them.
   bool runs = analyze || (sel != SEL_HUFF && eligible);
@@ -1007,7 +1017,7 @@ __device__ void plan_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, 
     reinterpret_cast<uint4*>(s_hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
     if (sel == SEL_LEARNED) stage_mlp(a.mlp_w, reinterpret_cast<float*>(s_sw));
   }
-  if (a.place_records && a.rec.counts[b] != 0) {
+  if (records != 0) {
     place_records(a, b, box, box + 3, s_scan64);
     fresh = false;
   }
@@ -1274,8 +1284,9 @@ __device__ __noinline__ void emit_many_runs(const EncodeArgs& a, uint32_t pre, u
 
 // The payload of codec block b (all threads of the CTA), after the plans of all the field's
 // blocks; block 0 also writes the header, section padding and books.  m: the block's
-// elements.  smem: payload_smem_bytes() of dynamic shared memory.
-__device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsigned char* smem) {
+// elements.  status: the field's, the same in every thread.  smem: payload_smem_bytes() of
+// dynamic shared memory.
+__device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, uint32_t status, unsigned char* smem) {
   uint32_t* s_buf = reinterpret_cast<uint32_t*>(smem);  // 16 KB: the payload; before it, the code book
   uint32_t* s_part = s_buf + kBufBytes / 4;             // 256 (+ 8)
   uint32_t* s_heads = s_part + kEncThreads + 8;         // 256
@@ -1295,6 +1306,7 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsign
   for (uint32_t k = tid; k < group; k += kEncThreads) before += __ldcg(&a.groups[k]) & kGroupBytes;
   const uint32_t nr = a.block_runs[b];
   const uint16_t* rv = block_run_store(a, b);
+  if (status & ERR_TIMEOUT) return;  // (every load above is on its way by now)
   before = warp_sum(before);
   if ((tid & 31) == 0) s_sum[wid] = before;
   PairPlan plan;
@@ -1365,7 +1377,7 @@ __global__ __launch_bounds__(kEncThreads, 4) void plan_kernel(EncodeArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (threadIdx.x == 0) block_box(a.g, blockIdx.x, s_box, s_box + 3);
   __syncthreads();
-  plan_body(a, blockIdx.x, s_box, smem);
+  plan_body(a, blockIdx.x, s_box, encode_status(a), smem);
 }
 
 __global__ __launch_bounds__(kEncThreads, 5) void payload_kernel(EncodeArgs a) {
@@ -1374,7 +1386,7 @@ __global__ __launch_bounds__(kEncThreads, 5) void payload_kernel(EncodeArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (threadIdx.x == 0) s_m = block_elems(a.g, blockIdx.x);
   __syncthreads();
-  payload_body(a, blockIdx.x, s_m, smem);
+  payload_body(a, blockIdx.x, s_m, encode_status(a), smem);
 }
 
 __device__ __forceinline__ int field_of_prefix(const uint32_t* prefix, int nfields, uint32_t c) {
@@ -1399,7 +1411,8 @@ __global__ __launch_bounds__(kEncThreads, 4) void plan_batch_kernel(const Encode
     block_box(tasks[f].g, blockIdx.x - tile0[f], s_box, s_box + 3);
   }
   __syncthreads();
-  plan_body(tasks[s_field], blockIdx.x - tile0[s_field], s_box, smem);
+  const EncodeArgs& a = tasks[s_field];
+  plan_body(a, blockIdx.x - tile0[s_field], s_box, encode_status(a), smem);
 }
 
 __global__ __launch_bounds__(kEncThreads, 5) void payload_batch_kernel(const EncodeArgs* __restrict__ tasks,
@@ -1413,7 +1426,8 @@ __global__ __launch_bounds__(kEncThreads, 5) void payload_batch_kernel(const Enc
     s_m = block_elems(tasks[f].g, blockIdx.x - tile0[f]);
   }
   __syncthreads();
-  payload_body(tasks[s_field], blockIdx.x - tile0[s_field], s_m, smem);
+  const EncodeArgs& a = tasks[s_field];
+  payload_body(a, blockIdx.x - tile0[s_field], s_m, encode_status(a), smem);
 }
 
 static size_t plan_smem_bytes() {
@@ -1462,7 +1476,7 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
   // which would pad the static shared memory of every kernel in this file
   extern __shared__ __align__(16) unsigned char smem_dyn[];
   unsigned char* smem_raw = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
-  __shared__ uint32_t s_word, s_box[6];
+  __shared__ uint32_t s_word, s_box[6], s_status;
   const int tid = threadIdx.x;
   // ---- phase 1: value ranges and bounds ---------------------------------------------
   while (true) {
@@ -1509,9 +1523,13 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
       await_field(&ea.st->books_done, 4u, ea.st, p.spin_limit);
       ready_field = f;
     }
-    if (tid == 0) block_box(ea.g, t - p.tile0[f], s_box, s_box + 3);
+    // (the status once, by thread 0: other CTAs' waits may expire meanwhile)
+    if (tid == 0) {
+      block_box(ea.g, t - p.tile0[f], s_box, s_box + 3);
+      s_status = encode_status(ea);
+    }
     __syncthreads();
-    plan_body(ea, t - p.tile0[f], s_box, smem_raw);
+    plan_body(ea, t - p.tile0[f], s_box, s_status, smem_raw);
     __syncthreads();
     if (tid == 0) {
       __threadfence();
@@ -1529,9 +1547,12 @@ __global__ __launch_bounds__(kPersistThreads, 4) void batch_persistent_kernel(co
       await_field(&ea.st->encode_done, ea.g.nblk, ea.st, p.spin_limit);
       ready_field = f;
     }
-    if (tid == 0) s_box[0] = block_elems(ea.g, t - p.tile0[f]);
+    if (tid == 0) {
+      s_box[0] = block_elems(ea.g, t - p.tile0[f]);
+      s_status = encode_status(ea);
+    }
     __syncthreads();
-    payload_body(ea, t - p.tile0[f], s_box[0], smem_raw);
+    payload_body(ea, t - p.tile0[f], s_box[0], s_status, smem_raw);
     __syncthreads();
   }
 }

@@ -1128,18 +1128,16 @@ __device__ __forceinline__ void construct_loop(const ConstructTask& one, const C
       mbar_wait(&S.bar[cur], (phase >> cur) & 1u, spin_limit);
       if (s_f[cur ^ 1] >= 0 && task(s_f[cur ^ 1])->use_tma && tma_ok)
         mbar_wait(&S.bar[cur ^ 1], (phase >> (cur ^ 1)) & 1u, spin_limit);
-      if (P) {
-        // the later phases still count on every tile: the current field's, the one
-        // claimed next and the ticket drawn after it are handed on unprocessed (the
-        // status already says that the results are void)
-        signal_field(field, ntile_acc);
-        auto abandon = [&](int f2) {
-          atomicOr(&task(f2)->a.st->status, ERR_TIMEOUT);
-          signal_field(f2, 1u);
-        };
-        if (s_f[cur ^ 1] >= 0) abandon(s_f[cur ^ 1]);
-        if (pending < ntiles) abandon(tasks ? find_field(tile0, nfields, pending, 0) : 0);
-      }
+      // the tile claimed next and the ticket drawn after it, perhaps of other fields, stay
+      // unprocessed: their fields' status says so too (encoding goes by it).  P: the later
+      // phases still count on every tile, so these are handed on
+      auto abandon = [&](int f2) {
+        atomicOr(&task(f2)->a.st->status, ERR_TIMEOUT);
+        if (P) signal_field(f2, 1u);
+      };
+      if (P) signal_field(field, ntile_acc);
+      if (s_f[cur ^ 1] >= 0) abandon(s_f[cur ^ 1]);
+      if (pending < ntiles) abandon(tasks ? find_field(tile0, nfields, pending, 0) : 0);
     }
     if (P) {
       if (tid == 0) {
