@@ -148,12 +148,13 @@ def decompress(archive: torch.Tensor, nbytes: int | None = None, out: torch.Tens
     head = None
     if dims is None or out is None:
         # the header crosses to the host once: its copy gives the shape here and drives the
-        # decompression (which compares it with the archive's own on the device)
+        # decompression (which compares it with the archive's own on the device), so it is
+        # read on the decompression's stream, behind what fills the archive there
         head = (C.c_uint8 * 128)()
         nd, esz = C.c_int(), C.c_int()
         shape = (C.c_uint64 * 3)()
         st = L.lib().csz_archive_head(C.c_void_p(archive.data_ptr()), archive.numel(), head, C.byref(nd), shape,
-                                      C.byref(esz), _stream_ptr(None))
+                                      C.byref(esz), _stream_ptr(stream))
         if dims is None:
             _check(st, "csz_archive_info")
             dims = tuple(shape[:nd.value])
