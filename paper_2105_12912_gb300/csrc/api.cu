@@ -520,8 +520,9 @@ csz_status csz_decompress(const uint8_t* d_ar, size_t bytes, float* d_out, uint6
 
 csz_status csz_archive_head(const uint8_t* d_ar, size_t bytes, uint8_t* h_header, int* ndim, uint64_t* dims,
                             int* elem_bytes, void* stream) {
-  if (!d_ar || !h_header) return CSZ_E_ARG;
-  if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;
+  if (!h_header) return CSZ_E_ARG;
+  if (bytes < (size_t)kHdr) return CSZ_E_CORRUPT;  // (an empty archive may have no address)
+  if (!d_ar) return CSZ_E_ARG;
   csz_status r = read_header(d_ar, h_header, static_cast<cudaStream_t>(stream));
   if (r != CSZ_OK) return r;
   r = csz_archive_info(h_header, kHdr, ndim, dims, nullptr, nullptr);
