@@ -154,6 +154,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // launch before it has completed and its writes are visible -- which that launch did in its
 // turn, so everything before it is too -- then lets the next launch's CTAs take places that
 // become free.  Does nothing in an ordinary launch.
+// Such a kernel is resident while the launch before it still writes, so what that launch (or
+// the caller's last one) writes is read by plain or L2 loads, never through the read-only
+// path (__ldg, const __restrict__): its loads are for data nobody writes while the kernel
+// lives, and a compiler may move them above the wait.
 __device__ __forceinline__ void chained_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -586,15 +590,14 @@ __device__ __forceinline__ uint32_t next_head(const uint32_t* head, const uint32
 // owner of step t gathers the unit's 16 bits from that code onwards.  Each unit is
 // written exactly once.  Returns the unit count.  scratch: >= 8*32 + 8 u32.
 __device__ inline uint32_t ihs_unit_gather(const uint16_t* sym, uint32_t N, int add,
-                                           const uint8_t* __restrict__ lens,
-                                           const uint64_t* __restrict__ codes, uint32_t lane,
+                                           const uint8_t* lens, const uint64_t* codes, uint32_t lane,
                                            uint32_t t, uint32_t skip) {
   uint32_t unit = 0;
   int have = 0;
   for (uint32_t tt = t; have < 16 && 32 * tt + lane < N; tt++) {
     const int s = sym[32 * tt + lane] + add;
-    const int L = __ldg(&lens[s]);
-    const uint64_t C = __ldg(&codes[s]);
+    const int L = lens[s];
+    const uint64_t C = codes[s];
     const int avail = L - (int)skip;
     const int take = min(avail, 16 - have);
     const uint32_t bits = (uint32_t)((C >> (avail - take)) & ((1ull << take) - 1ull));
@@ -606,14 +609,13 @@ __device__ inline uint32_t ihs_unit_gather(const uint16_t* sym, uint32_t N, int 
 }
 
 __device__ inline uint32_t ihs_encode_block(const uint16_t* sym, uint32_t N, int add,
-                                            const uint8_t* __restrict__ lens,
-                                            const uint64_t* __restrict__ codes, uint16_t* out16,
+                                            const uint8_t* lens, const uint64_t* codes, uint16_t* out16,
                                             uint32_t* scratch) {
   const uint32_t tid = threadIdx.x, l = tid & 31, w = tid >> 5;
   const uint32_t t0 = 16 * w;
   auto len_at = [&](uint32_t t) -> uint32_t {
     const uint32_t j = 32 * t + l;
-    return j < N ? (uint32_t)__ldg(&lens[sym[j] + add]) : 0u;
+    return j < N ? (uint32_t)lens[sym[j] + add] : 0u;
   };
   __syncthreads();
   uint32_t cum = 0;

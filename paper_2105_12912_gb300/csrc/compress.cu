@@ -900,7 +900,7 @@ __device__ __forceinline__ void plan_huff(PairPlan& P, const EncodeArgs& a, cons
     odd = 1u << 31;
 #pragma unroll
     for (int i = 0; i < 16; i++)
-      if ((P.e[i] & 31u) == kPackedLong) cum += __ldg(&a.lens[sym[i]]) - kPackedLong;
+      if ((P.e[i] & 31u) == kPackedLong) cum += a.lens[sym[i]] - kPackedLong;
   }
   pair_plan(P, cum | odd, s_part);
 }
@@ -935,7 +935,7 @@ struct RunPart {
         uint32_t L = e[i] & 31u;
         if (L == kPackedLong) {
           odd = 1u << 31;
-          L = __ldg(&lens[sym]);
+          L = lens[sym];
         }
         cum += L;
       }

@@ -462,7 +462,7 @@ struct IhsReader {
         // (bb lies at or above the second level's base: the lookup missed.  A damaged
         // stream can point past its cells.)
         const uint32_t c = (bb - bk.lut2_base) >> bk.lut2_shift;
-        const uint32_t e2 = c < bk.lut2_n ? (uint32_t)__ldg(&bk.lut2[c]) : 0u;
+        const uint32_t e2 = c < bk.lut2_n ? (uint32_t)bk.lut2[c] : 0u;
         const int l2 = lut2_len(e2);
         if (e2 != 0u && l2 <= 16 - sh) {
           l = l2;

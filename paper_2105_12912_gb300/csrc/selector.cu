@@ -88,11 +88,8 @@ __device__ __forceinline__ float dot32(const float (&w)[kMlpHid], const float* s
 }
 
 constexpr int kRedWarps = kTrainWarps / 2;  // the warps' sums meet in two turns
-__global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __restrict__ w,
-                                                                 const float* __restrict__ feat,
-                                                                 const float* __restrict__ tgt,
-                                                                 const uint8_t* __restrict__ valid,
-                                                                 uint64_t n, float* __restrict__ part) {
+__global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w, const float* feat, const float* tgt,
+                                                                 const uint8_t* valid, uint64_t n, float* part) {
   chained_begin();
   __shared__ float s_red[kRedWarps][kPart + kStage];
   __shared__ __align__(16) float s_act[kTrainWarps][4][kMlpHid];  // per warp: h1 and da2 of two rows
@@ -143,7 +140,7 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __
       for (int k = 0; k < 2; k++) {
         a1[k] = b1;
 #pragma unroll
-        for (int j = 0; j < kMlpIn; j++) x[k][j] = __ldg(&feat[row[k] * kMlpIn + j]);
+        for (int j = 0; j < kMlpIn; j++) x[k][j] = feat[row[k] * kMlpIn + j];
 #pragma unroll
         for (int j = 0; j < kMlpIn; j++) a1[k] = fmaf(w1[j], x[k][j], a1[k]);
         act[k][lane] = a1[k] > 0.0f ? a1[k] : 0.0f;
@@ -159,7 +156,7 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* __
 #pragma unroll
         for (int c = 0; c < kMlpOut; c++) {
           const float y = b3[c] + warp_sum_f(w3[c] * h2[k]);
-          const float e = k == 0 || both ? y - __ldg(&tgt[row[k] * kMlpOut + c]) : 0.0f;
+          const float e = k == 0 || both ? y - tgt[row[k] * kMlpOut + c] : 0.0f;
           loss = fmaf(e, e, loss);
           dy[k][c] = 2.0f * e;
         }
@@ -264,12 +261,9 @@ struct Sum2 {
 // they do.
 constexpr int kUpdThreads = 1024, kUpdParams = 32, kMaxParts = 512;
 constexpr float kPartScale = 1.0f / kMaxParts;
-__global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* __restrict__ part, int nparts,
-                                                                 float* __restrict__ w,
-                                                                 float* __restrict__ grad_out,
-                                                                 double* __restrict__ loss_out,
-                                                                 float* __restrict__ m, float* __restrict__ v,
-                                                                 uint32_t step, float lr, float c1, float c2) {
+__global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* part, int nparts, float* w,
+                                                                 float* grad_out, double* loss_out, float* m,
+                                                                 float* v, uint32_t step, float lr, float c1, float c2) {
   chained_begin();
   __shared__ Sum2 s_sum[32][kUpdParams + 1];
   __shared__ Sum2 s_tot[kUpdParams];
