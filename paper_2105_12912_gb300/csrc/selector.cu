@@ -127,7 +127,9 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w,
     const uint64_t mine = r0 + lane * nw;
     uint32_t todo = __ballot_sync(~0u, mine < n && (!valid || valid[mine]));
     while (todo) {
-      // two of the rows, or one (then the second repeats it and adds nothing)
+      // two of the rows, or one: then the second's place holds zeros from its inputs to its
+      // errors, so that it adds nothing whatever the weights and the first row's values are
+      // (a repeated row times an error of 0 would be a NaN where its activations overflow)
       uint64_t row[2];
       row[0] = r0 + (__ffs(todo) - 1) * nw;
       todo &= todo - 1;
@@ -135,28 +137,29 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w,
       row[1] = both ? r0 + (__ffs(todo) - 1) * nw : row[0];
       todo &= todo - 1;
       float x[2][kMlpIn], a1[2], a2[2], h2[2], dy[2][kMlpOut], da2[2], da1[2];
+      const bool live[2] = {true, both};
       // forward
 #pragma unroll
       for (int k = 0; k < 2; k++) {
         a1[k] = b1;
 #pragma unroll
-        for (int j = 0; j < kMlpIn; j++) x[k][j] = feat[row[k] * kMlpIn + j];
+        for (int j = 0; j < kMlpIn; j++) x[k][j] = live[k] ? feat[row[k] * kMlpIn + j] : 0.0f;
 #pragma unroll
         for (int j = 0; j < kMlpIn; j++) a1[k] = fmaf(w1[j], x[k][j], a1[k]);
-        act[k][lane] = a1[k] > 0.0f ? a1[k] : 0.0f;
+        act[k][lane] = live[k] && a1[k] > 0.0f ? a1[k] : 0.0f;
       }
       __syncwarp();
 #pragma unroll
       for (int k = 0; k < 2; k++) {
         a2[k] = dot32(w2r, act[k], b2);
-        h2[k] = a2[k] > 0.0f ? a2[k] : 0.0f;
+        h2[k] = live[k] && a2[k] > 0.0f ? a2[k] : 0.0f;
       }
 #pragma unroll
       for (int k = 0; k < 2; k++) {
 #pragma unroll
         for (int c = 0; c < kMlpOut; c++) {
           const float y = b3[c] + warp_sum_f(w3[c] * h2[k]);
-          const float e = k == 0 || both ? y - tgt[row[k] * kMlpOut + c] : 0.0f;
+          const float e = live[k] ? y - tgt[row[k] * kMlpOut + c] : 0.0f;
           loss = fmaf(e, e, loss);
           dy[k][c] = 2.0f * e;
         }
@@ -172,7 +175,7 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w,
           gb3[c] += dy[k][c];
           dh2 = fmaf(dy[k][c], w3[c], dh2);
         }
-        da2[k] = a2[k] > 0.0f ? dh2 : 0.0f;
+        da2[k] = live[k] && a2[k] > 0.0f ? dh2 : 0.0f;
         act[2 + k][lane] = da2[k];
         gb2 += da2[k];
       }
@@ -188,7 +191,7 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w,
           g2[j + 3] = fmaf(da2[k], h.w, g2[j + 3]);
         }
         const float dh1 = dot32(w2c, act[2 + k], 0.0f);
-        da1[k] = a1[k] > 0.0f ? dh1 : 0.0f;
+        da1[k] = live[k] && a1[k] > 0.0f ? dh1 : 0.0f;
 #pragma unroll
         for (int j = 0; j < kMlpIn; j++) g1[j] = fmaf(da1[k], x[k][j], g1[j]);
         gb1 += da1[k];
