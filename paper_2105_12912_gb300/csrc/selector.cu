@@ -87,6 +87,15 @@ __device__ __forceinline__ float dot32(const float (&w)[kMlpHid], const float* s
   return (acc[0] + acc[1]) + (acc[2] + acc[3]);
 }
 
+// x becomes the rounded sum of x and y; returns what rounding took from it (Knuth's TwoSum;
+// after an infinity a NaN that says nothing).
+__device__ __forceinline__ float two_sum(float& x, float y) {
+  const float s = __fadd_rn(x, y), b = __fsub_rn(s, x);
+  const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, b)), __fsub_rn(y, b));
+  x = s;
+  return e;
+}
+
 constexpr int kRedWarps = kTrainWarps / 2;  // the warps' sums meet in two turns
 __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w, const float* feat, const float* tgt,
                                                                  const uint8_t* valid, uint64_t n, float* part) {
@@ -222,30 +231,27 @@ __global__ __launch_bounds__(kTrainThreads) void mlp_grad_kernel(const float* w,
     }
     __syncthreads();
   }
+  // (rounded once: the CTA's sum has one rounding for every two warps and a last one)
   for (int p = threadIdx.x; p < kPart; p += kTrainThreads) {
-    float acc = 0.0f;
     const int q = padded_t(p);
+    float acc = s_red[0][q], low = 0.0f;
 #pragma unroll
-    for (int wv = 0; wv < kRedWarps; wv++) acc += s_red[wv][q];
-    part[(uint64_t)blockIdx.x * kPart + p] = acc;
+    for (int wv = 1; wv < kRedWarps; wv++) low = __fadd_rn(low, two_sum(acc, s_red[wv][q]));
+    part[(uint64_t)blockIdx.x * kPart + p] = isfinite(low) ? __fadd_rn(acc, low) : acc;
   }
 }
 
-// A sum in two floats (the second holds what rounding took from the first, by Knuth's
-// TwoSum): 48 bits or so.
-struct Sum2 {
-  float h, l;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    h = s;
-  }
-  __device__ __forceinline__ void add(const Sum2& o) {
+// A sum in three floats, each holding what rounding took from the one before: 72 bits, more
+// than a double's 53.
+struct Sum3 {
+  float h, m, l;
+  __device__ __forceinline__ void add(float x) { l = __fadd_rn(l, two_sum(m, two_sum(h, x))); }
+  __device__ __forceinline__ void add(const Sum3& o) {
     add(o.h);
-    l = __fadd_rn(l, o.l);
+    l = __fadd_rn(l, __fadd_rn(two_sum(m, o.m), o.l));
   }
-  __device__ __forceinline__ Sum2 shfl_xor(int o) const {
-    return Sum2{__shfl_xor_sync(~0u, h, o), __shfl_xor_sync(~0u, l, o)};
+  __device__ __forceinline__ Sum3 shfl_xor(int o) const {
+    return Sum3{__shfl_xor_sync(~0u, h, o), __shfl_xor_sync(~0u, m, o), __shfl_xor_sync(~0u, l, o)};
   }
 };
 
@@ -255,29 +261,27 @@ struct Sum2 {
 // Bound by latency.  A CTA takes 32 parameters; its 32 warps add every 32nd partial each
 // (all in flight, 128 bytes a row), warp w then adds parameter w's 32 sums across its lanes
 // -- always in the same order, so runs stay reproducible -- and warp 0 finishes the 32
-// parameters.  The sums run in pairs of floats: in doubles the FP64 pipe, 2 results a cycle
-// and SM, took most of the launch for adding, converting and one division a warp.  The
-// weights after 50 steps are as far from a 64-bit training run as with doubles (8.7e-8 of
-// their norm, mean of six fields either way).  Doubles are left for the one scale and the 32
-// products.  c1, c2: Adam's bias corrections of this step.
-// The partials are scaled down by kMaxParts, so that their sum overflows no earlier than
-// they do.
+// parameters.  The sums run in three floats: in doubles the FP64 pipe, 2 results a cycle and
+// SM, takes most of the launch for converting and adding (50 steps on 28,672 rows: 1186 us,
+// with the doubles spread over four times as many CTAs; 936 us so; 915 in pairs of floats,
+// which hold 48 bits).  Doubles are left for the last combination and the one scale, and for
+// sums that are not finite or overflow a float, which start again in them.  c1, c2: Adam's
+// bias corrections of this step.
 constexpr int kUpdThreads = 1024, kUpdParams = 32, kMaxParts = 512;
-constexpr float kPartScale = 1.0f / kMaxParts;
 __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* part, int nparts, float* w,
                                                                  float* grad_out, double* loss_out, float* m,
                                                                  float* v, uint32_t step, float lr, float c1, float c2) {
   chained_begin();
-  __shared__ Sum2 s_sum[32][kUpdParams + 1];
-  __shared__ Sum2 s_tot[kUpdParams];
+  __shared__ Sum3 s_sum[32][kUpdParams + 1];
+  __shared__ Sum3 s_tot[kUpdParams];
   __shared__ unsigned long long s_c[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int p0 = blockIdx.x * kUpdParams;
   {
-    Sum2 acc{0.0f, 0.0f};
+    Sum3 acc{0.0f, 0.0f, 0.0f};
     const int p = min(p0 + lane, kMlpParams);
 #pragma unroll 5
-    for (int g = wid; g < nparts; g += 32) acc.add(part[(uint64_t)g * kPart + p] * kPartScale);
+    for (int g = wid; g < nparts; g += 32) acc.add(part[(uint64_t)g * kPart + p]);
     s_sum[wid][lane] = acc;
   }
   // row counts: whole numbers
@@ -288,7 +292,7 @@ __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* pa
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
   if (lane == 0) s_c[wid] = cnt;
   __syncthreads();
-  Sum2 acc = s_sum[lane][wid];
+  Sum3 acc = s_sum[lane][wid];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc.add(acc.shfl_xor(o));
   if (lane == 0) s_tot[wid] = acc;
@@ -299,9 +303,12 @@ __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* pa
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
   const int p = p0 + lane;
   if (p > kMlpParams) return;
-  // (after an infinity the second float is a NaN that says nothing)
-  const Sum2 tot = s_tot[lane];
-  const double sum = ((double)tot.h + (isfinite(tot.l) ? (double)tot.l : 0.0)) / kPartScale;
+  const Sum3 tot = s_tot[lane];
+  double sum = (double)tot.h + ((double)tot.m + (double)tot.l);
+  if (!isfinite(sum)) {
+    sum = 0.0;
+    for (int g = 0; g < nparts; g++) sum += (double)part[(uint64_t)g * kPart + p];
+  }
   const double scale = cnt ? 1.0 / (3.0 * (double)cnt) : 0.0;
   if (p == kMlpParams) {
     if (loss_out) *loss_out = sum * scale;
@@ -327,8 +334,11 @@ int train_grid(uint64_t nrows) {
     cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
     if (g_sms <= 0) g_sms = 1;
   }
+  // a CTA an SM, or two in turn where a warp would add more than 32 rows into one FP32 sum
+  // (its rounding grows with them)
   const uint64_t want = (nrows + 4 * kTrainWarps - 1) / (4 * kTrainWarps);
-  const uint64_t cap = (uint64_t)(g_sms < kMaxParts ? g_sms : kMaxParts);
+  const int ctas = nrows > 32ull * kTrainWarps * (uint64_t)g_sms ? 2 * g_sms : g_sms;
+  const uint64_t cap = (uint64_t)(ctas < kMaxParts ? ctas : kMaxParts);
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
