@@ -429,9 +429,10 @@ csz_status enqueue_decode(const uint8_t* d_ar, size_t bytes, const uint8_t* h, b
       if (cudaMemsetAsync(da.scan_state, 0, 8ull * g.nblk, s) != cudaSuccess) return CSZ_E_CUDA;
     } else {
       // in the decoded run lengths' place (8 KB a block), read no more by then: 4 bytes a
-      // block row, at most 1 KB a block, each
+      // block row, at most 1 KB a block, each (the first up to 3 words a row more, for a
+      // pitch in 16-byte words, where a row has 65 blocks or more)
       da.gtotals = reinterpret_cast<int32_t*>(da.runl);
-      da.gstrips = da.gtotals + 256ull * g.nblk;
+      da.gstrips = da.gtotals + 512ull * g.nblk;
     }
   }
   if (f64) {

@@ -1253,7 +1253,12 @@ __device__ __forceinline__ void load_fused16(const DecodeArgs& a, uint32_t b, ui
   overlay_outliers(a, b, j0, n, q);
 }
 
-// Sums of the block's rows: totals[bx][row], row over the field's rows.
+// The word of block bx (along x) and row (of the field's rows) in gtotals.
+__device__ __forceinline__ uint64_t total_at(const DecodeArgs& a, uint32_t bx, uint64_t row, uint64_t nrows) {
+  return a.gpitch ? row * a.gpitch + bx : bx * nrows + row;
+}
+
+// Sums of the block's rows.
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) {
   chained_begin();
@@ -1272,7 +1277,7 @@ __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) 
   }
   const uint64_t nrows = (uint64_t)a.g.n[0] * a.g.n[1];
   if (p.valid && (ND == 3 || (threadIdx.x & 3) == 0))
-    a.gtotals[(b % a.g.g[2]) * nrows + (uint64_t)(org[0] + p.z) * a.g.n[1] + org[1] + p.y] = sum;
+    a.gtotals[total_at(a, b % a.g.g[2], (uint64_t)(org[0] + p.z) * a.g.n[1] + org[1] + p.y, nrows)] = sum;
 }
 
 // Row sums to the sums before each block, in place (a thread per row).
@@ -1297,6 +1302,31 @@ __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
   }
 }
 
+// The same, a CTA per row and eight blocks a thread, the row's words side by side: for fields
+// much wider than they have rows, where a thread per row walks along x alone (4 x 4 x 1 M
+// elements: 2239 -> 17 us of a decompression that takes 2708 -> 368 us; 16 x 1.5 M: 842 us).
+__global__ __launch_bounds__(1024) void gx_carry_wide_kernel(DecodeArgs a) {
+  chained_begin();
+  __shared__ int32_t s_scan[33];
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint32_t nb = a.g.g[2];
+  int4* t = reinterpret_cast<int4*>(a.gtotals + blockIdx.x * a.gpitch);
+  int32_t carry = 0;
+  for (uint32_t i0 = 0; i0 < nb; i0 += 8 * blockDim.x) {
+    // (what lies between the row's end and its pitch comes behind every sum that is used)
+    const uint32_t i = i0 + 8 * threadIdx.x;
+    int4 v = make_int4(0, 0, 0, 0), w = v;
+    if (i < nb) v = t[i / 4];
+    if (i + 4 < nb) w = t[i / 4 + 1];
+    int32_t all;
+    const int32_t s0 = carry + block_excl_scan<int32_t>(v.x + v.y + v.z + v.w + w.x + w.y + w.z + w.w, s_scan, &all);
+    const int32_t s1 = s0 + v.x + v.y + v.z + v.w;
+    if (i < nb) t[i / 4] = make_int4(s0, s0 + v.x, s0 + v.x + v.y, s0 + v.x + v.y + v.z);
+    if (i + 4 < nb) t[i / 4 + 1] = make_int4(s1, s1 + w.x, s1 + w.x + w.y, s1 + w.x + w.y + w.z);
+    carry += all;
+  }
+}
+
 // Partial sums along x, over the whole row, and along y, within the block, of one block.
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
@@ -1311,7 +1341,8 @@ __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
   const RowPiece p = row_piece<ND>(w);
   int32_t k[16];
   load_fused16(a, b, p.j0, p.n, k);
-  int32_t carry = p.valid ? a.gtotals[(b % a.g.g[2]) * nrows + (uint64_t)(org[0] + p.z) * ny + org[1] + p.y] : 0;
+  int32_t carry =
+      p.valid ? a.gtotals[total_at(a, b % a.g.g[2], (uint64_t)(org[0] + p.z) * ny + org[1] + p.y, nrows)] : 0;
 #pragma unroll
   for (int i = 1; i < 16; i++) k[i] += k[i - 1];
   if (ND == 2) {
@@ -1502,6 +1533,24 @@ __global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state)
   }
 }
 
+// The last pass of 2-D fields: a thread per column and eight rows (which lie in one strip).
+__global__ __launch_bounds__(256) void gfinal_rows_kernel(DecodeArgs a) {
+  chained_begin();
+  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  const uint32_t ny = a.g.n[1], nx = a.g.n[2], nxb = (nx + 255) / 256;
+  const uint32_t y0 = 8 * (blockIdx.x / nxb), x = 256 * (blockIdx.x % nxb) + threadIdx.x;
+  if (x >= nx) return;
+  float* out = a.out + (uint64_t)y0 * nx + x;
+  const int32_t* q = reinterpret_cast<const int32_t*>(out);
+  const int32_t before = a.gstrips[(uint64_t)(y0 / a.g.blk[1]) * nx + x];
+  int32_t v[8];
+#pragma unroll
+  for (uint32_t i = 0; i < 8; i++) v[i] = y0 + i < ny ? q[(uint64_t)i * nx] : 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 8; i++)
+    if (y0 + i < ny) __stcs(&out[(uint64_t)i * nx], scale(v[i] + before, a.ebx2_f));
+}
+
 // Verbatim patches (after the last pass).
 __global__ void gpatch_kernel(DecodeArgs a) {
   chained_begin();
@@ -1520,7 +1569,7 @@ __global__ void gpatch_kernel(DecodeArgs a) {
 }
 
 // The global reconstruction's launches (after set-up, decoding and run expansion).
-cudaError_t launch_global_reconstruct(const DecodeArgs& a, cudaStream_t s) {
+cudaError_t launch_global_reconstruct(DecodeArgs a, cudaStream_t s) {
   trace_begin(K_RECONSTRUCT, s);
   const int nd = a.g.ndim;
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
@@ -1528,13 +1577,36 @@ cudaError_t launch_global_reconstruct(const DecodeArgs& a, cudaStream_t s) {
   if (nd == 1) {
     launch_chained(g1d_kernel, a.g.nblk, 256, 0, s, a, a.scan_state);
   } else {
-    if (nd == 2) launch_chained(grow_totals_kernel<2>, a.g.nblk, kRecThreads, 0, s, a);
-    else launch_chained(grow_totals_kernel<3>, a.g.nblk, kRecThreads, 0, s, a);
-    launch_chained(gx_carry_kernel, ctas(nz * ny), 256, 0, s, a);
-    if (nd == 2) launch_chained(gblock_kernel<2>, a.g.nblk, kRecThreads, 0, s, a);
-    else launch_chained(gblock_kernel<3>, a.g.nblk, kRecThreads, 0, s, a);
+    // a block's CTA needs no more threads than the field's rows and columns have work for
+    // (2-D: 64 columns by 16 rows a band, 3-D: 16 rows a plane)
+    const unsigned threads = nd == 2 ? 64u * (unsigned)((imin(64, ny) + 15) / 16) : (16u * imin(16, nz) + 31u) & ~31u;
+    // Row sums: a thread per row walks along its blocks alone, a CTA per row takes thousands at
+    // a time but the SMs hold few of them (eight of 256 threads an SM, or two of 1024 for as few
+    // rows).  A call with a thread and with a CTA per row: 16 rows of 40, 84 and 800 blocks 44 and
+    // 45, 46 and 46, 70 and 46 us; 3000 rows of 40, 84 and 400 blocks 87 and 89, 127 and 124, 445
+    // and 427 us; 8000 rows of 84 and 160 blocks 272 and 277, 530 and 531 us.  Hence the line.
+    const uint64_t nrows = nz * ny;
+    static int sms = 0;
+    if (sms == 0) {
+      int dev = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    const bool wide = a.g.g[2] > 64 + nrows / 80;
+    a.gpitch = wide ? (a.g.g[2] + 3ull) & ~3ull : 0;
+    if (nd == 2) launch_chained(grow_totals_kernel<2>, a.g.nblk, threads, 0, s, a);
+    else launch_chained(grow_totals_kernel<3>, a.g.nblk, threads, 0, s, a);
+    if (wide)
+      launch_chained(gx_carry_wide_kernel, (unsigned)nrows, nrows <= 2ull * sms ? 1024 : 256, 0, s, a);
+    else
+      launch_chained(gx_carry_kernel, ctas(nrows), 256, 0, s, a);
+    if (nd == 2) launch_chained(gblock_kernel<2>, a.g.nblk, threads, 0, s, a);
+    else launch_chained(gblock_kernel<3>, a.g.nblk, threads, 0, s, a);
     launch_chained(gy_carry_kernel, ctas(nz * nx), 256, 0, s, a);
-    launch_chained(gfinal_kernel, ctas(ny * nx), 256, 0, s, a);
+    if (nd == 2 && nx >= 256)
+      launch_chained(gfinal_rows_kernel, (unsigned)((nx + 255) / 256 * ((ny + 7) / 8)), 256, 0, s, a);
+    else
+      launch_chained(gfinal_kernel, ctas(ny * nx), 256, 0, s, a);
   }
   if (a.n_rec) launch_chained(gpatch_kernel, (unsigned)((a.n_rec + 255) / 256 < 1024 ? (a.n_rec + 255) / 256 : 1024), 256, 0, s, a);
   trace_end(K_RECONSTRUCT, s);

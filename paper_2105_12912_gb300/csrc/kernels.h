@@ -189,7 +189,8 @@ struct DecodeArgs {
   uint64_t* prep_lb;   // set-up chunks' look-back states (2 per 1024 blocks), zeroed per call
   int global;          // global (unchunked) Lorenzo archive: partial sums over the whole field
   uint64_t* scan_state;  // 1-D: their look-back states (one per block), zeroed per call
-  int32_t* gtotals;      // 2-D, 3-D: row sums by block along x, then the sums before each
+  int32_t* gtotals;      // 2-D, 3-D: row sums by block along x, then the sums before each,
+  uint64_t gpitch;       // [block][row], or where this is not 0 [row][block] at this pitch
   int32_t* gstrips;      // and the sums before each strip of blocks along y
   int dead;            // batches: the header failed validation, do nothing
   int check_hdr;       // the arguments come from a host copy of the header (hdr): the
