@@ -801,6 +801,73 @@ __device__ __forceinline__ void st_piece(void* p, const int32_t (&k)[16]) {
     reinterpret_cast<int4*>(p)[c] = make_int4(k[4 * c], k[4 * c + 1], k[4 * c + 2], k[4 * c + 3]);
 }
 
+// Edge blocks of 1-D and 2-D fields under the global predictor, by box element, then by dense
+// slot (not inlined: beside the full blocks' path its 17 elements a thread spill, and a field
+// thinner than a block has no others: 16 x 1.5 M elements, construct 589 us inlined, 366 so).
+// Returns error bits.
+template <int ND, typename E>
+__device__ __noinline__ uint32_t edge_codes_global(const ConstructArgs& A, SmemT<E, kHaloMax>& S, E* in,
+                                                   const uint32_t* w, uint32_t m, int32_t* dglob) {
+  static_assert(ND < 3, "3-D edge blocks go by rows (post_edge_rows)");
+  using H = Halo<ND>;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const Pq<E> pq(S.pq);
+  const int32_t r = (int32_t)A.radius;
+  int32_t* K = reinterpret_cast<int32_t*>(in);
+  uint32_t err = 0;
+  constexpr uint32_t NB = H::X * H::Y * H::Z;
+  constexpr uint32_t PER = (NB + kThreads - 1) / kThreads;
+  constexpr int hy = ND >= 2 ? 1 : 0;
+  if (tid < kSlots / 32) S.patch[tid] = 0;
+  __syncthreads();
+  // prequantize every box element the predictor reads (x >= -1) into registers
+  int32_t kv[PER];
+#pragma unroll
+  for (uint32_t i = 0; i < PER; i++) {
+    const uint32_t p = tid + kThreads * i;
+    kv[i] = 0;
+    if (p < NB) {
+      const int x = (int)(p % H::X) - (int)kHaloPadX, y = (int)(p / H::X) - hy;
+      if (x >= -1) {
+        bool patch = false;
+        if (!pq.fast(in[p], kv[i])) err |= pq.full(in[p], kv[i], patch);
+        if (patch && x >= 0 && y >= 0 && (uint32_t)x < w[2] && (uint32_t)y < w[1]) {
+          const uint32_t j = (uint32_t)y * w[2] + (uint32_t)x;
+          atomicOr(&S.patch[j >> 5], 1u << (j & 31));
+        }
+      }
+    }
+  }
+  __syncthreads();  // every element read: the box now carries k
+#pragma unroll
+  for (uint32_t i = 0; i < PER; i++) {
+    const uint32_t p = tid + kThreads * i;
+    if (p < NB) K[p] = kv[i];
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int i = 0; i < kPer; i++) {
+    const uint32_t j = tid + kThreads * i;
+    const bool inb = j < m;
+    uint32_t q = 0;
+    if (inb) {
+      const uint32_t y = ND == 2 ? j / w[2] : 0u, x = j - y * w[2];
+      const uint32_t p = (y + hy) * H::X + (x + kHaloPadX);
+      int32_t d = K[p] - K[p - 1];
+      if (ND >= 2) d -= K[p - H::X] - K[p - H::X - 1];
+      const uint32_t u = (uint32_t)(d + r);
+      q = u - 1u < (uint32_t)(2 * r - 1) ? u : 0u;  // |delta| < r
+      atomicAdd(&S.hc[q], 1u);
+      if (q == 0) dglob[j] = d;
+    }
+    S.c[j] = (uint16_t)q;  // zero beyond m
+    const uint32_t ob = __ballot_sync(~0u, inb && q == 0);
+    if (lane == 0) S.outl[j >> 5] = ob;
+  }
+  __syncthreads();
+  return err;
+}
+
 // Codes, records and histograms of codec block b under the global predictor: the mixed
 // difference (1 - S_x)(1 - S_y)(1 - S_z) k over the halo'd box (the paper's 1/2/3-D
 // predictor, Sec. IV-B2, with no chunk restarts), then the tail.
@@ -893,57 +960,7 @@ __device__ void process_tile_global(const ConstructArgs& A, uint32_t b, const ui
     tile_tail<ND == 3>(A, b, S, m, full, err, n_rec_acc, n_patch_acc);
     return;
   }
-  // edge blocks of 1-D and 2-D fields: by box element, then by dense slot
-  constexpr uint32_t NB = H::X * H::Y * H::Z;
-  constexpr uint32_t PER = (NB + kThreads - 1) / kThreads;
-  constexpr int hy = ND >= 2 ? 1 : 0;
-  if (tid < kSlots / 32) S.patch[tid] = 0;
-  __syncthreads();
-  // prequantize every box element the predictor reads (x >= -1) into registers
-  int32_t kv[PER];
-#pragma unroll
-  for (uint32_t i = 0; i < PER; i++) {
-    const uint32_t p = tid + kThreads * i;
-    kv[i] = 0;
-    if (p < NB) {
-      const int x = (int)(p % H::X) - (int)kHaloPadX, y = (int)(p / H::X) - hy;
-      if (x >= -1) {
-        bool patch = false;
-        if (!pq.fast(in[p], kv[i])) err |= pq.full(in[p], kv[i], patch);
-        if (patch && x >= 0 && y >= 0 && (uint32_t)x < w[2] && (uint32_t)y < w[1]) {
-          const uint32_t j = (uint32_t)y * w[2] + (uint32_t)x;
-          atomicOr(&S.patch[j >> 5], 1u << (j & 31));
-        }
-      }
-    }
-  }
-  __syncthreads();  // every element read: the box now carries k
-#pragma unroll
-  for (uint32_t i = 0; i < PER; i++) {
-    const uint32_t p = tid + kThreads * i;
-    if (p < NB) K[p] = kv[i];
-  }
-  __syncthreads();
-#pragma unroll 4
-  for (int i = 0; i < kPer; i++) {
-    const uint32_t j = tid + kThreads * i;
-    const bool inb = j < m;
-    uint32_t q = 0;
-    if (inb) {
-      const uint32_t y = ND == 2 ? j / w[2] : 0u, x = j - y * w[2];
-      const uint32_t p = (y + hy) * H::X + (x + kHaloPadX);
-      int32_t d = K[p] - K[p - 1];
-      if (ND >= 2) d -= K[p - H::X] - K[p - H::X - 1];
-      const uint32_t u = (uint32_t)(d + r);
-      q = u - 1u < (uint32_t)(2 * r - 1) ? u : 0u;  // |delta| < r
-      atomicAdd(&S.hc[q], 1u);
-      if (q == 0) dglob[j] = d;
-    }
-    S.c[j] = (uint16_t)q;  // zero beyond m
-    const uint32_t ob = __ballot_sync(~0u, inb && q == 0);
-    if (lane == 0) S.outl[j >> 5] = ob;
-  }
-  __syncthreads();
+  if constexpr (ND < 3) err |= edge_codes_global<ND, E>(A, S, in, box + 3, m, dglob);
   run_head_words(S.c, m, S.head);
   __syncthreads();
   tile_tail<false>(A, b, S, m, false, err, n_rec_acc, n_patch_acc);
