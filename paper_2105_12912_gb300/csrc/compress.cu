@@ -809,15 +809,12 @@ __device__ __noinline__ void place_records(const EncodeArgs& a, uint32_t b, cons
   }
 }
 
-// The nr runs of a block: their values and lengths, in order, from its codes and the run
-// starts that construction left as bits.  A thread takes 16 consecutive codes; runs before
-// them are counted in the bit words, which every warp reads for itself, so one barrier
-// comes before the lengths and one after them.  s_at: scratch, the run starts.  (Finding the
-// starts again from codes in shared memory took three more barriers, with one warp's index of
-// the words between them: 40 mixed fields, most of their blocks in runs, compression 553 ->
-// 511 us.)  All threads.
-__device__ __noinline__ void extract_runs(const uint16_t* codes, const uint32_t* heads, uint32_t m, uint32_t nr,
-                                          uint16_t* s_at, uint16_t* s_rv, uint16_t* s_rl) {
+// The runs of a block: their values and starts, in order, from its codes and the run starts
+// that construction left as bits.  A thread takes 16 consecutive codes; runs before them are
+// counted in the bit words, which every warp reads for itself.  All threads; a barrier
+// follows at the caller.
+__device__ __forceinline__ void scatter_runs(const uint16_t* codes, const uint32_t* heads, uint16_t* s_at,
+                                             uint16_t* s_rv) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint4* src = reinterpret_cast<const uint4*>(codes + 16 * tid);
   const uint4 c0 = __ldcg(&src[0]), c1 = __ldcg(&src[1]), w4 = __ldcg(&reinterpret_cast<const uint4*>(heads)[lane]);
@@ -833,8 +830,23 @@ __device__ __noinline__ void extract_runs(const uint16_t* codes, const uint32_t*
       run++;
     }
   }
+}
+
+// Length of run i of nr in a block of m codes, the starts being at.
+__device__ __forceinline__ uint32_t run_length(const uint16_t* at, uint32_t i, uint32_t nr, uint32_t m) {
+  return (i + 1 < nr ? at[i + 1] : m) - at[i];
+}
+
+// The nr runs of a block: their values and lengths, with one barrier before the lengths and one
+// after them.  s_at: scratch, the run starts.  (Finding the starts again from codes in shared
+// memory took three more barriers, with one warp's index of the words between them: 40 mixed
+// fields, most of their blocks in runs, compression 553 -> 511 us.)  All threads.
+__device__ __noinline__ void extract_runs(const uint16_t* codes, const uint32_t* heads, uint32_t m, uint32_t nr,
+                                          uint16_t* s_at, uint16_t* s_rv, uint16_t* s_rl) {
+  const uint32_t tid = threadIdx.x;
+  scatter_runs(codes, heads, s_at, s_rv);
   __syncthreads();
-  for (uint32_t i = tid; i < nr; i += kEncThreads) s_rl[i] = (uint16_t)((i + 1 < nr ? s_at[i + 1] : m) - s_at[i]);
+  for (uint32_t i = tid; i < nr; i += kEncThreads) s_rl[i] = (uint16_t)run_length(s_at, i, nr, m);
   __syncthreads();
 }
 
@@ -1369,6 +1381,49 @@ __device__ void payload_body(const EncodeArgs& a, uint32_t b, uint32_t m, uint32
   if (b == 0) finish_field(a);
 }
 
+// Forced RLE: a block's size is its run count's, so its plan needs no runs, and its payload
+// takes them from the codes.  (A store and a reload of every run between the two, as for blocks
+// picked by size, took more than the rest where runs are short: 100x500x500 walk, rel 1e-4,
+// compression 427 us; now 271.)  Kernels of their own, for the registers of the others.
+__device__ void plan_rle_body(const EncodeArgs& a, uint32_t b, const uint32_t* box, unsigned char* smem) {
+  const uint32_t nr = a.block_runs[b], records = a.rec.counts[b];
+  if (encode_status(a) & ERR_TIMEOUT) return;
+  if (records != 0) place_records(a, b, box, box + 3, reinterpret_cast<uint64_t*>(smem));
+  if (threadIdx.x == 0) {
+    a.ar[a.off_codec + b] = (uint8_t)CODEC_RLE;
+    reinterpret_cast<uint32_t*>(a.ar + a.off_bb)[b] = 4 * nr;
+    atomicAdd(reinterpret_cast<unsigned long long*>(a.groups) + b / kGroup, (unsigned long long)(4 * nr) | 1ull << 40);
+  }
+}
+
+__device__ void payload_rle_body(const EncodeArgs& a, uint32_t b, uint32_t m, unsigned char* smem) {
+  uint16_t* s_rv = reinterpret_cast<uint16_t*>(smem);  // 4096 run values, 4096 run starts
+  uint16_t* s_at = s_rv + kSlots;
+  __shared__ uint64_t s_sum[kEncThreads / 32];
+  const uint32_t tid = threadIdx.x;
+  const uint32_t* bb = reinterpret_cast<const uint32_t*>(a.ar + a.off_bb);
+  const uint32_t nr = a.block_runs[b], group = b / kGroup;
+  uint64_t before = tid < b % kGroup ? (uint64_t)__ldcg(&bb[group * kGroup + tid]) : 0ull;
+  for (uint32_t k = tid; k < group; k += kEncThreads) before += __ldcg(&a.groups[k]) & kGroupBytes;
+  uint64_t dst_off = a.off_rec + 8ull * __ldcg(&a.st->n_rec);
+  if (encode_status(a) & ERR_TIMEOUT) return;
+  scatter_runs(a.codes + (uint64_t)b * kSlots, a.masks + (uint64_t)b * kMaskWords + 2 * (kSlots / 32), s_at, s_rv);
+  before = warp_sum(before);
+  if ((tid & 31) == 0) s_sum[tid >> 5] = before;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kEncThreads / 32; w++) dst_off += s_sum[w];
+  if (dst_off + 4 * nr > a.cap) {
+    if (tid == 0) atomicOr(&a.st->status, ERR_CAPACITY);
+  } else {
+    // nr values, then nr lengths, two a word
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.ar + dst_off);
+    auto unit = [&](uint32_t i) -> uint32_t { return i < nr ? s_rv[i] : run_length(s_at, i - nr, nr, m); };
+    for (uint32_t i = tid; i < nr; i += kEncThreads) dst[i] = unit(2 * i) | unit(2 * i + 1) << 16;
+  }
+  if (b == 0) finish_field(a);
+}
+
 // (four CTAs an SM: with the registers of five the plan spills, 3-D 512^3 compression 818
 // against 805 us, 40 mixed fields 486 against 474; the payload's place is better at five)
 __global__ __launch_bounds__(kEncThreads, 4) void plan_kernel(EncodeArgs a) {
@@ -1387,6 +1442,24 @@ __global__ __launch_bounds__(kEncThreads, 5) void payload_kernel(EncodeArgs a) {
   if (threadIdx.x == 0) s_m = block_elems(a.g, blockIdx.x);
   __syncthreads();
   payload_body(a, blockIdx.x, s_m, encode_status(a), smem);
+}
+
+__global__ __launch_bounds__(kEncThreads) void plan_rle_kernel(EncodeArgs a) {
+  chained_begin();
+  __shared__ uint32_t s_box[6];
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (threadIdx.x == 0) block_box(a.g, blockIdx.x, s_box, s_box + 3);
+  __syncthreads();
+  plan_rle_body(a, blockIdx.x, s_box, smem);
+}
+
+__global__ __launch_bounds__(kEncThreads) void payload_rle_kernel(EncodeArgs a) {
+  chained_begin();
+  __shared__ uint32_t s_m;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (threadIdx.x == 0) s_m = block_elems(a.g, blockIdx.x);
+  __syncthreads();
+  payload_rle_body(a, blockIdx.x, s_m, smem);
 }
 
 __device__ __forceinline__ int field_of_prefix(const uint32_t* prefix, int nfields, uint32_t c) {
@@ -1640,6 +1713,12 @@ cudaError_t launch_codebook(const BookArgs& a, cudaStream_t s) {
 
 cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s) {
   trace_begin(K_ENCODE, s);
+  if (a.select == SEL_RLE && !a.analyze) {
+    launch_chained(plan_rle_kernel, a.g.nblk, kEncThreads, 33 * 8, s, a);
+    launch_chained(payload_rle_kernel, a.g.nblk, kEncThreads, 4 * kSlots, s, a);
+    trace_end(K_ENCODE, s);
+    return cudaGetLastError();
+  }
   launch_chained(plan_kernel, a.g.nblk, kEncThreads, plan_smem_bytes(), s, a);
   if (!a.analyze) launch_chained(payload_kernel, a.g.nblk, kEncThreads, payload_smem_bytes(), s, a);
   trace_end(K_ENCODE, s);
