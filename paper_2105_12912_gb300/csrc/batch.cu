@@ -181,6 +181,37 @@ cudaError_t enqueue_plan(const csz_batch* b, cudaStream_t s) {
   return b->persistent ? enqueue_persistent(b, b->persist_grid, s) : enqueue(b, b->construct_grid, s);
 }
 
+// The plan as a graph, captured on a private stream (the caller's may be the legacy default
+// stream, which cannot be captured).  *step names what failed.
+cudaError_t capture_plan(const csz_batch* b, cudaGraphExec_t* exec, const char** step) {
+  const bool tracing = trace_suspend();
+  cudaGraph_t graph = nullptr;
+  cudaStream_t cap = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+  *step = "capture stream";
+  if (e == cudaSuccess) {
+    e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    *step = "begin capture";
+  }
+  if (e == cudaSuccess) {
+    const cudaError_t e2 = enqueue_plan(b, cap);
+    e = cudaStreamEndCapture(cap, &graph);
+    *step = "end capture";
+    if (e == cudaSuccess && e2 != cudaSuccess) {
+      e = e2;
+      *step = "captured launches";
+    }
+  }
+  if (e == cudaSuccess) {
+    e = cudaGraphInstantiate(exec, graph, 0);
+    *step = "instantiate";
+  }
+  if (graph) cudaGraphDestroy(graph);
+  if (cap) cudaStreamDestroy(cap);
+  trace_resume(tracing);
+  return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -372,8 +403,9 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
 
   // The plan: one persistent launch (default) or the staged launches, and its grid.
   // With CSZ_BATCH_AUTOTUNE every allowed candidate is timed on the batch (resident
-  // CTAs per SM 1..4 for either plan) and the fastest is kept; the archives do not
-  // depend on the choice.
+  // CTAs per SM 1..4 for either plan); each plan's fastest grid is kept, and of the two
+  // plans the one whose graph replays faster.  The archives do not depend on the choice.
+  float best_staged = 0.0f, best_persist = 0.0f;  // (0: not timed)
   const bool allow_staged = (autotune & CSZ_BATCH_STAGED) || !(autotune & CSZ_BATCH_PERSISTENT);
   const int pmax = persist_grid_max();
   const bool allow_persist = pmax > 0 && ((autotune & CSZ_BATCH_PERSISTENT) || !(autotune & CSZ_BATCH_STAGED));
@@ -389,7 +421,6 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    float best = 0.0f;
     auto time_it = [&](bool persist, int grid, float& ms) {
       for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {
         cudaEventRecord(e0, s);
@@ -406,8 +437,8 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
       time_it(false, grid, ms);
       if (e != cudaSuccess) break;
       b->tuned_ms[k - 1] = ms;
-      if (best == 0.0f || ms < best) {
-        best = ms;
+      if (best_staged == 0.0f || ms < best_staged) {
+        best_staged = ms;
         b->tuned_grid = grid;
         b->construct_grid = grid;
         b->persistent = 0;
@@ -421,8 +452,8 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
       time_it(true, grid, ms);
       if (e != cudaSuccess) break;
       b->persist_ms[k - 1] = ms;
-      if (best == 0.0f || ms < best) {
-        best = ms;
+      if (best_persist == 0.0f || ms < best_persist) {
+        best_persist = ms;
         b->persist_grid = grid;
         b->persistent = 1;
       }
@@ -436,33 +467,40 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
     }
   }
 
-  // capture the launch sequence once, on a private stream (the caller's may be the
-  // legacy default stream, which cannot be captured); replays go to any stream
-  const bool tracing = trace_suspend();
-  cudaGraph_t graph = nullptr;
-  cudaStream_t cap = nullptr;
-  e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-  const char* step = "capture stream";
-  if (e == cudaSuccess) {
-    e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-    step = "begin capture";
-  }
-  if (e == cudaSuccess) {
-    const cudaError_t e2 = enqueue_plan(b, cap);
-    e = cudaStreamEndCapture(cap, &graph);
-    step = "end capture";
-    if (e == cudaSuccess && e2 != cudaSuccess) {
-      e = e2;
-      step = "captured launches";
+  // capture the launch sequence once; replays go to any stream
+  const char* step = "";
+  if (best_staged > 0.0f && best_persist > 0.0f) {
+    // Both plans' best grids, as they will run: in a graph, where the staged plan's launches
+    // follow each other more closely than the tuner's did (4 x 64 K elements, forced RLE:
+    // replays of 53 and 62 us, while the launches by themselves favoured the second).
+    cudaGraphExec_t exec[2] = {};
+    float ms[2] = {};
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    for (int k = 0; k < 2 && e == cudaSuccess; k++) {
+      b->persistent = k;
+      e = capture_plan(b, &exec[k], &step);
     }
+    if (e == cudaSuccess) e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    for (int rep = 0; rep < 8 && e == cudaSuccess; rep++) {  // (in turn; the first pair warms up)
+      const int k = rep & 1;
+      step = "autotune replay";
+      e = cudaEventRecord(e0, s);
+      if (e == cudaSuccess) e = cudaGraphLaunch(exec[k], s);
+      if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+      float t = 0.0f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+      if (rep >= 2 && (ms[k] == 0.0f || t < ms[k])) ms[k] = t;
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    b->persistent = ms[1] < ms[0] ? 1 : 0;
+    b->exec = exec[b->persistent];
+    if (exec[1 - b->persistent]) cudaGraphExecDestroy(exec[1 - b->persistent]);
+  } else {
+    e = capture_plan(b, &b->exec, &step);
   }
-  if (e == cudaSuccess) {
-    e = cudaGraphInstantiate(&b->exec, graph, 0);
-    step = "instantiate";
-  }
-  if (graph) cudaGraphDestroy(graph);
-  if (cap) cudaStreamDestroy(cap);
-  trace_resume(tracing);
   if (failed(e, step)) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     delete b;
