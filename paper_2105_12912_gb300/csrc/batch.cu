@@ -410,14 +410,12 @@ csz_status csz_batch_create(int nfields, const csz_field* fields, const csz_opti
   const int pmax = persist_grid_max();
   const bool allow_persist = pmax > 0 && ((autotune & CSZ_BATCH_PERSISTENT) || !(autotune & CSZ_BATCH_STAGED));
   const int full = construct_grid(tiles);
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   b->tuned_grid = full;
   b->construct_grid = full;
   b->persist_grid = pmax;
   b->persistent = allow_persist ? 1 : 0;
-  if ((autotune & CSZ_BATCH_AUTOTUNE) && sms > 0) {
+  if (autotune & CSZ_BATCH_AUTOTUNE) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -708,11 +706,8 @@ csz_status csz_batch_dec_create(int nfields, const csz_dfield* fields, void* d_w
   int common_nd = gs[0].ndim;
   uint64_t blocks = 0;
   for (const Geom& g : gs) blocks += g.nblk;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   uint32_t rounds = kDecChunkRounds;
-  while (rounds > 1 && blocks / (rounds * (uint32_t)kDecShapes[1] / 2) < (uint64_t)kDecChunkWaves * (uint32_t)(sms > 0 ? sms : 1))
+  while (rounds > 1 && blocks / (rounds * (uint32_t)kDecShapes[1] / 2) < (uint64_t)kDecChunkWaves * (uint32_t)sm_count())
     rounds /= 2;
   for (int f = 1; f < nfields; f++)
     if (gs[f].ndim != common_nd) common_nd = 0;

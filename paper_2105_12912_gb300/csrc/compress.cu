@@ -1644,26 +1644,24 @@ size_t persist_len_book_bytes() { return book_mem_bytes(kNsymLen); }
 
 template <int ND>
 static int persist_occupancy() {
-  static int occ = -1;
-  if (occ < 0) {
+  static PerDevice occ_and_one;
+  return occ_and_one.get([] {
+    int occ = 0;
     const int sm = (int)persist_smem_bytes();
     if (cudaFuncSetAttribute(batch_persistent_kernel<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) !=
             cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batch_persistent_kernel<ND>, kPersistThreads, sm) !=
             cudaSuccess)
       occ = 0;
-  }
-  return occ;
+    return occ + 1;
+  }) - 1;
 }
 
 int persist_grid_max() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int occ = persist_occupancy<0>();
   for (int o : {persist_occupancy<1>(), persist_occupancy<2>(), persist_occupancy<3>()})
     if (o < occ) occ = o;
-  return occ * (sms > 0 ? sms : 0);
+  return occ * sm_count();
 }
 
 cudaError_t launch_batch_persistent(const PersistArgs& p, int grid, int nd, cudaStream_t s) {
@@ -1728,15 +1726,8 @@ cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s) {
 }
 
 uint32_t range_ctas(uint64_t n) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
-  }
-  const uint64_t want = (n / 4 + 255) / 256;
-  const uint64_t grid = want < (uint64_t)sms * 8 ? want : (uint64_t)sms * 8;
+  const uint64_t want = (n / 4 + 255) / 256, most = 8ull * sm_count();
+  const uint64_t grid = want < most ? want : most;
   return grid ? (uint32_t)grid : 1u;
 }
 

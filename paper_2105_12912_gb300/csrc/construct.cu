@@ -30,21 +30,16 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const EncodeTiledFn fn = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+    const bool found = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                           cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess;
+    return found ? reinterpret_cast<EncodeTiledFn>(p) : EncodeTiledFn(nullptr);
+  }();
   return fn;
 }
-
-int g_sms = 0;
 
 }  // namespace
 
@@ -97,19 +92,10 @@ void prepare_construct_task(ConstructTask& T) {
 template <int ND, typename E, bool G>
 int grid_of(uint32_t ntiles) {
   using SM = SmemT<E, G ? kHaloMax : kSlots>;
-  static int occ = 0;
-  if (g_sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_sms <= 0) g_sms = 1;
-  }
-  if (occ == 0) {
-    cudaFuncSetAttribute(construct_kernel<ND, E, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, construct_kernel<ND, E, G>, kThreads, sizeof(SM));
-    if (occ <= 0) occ = 1;
-  }
-  const uint64_t cap = (uint64_t)g_sms * occ;
+  static PerDevice occ;
+  const uint64_t cap = (uint64_t)sm_count() * occ.get([] {
+    return allow_and_count(construct_kernel<ND, E, G>, kThreads, sizeof(SM), sizeof(SM));
+  });
   return (int)(ntiles < cap ? (ntiles ? ntiles : 1) : cap);
 }
 

@@ -1586,18 +1586,12 @@ cudaError_t launch_global_reconstruct(DecodeArgs a, cudaStream_t s) {
     // 45, 46 and 46, 70 and 46 us; 3000 rows of 40, 84 and 400 blocks 87 and 89, 127 and 124, 445
     // and 427 us; 8000 rows of 84 and 160 blocks 272 and 277, 530 and 531 us.  Hence the line.
     const uint64_t nrows = nz * ny;
-    static int sms = 0;
-    if (sms == 0) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
     const bool wide = a.g.g[2] > 64 + nrows / 80;
     a.gpitch = wide ? (a.g.g[2] + 3ull) & ~3ull : 0;
     if (nd == 2) launch_chained(grow_totals_kernel<2>, a.g.nblk, threads, 0, s, a);
     else launch_chained(grow_totals_kernel<3>, a.g.nblk, threads, 0, s, a);
     if (wide)
-      launch_chained(gx_carry_wide_kernel, (unsigned)nrows, nrows <= 2ull * sms ? 1024 : 256, 0, s, a);
+      launch_chained(gx_carry_wide_kernel, (unsigned)nrows, nrows <= 2ull * sm_count() ? 1024 : 256, 0, s, a);
     else
       launch_chained(gx_carry_kernel, ctas(nrows), 256, 0, s, a);
     if (nd == 2) launch_chained(gblock_kernel<2>, a.g.nblk, threads, 0, s, a);
@@ -1812,26 +1806,18 @@ cudaError_t launch_decode_stages(const DecodeArgs& a, cudaStream_t s) {
     // warps per CTA: a stream is a chain of dependent steps, so a field with fewer streams
     // than the chip's SMs take at full occupancy spreads them over more, smaller CTAs
     // (each stages its own tables)
-    static int sms = 0, occ[4][4][3] = {};
     auto k = nd == 1 ? stream_decode_kernel<1, E> : (nd == 2 ? stream_decode_kernel<2, E> : stream_decode_kernel<3, E>);
-    if (sms == 0) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      for (auto kk : {stream_decode_kernel<1, E>, stream_decode_kernel<2, E>, stream_decode_kernel<3, E>})
-        cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stream_smem_bytes(3, kStreamWarps));
-    }
+    const int sms = sm_count();
     const uint64_t streams = 2ull * a.g.nblk;
     const int wi = streams >= 32ull * sms ? 2 : (streams >= 8ull * sms ? 1 : 0);
     const int warps = 4 << wi;
     static_assert(kStreamWarps == 16, "4, 8 or 16 warps");
     const size_t smem = stream_smem_bytes(nluts, warps);
-    if (occ[nd][nluts][wi] == 0) {
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[nd][nluts][wi], k, 32 * warps, smem);
-      if (occ[nd][nluts][wi] <= 0) occ[nd][nluts][wi] = 1;
-    }
+    static PerDevice occ[4][4][3];
+    const int per_sm = occ[nd][nluts][wi].get(
+        [&] { return allow_and_count(k, 32 * warps, smem, stream_smem_bytes(3, kStreamWarps)); });
     const uint64_t want = (streams + warps - 1) / warps;
-    const uint64_t cap = (uint64_t)sms * occ[nd][nluts][wi];
+    const uint64_t cap = (uint64_t)sms * per_sm;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
     trace_begin(K_STREAM_DECODE, s);
     launch_chained(k, grid, 32 * warps, smem, s, a);

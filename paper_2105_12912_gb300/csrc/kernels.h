@@ -3,12 +3,54 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 
 namespace cszp {
+
+// A value found once per device, by whichever thread comes first while the others wait: an SM
+// count, or a kernel's occupancy together with the shared-memory limit that is set for it
+// (the limit is the device's, and a launch before it is set is refused).
+class PerDevice {
+ public:
+  template <typename F>
+  int get(F find) {  // find() > 0
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return find();
+    std::lock_guard<std::mutex> lock(mu_);
+    if (v_[dev] == 0) v_[dev] = find();
+    return v_[dev];
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::mutex mu_;
+  int v_[kDevices] = {};
+};
+
+inline int sm_count() {
+  static PerDevice sms;
+  return sms.get([] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+  });
+}
+
+// CTAs of `threads` threads and `smem` bytes of dynamic shared memory that an SM holds (at
+// least 1), after allowing the kernel `most` bytes.
+template <typename K>
+inline int allow_and_count(K kernel, int threads, size_t smem, size_t most) {
+  int occ = 0;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
+  return occ > 0 ? occ : 1;
+}
 
 // A launch whose CTAs may take their places on the SMs while the launch before it on the
 // stream still runs (programmatic dependent launch): the kernel begins with

@@ -325,19 +325,12 @@ __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* pa
   }
 }
 
-int g_sms = 0;
-
 int train_grid(uint64_t nrows) {
-  if (g_sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_sms <= 0) g_sms = 1;
-  }
+  const int sms = sm_count();
   // a CTA an SM, or two in turn where a warp would add more than 32 rows into one FP32 sum
   // (its rounding grows with them)
   const uint64_t want = (nrows + 4 * kTrainWarps - 1) / (4 * kTrainWarps);
-  const int ctas = nrows > 32ull * kTrainWarps * (uint64_t)g_sms ? 2 * g_sms : g_sms;
+  const int ctas = nrows > 32ull * kTrainWarps * (uint64_t)sms ? 2 * sms : sms;
   const uint64_t cap = (uint64_t)(ctas < kMaxParts ? ctas : kMaxParts);
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
