@@ -381,7 +381,9 @@ const char* csz_status_string(int status);
 /*
  * Kernel tracing (benchmarking aid; process-global, not thread-safe).
  * csz_kernel_count() kernels are numbered 0..count-1 and named by csz_kernel_name().
- * Launch counts are always kept.  While tracing is enabled every launch is bracketed
+ * Launch counts are always kept; a stage of several launches has the further ones
+ * counted under a name of their own, without time ("encode_payload": its time is in
+ * "encode"; "global_passes": in "reconstruct").  While tracing is enabled every launch is bracketed
  * by CUDA events on the caller's stream and the elapsed milliseconds are added to the
  * kernel's total at the call's synchronisation.  While tracing is enabled,
  * csz_batch_compress and csz_batch_decompress launch their kernels one by one instead

@@ -111,6 +111,7 @@ void trace_end(int id, cudaStream_t s) {
   cudaEventRecord(g_trace.ev[id][1], s);
   g_trace.armed[id] = true;
 }
+void trace_further(int id, int launches) { g_trace.launches[id] += launches; }
 bool trace_suspend() {
   const bool on = g_trace.on;
   g_trace.on = false;
@@ -124,7 +125,7 @@ void trace_count_batch(bool persistent) {
     g_trace.launches[K_BATCH]++;
     return;
   }
-  for (int k : {K_RANGE, K_CONSTRUCT, K_CODEBOOK, K_ENCODE}) g_trace.launches[k]++;
+  for (int k : {K_RANGE, K_CONSTRUCT, K_CODEBOOK, K_ENCODE, K_ENCODE_PAYLOAD}) g_trace.launches[k]++;
 }
 void trace_count_decode_batch() {
   for (int k : {K_DEC_HEADER, K_DEC_SETUP, K_STREAM_DECODE, K_RECONSTRUCT}) g_trace.launches[k]++;
@@ -136,7 +137,7 @@ extern "C" {
 static const char* const kKernelNames[K_COUNT] = {
     "range", "abs_params", "construct", "codebook", "encode", "dec_setup",
     "stream_decode", "rle_expand", "reconstruct", "mlp_predict", "mlp_grad", "mlp_update", "dec_status",
-    "dec_header", "batch_persistent"};
+    "dec_header", "batch_persistent", "encode_payload", "global_passes"};
 
 int csz_kernel_count(void) { return K_COUNT; }
 

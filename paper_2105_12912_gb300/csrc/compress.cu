@@ -1716,11 +1716,15 @@ cudaError_t launch_encode(const EncodeArgs& a, cudaStream_t s) {
   if (a.select == SEL_RLE && !a.analyze) {
     launch_chained(plan_rle_kernel, a.g.nblk, kEncThreads, 33 * 8, s, a);
     launch_chained(payload_rle_kernel, a.g.nblk, kEncThreads, 4 * kSlots, s, a);
+    trace_further(K_ENCODE_PAYLOAD, 1);
     trace_end(K_ENCODE, s);
     return cudaGetLastError();
   }
   launch_chained(plan_kernel, a.g.nblk, kEncThreads, plan_smem_bytes(), s, a);
-  if (!a.analyze) launch_chained(payload_kernel, a.g.nblk, kEncThreads, payload_smem_bytes(), s, a);
+  if (!a.analyze) {
+    launch_chained(payload_kernel, a.g.nblk, kEncThreads, payload_smem_bytes(), s, a);
+    trace_further(K_ENCODE_PAYLOAD, 1);
+  }
   trace_end(K_ENCODE, s);
   return cudaGetLastError();
 }
@@ -1767,6 +1771,7 @@ cudaError_t launch_encode_batch(const EncodeArgs* d_tasks, const uint32_t* d_til
   // (chained to the plans: two launches cost a small batch about as much as the one they
   // replaced; 4 x 64 K elements, forced RLE, staged: 54 -> 53 us, 52 in one launch)
   launch_chained(payload_batch_kernel, ntiles, kEncThreads, payload_smem_bytes(), s, d_tasks, d_tile0, nfields);
+  trace_further(K_ENCODE_PAYLOAD, 1);
   trace_end(K_ENCODE, s);
   return cudaGetLastError();
 }

@@ -1602,6 +1602,7 @@ cudaError_t launch_global_reconstruct(DecodeArgs a, cudaStream_t s) {
     else
       launch_chained(gfinal_kernel, ctas(ny * nx), 256, 0, s, a);
   }
+  trace_further(K_GLOBAL_PASSES, (nd == 1 ? 0 : 4) + (a.n_rec ? 1 : 0));
   if (a.n_rec) launch_chained(gpatch_kernel, (unsigned)((a.n_rec + 255) / 256 < 1024 ? (a.n_rec + 255) / 256 : 1024), 256, 0, s, a);
   trace_end(K_RECONSTRUCT, s);
   return cudaGetLastError();

@@ -256,10 +256,14 @@ enum KernelId : int {
   K_DEC_STATUS,
   K_DEC_HEADER,
   K_BATCH,  // the batched persistent compression kernel
+  // further launches of a stage, counted here; their time is in the stage's own entry
+  K_ENCODE_PAYLOAD,  // K_ENCODE's second launch
+  K_GLOBAL_PASSES,   // K_RECONSTRUCT's after the first, global prediction
   K_COUNT
 };
 void trace_begin(int id, cudaStream_t s);
 void trace_end(int id, cudaStream_t s);
+void trace_further(int id, int launches);  // count launches without events of their own
 bool trace_suspend();           // stop event tracing (stream capture); returns the old state
 bool trace_on();                // event tracing is enabled
 void trace_fold();              // fold the recorded events into the totals (after a synchronisation)
