@@ -20,6 +20,11 @@ namespace cszp {
 
 __device__ __forceinline__ void flag(DevState* st, uint32_t bits) { atomicOr(&st->status, bits); }
 
+// A field whose set-up found it corrupt, or whose set-up gave up a wait, has no payload
+// offsets, block lists or run codes that may be used as such: the launches that follow leave
+// its output alone.
+__device__ __forceinline__ bool undecodable(uint32_t status) { return (status & (ERR_CORRUPT | ERR_TIMEOUT)) != 0; }
+
 // =================================================================================
 // archive validation and offsets
 // =================================================================================
@@ -792,7 +797,7 @@ __device__ void stream_decode_body(const DecodeArgs& a, uint32_t b_begin, uint32
   // that a corruption flagged by another CTA meanwhile cannot split this CTA
   __shared__ uint32_t s_next;  // batches: the chunk's next stream slot
   if (threadIdx.x == 0) {
-    s_go = !(a.st->status & ERR_CORRUPT);
+    s_go = !undecodable(a.st->status);
     s_next = 0;
   }
   const bool huff = (a.flags & 1u) != 0, rle = (a.flags & 2u) != 0;
@@ -1013,7 +1018,7 @@ __global__ __launch_bounds__(kRecThreads) void rle_expand_kernel(DecodeArgs a) {
   if (codec != CODEC_RLE && codec != CODEC_RLE_HUFF) return;
   // the status is read once, by thread 0, and acted on after the barrier, so that a
   // corruption flagged by another CTA meanwhile cannot split this CTA's threads
-  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT);
+  if (threadIdx.x == 0) S.go = !undecodable(a.st->status);
   __syncthreads();
   if (!S.go) return;
   uint32_t org[3], w[3], c[8];
@@ -1226,7 +1231,7 @@ __global__ __launch_bounds__(kRecThreads, 6) void reconstruct_kernel(DecodeArgs 
   if (a.dead) return;
   // the status is read once, by thread 0 (run expansions in other CTAs may flag
   // corruption meanwhile), so every thread takes the same path
-  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT) && blockIdx.x < a.st->n_slow;
+  if (threadIdx.x == 0) S.go = !undecodable(a.st->status) && blockIdx.x < a.st->n_slow;
   __syncthreads();
   if (!S.go) return;
   reconstruct_body<ND, E>(a, a.slowblk[blockIdx.x], S);
@@ -1262,7 +1267,7 @@ __device__ __forceinline__ uint64_t total_at(const DecodeArgs& a, uint32_t bx, u
 template <int ND>
 __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint32_t b = blockIdx.x;
   uint32_t org[3], w[3];
   block_box(a.g, b, org, w);
@@ -1283,7 +1288,7 @@ __global__ __launch_bounds__(kRecThreads) void grow_totals_kernel(DecodeArgs a) 
 // Row sums to the sums before each block, in place (a thread per row).
 __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint64_t nrows = (uint64_t)a.g.n[0] * a.g.n[1];
   const uint64_t row = blockIdx.x * 256ull + threadIdx.x;
   if (row >= nrows) return;
@@ -1308,7 +1313,7 @@ __global__ __launch_bounds__(256) void gx_carry_kernel(DecodeArgs a) {
 __global__ __launch_bounds__(1024) void gx_carry_wide_kernel(DecodeArgs a) {
   chained_begin();
   __shared__ int32_t s_scan[33];
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint32_t nb = a.g.g[2];
   int4* t = reinterpret_cast<int4*>(a.gtotals + blockIdx.x * a.gpitch);
   int32_t carry = 0;
@@ -1333,7 +1338,7 @@ __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
   chained_begin();
   __shared__ __align__(16) int32_t s_k[kSlots];
   __shared__ int32_t s_band[4][64];
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint32_t b = blockIdx.x, tid = threadIdx.x;
   uint32_t org[3], w[3];
   block_box(a.g, b, org, w);
@@ -1394,7 +1399,7 @@ __global__ __launch_bounds__(kRecThreads) void gblock_kernel(DecodeArgs a) {
 // strips before it (a thread per plane and column): gstrips[(z gy + by) nx + x].
 __global__ __launch_bounds__(256) void gy_carry_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
   const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
   if (c >= nz * nx) return;
@@ -1420,7 +1425,7 @@ __global__ __launch_bounds__(256) void gy_carry_kernel(DecodeArgs a) {
 // column; 2-D fields have one plane), scaled.
 __global__ __launch_bounds__(256) void gfinal_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint64_t nz = a.g.n[0], ny = a.g.n[1], nx = a.g.n[2];
   const uint64_t c = blockIdx.x * 256ull + threadIdx.x;
   if (c >= ny * nx) return;
@@ -1491,7 +1496,7 @@ __global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state)
   __shared__ int32_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid == 0) {
-    s_go = !(a.st->status & ERR_CORRUPT);
+    s_go = !undecodable(a.st->status);
     s_tile = atomicAdd(&a.st->ticket_construct, 1u);
   }
   __syncthreads();
@@ -1536,7 +1541,7 @@ __global__ __launch_bounds__(256) void g1d_kernel(DecodeArgs a, uint64_t* state)
 // The last pass of 2-D fields: a thread per column and eight rows (which lie in one strip).
 __global__ __launch_bounds__(256) void gfinal_rows_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint32_t ny = a.g.n[1], nx = a.g.n[2], nxb = (nx + 255) / 256;
   const uint32_t y0 = 8 * (blockIdx.x / nxb), x = 256 * (blockIdx.x % nxb) + threadIdx.x;
   if (x >= nx) return;
@@ -1554,7 +1559,7 @@ __global__ __launch_bounds__(256) void gfinal_rows_kernel(DecodeArgs a) {
 // Verbatim patches (after the last pass).
 __global__ void gpatch_kernel(DecodeArgs a) {
   chained_begin();
-  if (a.dead || (a.st->status & ERR_CORRUPT)) return;
+  if (a.dead || undecodable(a.st->status)) return;
   const uint2* rec = reinterpret_cast<const uint2*>(a.ar + a.off_rec);
   const uint64_t ny = a.g.n[1], nx = a.g.n[2];
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < a.n_rec; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -1727,7 +1732,7 @@ __global__ __launch_bounds__(kRecThreads, 6) void reconstruct_batch_kernel(const
   if (a.fuse && a.ar[a.off_codec + b] == CODEC_HUFF && block_is_full(a.g, b)) return;
   // the status is read once, by thread 0 (run expansions in other CTAs may flag
   // corruption meanwhile), so every thread takes the same path
-  if (threadIdx.x == 0) S.go = !(a.st->status & ERR_CORRUPT);
+  if (threadIdx.x == 0) S.go = !undecodable(a.st->status);
   __syncthreads();
   if (!S.go) return;
   if (a.g.ndim == 1) reconstruct_body<1, float>(a, b, S);

@@ -41,3 +41,21 @@ def test_nothing_is_encoded(probe, shape, select):
         assert bool((out == 0xa5).all())
     ar, nb, _ = api.compress(x, 1e-3, select=select, workspace=ws)
     assert torch.equal(ar[:nb], keep)
+
+
+@pytest.mark.parametrize("global_lorenzo", [False, True])
+@pytest.mark.parametrize("shape", [(9000,), (70, 200), (20, 40, 35)])
+def test_nothing_is_decoded(probe, shape, global_lorenzo):
+    """The same after an expired wait in decompression's set-up: the output stays as it was."""
+    from paper_2105_12912_gb300 import api
+    x = torch.cumsum(torch.randn(shape, generator=torch.Generator().manual_seed(4)), -1)
+    x[: shape[0] // 3] = 0.0
+    x = x.cuda()
+    ws = api.Workspace()
+    ar, nb, hdr = api.compress_with_header(x, 1e-3, radius=32, workspace=ws, global_lorenzo=global_lorenzo)
+    out = torch.full_like(x, -7.0)
+    assert probe.probe_decode(C.c_void_p(ar.data_ptr()), C.c_uint64(nb), hdr, len(shape), (C.c_uint64 * 3)(*shape),
+                              C.c_void_p(ws.buf.data_ptr()), C.c_void_p(out.data_ptr())) == 0
+    assert bool((out == -7.0).all())
+    y, st = api.decompress(ar, nb, workspace=ws)
+    assert st == 0 and float((x.double() - y.double()).abs().max()) <= api.header(ar)["eb_f"]

@@ -62,3 +62,53 @@ extern "C" int probe_encode(const float* x, int ndim, const uint64_t* dims, int 
   if (launch_encode(a, nullptr) != cudaSuccess) return 3;
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : 4;
 }
+
+// The decoding launches (csz_decompress's) of an FP32 archive whose header is hdr, with the
+// status set before them.
+extern "C" int probe_decode(const uint8_t* ar, uint64_t bytes, const uint8_t* hdr, int ndim, const uint64_t* dims,
+                            void* ws, float* out) {
+  Geom g;
+  if (!make_geom(ndim, dims, g)) return 1;
+  const Layout L = layout(g);
+  DevState* st = at<DevState>(ws, L.st);
+  const uint32_t bit = ERR_TIMEOUT;
+  if (cudaMemset(st, 0, L.hist_code - L.st) != cudaSuccess) return 2;
+  if (cudaMemset(at<void>(ws, L.lb_e), 0, 8ull * g.nblk) != cudaSuccess) return 2;
+  if (cudaMemcpy(&st->status, &bit, sizeof(bit), cudaMemcpyHostToDevice) != cudaSuccess) return 2;
+  float eb = 0.0f;
+  DecodeArgs a;
+  memset(&a, 0, sizeof(a));
+  memcpy(&eb, hdr + 48, 4);
+  memcpy(&a.radius, hdr + 52, 4);
+  memcpy(&a.flags, hdr + 60, 4);
+  memcpy(&a.n_rec, hdr + 72, 8);
+  memcpy(&a.payload, hdr + 96, 8);
+  memcpy(a.n_codec, hdr + 116, 12);
+  a.g = g;
+  a.st = st;
+  a.ar = ar;
+  a.bytes = bytes;
+  a.off_codec = kHdr;
+  a.off_bb = kHdr + a8(g.nblk);
+  a.off_rec = a.off_bb + a8(4ull * g.nblk);
+  a.off_pay = a.off_rec + 8 * a.n_rec;
+  a.off_books = a.off_pay + a8(a.payload);
+  a.ebx2_f = 2.0f * eb;
+  a.blk_off = at<uint64_t>(ws, L.blk_off);
+  a.rec_start = at<uint32_t>(ws, L.rec_start);
+  a.tabs = at<DecTab>(ws, L.tabs);
+  a.codes = at<uint16_t>(ws, L.codes);
+  a.runv = a.codes;
+  a.runl = at<uint16_t>(ws, L.runl);
+  a.runblk = at<uint32_t>(ws, L.runblk);
+  a.slowblk = at<uint32_t>(ws, L.slowblk);
+  a.prep_lb = at<uint64_t>(ws, L.prep_lb);
+  a.global = (a.flags & kFlagGlobal) != 0;
+  a.fuse = !a.global;
+  a.scan_state = at<uint64_t>(ws, L.lb_e);
+  a.gtotals = reinterpret_cast<int32_t*>(a.runl);
+  a.gstrips = a.gtotals + 512ull * g.nblk;
+  a.out = out;
+  if (launch_decode(a, nullptr) != cudaSuccess) return 3;
+  return cudaDeviceSynchronize() == cudaSuccess ? 0 : 4;
+}
