@@ -10,6 +10,7 @@
 //                                     MLP pick
 //   payload_kernel                    per block: its place among the payloads, payload;
 //                                     block 0: header, padding, books
+//                                     (plan_rle_kernel, payload_rle_kernel: RLE forced)
 // Batches run the same bodies either as one launch per stage (the *_batch kernels)
 // or as the phases of one persistent kernel (batch_persistent_kernel).
 #include "common.cuh"
@@ -329,10 +330,6 @@ __device__ void rank_merge_sort_u64(uint64_t* a, uint64_t* b, int L) {
   }
 }
 
-// One CTA per book: 0 quant codes [1024], 1 run values [1024], 2 run lengths [4096].
-// Shared memory (bytes): len 4K | sym 8K | parent by node 16K | region A 32K (sort keys,
-// live node list, canonical scratch) | region B 32K (sort scratch, new nodes, depth
-// pass): 92 KB, two such CTAs an SM.
 // =================================================================================
 // record offsets: exclusive prefix of the blocks' record counts (one CTA)
 // =================================================================================
@@ -363,9 +360,11 @@ __device__ void record_offsets_body(const BookArgs& a) {
   }
 }
 
-// Working memory of one book over nsym symbols: len nsym B | sym 2 nsym | parent by node
+// One CTA per book: 0 quant codes [1024], 1 run values [1024], 2 run lengths [4096].
+// Working memory of one over nsym symbols: len nsym B | sym 2 nsym | parent by node
 // 4 nsym | region A 8 nsym (sort keys, live node list, canonical scratch) | region B
-// 8 nsym (sort scratch, new nodes, depth pass).
+// 8 nsym (sort scratch, new nodes, depth pass): 92 KB for the run lengths, two such CTAs
+// an SM.
 __host__ __device__ constexpr uint32_t book_mem_bytes(int nsym) { return 23u * (uint32_t)nsym; }
 
 // Keys of live nodes: (weight, internal, node id), the order in which the sequential
@@ -603,10 +602,6 @@ __global__ __launch_bounds__(kBookThreads) void codebook_batch_kernel(const Book
 static size_t codebook_smem_bytes() { return book_mem_bytes(kNsymLen); }
 
 // =================================================================================
-// per-block selection and encoding
-// =================================================================================
-
-// =================================================================================
 // header, section padding and books
 // =================================================================================
 __device__ void finalize_body(const FinalizeArgs& a) {
@@ -676,6 +671,9 @@ __device__ void finalize_body(const FinalizeArgs& a) {
   }
 }
 
+// =================================================================================
+// per-block selection and encoding
+// =================================================================================
 constexpr int kEncThreads = 256;
 constexpr int kBufBytes = 16384;  // payload assembly buffer
 

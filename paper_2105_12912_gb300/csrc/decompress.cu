@@ -1704,10 +1704,10 @@ __global__ __launch_bounds__(1024) void dec_setup_batch_kernel(const DecodeArgs*
   else dec_records_body(a, role - nprep - 3, nroles - nprep - 3);
 }
 
-// entropy decoding: per field ceil(nblk / (W / 2)) CTAs of W warps (W = blockDim.x / 32,
-// chosen by the batch's tuner: 8, 16 or 32), one stream per warp; ND != 0 (the
-// batch's common dimensionality): full Huffman blocks reconstructed in the decoding
-// warps, as for single fields
+// entropy decoding: per field ceil(nblk / (rounds W / 2)) CTAs of W warps (W = blockDim.x /
+// 32, chosen by the batch's tuner: 8, 16 or 32), whose warps draw the streams of the CTA's
+// blocks one at a time; ND != 0 (the batch's common dimensionality): full Huffman blocks
+// reconstructed in the decoding warps, as for single fields
 template <int ND>
 __global__ __launch_bounds__(1024) void stream_decode_batch_kernel(const DecodeArgs* __restrict__ tasks,
                                                                    const uint32_t* __restrict__ chunk0, int nfields,

@@ -295,9 +295,9 @@ cudaError_t launch_encode_batch(const EncodeArgs* d_tasks, const uint32_t* d_til
                                 cudaStream_t s);
 
 // Batched compression as one persistent kernel: every CTA goes through the same
-// four phases in order, taking work items from one ticket per phase -- value-range
+// five phases in order, taking work items from one ticket per phase -- value-range
 // CTAs (cta0 prefix), construction tiles, the four book-phase items of each field,
-// encoding blocks -- and waits (bounded) only on the hand-over counters of
+// block plans, block payloads -- and waits (bounded) only on the hand-over counters of
 // DevState that an earlier phase releases, so the whole batch is one launch.
 struct PersistArgs {
   const RangeTask* rtasks;
@@ -331,7 +331,7 @@ struct DecodeBatchLaunch {
   int nfields;
   const uint32_t* setup0;  // nfields + 1: set-up CTAs (prep, 3 tables, records)
   uint32_t nsetup;
-  const uint32_t* chunk0;  // nfields + 1: stream-decode CTAs (kStreamWarpsPerCta / 2 blocks each)
+  const uint32_t* chunk0;  // nfields + 1: stream-decode CTAs
   uint32_t nchunks;
   const uint32_t* tile0;   // nfields + 1: codec blocks
   uint32_t ntiles;

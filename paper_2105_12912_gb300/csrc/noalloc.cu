@@ -10,9 +10,9 @@
 
 namespace {
 
-// Scratch for any archive of at most kStaticMaxBlocks codec blocks: the workspace of
-// a 64-block shape is about 1.16 MiB, and the last 256 bytes hold the call's status
-// word.  Every GPU that loads the library holds this array until the process exits.
+// Scratch for any archive of at most kStaticMaxBlocks codec blocks: the decompression
+// workspace of a 64-block shape is 1.22 MiB (26 KB less than there is), and the last 256
+// bytes hold the call's status word.  Every GPU that loads the library holds this array until the process exits.
 constexpr size_t kStaticScratchBytes = 1280 * 1024;
 constexpr size_t kStatusBytes = 256;
 constexpr size_t kStaticWorkspaceBytes = kStaticScratchBytes - kStatusBytes;
