@@ -258,31 +258,30 @@ struct Sum3 {
 // Sum of the CTA partials, scaled to the mean over rows and outputs; optionally one Adam
 // step on the weights.  Parameter kMlpParams is the loss.
 //
-// Bound by latency.  A CTA takes 32 parameters; its 32 warps add every 32nd partial each
-// (all in flight, 128 bytes a row), warp w then adds parameter w's 32 sums across its lanes
-// -- always in the same order, so runs stay reproducible -- and warp 0 finishes the 32
-// parameters.  The sums run in three floats: in doubles the FP64 pipe, 2 results a cycle and
-// SM, takes most of the launch for converting and adding (50 steps on 28,672 rows: 1186 us,
-// with the doubles spread over four times as many CTAs; 936 us so; 915 in pairs of floats,
-// which hold 48 bits).  Doubles are left for the last combination and the one scale, and for
-// sums that are not finite or overflow a float, which start again in them.  c1, c2: Adam's
-// bias corrections of this step.
-constexpr int kUpdThreads = 1024, kUpdParams = 32, kMaxParts = 512;
+// Bound by latency, then by issue: the CTAs start as the gradient launch ends, many of them on
+// the first SMs that become free.  So a CTA takes 8 parameters: a warp reads 8 of four partials
+// at a time (32 bytes each, all in flight) and adds every 32nd, and the sums meet by shuffles
+// and through shared memory, always in the same order, so runs stay reproducible.  The sums run
+// in three floats: in doubles the FP64 pipe, 2 results a cycle and SM, takes most of the launch
+// for converting and adding (50 steps on 28,672 rows: 1186 us in doubles where pairs of floats,
+// which hold 48 bits, take 915; in turn with pairs, 849 and 855 us so, and 915 and 936 with 32
+// parameters a CTA).  Doubles are left for the last combination and the one scale, and for sums
+// that are not finite or overflow a float, which start again in them.  c1, c2: Adam's bias
+// corrections of this step.
+constexpr int kUpdThreads = 256, kUpdWarps = kUpdThreads / 32, kUpdParams = 8, kMaxParts = 512;
 __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* part, int nparts, float* w,
                                                                  float* grad_out, double* loss_out, float* m,
                                                                  float* v, uint32_t step, float lr, float c1, float c2) {
   chained_begin();
-  __shared__ Sum3 s_sum[32][kUpdParams + 1];
-  __shared__ Sum3 s_tot[kUpdParams];
-  __shared__ unsigned long long s_c[32];
+  __shared__ Sum3 s_sum[kUpdWarps][kUpdParams];
+  __shared__ unsigned long long s_c[kUpdWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int p0 = blockIdx.x * kUpdParams;
+  const int p = blockIdx.x * kUpdParams + (lane & 7);
+  Sum3 acc{0.0f, 0.0f, 0.0f};
   {
-    Sum3 acc{0.0f, 0.0f, 0.0f};
-    const int p = min(p0 + lane, kMlpParams);
+    const int q = min(p, kMlpParams);
 #pragma unroll 5
-    for (int g = wid; g < nparts; g += 32) acc.add(part[(uint64_t)g * kPart + p]);
-    s_sum[wid][lane] = acc;
+    for (int g = 4 * wid + (lane >> 3); g < nparts; g += 4 * kUpdWarps) acc.add(part[(uint64_t)g * kPart + q]);
   }
   // row counts: whole numbers
   unsigned long long cnt = 0;
@@ -290,21 +289,21 @@ __global__ __launch_bounds__(kUpdThreads) void mlp_update_kernel(const float* pa
     cnt += (unsigned long long)part[(uint64_t)g * kPart + kMlpParams + 1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
+  acc.add(acc.shfl_xor(8));
+  acc.add(acc.shfl_xor(16));
+  if (lane < kUpdParams) s_sum[wid][lane] = acc;
   if (lane == 0) s_c[wid] = cnt;
   __syncthreads();
-  Sum3 acc = s_sum[lane][wid];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc.add(acc.shfl_xor(o));
-  if (lane == 0) s_tot[wid] = acc;
-  __syncthreads();
   if (wid) return;
-  cnt = s_c[lane];
+  acc = s_sum[lane >> 3][lane & 7];
+  acc.add(s_sum[4 + (lane >> 3)][lane & 7]);
+  acc.add(acc.shfl_xor(8));
+  acc.add(acc.shfl_xor(16));
+  cnt = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(~0u, cnt, o);
-  const int p = p0 + lane;
-  if (p > kMlpParams) return;
-  const Sum3 tot = s_tot[lane];
-  double sum = (double)tot.h + ((double)tot.m + (double)tot.l);
+  for (int k = 0; k < kUpdWarps; k++) cnt += s_c[k];
+  if (lane >= kUpdParams || p > kMlpParams) return;
+  double sum = (double)acc.h + ((double)acc.m + (double)acc.l);
   if (!isfinite(sum)) {
     sum = 0.0;
     for (int g = 0; g < nparts; g++) sum += (double)part[(uint64_t)g * kPart + p];
